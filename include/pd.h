@@ -44,7 +44,7 @@ typedef enum {
     PD_EINVAL = 1,      /* invalid argument (sizes, ranges, null pointers) */
     PD_ENOMEM = 2,      /* device or host allocation failed */
     PD_ECUDA = 3,       /* a CUDA runtime call or kernel launch failed */
-    PD_ETIMEOUT = 4,    /* a bounded device wait gave up (status word set) */
+    PD_ETIMEOUT = 4,    /* a bounded device wait gave up (pd_state_report) */
     PD_ENOTCONV = 5,    /* power iteration did not reach its tolerance */
     PD_ENOTSUP = 6      /* valid but unsupported configuration */
 } pd_status;
@@ -343,7 +343,9 @@ pd_status pd_synthesis_iterate(pd_plan* plan, pd_state* st, const pd_params* par
  * rank's active blocks, gridding of their dual change into the state's U, the sparsity
  * dual update). The caller then sums U over the ranks (pd_state_u gives the device
  * pointer of the state's U, complex [Kx/4][Ky][4] column panels, Kx*Ky elements; the
- * sum must go to another buffer, since U keeps this rank's own part).
+ * sum must go to another buffer, since U keeps this rank's own part). U stands for G^T v up
+ * to the symmetry of a real image: most visibilities with u < 0 are gridded as their
+ * conjugates at -(u, v), which leaves Re(Z^T F^H U) as it is; pd_iterate_primal takes either.
  * pd_iterate_primal: steps 17-18 with the summed U (device, same layout; NULL = the
  * state's own U). adaptive must be 0 (the residual norms would differ between ranks).
  * Both asynchronous on `stream`; pd_iterate_dual + pd_iterate_primal(NULL) equals one
@@ -385,7 +387,9 @@ pd_status pd_state_report(const pd_plan* plan, const pd_state* st, int64_t* t, d
 /*
  * Checkpoint: the full state as one host byte buffer. pd_state_save writes
  * pd_state_bytes() bytes to host `buf`; pd_state_load restores it (same plan).
- * The counter-based draws make a resumed run identical to an uninterrupted one.
+ * The counter-based draws make a resumed run identical to an uninterrupted one. v and y are
+ * stored by the base cells of the points in tiles of `tile` (0: 32) cells, independently of the
+ * plan's internal order; the first save or load of a plan sorts the points once on the host.
  */
 size_t pd_state_bytes(const pd_plan* plan);
 pd_status pd_state_save(const pd_plan* plan, const pd_state* st, void* buf, void* stream);

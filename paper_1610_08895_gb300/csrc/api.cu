@@ -160,45 +160,83 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     p->csr_cplx = dde > 0;
     g.J = Jfoot;   // tiles, windows and halos follow the footprint; weights use kb_J
     g.beta = d->kb_beta > 0 ? d->kb_beta : kb_beta_default(p->kb_J);
-    // default tile: 32 cells (the densest tiles bound the gridding critical path); at least
-    // two tiles per grid side, for the colour classes of the gridding
-    int T = d->tile ? d->tile : 32;
-    while (T > std::min(g.Kx, g.Ky) / 2) T >>= 1;
-    while (T < g.J) T <<= 1;
+    // default tile: 16 cells, so that small grids still make enough work items and dense ones
+    // no long ones; 32 for FP32 grids of 2048^2 cells and more, whose items fill the GPU anyway
+    // and then spend less on windows. At least two tiles per grid side, for the tile colours.
+    const bool fly32 = d->precision == PD_F32 && d->g_mode == PD_G_ON_THE_FLY && d->kernel_width <= 8;
+    int T = d->tile ? d->tile : (fly32 && (int64_t)g.Kx * g.Ky >= (int64_t)2048 * 2048 ? 32 : 16);
+    auto fit = [&](int t) {
+        while (t > std::min(g.Kx, g.Ky) / 2) t >>= 1;
+        while (t < g.J) t <<= 1;
+        return t;
+    };
+    T = fit(T);
+    p->ck_tile = fit(d->tile ? d->tile : 32);
     if (T > std::min(g.Kx, g.Ky) / 2) return fail(PD_ENOTSUP, "grid side below twice the kernel width");
     g.tile = T; g.logT = ilog2(T);
     g.ntx = g.Kx / T; g.nty = g.Ky / T; g.ntiles = g.ntx * g.nty;
-    g.ext = T + g.J - 1; g.halo_lo = g.J / 2 - 1; g.halo_hi = g.J / 2;
+    g.ext = T + g.J - 1;
+    const int halo_lo = g.J / 2 - 1;   // footprint cells before the base cell floor(g)
     p->M = d->nvis; p->d = d->nblocks; p->b = d->nbases; p->L = d->levels;
     p->basis_ids.assign(d->basis_ids, d->basis_ids + d->nbases);
     p->n_wavelet = 0;
     for (int id : p->basis_ids) p->n_wavelet += id > 0;
     CU(cudaGetDevice(&p->device));
     CU(cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device));
+    CU(cudaDeviceGetAttribute(&p->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
 
-    // ---- visibilities: base cell, fraction, (tile, block) order
+    // ---- visibilities: first footprint cell, fraction, (tile, block) order
     const int64_t M = p->M;
     std::vector<int32_t> bx(M), by(M);
     std::vector<double> frx(M), fry(M);
+    std::vector<unsigned char> flip(M, 0);
+    // integer part and fraction; a fraction that rounds to 1 in the working precision moves to
+    // the next cell
+    auto split = [&](double x, double& fl, double& fr) {
+        fl = std::floor(x);
+        fr = x - fl;
+        if (p->prec == PD_F32 && (float)fr >= 1.0f) { fl += 1.0; fr = 0.0; }
+    };
+    auto base_cell = [&](double x, double y) {
+        double flx, fly, fr;
+        split(x, flx, fr);
+        split(y, fly, fr);
+        return (int32_t)(((((int64_t)fly % g.Ky) + g.Ky) % g.Ky) << 16 | ((((int64_t)flx % g.Kx) + g.Kx) % g.Kx));
+    };
+    // neither fraction x nor its mirror image 1 - x rounds to a grid line
+    auto inside = [&](double x) {
+        const double fr = x - std::floor(x);
+        return p->prec == PD_F32 ? (float)fr > 0.0f && (float)fr < 1.0f && (float)(1.0 - fr) < 1.0f
+                                 : fr > 0.0 && fr < 1.0 && 1.0 - fr < 1.0;
+    };
+    p->h_base.resize(M);
     for (int64_t m = 0; m < M; ++m) {
         const double u = d->uv[2 * m], v = d->uv[2 * m + 1];
         if (!(u >= -M_PI && u < M_PI && v >= -M_PI && v < M_PI))
             return fail(PD_EINVAL, "uv points must lie in [-pi, pi)^2");
         const int blk = d->block_of_vis[m];
         if (blk < 0 || blk >= p->d) return fail(PD_EINVAL, "block_of_vis out of range");
-        const double gxv = u * g.Kx / (2.0 * M_PI), gyv = v * g.Ky / (2.0 * M_PI);
-        double flx = std::floor(gxv), fly = std::floor(gyv);
-        double fx = gxv - flx, fy = gyv - fly;
-        // a fraction that rounds to 1 in the working precision moves to the next cell
-        if (p->prec == PD_F32) {
-            if ((float)fx >= 1.0f) { flx += 1.0; fx = 0.0; }
-            if ((float)fy >= 1.0f) { fly += 1.0; fy = 0.0; }
+        double gxv = u * g.Kx / (2.0 * M_PI), gyv = v * g.Ky / (2.0 * M_PI);
+        p->h_base[m] = base_cell(gxv, gyv);
+        // Held at -(u, v) as its conjugate. A point on a grid line (to the working precision)
+        // stays where it is: its taps reach J/2 cells to one side only, and the mirrored ones
+        // would to the other.
+        if (!dde && u < 0 && inside(gxv) && inside(gyv)) {
+            gxv = -gxv;
+            gyv = -gyv;
+            flip[m] = 1;
         }
-        bx[m] = (int32_t)((((int64_t)flx % g.Kx) + g.Kx) % g.Kx);
-        by[m] = (int32_t)((((int64_t)fly % g.Ky) + g.Ky) % g.Ky);
+        double flx, fly, fx, fy;
+        split(gxv, flx, fx);
+        split(gyv, fly, fy);
+        // the footprint's first cell, halo_lo cells before the base cell
+        bx[m] = (int32_t)((((int64_t)flx - halo_lo) % g.Kx + g.Kx) % g.Kx);
+        by[m] = (int32_t)((((int64_t)fly - halo_lo) % g.Ky + g.Ky) % g.Ky);
         frx[m] = fx;
         fry[m] = fy;
     }
+    // a fifth of an SM's share of the points (five CTAs per SM), at least four rounds of a CTA
+    const int degrid_part = (int)std::max<int64_t>(1024, M / ((int64_t)p->num_sms * 5));
     const int64_t nbucket = (int64_t)g.ntiles * p->d;
     std::vector<int32_t> order(M);
     {
@@ -243,7 +281,7 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
             p->max_tile_segs = std::max(p->max_tile_segs, tile_seg_start[t + 1] - tile_seg_start[t]);
         if (p->max_tile_segs > 1024)
             return fail(PD_ENOTSUP, "more than 1024 blocks share one gridding tile; use a smaller tile");
-        // within each segment: by 8 x 8 super-cell, then row-major by base cell (stable: ties
+        // within each segment: by 8 x 8 super-cell, then row-major by cell (stable: ties
         // keep user order), so that the points of one super-cell row are consecutive
         p->nsc_side = std::max(1, g.tile / SC);
         auto scell_of = [&](int32_t m) {
@@ -268,14 +306,6 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
             }
         }
         p->h_sc_start = std::move(sc_start);
-        // segments of each block (tile order) for the fixed-order block reductions
-        std::vector<int32_t> bss(p->d + 1, 0), bsl(p->nseg);
-        for (int64_t sg = 0; sg < p->nseg; ++sg) bss[seg_block[sg] + 1]++;
-        for (int i = 0; i < p->d; ++i) bss[i + 1] += bss[i];
-        {
-            std::vector<int32_t> fill(bss.begin(), bss.end() - 1);
-            for (int64_t sg = 0; sg < p->nseg; ++sg) bsl[fill[seg_block[sg]]++] = (int32_t)sg;
-        }
         // tiles by decreasing visibility count (heaviest scheduled first)
         std::vector<int32_t> tord(g.ntiles);
         std::iota(tord.begin(), tord.end(), 0);
@@ -285,8 +315,33 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         for (int t = 0; t < g.ntiles; ++t) p->ntiles_nonempty += tcount(t) > 0;
         p->h_tile_seg_start = tile_seg_start;
         p->h_seg_block = seg_block;
-        p->h_block_seg_start = bss;
-        p->h_block_seg_list = bsl;
+        // degridding items: a tile's points in parts of about degrid_part (parts of a heavy tile go
+        // to several CTAs), heaviest tile first; the slots of seg_part and the blocks' lists of them
+        std::vector<int32_t> bss(p->d + 1, 0), bsl;
+        std::vector<SegSlot> slots;
+        {
+            std::vector<std::vector<int32_t>> of(p->d);
+            for (int k = 0; k < p->ntiles_nonempty; ++k) {
+                const int t = tord[k], s0 = tile_seg_start[t], ns = tile_seg_start[t + 1] - s0;
+                const int n = tcount(t), q0 = seg_start[s0], parts = std::max(1, (n + degrid_part - 1) / degrid_part);
+                for (int q = 0; q < parts; ++q) {
+                    p->h_ditems.push_back(TileItem{t, q, parts, (int32_t)slots.size(), s0, ns, 0, 0});
+                    // the part's share when every block is active
+                    const int lo = q0 + (int)((int64_t)n * q / parts), hi = q0 + (int)((int64_t)n * (q + 1) / parts);
+                    for (int sg = s0; sg < s0 + ns; ++sg) {
+                        of[seg_block[sg]].push_back((int32_t)slots.size());
+                        const int a = std::max(lo, seg_start[sg]), b2 = std::min(hi, seg_start[sg + 1]);
+                        slots.push_back(SegSlot{a, std::max(a, b2)});
+                    }
+                }
+            }
+            for (int i = 0; i < p->d; ++i) {
+                bsl.insert(bsl.end(), of[i].begin(), of[i].end());
+                bss[i + 1] = (int32_t)bsl.size();
+            }
+            p->nslot = (int64_t)slots.size();
+            p->n_ditems = (int)p->h_ditems.size();
+        }
 
         auto& A = p->allocs;
         size_t& B = p->device_bytes;
@@ -294,8 +349,12 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         ALLOC(p->seg_start, seg_start.size());
         ALLOC(p->seg_block, seg_block.size());
         ALLOC(p->tile_seg_start, tile_seg_start.size());
-        ALLOC(p->block_seg_start, bss.size());
-        ALLOC(p->block_seg_list, bsl.size());
+        ALLOC(p->block_slot_start, bss.size());
+        ALLOC(p->block_slot_list, bsl.size());
+        ALLOC(p->ditems, p->h_ditems.size());
+        ALLOC(p->slot_range, slots.size());
+        CU(upload(p->ditems, p->h_ditems));
+        CU(upload(p->slot_range, slots));
         ALLOC(p->tile_order, tord.size());
         ALLOC(p->seg_sc_start, p->h_sc_start.size());
         CU(upload(p->seg_sc_start, p->h_sc_start));
@@ -304,21 +363,46 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         {
             // tiles of each colour in heaviest-first order
             const int q = g.ntiles / 4;
-            std::vector<int32_t> col((size_t)g.ntiles), fill(4, 0), cc(4, q);
+            std::vector<int32_t> col((size_t)g.ntiles), fill(4, 0), cc(4, 0);
             for (int k = 0; k < g.ntiles; ++k) {
                 const int c = tile_colour(tord[k], g.ntx);
                 col[(size_t)c * q + fill[c]++] = tord[k];
+                cc[c] += k < p->ntiles_nonempty;
             }
             ALLOC(p->colour_tiles, col.size());
             ALLOC(p->colour_counts, 4);
             CU(upload(p->colour_tiles, col));
             CU(upload(p->colour_counts, cc));
         }
+        // the FP32 gridding's work items
+        grid_setup(p);
+        {
+            std::vector<int4> info(g.ntiles);
+            std::vector<int2> items;
+            for (int k = 0, c = 0; c < 4; ++c)     // colour by colour, heaviest tile first
+                for (int t : tord) {
+                    if (tile_colour(t, g.ntx) != c) continue;
+                    const int parts = p->grid_part ? std::max(1, (tcount(t) + p->grid_part - 1) / p->grid_part) : 1;
+                    info[t] = make_int4(tile_seg_start[t], tile_seg_start[t + 1] - tile_seg_start[t], parts, k++);
+                    if (tcount(t) > 0)
+                        for (int q = 0; q < parts; ++q) items.push_back(make_int2(t, q));
+                }
+            p->n_items = (int)items.size();
+            const std::vector<int32_t> ni(1, p->n_items);
+            ALLOC(p->tile_info, info.size());
+            ALLOC(p->items, items.size());
+            ALLOC(p->nitems, 1);
+            ALLOC(p->pend, g.ntiles);
+            CU(upload(p->tile_info, info));
+            CU(upload(p->items, items));
+            CU(upload(p->nitems, ni));
+            CU(cudaMemset(p->pend, 0, g.ntiles * sizeof(int32_t)));
+        }
         CU(upload(p->seg_start, seg_start));
         CU(upload(p->seg_block, seg_block));
         CU(upload(p->tile_seg_start, tile_seg_start));
-        CU(upload(p->block_seg_start, bss));
-        CU(upload(p->block_seg_list, bsl));
+        CU(upload(p->block_slot_start, bss));
+        CU(upload(p->block_slot_list, bsl));
         CU(upload(p->tile_order, tord));
     }
     auto& A = p->allocs;
@@ -344,14 +428,16 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         CU(dalloc_bytes(A, B, &p->fx, M * p->rsz));
         CU(dalloc_bytes(A, B, &p->fy, M * p->rsz));
         CU(upload(p->cell, cell));
+        for (int64_t i = 0; i < M; ++i)
+            if (flip[order[i]]) order[i] = (int32_t)((uint32_t)order[i] | 0x80000000u);
         CU(upload(p->perm, order));
         CU(upload_real(p->fx, fxs, p->prec));
         CU(upload_real(p->fy, fys, p->prec));
     }
     {
-        std::vector<int32_t> counts = {(int32_t)p->nseg, g.ntiles};
+        std::vector<int32_t> counts = {(int32_t)p->nseg, p->ntiles_nonempty, p->n_ditems};
         std::vector<int32_t> ob(p->d, 1), obs(p->b, 1);
-        ALLOC(p->counts_all, 2);
+        ALLOC(p->counts_all, 3);
         ALLOC(p->ones_block, ob.size());
         ALLOC(p->ones_basis, obs.size());
         CU(upload(p->counts_all, counts));
@@ -364,14 +450,24 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         CU(dalloc_bytes(A, B, &p->cy, g.ny * p->rsz));
         CU(dalloc_bytes(A, B, &p->twx, g.Kx * p->csz));
         CU(dalloc_bytes(A, B, &p->twy, g.Ky * p->csz));
-        CU(upload_real(p->cx, deapodisation(g.nx, g.Kx, p->kb_J, g.beta), p->prec));
-        CU(upload_real(p->cy, deapodisation(g.ny, g.Ky, p->kb_J, g.beta), p->prec));
+        CU(dalloc_bytes(A, B, &p->cxl, g.nx * p->rsz));
+        CU(dalloc_bytes(A, B, &p->cyl, g.ny * p->rsz));
+        auto put = [&](void* hi, void* lo, std::vector<double> c) {
+            cudaError_t e = upload_real(hi, c, p->prec);
+            for (double& x : c) x -= p->prec == PD_F32 ? (double)(float)x : x;
+            return e ? e : upload_real(lo, c, p->prec);
+        };
+        CU(put(p->cx, p->cxl, deapodisation(g.nx, g.Kx, p->kb_J, g.beta)));
+        CU(put(p->cy, p->cyl, deapodisation(g.ny, g.Ky, p->kb_J, g.beta)));
         CU(upload_real(p->twx, twiddles(g.Kx), p->prec));
         CU(upload_real(p->twy, twiddles(g.Ky), p->prec));
         {
             std::vector<double> kp = kb_tap_polynomials(p->kb_J, g.beta, KB_DEG);
             for (int a = 0; a < p->kb_J; ++a)
+            {
                 for (int k = 0; k <= KB_DEG; ++k) p->kbpoly.c[a][k] = (float)kp[(size_t)a * (KB_DEG + 1) + k];
+                p->kbpoly.lo[a] = (float)(kp[(size_t)a * (KB_DEG + 1)] - (double)p->kbpoly.c[a][0]);
+            }
         }
         p->h_filt.assign((size_t)p->b * MAX_FILTER, 0.0);
         p->h_filt_len.assign(p->b, 0);
@@ -398,7 +494,7 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         CU(cudaMemset(p->gridb, 0, half_cols * g.Ky * p->csz));
         CU(dalloc_bytes(A, B, &p->gridu, K * p->csz));
         CU(dalloc_bytes(A, B, &p->rbuf, (size_t)M * p->csz));
-        ALLOC(p->seg_part, 2 * std::max<int64_t>(p->nseg, 1));
+        ALLOC(p->seg_part, 2 * std::max<int64_t>(p->nslot, 1));
         ALLOC(p->blk_norm, 2 * p->d);
         CU(dalloc_bytes(A, B, &p->blk_scale, p->d * p->rsz));
         const size_t llsz = (size_t)p->b * (g.ny / 2) * (g.nx / 2) * p->rsz;
@@ -408,7 +504,8 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         CU(dalloc_bytes(A, B, &p->synpart, (size_t)p->b * N * p->rsz));
         p->red_len = 1024;
         ALLOC(p->red, p->red_len + 8);
-        ALLOC(p->sched, 8);
+        ALLOC(p->sched, 16);
+        CU(cudaMemset(p->sched, 0, 16 * sizeof(int32_t)));
         CU(cudaMemset(p->ds, 0, (size_t)p->b * N * p->rsz));
     }
     if (p->g_mode == PD_G_CSR) {
@@ -443,39 +540,42 @@ extern "C" pd_status pd_plan_info(const pd_plan* p, int32_t* ky, int32_t* kx, do
 // Scratch of a batch of operator applications (one launch per pass for the whole batch):
 // the plan's own buffers for one image, otherwise buffers kept by the plan and grown to
 // the largest batch seen (the device is synchronised before the old ones are freed).
-static pd_status ensure_batch(pd_plan* p, int batch, void** t1, void** gb, void** gu) {
+static pd_status ensure_batch(pd_plan* p, int batch, void** t1, void** gb, void** gu, int32_t** pend) {
     if (batch == 1) {
-        *t1 = p->t1; *gb = p->gridb; *gu = p->gridu;
+        *t1 = p->t1; *gb = p->gridb; *gu = p->gridu; *pend = p->pend;
         return PD_OK;
     }
     if (batch > p->batch_cap) {
         CU(cudaDeviceSynchronize());
-        for (void* q : {p->bt1, p->bgb, p->bgu})
+        for (void* q : {p->bt1, p->bgb, p->bgu, (void*)p->bpend})
             if (q) {
                 cudaFree(q);
                 p->allocs.erase(std::remove(p->allocs.begin(), p->allocs.end(), q), p->allocs.end());
             }
         p->bt1 = p->bgb = p->bgu = nullptr;
+        p->bpend = nullptr;
         p->batch_cap = 0;
         const size_t half = (size_t)(p->g.nx / 4 + 1) * 4;
         size_t dummy = 0;
         if (dalloc_bytes(p->allocs, dummy, &p->bt1, batch * half * p->g.ny * p->csz) ||
             dalloc_bytes(p->allocs, dummy, &p->bgb, batch * half * p->g.Ky * p->csz) ||
-            dalloc_bytes(p->allocs, dummy, &p->bgu, (size_t)batch * p->g.Kx * p->g.Ky * p->csz))
+            dalloc_bytes(p->allocs, dummy, &p->bgu, (size_t)batch * p->g.Kx * p->g.Ky * p->csz) ||
+            dalloc(p->allocs, dummy, &p->bpend, (size_t)batch * p->g.ntiles))
             return fail(PD_ENOMEM, "batch scratch allocation failed");
         // the unused slots of the last column panel of the half grids stay zero
         CU(cudaMemset(p->bt1, 0, batch * half * p->g.ny * p->csz));
         CU(cudaMemset(p->bgb, 0, batch * half * p->g.Ky * p->csz));
         p->batch_cap = batch;
     }
-    *t1 = p->bt1; *gb = p->bgb; *gu = p->bgu;
+    *t1 = p->bt1; *gb = p->bgb; *gu = p->bgu; *pend = p->bpend;
     return PD_OK;
 }
 
 template <typename R>
 static pd_status apply_phi_t(pd_plan* p, const void* x, void* y, int batch, cudaStream_t s) {
     void *t1, *gb, *gu;
-    pd_status st = ensure_batch(p, batch, &t1, &gb, &gu);
+    int32_t* pend;
+    pd_status st = ensure_batch(p, batch, &t1, &gb, &gu, &pend);
     if (st != PD_OK) return st;
     CU(fwd_fft<R>(p, (const R*)x, (cplx_t<R>*)gb, s, batch, (cplx_t<R>*)t1));
     CU(degrid_plain<R>(p, (const cplx_t<R>*)gb, (cplx_t<R>*)y, s, batch));
@@ -484,9 +584,10 @@ static pd_status apply_phi_t(pd_plan* p, const void* x, void* y, int batch, cuda
 template <typename R>
 static pd_status apply_phi_adj_t(pd_plan* p, const void* y, void* x, int batch, cudaStream_t s) {
     void *t1, *gb, *gu;
-    pd_status st = ensure_batch(p, batch, &t1, &gb, &gu);
+    int32_t* pend;
+    pd_status st = ensure_batch(p, batch, &t1, &gb, &gu, &pend);
     if (st != PD_OK) return st;
-    CU(grid_plain<R>(p, (const cplx_t<R>*)y, (cplx_t<R>*)gu, s, batch));
+    CU(grid_plain<R>(p, (const cplx_t<R>*)y, (cplx_t<R>*)gu, s, batch, pend));
     CU(inv_fft<R>(p, (const cplx_t<R>*)gu, (R*)x, nullptr, s, batch, (cplx_t<R>*)t1));
     return PD_OK;
 }
@@ -633,8 +734,7 @@ extern "C" pd_status pd_state_create(pd_plan* p, pd_state** out) {
               !dalloc(A, B, &st->res_norm, p->d) && !dalloc(A, B, &st->p_block, p->d) &&
               !dalloc(A, B, &st->p_basis, p->b) && !dalloc(A, B, &st->block_active, p->d) &&
               !dalloc(A, B, &st->basis_active, p->b) &&
-              !dalloc(A, B, &st->act_tiles, p->g.ntiles) && !dalloc(A, B, &st->tile_active, p->g.ntiles) &&
-              !dalloc(A, B, &st->act_col, p->g.ntiles) && !dalloc(A, B, &st->counts, 6) && !dalloc(A, B, &st->t, 1) && !dalloc(A, B, &st->diag, 2) &&
+              !dalloc(A, B, &st->tile_active, p->g.ntiles) && !dalloc(A, B, &st->counts, 2) && !dalloc(A, B, &st->t, 1) && !dalloc(A, B, &st->diag, 2) &&
               !dalloc(A, B, &st->prim_part, 2 * (size_t)inv_rows_ctas(p)) && !dalloc(A, B, &st->status, 1);
     if (!ok) {
         pd_state_destroy(st);
@@ -757,12 +857,13 @@ static cudaError_t enqueue_dual(pd_plan* p, pd_state* st, const pd_params* prm, 
         return e;
     if (concurrent && (e = cudaEventRecord(st->ev_join, ps))) return e;
     if ((e = fwd_fft<R>(p, (const R*)st->xt, (cplx_t<R>*)p->gridb, s))) return e;
-    DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm};
-    if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, st->act_tiles, st->counts, s))) return e;
+    DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm, st->tile_active,
+                p->ditems, p->counts_all + 2, p->items, p->nitems};
+    if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, s))) return e;
     {
         const int q = p->g.ntiles / 4;
-        const int32_t* lists[4] = {st->act_col, st->act_col + q, st->act_col + 2 * q, st->act_col + 3 * q};
-        if ((e = grid_dual<R>(p, da, lists, st->counts + 2, (cplx_t<R>*)st->u, s))) return e;
+        const int32_t* lists[4] = {p->colour_tiles, p->colour_tiles + q, p->colour_tiles + 2 * q, p->colour_tiles + 3 * q};
+        if ((e = grid_dual<R>(p, da, lists, p->colour_counts, (cplx_t<R>*)st->u, s))) return e;
     }
     return cudaSuccess;
 }
@@ -804,18 +905,21 @@ static cudaError_t ensure_per_block(pd_plan* p, pd_state* st) {
     for (int j = 0; j < b; ++j) eyeb[(size_t)j * b + j] = 1;
     // each block's tiles, all of them (degridding) and by colour (gridding)
     std::vector<std::vector<int32_t>> tl(d), tc((size_t)4 * d);
+    std::vector<std::vector<TileItem>> td(nt);
+    for (const TileItem& ti : p->h_ditems) td[ti.tile].push_back(ti);
     for (int t = 0; t < nt; ++t)
         for (int sg = p->h_tile_seg_start[t]; sg < p->h_tile_seg_start[t + 1]; ++sg) {
             const int blk = p->h_seg_block[sg];
             tl[blk].push_back(t);
             tc[(size_t)4 * blk + tile_colour(t, p->g.ntx)].push_back(t);
         }
-    std::vector<int32_t> tiles, counts((size_t)2 * d, 0), col, ccounts((size_t)4 * d, 0);
+    std::vector<TileItem> tiles;
+    std::vector<int32_t> counts(d, 0), col, ccounts((size_t)4 * d, 0);
     st->h_pb_off.assign((size_t)5 * d + 1, 0);   // [d + 1] all-tile offsets, then [4 d] colour offsets
     for (int i = 0; i < d; ++i) {
         st->h_pb_off[i] = (int32_t)tiles.size();
-        tiles.insert(tiles.end(), tl[i].begin(), tl[i].end());
-        counts[2 * i + 1] = (int32_t)tl[i].size();
+        for (int32_t t : tl[i]) tiles.insert(tiles.end(), td[t].begin(), td[t].end());
+        counts[i] = (int32_t)tiles.size() - st->h_pb_off[i];
         for (int c = 0; c < 4; ++c) {
             st->h_pb_off[d + 1 + 4 * i + c] = (int32_t)col.size();
             col.insert(col.end(), tc[(size_t)4 * i + c].begin(), tc[(size_t)4 * i + c].end());
@@ -823,17 +927,37 @@ static cudaError_t ensure_per_block(pd_plan* p, pd_state* st) {
         }
     }
     st->h_pb_off[d] = (int32_t)tiles.size();
+    // k_grid_mma's items of each block: its tiles heaviest first, as in the plan's list
+    std::vector<int2> items;
+    std::vector<int32_t> nitems(d, 0);
+    st->h_pb_item_off.assign(d, 0);
+    if (p->grid_smem) {
+        std::vector<int4> info(nt);
+        cudaError_t e0 = cudaMemcpy(info.data(), p->tile_info, nt * sizeof(int4), cudaMemcpyDeviceToHost);
+        if (e0) return e0;
+        for (int i = 0; i < d; ++i) {
+            st->h_pb_item_off[i] = (int32_t)items.size();
+            std::vector<int32_t> o = tl[i];
+            std::sort(o.begin(), o.end(), [&](int32_t a, int32_t c) { return info[a].w < info[c].w; });
+            for (int32_t t : o)
+                for (int q = 0; q < info[t].z; ++q) items.push_back(make_int2(t, q));
+            nitems[i] = (int32_t)items.size() - st->h_pb_item_off[i];
+        }
+    }
     cudaError_t e;
     auto& A = st->allocs;
     size_t& B = st->device_bytes;
+    if ((e = dalloc(A, B, &st->pb_items, std::max<size_t>(items.size(), 1))) || (e = dalloc(A, B, &st->pb_nitems, d)) ||
+        (e = upload(st->pb_items, items)) || (e = upload(st->pb_nitems, nitems)))
+        return e;
     if ((e = dalloc(A, B, &st->pb_eye_blocks, eyed.size())) || (e = dalloc(A, B, &st->pb_eye_bases, eyeb.size())) ||
-        (e = dalloc(A, B, &st->pb_tiles, std::max<size_t>(tiles.size(), 1))) ||
+        (e = dalloc(A, B, &st->pb_ditems, std::max<size_t>(tiles.size(), 1))) ||
         (e = dalloc(A, B, &st->pb_counts, counts.size())) ||
         (e = dalloc(A, B, &st->pb_col, std::max<size_t>(col.size(), 1))) ||
         (e = dalloc(A, B, &st->pb_ccounts, ccounts.size())))
         return e;
     if ((e = upload(st->pb_eye_blocks, eyed)) || (e = upload(st->pb_eye_bases, eyeb)) ||
-        (e = upload(st->pb_tiles, tiles)) || (e = upload(st->pb_counts, counts)) || (e = upload(st->pb_col, col)) ||
+        (e = upload(st->pb_ditems, tiles)) || (e = upload(st->pb_counts, counts)) || (e = upload(st->pb_col, col)) ||
         (e = upload(st->pb_ccounts, ccounts)))
         return e;
     st->h_act.assign(d, 0);
@@ -858,15 +982,20 @@ static cudaError_t enqueue_iteration_per_block(pd_plan* p, pd_state* st, const p
     for (int i = 0; i < d; ++i) {
         if (!st->h_act[i]) continue;
         DualArgs da{st->y, st->v, st->pb_eye_blocks + (size_t)i * d, st->eps, st->res_norm};
-        if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, st->pb_tiles + st->h_pb_off[i],
-                                st->pb_counts + 2 * i, s)))
-            return e;
+        da.ditems = st->pb_ditems + st->h_pb_off[i];
+        da.nditems = st->pb_counts + i;
+        if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, s))) return e;
     }
     for (int i = 0; i < d; ++i) {
         if (!st->h_act[i]) continue;
         DualArgs da{st->y, st->v, st->pb_eye_blocks + (size_t)i * d, st->eps, st->res_norm};
         const int32_t* lists[4];
         for (int c = 0; c < 4; ++c) lists[c] = st->pb_col + st->h_pb_off[d + 1 + 4 * i + c];
+        if (p->grid_smem) {
+            if ((e = grid_begin(p, da.block_active, p->pend, nullptr, 0, 1, s))) return e;
+            da.items = st->pb_items + st->h_pb_item_off[i];
+            da.nitems = st->pb_nitems + i;
+        }
         if ((e = grid_dual<R>(p, da, lists, st->pb_ccounts + 4 * i, (cplx_t<R>*)st->u, s))) return e;
     }
     for (int j = 0; j < b; ++j) {
@@ -949,12 +1078,13 @@ static cudaError_t enqueue_synthesis(pd_plan* p, pd_state* st, const pd_params* 
     if ((e = select_active(p, st, sa, s))) return e;                                      // step 3
     if ((e = psi_plain<R>(p, (const R*)st->syn_at, (R*)st->xt, s))) return e;            // x~ = Psi alpha~
     if ((e = fwd_fft<R>(p, (const R*)st->xt, (cplx_t<R>*)p->gridb, s))) return e;        // b~ = F Z x~
-    DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm};
-    if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, st->act_tiles, st->counts, s))) return e;
+    DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm, st->tile_active,
+                p->ditems, p->counts_all + 2, p->items, p->nitems};
+    if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, s))) return e;
     {
         const int q = p->g.ntiles / 4;
-        const int32_t* lists[4] = {st->act_col, st->act_col + q, st->act_col + 2 * q, st->act_col + 3 * q};
-        if ((e = grid_dual<R>(p, da, lists, st->counts + 2, (cplx_t<R>*)st->u, s))) return e;
+        const int32_t* lists[4] = {p->colour_tiles, p->colour_tiles + q, p->colour_tiles + 2 * q, p->colour_tiles + 3 * q};
+        if ((e = grid_dual<R>(p, da, lists, p->colour_counts, (cplx_t<R>*)st->u, s))) return e;
     }
     if ((e = inv_fft<R>(p, (const cplx_t<R>*)st->u, (R*)st->st, nullptr, s))) return e;  // Re(Phi^H v)
     if ((e = synth_dual<R>(p, (const R*)st->xt, (R*)st->syn_u, (R*)st->st, prm->sigma, prm->varsigma, s)))
@@ -1135,22 +1265,62 @@ extern "C" pd_status pd_state_report(const pd_plan* p, const pd_state* st, int64
     if (p_block) CU(cudaMemcpyAsync(p_block, st->p_block, p->d * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (block_active) CU(cudaMemcpyAsync(block_active, st->block_active, p->d * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (basis_active) CU(cudaMemcpyAsync(basis_active, st->basis_active, p->b * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    int32_t gave_up = 0;
+    CU(cudaMemcpyAsync(&gave_up, p->sched + 10, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (work) CU(cudaMemcpyAsync(work, st->counts, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
+    if (gave_up) {
+        CU(cudaMemsetAsync(p->sched + 10, 0, sizeof(int32_t), s));
+        return fail(PD_ETIMEOUT, "a wait of the gridding gave up: the state is not valid");
+    }
     if (t) *t = th;
     if (dx2) *dx2 = dg[0];
     if (x2) *x2 = dg[1];
     return PD_OK;
 }
 
-// checkpoint layout: x, xt, s, st, v, u, y (working precision), eps, res_norm, p_block, p_basis, t
-struct Part { void* dev; size_t bytes; };
+// checkpoint layout: x, xt, s, st, v, u, y (working precision), eps, res_norm, p_block, p_basis, t;
+// v and y (vis) by (tile, block, super-cell, row, column, user index) of the points' base cells
+// in tiles of ck_tile cells, unconjugated
+struct Part { void* dev; size_t bytes; bool vis; };
 static std::vector<Part> state_parts(const pd_plan* p, const pd_state* st) {
     const size_t N = (size_t)p->g.nx * p->g.ny, K = (size_t)p->g.Kx * p->g.Ky;
-    return {{st->x, N * p->rsz}, {st->xt, N * p->rsz}, {st->s, N * p->b * p->rsz}, {st->st, N * p->rsz},
-            {st->v, p->M * p->csz}, {st->u, K * p->csz}, {st->y, p->M * p->csz}, {st->eps, p->d * sizeof(double)},
-            {st->res_norm, p->d * sizeof(double)}, {st->p_block, p->d * sizeof(double)},
-            {st->p_basis, p->b * sizeof(double)}, {st->t, sizeof(int64_t)}};
+    return {{st->x, N * p->rsz, false}, {st->xt, N * p->rsz, false}, {st->s, N * p->b * p->rsz, false},
+            {st->st, N * p->rsz, false}, {st->v, p->M * p->csz, true}, {st->u, K * p->csz, false},
+            {st->y, p->M * p->csz, true}, {st->eps, p->d * sizeof(double), false},
+            {st->res_norm, p->d * sizeof(double), false}, {st->p_block, p->d * sizeof(double), false},
+            {st->p_basis, p->b * sizeof(double), false}, {st->t, sizeof(int64_t), false}};
+}
+static pd_status ensure_ck(pd_plan* p) {
+    if (p->ck_perm) return PD_OK;
+    const int64_t M = p->M;
+    std::vector<int32_t> perm(M), seg(p->nseg + 1);
+    CU(cudaMemcpy(perm.data(), p->perm, M * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(seg.data(), p->seg_start, (p->nseg + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    struct Key {
+        int64_t bucket;       // tile, block
+        int64_t in;           // super-cell, row, column
+        int32_t user, at;
+    };
+    std::vector<Key> key(M);
+    const int T = p->ck_tile, logT = ilog2(T), ntx = p->g.Kx / T, side = std::max(1, T / SC);
+    for (int64_t sg = 0; sg < p->nseg; ++sg)
+        for (int32_t i = seg[sg]; i < seg[sg + 1]; ++i) {
+            const int32_t m = vis_index(perm[i]), c = p->h_base[m], by = c >> 16, bx = c & 0xFFFF;
+            const int ly = by & (T - 1), lx = bx & (T - 1);
+            key[i] = Key{((int64_t)(by >> logT) * ntx + (bx >> logT)) * p->d + p->h_seg_block[sg],
+                         (((int64_t)(ly / SC) * side + lx / SC) << 32) | c, m,
+                         (int32_t)((uint32_t)i | ((uint32_t)perm[i] & 0x80000000u))};
+        }
+    std::sort(key.begin(), key.end(), [](const Key& a, const Key& b) {
+        if (a.bucket != b.bucket) return a.bucket < b.bucket;
+        return a.in != b.in ? a.in < b.in : a.user < b.user;
+    });
+    std::vector<int32_t> out(M);
+    for (int64_t i = 0; i < M; ++i) out[i] = key[i].at;
+    CU(dalloc(p->allocs, p->device_bytes, &p->ck_perm, M));
+    CU(upload(p->ck_perm, out));
+    return PD_OK;
 }
 extern "C" size_t pd_state_bytes(const pd_plan* p) {
     if (!p) return 0;
@@ -1161,10 +1331,16 @@ extern "C" size_t pd_state_bytes(const pd_plan* p) {
 }
 extern "C" pd_status pd_state_save(const pd_plan* p, const pd_state* st, void* buf, void* stream) {
     if (!p || !st || !buf || st->plan != p) return fail(PD_EINVAL, "pd_state_save: bad argument");
+    pd_status e = ensure_ck(st->plan);
+    if (e != PD_OK) return e;
     cudaStream_t s = (cudaStream_t)stream;
     unsigned char* c = (unsigned char*)buf;
     for (const Part& q : state_parts(p, st)) {
-        CU(cudaMemcpyAsync(c, q.dev, q.bytes, cudaMemcpyDeviceToHost, s));
+        if (q.vis) {      // through the plan's residual scratch
+            if (p->prec == PD_F64) CU(gather_by<double>(p, p->ck_perm, (const double2*)q.dev, (double2*)p->rbuf, s));
+            else CU(gather_by<float>(p, p->ck_perm, (const float2*)q.dev, (float2*)p->rbuf, s));
+        }
+        CU(cudaMemcpyAsync(c, q.vis ? p->rbuf : q.dev, q.bytes, cudaMemcpyDeviceToHost, s));
         c += q.bytes;
     }
     CU(cudaStreamSynchronize(s));
@@ -1172,10 +1348,16 @@ extern "C" pd_status pd_state_save(const pd_plan* p, const pd_state* st, void* b
 }
 extern "C" pd_status pd_state_load(const pd_plan* p, pd_state* st, const void* buf, void* stream) {
     if (!p || !st || !buf || st->plan != p) return fail(PD_EINVAL, "pd_state_load: bad argument");
+    pd_status e = ensure_ck(st->plan);
+    if (e != PD_OK) return e;
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned char* c = (const unsigned char*)buf;
     for (const Part& q : state_parts(p, st)) {
-        CU(cudaMemcpyAsync(q.dev, c, q.bytes, cudaMemcpyHostToDevice, s));
+        CU(cudaMemcpyAsync(q.vis ? p->rbuf : q.dev, c, q.bytes, cudaMemcpyHostToDevice, s));
+        if (q.vis) {
+            if (p->prec == PD_F64) CU(scatter_by<double>(p, p->ck_perm, (const double2*)p->rbuf, (double2*)q.dev, s));
+            else CU(scatter_by<float>(p, p->ck_perm, (const float2*)p->rbuf, (float2*)q.dev, s));
+        }
         c += q.bytes;
     }
     CU(cudaStreamSynchronize(s));

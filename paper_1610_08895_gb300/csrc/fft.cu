@@ -179,6 +179,16 @@ template <typename R, int N> struct PassShape {
     static constexpr int MIN_CTAS_COLS = NT_COLS <= 512 ? 2 : 1;
 };
 
+// v cx cy with one rounding in FP32 (factors as value + remainder); plainly in FP64.
+template <typename R> __device__ __forceinline__ R deapodise(R v, R cx, R cxl, R cy, R cyl) {
+    if constexpr (sizeof(R) == 4) {
+        const float p = cx * cy, q = fmaf(cx, cy, -p) + fmaf(cx, cyl, cxl * cy);
+        return fmaf(v, p, v * q);
+    } else {
+        return v * cx * cy;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Forward row pass (Z, then F along x) of two image rows a = iy0 + 2 pr, b = a + 1 per
 // pair: z = Z x_a + i Z x_b. Sequence 2 pr holds z for the even outputs, 2 pr + 1 the
@@ -187,7 +197,8 @@ template <typename R, int N> struct PassShape {
 template <typename R, int N>
 __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN_CTAS_ROWS) k_fwd_rows(
     const R* __restrict__ x, cplx_t<R>* __restrict__ t1, const R* __restrict__ cx, const R* __restrict__ cy,
-    const cplx_t<R>* __restrict__ twx, int ny, int64_t t1_stride) {
+    const R* __restrict__ cxl, const R* __restrict__ cyl, const cplx_t<R>* __restrict__ twx, int ny,
+    int64_t t1_stride) {
     using C2 = cplx_t<R>;
     using S = Shape<R, N>;
     using P = PassShape<R, N>;
@@ -201,9 +212,10 @@ __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN
     batched_loop<4, NT>(P::PAIRS * N, [&](int e) {
         const int pr = e / N, ix = e % N;
         const int a = iy0 + 2 * pr;
-        const R c = cx[ix];
+        const R c = cx[ix], cl = cxl[ix];
         const int lc = ix - N / 2;
-        return In{x[(int64_t)a * N + ix] * c * cy[a], x[(int64_t)(a + 1) * N + ix] * c * cy[a + 1],
+        return In{deapodise(x[(int64_t)a * N + ix], c, cl, cy[a], cyl[a]),
+                  deapodise(x[(int64_t)(a + 1) * N + ix], c, cl, cy[a + 1], cyl[a + 1]),
                   __ldg(&twx[lc & (Kx - 1)])};
     }, [&](int e, const In& v) {
         const int pr = e / N, ix = e % N;
@@ -320,7 +332,7 @@ __global__ void __launch_bounds__(PassShape<R, N>::NT_COLS, PassShape<R, N>::MIN
 template <typename R, int N>
 __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN_CTAS_ROWS) k_inv_rows(
     const cplx_t<R>* __restrict__ t1, R* __restrict__ out, const R* __restrict__ cx, const R* __restrict__ cy,
-    const cplx_t<R>* __restrict__ twx, int ny, int mode, R tau, R sigma, R varsigma, R* __restrict__ xs,
+    const R* __restrict__ cxl, const R* __restrict__ cyl, const cplx_t<R>* __restrict__ twx, int ny, int mode, R tau, R sigma, R varsigma, R* __restrict__ xs,
     R* __restrict__ xt, const R* __restrict__ st_, double* __restrict__ part, int64_t t1_stride) {
     using C2 = cplx_t<R>;
     using S = Shape<R, N>;
@@ -357,11 +369,11 @@ __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN
         const C2 w = cconj(__ldg(&twx[lc & (Kx - 1)]));
         const C2* ev = s + (2 * pr) * S::PN;
         const C2 z = cadd(ev[m], cmul(w, ev[S::PN + m]));
-        const R c = cx[ix];
+        const R c = cx[ix], cl = cxl[ix];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int iy = iy0 + 2 * pr + h;
-            const R g = (h ? z.y : z.x) * c * cy[iy];
+            const R g = deapodise(h ? z.y : z.x, c, cl, cy[iy], cyl[iy]);
             const int64_t idx = (int64_t)iy * N + ix;
             if (mode == 0) {
                 out[idx] = g;
@@ -412,7 +424,8 @@ static cudaError_t launch_fwd_rows(const pd_plan* p, const R* x, cplx_t<R>* t1, 
     cudaError_t e;
     if ((e = ensure_smem(k_fwd_rows<R, N>, P::SMEM_ROWS))) return e;
     k_fwd_rows<R, N><<<dim3(p->g.ny / (2 * P::PAIRS), batch), P::NT_ROWS, P::SMEM_ROWS, s>>>(
-        x, t1, (const R*)p->cx, (const R*)p->cy, (const cplx_t<R>*)p->twx, p->g.ny, t1_elems(p));
+        x, t1, (const R*)p->cx, (const R*)p->cy, (const R*)p->cxl, (const R*)p->cyl,
+            (const cplx_t<R>*)p->twx, p->g.ny, t1_elems(p));
     return cudaGetLastError();
 }
 template <typename R, int N>
@@ -444,11 +457,13 @@ static cudaError_t launch_inv_rows(const pd_plan* p, const cplx_t<R>* t1, R* out
     const int ctas = p->g.ny / (2 * P::PAIRS);
     if (pa == nullptr)
         k_inv_rows<R, N><<<dim3(ctas, batch), P::NT_ROWS, P::SMEM_ROWS, s>>>(
-            t1, out, (const R*)p->cx, (const R*)p->cy, (const cplx_t<R>*)p->twx, p->g.ny, 0, R(0), R(0), R(0),
+            t1, out, (const R*)p->cx, (const R*)p->cy, (const R*)p->cxl, (const R*)p->cyl,
+            (const cplx_t<R>*)p->twx, p->g.ny, 0, R(0), R(0), R(0),
             nullptr, nullptr, nullptr, nullptr, t1_elems(p));
     else
         k_inv_rows<R, N><<<ctas, P::NT_ROWS, P::SMEM_ROWS, s>>>(
-            t1, nullptr, (const R*)p->cx, (const R*)p->cy, (const cplx_t<R>*)p->twx, p->g.ny, 1, (R)pa->tau,
+            t1, nullptr, (const R*)p->cx, (const R*)p->cy, (const R*)p->cxl, (const R*)p->cyl,
+            (const cplx_t<R>*)p->twx, p->g.ny, 1, (R)pa->tau,
             (R)pa->sigma, (R)pa->varsigma, (R*)pa->x, (R*)pa->xt, (const R*)pa->st, pa->part, t1_elems(p));
     return cudaGetLastError();
 }

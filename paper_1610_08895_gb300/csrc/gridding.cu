@@ -4,22 +4,23 @@
 // update of Algorithm 1 step 8 (l2-ball projection, eq. proj-L2) and the
 // gridding of the dual change for step 9.
 //
-// Visibilities are stored in (tile, block, super-cell, row, column) order of
-// their base cell: each (tile, block) pair is a contiguous segment. Per tile, the
+// Visibilities are stored in (tile, block, super-cell, row, column) order of the first
+// cell of their footprint: each (tile, block) pair is a contiguous segment. Per tile, the
 // segments of active blocks are listed in shared memory and worked on as one
-// concatenated range, so inactive blocks cost nothing and batches stay full. A point at continuous grid coordinate g has base cell floor(g) (kept
-// mod K) and fraction g - floor(g) (working precision, computed in FP64 at plan
+// concatenated range, so inactive blocks cost nothing and batches stay full. A point at
+// continuous grid coordinate g has base cell floor(g) (kept mod K) and fraction g - floor(g) (working precision, computed in FP64 at plan
 // time); its taps are the cells floor(g) - J/2 + 1 ... floor(g) + J/2 (mod K),
-// with weight phi(fraction + J/2 - 1 - a) for tap a.
+// with weight phi(fraction + J/2 - 1 - a) for tap a; what is stored is the first of them.
 //
 // Both directions work tile by tile (one CTA owns a T x T tile at a time) on the
-// tile plus a halo of J/2 - 1 cells before and J/2 after:
+// tile plus a halo of J - 1 cells after it:
 // * degridding stages that window of F Z x (held as its half grid: the columns
 //   kx <= nx, the others by conjugate symmetry) in shared memory and gathers from it;
 // * gridding accumulates the window in shared memory and adds the whole window
-//   (tile and halo) to U. The tiles are gridded in four launches, one per tile colour
-//   (tile row and column parity): the windows of two tiles of one colour are disjoint,
-//   so no two CTAs of a launch touch the same cell of U. No global atomics.
+//   (tile and halo) to U. The windows of two tiles of one colour (tile row and column
+//   parity) are disjoint. In FP32 with J <= 8 (k_grid_mma) one launch takes the tiles colour
+//   by colour and adds overlapping windows in the order of the tiles; the other kernels take
+//   one launch per colour. Either way every cell's sum has a fixed order.
 #include <algorithm>
 
 #include "gridding.cuh"
@@ -51,6 +52,43 @@ __device__ __forceinline__ void degrid_load(DegridIn<R>& in, int pos, int& j, co
     }
 }
 
+// Stage the E x E window of the half grid at (oy, ox) in shared memory (pitch EP, even) twice,
+// the second copy (E * EP further) shifted left by one column. The window starts on a column
+// panel, so a thread takes two cells (16 bytes) at a time, consecutive threads along a panel,
+// with all of a thread's loads of a batch in flight.
+__device__ __forceinline__ void stage_window_pairs(float2* win, const float2* __restrict__ gh, int oy, int ox, int E,
+                                                   int EP, const Geo& g) {
+    constexpr int UB = 2;
+    const int per = 2 * E, slots = ((E + 3) >> 2) * per;       // slots of a panel: (row, half)
+    for (int i0 = threadIdx.x; i0 < slots; i0 += UB * (int)blockDim.x) {
+        float4 q[UB];
+        int o[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int i = i0 + u * (int)blockDim.x;
+            const int pn = i / per, r = i - pn * per;
+            const int ey = r >> 1, ex = 4 * pn + 2 * (r & 1);
+            o[u] = i < slots && ex < E ? ey * EP + ex : -1;
+            if (o[u] < 0) continue;
+            const int ky = (oy + ey) & (g.Ky - 1), kx = (ox + ex) & (g.Kx - 1);
+            if (kx < g.nx) {
+                q[u] = *reinterpret_cast<const float4*>(gh + panel_off(ky, kx, g.Ky));
+            } else {
+                const float2 a = half_grid_at(gh, ky, kx, g), b = half_grid_at(gh, ky, kx + 1, g);
+                q[u] = make_float4(a.x, a.y, b.x, b.y);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            if (o[u] < 0) continue;
+            *reinterpret_cast<float4*>(win + o[u]) = q[u];
+            float2* w2 = win + E * EP + o[u];
+            if (o[u] > 0) w2[-1] = make_float2(q[u].x, q[u].y);   // column 0 goes to the row above's spare slot
+            w2[0] = make_float2(q[u].z, q[u].w);
+        }
+    }
+}
+
 // MODE 0 (plain): out_user[perm[m]] = (G grid)_m for every visibility of the listed tiles.
 // MODE 1 (pd): for visibilities of active blocks r = v + G b - y, with FP64 sums of
 // ||r||^2 and ||G b - y||^2 per (tile, block) segment (per-warp slots, summed in warp order).
@@ -62,11 +100,12 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
                                                 const int32_t* __restrict__ perm,
                                                 const int32_t* __restrict__ seg_start,
                                                 const int32_t* __restrict__ seg_block,
-                                                const int32_t* __restrict__ tile_seg_start,
-                                                const int32_t* __restrict__ active, const int32_t* __restrict__ list,
-                                                const int32_t* __restrict__ count, double* __restrict__ seg_part,
+                                                const int32_t* __restrict__ active,
+                                                const TileItem* __restrict__ items,
+                                                const int32_t* __restrict__ nitems,
+                                                const int32_t* __restrict__ tile_on, double* __restrict__ seg_part,
                                                 int max_segs, Geo g, R two_over_j, R beta, const KbPoly kp,
-                                                int* __restrict__ next_tile, int batch, int64_t gstride,
+                                                int* __restrict__ sched, int batch, int64_t gstride,
                                                 int64_t ostride) {
     using C2 = cplx_t<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -79,42 +118,47 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
     double* part = reinterpret_cast<double*>(win + (PAIRS ? 2 : 1) * g.ext * EP);  // [8 warps][max_segs][2]
     int* act_seg = reinterpret_cast<int*>(part + 16 * max_segs);        // [max_segs]
     int* act_pre = act_seg + max_segs;                                   // [max_segs + 1]
-    __shared__ int nact_s, tile_s;
-    const int E = g.ext, T = g.tile, H = g.halo_lo;
+    __shared__ int nact_s, item_s;
+    __shared__ TileItem ti_s;
+    const int E = g.ext, T = g.tile;
     const int warp = threadIdx.x >> 5;
-    const int n = *count;
+    const int n = *nitems;
+    if (threadIdx.x == 0) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
     for (;;) {
-        // tiles are taken from the heaviest-first list one at a time by whichever CTA is free
-        if (threadIdx.x == 0) tile_s = atomicAdd(next_tile, 1);
         __syncthreads();
-        const int w = tile_s;
+        const int w = item_s;
         if (w >= n * batch) break;
-        // work item w: tile w / batch of the list for image w mod batch (a batch of plain
-        // applications; the heaviest tiles of every image come first)
-        const int t = list[w / batch], img = w % batch;
+        // item w / batch of the heaviest-first list for image w mod batch (a batch of plain applications)
+        const TileItem ti = ti_s;
+        const int t = ti.tile, img = w % batch;
         const cplx_t<R>* gimg = grid + (int64_t)img * gstride;
         cplx_t<R>* oimg = MODE == 0 ? out + (int64_t)img * ostride : out;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
         const int oy = ty * T, ox = tx * T;
-        const int seg0 = tile_seg_start[t], nseg_t = tile_seg_start[t + 1] - seg0;
+        const int seg0 = ti.seg0, nseg_t = ti.nseg;
         list_active_segments(seg0, nseg_t, seg_block, MODE == 1 ? active : nullptr, seg_start, act_seg, act_pre,
                              &nact_s);
-        for (int i = threadIdx.x; i < E * E; i += blockDim.x) {
-            const int ey = i / E, ex = i - ey * E;
-            const C2 gv = half_grid_at(gimg, (oy - H + ey) & (g.Ky - 1), (ox - H + ex) & (g.Kx - 1), g);
-            win[ey * EP + ex] = gv;
-            if (PAIRS && ex > 0) win[E * EP + ey * EP + ex - 1] = gv;
+        if constexpr (PAIRS) {
+            stage_window_pairs(win, gimg, oy, ox, E, EP, g);
+        } else {
+            for (int i = threadIdx.x; i < E * E; i += blockDim.x) {
+                const int ey = i / E, ex = i - ey * E;
+                win[ey * EP + ex] = half_grid_at(gimg, (oy + ey) & (g.Ky - 1), (ox + ex) & (g.Kx - 1), g);
+            }
         }
         if (MODE == 1)
             for (int i = threadIdx.x; i < 16 * nseg_t; i += blockDim.x) part[i] = 0.0;
         __syncthreads();
-        const int nact = nact_s, total = act_pre[nact];
+        // this part's positions of the tile's active points
+        const int nact = nact_s, all = act_pre[nact];
+        const int first = (int)((int64_t)all * ti.part / ti.parts), total = (int)((int64_t)all * (ti.part + 1) / ti.parts);
         double* mypart = part + 2 * nseg_t * warp;
         int j = 0;   // segment cursor: positions only grow, so it only moves forward
         // the inputs of the point blockDim.x positions ahead are loaded while this one is worked on
         DegridIn<R> nx{};
-        if ((int)threadIdx.x < total) degrid_load<R, MODE>(nx, threadIdx.x, j, act_seg, act_pre, seg_start, cell, fxs, fys, y, v);
-        for (int base = 0; base < total; base += blockDim.x) {
+        if (first + (int)threadIdx.x < total)
+            degrid_load<R, MODE>(nx, first + threadIdx.x, j, act_seg, act_pre, seg_start, cell, fxs, fys, y, v);
+        for (int base = first; base < total; base += blockDim.x) {
             const int pos = base + threadIdx.x;
             const bool ok = pos < total;
             const DegridIn<R> in = nx;
@@ -161,7 +205,7 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
                     }
                 }
                 if (MODE == 0) {
-                    oimg[perm[m]] = mk<C2>(sx, sy);
+                    oimg[vis_index(perm[m])] = vis_conj(perm[m], mk<C2>(sx, sy));
                 } else {
                     const R dx = sx - in.yy.x, dy = sy - in.yy.y;
                     const C2 r = mk<C2>(in.vv.x + dx, in.vv.y + dy);
@@ -173,6 +217,7 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
             if (MODE == 1) warp_seg_add(ok, jcur, ar, ad, mypart);
         }
         __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
         if (MODE == 1) {
             for (int k = threadIdx.x; k < nact; k += blockDim.x) {
                 double sr = 0.0, sd = 0.0;
@@ -180,15 +225,16 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
                     sr += part[2 * nseg_t * wp + 2 * k];
                     sd += part[2 * nseg_t * wp + 2 * k + 1];
                 }
-                seg_part[2 * act_seg[k]] = sr;
-                seg_part[2 * act_seg[k] + 1] = sd;
+                const int64_t slot = (int64_t)ti.slot0 + act_seg[k] - seg0;
+                seg_part[2 * slot] = sr;
+                seg_part[2 * slot + 1] = sd;
             }
         }
-        __syncthreads();
     }
+    if (threadIdx.x == 0) leave_items(sched);
 }
 
-// Per-block FP64 norms summed over the block's segments in a fixed order (one warp per
+// Per-block FP64 norms summed over the block's seg_part slots in a fixed order (one warp per
 // block: lane-strided partial sums, then a fixed shuffle tree), the ball scale
 // c_i = max(0, 1 - eps_i/||r_i||) of step 8 (so v_new = c_i r_i = z - P_B(z)), and the
 // residual norm ||G_i b - y_i|| for the adaptive probabilities of Sec. 4.
@@ -233,7 +279,8 @@ __global__ void __launch_bounds__(256) k_grid(const cplx_t<R>* __restrict__ src,
                                               const int32_t* __restrict__ seg_block,
                                               const int32_t* __restrict__ tile_seg_start,
                                               const int32_t* __restrict__ list, const int32_t* __restrict__ count,
-                                              cplx_t<R>* __restrict__ U, int max_segs,
+                                              const int32_t* __restrict__ tile_on, cplx_t<R>* __restrict__ U,
+                                              int max_segs,
                                               Geo g, R two_over_j, R beta, const KbPoly kp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     R* acc = reinterpret_cast<R*>(smraw);   // [ext*ext] re then [ext*ext] im
@@ -244,6 +291,7 @@ __global__ void __launch_bounds__(256) k_grid(const cplx_t<R>* __restrict__ src,
     const int n = *count;
     for (int w = blockIdx.x; w < n; w += gridDim.x) {
         const int t = list[w];
+        if (tile_on && !tile_on[t]) continue;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
         const int oy = ty * g.tile, ox = tx * g.tile;
         const int seg0 = tile_seg_start[t], nseg_t = tile_seg_start[t + 1] - seg0;
@@ -374,7 +422,7 @@ __device__ __forceinline__ void grid_load(GridIn<R>& in, int pos, int& j, const 
         in.b = v[m];
         in.sc = rscale[j];
     } else {
-        in.a = src[perm[m]];
+        in.a = vis_conj(perm[m], src[vis_index(perm[m])]);
     }
 }
 
@@ -385,13 +433,13 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
     const R* __restrict__ fxs, const R* __restrict__ fys, const int32_t* __restrict__ perm,
     const int32_t* __restrict__ seg_start, const int32_t* __restrict__ seg_block,
     const int32_t* __restrict__ tile_seg_start, const int32_t* __restrict__ sc_start,
-    const int32_t* __restrict__ list, const int32_t* __restrict__ count, cplx_t<R>* __restrict__ U, int max_segs,
-    Geo g, R two_over_j, R beta, const KbPoly kp, int* __restrict__ next_tile, int batch, int64_t istride,
-    int64_t ustride) {
+    const int32_t* __restrict__ list, const int32_t* __restrict__ count, const int32_t* __restrict__ tile_on,
+    cplx_t<R>* __restrict__ U, int max_segs, Geo g, R two_over_j, R beta, const KbPoly kp,
+    int* __restrict__ next_tile, int batch, int64_t istride, int64_t ustride) {
     static_assert(J <= 8 && J % 2 == 0, "class ownership needs J <= 8");
     using C2 = cplx_t<R>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int T = g.tile, E = g.ext, WR = T + 7, WS = WR * GW_WP;
+    const int T = g.tile, WR = T + 7, WS = WR * GW_WP;
     const int nsd = T / 8 > 0 ? T / 8 : 1, nsc = nsd * nsd;    // super-cells per side, per tile
     const int nw = blockDim.x >> 5;                             // = nsd
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -413,7 +461,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
     const int n = *count;
     for (;;) {
         // tiles are taken from the heaviest-first list one at a time by whichever CTA is free
-        if (threadIdx.x == 0) tile_s = atomicAdd(next_tile, 1);
+        if (threadIdx.x == 0) tile_s = claim_tile(next_tile, list, n, batch, tile_on);
         __syncthreads();
         const int w = tile_s;
         if (w >= n * batch) break;
@@ -562,59 +610,585 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
     }
 }
 
+// ---------------------------------------------------------------- gridding, FP32, J <= 8
+// The window of one super-cell (8 x 8 footprint origins) is a 16 x 16 patch, and gridding
+// its points is a contraction over them: patch[r][c] = sum_m wy_m[r] (d_m wx_m[c]). A warp
+// runs it on the tensor cores: M = 16 patch rows, N = 2 x 16 patch columns (re, im), K = 16
+// points. Every FP32 operand is split exactly into three bf16 values (8 + 8 + 8 significant
+// bits), and the six products down to 2^-16 of the leading one are accumulated, smallest
+// first: what is dropped is below the rounding of an FP32 product. The sum of 16 points is
+// then added to FP32 registers (the tensor core truncates its sums, so no chain goes
+// through it).
+// A CTA works on one part of a tile at a time. The part's points, super-cell by super-cell
+// (each padded to a multiple of 16), are cut into chunks of 32 that are shared out evenly
+// among the CTA's working warps; at the end of a super-cell (or of its share) a warp stores
+// the patch to the slot super-cell + warp, which no other pair has; the slots are then summed,
+// in a fixed order, into the part's window. One more warp keeps the others fed: it claims
+// the next item and lists its points while they work on the current one, and it adds the
+// finished window to U with bulk reductions, one per column panel (rows of a panel are
+// contiguous in U), while they work on the next.
+// What bounds it: instruction issue (about 30 warp instructions a point, 12 of them in the
+// contraction; the split's logic operations share the half-rate ALU pipe) with 16 warps per
+// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 356 us, against 462 us
+// for the FP32 FMA kernel below it in four launches (same windows); 65,536 points on 512^2,
+// where the densest tile was the critical path of each launch: 28 against 154 us; 1.05M on
+// 1024^2: 38 against 233 us. Slower there: 2048-point parts (459 us), 3 or 15 working warps
+// (442, 448 us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the
+// tiles' weight instead of their colour (3.3 ms: chains of neighbours).
+// Staging (one lane per point) writes the taps by class (patch row / column mod 8),
+// negated when the tap falls in the upper half of the patch: 18 floats a point, each read
+// once, by the lane whose fragment needs it.
+constexpr int GM_F = 18;       // floats per staged point: 8 row classes, 8 column classes, re, im
+constexpr int GM_WP = 18;      // patch pitch (complex)
+constexpr int GM_PS = 16 * GM_WP;   // patch slot (complex)
+constexpr int GM_MAXW = 16;    // warps per CTA, the feeding one included
+constexpr int GM_SPIN = 1 << 22;
+
+__device__ __forceinline__ int ld_acquire(const int32_t* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// One work item, listed by the feeding warp: which tile and part, and its chunks.
+struct GridItem {
+    int tile, img, part, parts;   // tile < 0: none left
+    int nact, total, cbeg, nchunk;
+};
+
+// Shared memory of a CTA with nc working warps (ms: most segments of a tile); the item
+// lists are kept twice.
+__host__ __device__ constexpr size_t grid_mma_lists(int nsc, int ms) {
+    return (size_t)nsc * sizeof(int2) + (size_t)(nsc + 1) * sizeof(int) + (size_t)ms * sizeof(float) +
+           (size_t)(2 * nsc * ms + 1) * sizeof(int);
+}
+__host__ __device__ constexpr size_t grid_mma_smem(int T, int nc, int ms) {
+    const int nsd = T / 8, nsc = nsd * nsd;
+    return (size_t)(T + 8) * (T + 8) * sizeof(float2) + (size_t)(nsc + nc) * GM_PS * sizeof(float2) +
+           (size_t)nc * 32 * GM_F * sizeof(float) + 2 * ((grid_mma_lists(nsc, ms) + 15) / 16 * 16) +
+           (size_t)ms * sizeof(int);
+}
+
+__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// x = s0 + s1 + s2, each part with its low 16 bits zero: exact in bf16. s0 is rounded to
+// nearest, so that the parts' signs differ and the dropped products have no bias (truncated
+// parts measured twice the error of the sum of 16 products: 9.1e-8 against 4.9e-8, and a
+// chain of FP32 multiply-adds 7.3e-8).
+__device__ __forceinline__ void split3(float x, uint32_t* s) {
+    s[0] = (__float_as_uint(x) + 0x8000u) & 0xffff0000u;
+    const float r = x - __uint_as_float(s[0]);
+    s[1] = __float_as_uint(r) & 0xffff0000u;
+    s[2] = __float_as_uint(r - __uint_as_float(s[1]));
+}
+// the upper halves of a (low) and b (high)
+__device__ __forceinline__ uint32_t pack_hi(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+// 0xffff in the half of each negative operand
+__device__ __forceinline__ uint32_t sign_mask(float a, float b) {
+    uint32_t m;
+    asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(m) : "r"(__float_as_uint(a)), "r"(__float_as_uint(b)));
+    return m;
+}
+
+// acc += the 16 staged points of group grp, all of one super-cell.
+// acc[n][e]: n = {re low, re high, im low, im high} columns, e = the fragment's 4 elements.
+__device__ __forceinline__ void grid_mma_group(const float* __restrict__ st, int grp, int g, int t, float (*acc)[4]) {
+    const int p0 = 16 * grp + 4 * t;
+    const int ps = p0 ^ ((g & 1) << 4);
+    const float4 wy = *reinterpret_cast<const float4*>(st + g * 32 + ps);
+    const float4 wx = *reinterpret_cast<const float4*>(st + (8 + g) * 32 + ps);
+    const float4 dr = *reinterpret_cast<const float4*>(st + 16 * 32 + p0);
+    const float4 di = *reinterpret_cast<const float4*>(st + 17 * 32 + p0);
+    uint32_t A[3][4];
+    {
+        const uint32_t m0 = sign_mask(wy.x, wy.y), m1 = sign_mask(wy.z, wy.w);
+        uint32_t s[4][3];
+        split3(fabsf(wy.x), s[0]); split3(fabsf(wy.y), s[1]); split3(fabsf(wy.z), s[2]); split3(fabsf(wy.w), s[3]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const uint32_t u = pack_hi(s[0][i], s[1][i]), v = pack_hi(s[2][i], s[3][i]);
+            A[i][0] = u & ~m0; A[i][1] = u & m0; A[i][2] = v & ~m1; A[i][3] = v & m1;
+        }
+    }
+    const uint32_t m0 = sign_mask(wx.x, wx.y), m1 = sign_mask(wx.z, wx.w);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                       // real, imaginary part
+        const float4 dv = h ? di : dr;
+        uint32_t s[4][3], u[3], v[3];
+        split3(fabsf(wx.x) * dv.x, s[0]); split3(fabsf(wx.y) * dv.y, s[1]);
+        split3(fabsf(wx.z) * dv.z, s[2]); split3(fabsf(wx.w) * dv.w, s[3]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) { u[i] = pack_hi(s[0][i], s[1][i]); v[i] = pack_hi(s[2][i], s[3][i]); }
+#pragma unroll
+        for (int hi = 0; hi < 2; ++hi) {                // low, high half of the patch columns
+            uint32_t b0[3], b1[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                b0[i] = hi ? u[i] & m0 : u[i] & ~m0;
+                b1[i] = hi ? v[i] & m1 : v[i] & ~m1;
+            }
+            float d[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(d, A[2], b0[0], b1[0]);
+            mma_bf16(d, A[0], b0[2], b1[2]);
+            mma_bf16(d, A[1], b0[1], b1[1]);
+            mma_bf16(d, A[1], b0[0], b1[0]);
+            mma_bf16(d, A[0], b0[1], b1[1]);
+            float m[4] = {0.f, 0.f, 0.f, 0.f};              // apart: products of 8-bit values, mostly exact
+            mma_bf16(m, A[0], b0[0], b1[0]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[2 * h + hi][e] += m[e] + d[e];
+        }
+    }
+}
+
+// w[0..J) (tap a falls in class (o + a) mod 8) into class order, negated for o + a >= 8,
+// zero for classes without a tap
+template <int J> __device__ __forceinline__ void class_order(const float* w, int o, float* out) {
+#pragma unroll
+    for (int a = 0; a < 8; ++a) out[a] = a < J ? w[a] : 0.f;
+#pragma unroll
+    for (int sh = 1; sh < 8; sh <<= 1) {
+        const bool on = (o & sh) != 0;
+        float q[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) q[c] = on ? out[(c - sh) & 7] : out[c];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) out[c] = q[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) out[c] = c < o ? -out[c] : out[c];
+}
+
+// The lists of one item in shared memory.
+struct GridLists {
+    int2* sinfo;      // [nsc] first slot and number of slots of each super-cell
+    int* ps;          // [nsc + 1] padded start of each super-cell
+    float* rscale;    // [ms] ball scale of each active segment
+    int* rstart;      // [nsc * ms] first point of each range (super-cell * nact + segment)
+    int* rpre;        // [nsc * ms + 1] prefix sums of the ranges' lengths
+    __device__ GridLists(unsigned char* base, int nsc, int ms) {
+        sinfo = reinterpret_cast<int2*>(base);
+        ps = reinterpret_cast<int*>(sinfo + nsc);
+        rscale = reinterpret_cast<float*>(ps + nsc + 1);
+        rstart = reinterpret_cast<int*>(rscale + ms);
+        rpre = rstart + nsc * ms;
+    }
+};
+
+// The point at position pos of the item's padded order (super-cell sc from ps[sc] on); sc,
+// k and jj are this lane's super-cell, range and active-segment cursors (k = sc * nact +
+// jj), moved forward to it. False past the super-cell's points.
+template <int MODE>
+__device__ __forceinline__ bool grid_mma_load(GridIn<float>& in, int pos, int& sc, int& k, int& jj, int nsc, int nact,
+                                              const GridLists& L, const float2* __restrict__ src,
+                                              const float2* __restrict__ rbuf, const float2* __restrict__ v,
+                                              const int32_t* __restrict__ cell, const float* __restrict__ fxs,
+                                              const float* __restrict__ fys, const int32_t* __restrict__ perm) {
+    while (sc + 1 < nsc && L.ps[sc + 1] <= pos) ++sc;
+    const int up = pos - L.ps[sc] + L.rpre[sc * nact];
+    if (up >= L.rpre[(sc + 1) * nact]) return false;
+    while (L.rpre[k + 1] <= up) {
+        ++k;
+        jj = jj + 1 == nact ? 0 : jj + 1;
+    }
+    const int m = L.rstart[k] + up - L.rpre[k];
+    in.m = m;
+    in.fx = fxs[m];
+    in.fy = fys[m];
+    in.c = cell[m];
+    if (MODE == 1) {
+        in.a = rbuf[m];
+        in.b = v[m];
+        in.sc = L.rscale[jj];
+    } else {
+        const int q = perm[m];
+        in.a = vis_conj(q, src[vis_index(q)]);
+    }
+    return true;
+}
+
+template <int J, int MODE>
+__global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
+    const float2* __restrict__ src, const float2* __restrict__ rbuf, float2* __restrict__ v,
+    const float* __restrict__ scale, const int32_t* __restrict__ active, const int32_t* __restrict__ cell,
+    const float* __restrict__ fxs, const float* __restrict__ fys, const int32_t* __restrict__ perm,
+    const int32_t* __restrict__ seg_start, const int32_t* __restrict__ seg_block,
+    const int32_t* __restrict__ sc_start, const int4* __restrict__ tile_info, const int32_t* __restrict__ tile_on,
+    const int2* __restrict__ items, const int32_t* __restrict__ nitems, int32_t* pend, float2* U, int max_segs, Geo g,
+    const KbPoly kp, int* sched, int batch, int64_t istride, int64_t ustride) {
+    static_assert(J <= 8 && J % 2 == 0, "a super-cell's window is 16 x 16 for J <= 8");
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int T = g.tile, nsd = T >> 3, nsc = nsd * nsd, W = T + 8;
+    const int nc = (blockDim.x >> 5) - 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NT = blockDim.x, NCT = nc * 32;                   // all threads, working threads
+    float2* wbuf = reinterpret_cast<float2*>(smraw);            // [W / 4][W][4] the window, in U's panel layout
+    float2* slots = wbuf + W * W;                               // [nsc + nc][16][GM_WP]
+    float* st = reinterpret_cast<float*>(slots + (size_t)(nsc + nc) * GM_PS) + (size_t)warp * 32 * GM_F;   // [GM_F][32]
+    unsigned char* lbase = reinterpret_cast<unsigned char*>(slots + (size_t)(nsc + nc) * GM_PS) +
+                           (size_t)nc * 32 * GM_F * sizeof(float);
+    const size_t lsz = (grid_mma_lists(nsc, max_segs) + 15) / 16 * 16;
+    __shared__ GridItem item_s[2];
+    // barriers: 1, 2 item listed (even, odd); 3 slots written; 4 window written; 5 window free; 6 halfway
+    if (warp == nc) {
+        // ---------------------------------------------------------------- the feeding warp
+        int* act_seg = reinterpret_cast<int*>(lbase + 2 * lsz);
+        const int nitem = *nitems * batch;
+        // claims the next item with an active block (items are claimed in order by whichever CTA is
+        // free; item w: items[w / batch] for image w mod batch of a batch) and lists it in buffer b
+        auto prepare = [&](int b) -> bool {
+            const GridLists L(lbase + b * lsz, nsc, max_segs);
+            int w;
+            int2 it;
+            int4 ti;
+            for (;;) {
+                w = lane == 0 ? atomicAdd(sched, 1) : 0;
+                w = __shfl_sync(0xffffffffu, w, 0);
+                if (w >= nitem) {
+                    if (lane == 0) item_s[b].tile = -1;
+                    return false;
+                }
+                it = items[w / batch];
+                ti = tile_info[it.x];
+                if (!tile_on || tile_on[it.x]) break;
+            }
+            int nact = 0;
+            const unsigned below = (1u << lane) - 1u;
+            for (int base = 0; base < ti.y; base += 32) {
+                const int k = base + lane;
+                int blk = 0;
+                bool on = k < ti.y;
+                if (on) blk = seg_block[ti.x + k];
+                if (MODE == 1 && on) on = active[blk] != 0;
+                const unsigned bal = __ballot_sync(0xffffffffu, on);
+                if (on) {
+                    const int pos = nact + __popc(bal & below);
+                    act_seg[pos] = ti.x + k;
+                    if (MODE == 1) L.rscale[pos] = scale[blk];
+                }
+                nact += __popc(bal);
+            }
+            __syncwarp();
+            // ranges super-cell * nact + segment, with the prefix sums of their lengths
+            const int nr = nact * nsc;
+            int tot = 0;
+            if (lane == 0) L.rpre[0] = 0;
+            for (int base = 0; base < nr; base += 128) {
+                int s0[4], s1[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = base + u * 32 + lane;
+                    s0[u] = s1[u] = 0;
+                    if (k < nr) {
+                        const int sc = k / nact;
+                        const int32_t* p = sc_start + (int64_t)act_seg[k - sc * nact] * (nsc + 1) + sc;
+                        s0[u] = p[0];
+                        s1[u] = p[1];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int k = base + u * 32 + lane;
+                    int incl = s1[u] - s0[u];
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int yv = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += yv;
+                    }
+                    if (k < nr) {
+                        L.rstart[k] = s0[u];
+                        L.rpre[k + 1] = tot + incl;
+                    }
+                    tot += __shfl_sync(0xffffffffu, incl, 31);
+                }
+            }
+            __syncwarp();
+            // every super-cell starts at a multiple of 16, so that the 16 points of a group share it
+            int padded = 0;
+            for (int base = 0; base < nsc; base += 32) {
+                const int sc = base + lane;
+                const int pl = sc < nsc && nact ? (L.rpre[(sc + 1) * nact] - L.rpre[sc * nact] + 15) & ~15 : 0;
+                int incl = pl;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int yv = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += yv;
+                }
+                if (sc < nsc) L.ps[sc] = padded + incl - pl;
+                padded += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) L.ps[nsc] = padded;
+            __syncwarp();
+            // this part's chunks of the tile, shared out to nu warps with at least one chunk each
+            const int allch = (padded + 31) >> 5;
+            const int cbeg = (int)((int64_t)allch * it.y / ti.z);
+            const int nchunk = (int)((int64_t)allch * (it.y + 1) / ti.z) - cbeg, nu = min(nc, nchunk);
+            for (int sc = lane; sc < nsc; sc += 32) {
+                const int c0 = max((L.ps[sc] >> 5) - cbeg, 0), c1 = min(((L.ps[sc + 1] - 1) >> 5) - cbeg, nchunk - 1);
+                int2 si = make_int2(0, 0);
+                if (L.ps[sc + 1] > L.ps[sc] && c0 <= c1) {   // chunk c belongs to warp ((c + 1) nu - 1) / nchunk
+                    const int w0 = ((c0 + 1) * nu - 1) / nchunk, w1 = ((c1 + 1) * nu - 1) / nchunk;
+                    si = make_int2(sc + w0, w1 - w0 + 1);
+                }
+                L.sinfo[sc] = si;
+            }
+            if (lane == 0) item_s[b] = GridItem{it.x, w % batch, it.y, ti.z, nact, padded, cbeg, nchunk};
+            return true;
+        };
+        bool have = prepare(0);
+        __syncwarp();
+        bar_arrive(1, NT);
+        for (int i = 0; have; ++i) {
+            const int b = i & 1;
+            bar_sync(6, 64);                                    // the working warps are halfway through item i
+            const bool next = prepare(b ^ 1);
+            __syncwarp();
+            bar_arrive(1 + (b ^ 1), NT);
+            bar_sync(4, NT);                                    // item i's window is complete
+            // The windows of neighbouring tiles overlap, and so do a tile's parts: they are added to
+            // U in the order of the items, so that the sums do not depend on timing. Earlier items
+            // are claimed earlier and a CTA takes its items in order, so the first unfinished one
+            // is being worked on and never waits: this wait ends. Its limit is a safeguard (some
+            // seconds), after which the launch goes on and sets its error flag.
+            const GridItem& im = item_s[b];
+            const int ty = im.tile / g.ntx, tx = im.tile - ty * g.ntx;
+            int32_t* pd = pend + (int64_t)im.img * g.ntiles;
+            if (lane < 9) {
+                const int t2 = ((ty + lane / 3 - 1) & (g.nty - 1)) * g.ntx + ((tx + lane % 3 - 1) & (g.ntx - 1));
+                const int upto = t2 == im.tile ? im.parts - im.part : 0;
+                if (t2 == im.tile || tile_info[t2].w < tile_info[im.tile].w) {
+                    int tries = 0;
+                    while (ld_acquire(pd + t2) > upto)
+                        if (++tries > GM_SPIN) { atomicExch(sched + 2, 1); break; }
+                }
+            }
+            __syncwarp();
+            asm volatile("fence.proxy.async;" ::: "memory");
+            // panel pn of the window: W rows of 32 bytes, in two pieces where they wrap around the grid
+            float2* Uimg = U + (int64_t)im.img * ustride;
+            const int oy = ty * T, r0 = min(W, g.Ky - oy);
+            for (int pn = lane; pn < W / 4; pn += 32) {
+                float2* dst = Uimg + panel_off(oy, (tx * T + 4 * pn) & (g.Kx - 1), g.Ky);
+                const uint32_t sa = (uint32_t)__cvta_generic_to_shared(wbuf + pn * W * 4);
+                asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst),
+                             "r"(sa), "r"(r0 * 32) : "memory");
+                if (r0 < W)
+                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
+                                     dst - (int64_t)oy * PW), "r"(sa + r0 * 32), "r"((W - r0) * 32) : "memory");
+            }
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            __syncwarp();
+            if (next) bar_arrive(5, NT);                        // the window's buffer is free
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            asm volatile("fence.proxy.async;" ::: "memory");
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) atomicSub(pd + im.tile, 1);
+            have = next;
+        }
+        // the last CTA to leave sets the counters back for the next launch
+        if (lane == 0 && atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
+            sched[0] = 0;
+            sched[1] = 0;
+        }
+        return;
+    }
+    // -------------------------------------------------------------------- the working warps
+    const int fg = lane >> 2, ft = lane & 3;                    // fragment row / column of this lane
+    // where this warp stands in the current item
+    GridIn<float> in{};
+    int sc, k, jj, ch0, ch1, nact, total, oy, ox;
+    const float2* simg = src;
+    bool ok;
+    auto setup = [&](int b) {
+        const GridItem& im = item_s[b];
+        const GridLists L(lbase + b * lsz, nsc, max_segs);
+        const int ty = im.tile / g.ntx;
+        oy = ty * T;
+        ox = (im.tile - ty * g.ntx) * T;
+        nact = im.nact;
+        total = im.total;
+        if (MODE == 0) simg = src + (int64_t)im.img * istride;
+        const int nu = min(nc, im.nchunk);
+        ch0 = warp < nu ? im.cbeg + (int)((int64_t)im.nchunk * warp / nu) : 0;
+        ch1 = warp < nu ? im.cbeg + (int)((int64_t)im.nchunk * (warp + 1) / nu) : 0;
+        sc = k = jj = 0;
+        ok = false;
+        if (ch0 < ch1) {
+            const int pos = ch0 * 32 + lane;
+            int hi = nsc;     // last super-cell with ps[sc] <= pos
+            while (hi - sc > 1) {
+                const int mid = (sc + hi) >> 1;
+                if (L.ps[mid] <= pos) sc = mid; else hi = mid;
+            }
+            const int nr = nact * nsc, up = min(pos - L.ps[sc] + L.rpre[sc * nact], L.rpre[nr] - 1);
+            hi = nr;          // last range with rpre[k] <= up
+            while (hi - k > 1) {
+                const int mid = (k + hi) >> 1;
+                if (L.rpre[mid] <= up) k = mid; else hi = mid;
+            }
+            jj = k % nact;
+            ok = pos < total && grid_mma_load<MODE>(in, pos, sc, k, jj, nsc, nact, L, simg, rbuf, v, cell, fxs, fys, perm);
+        }
+    };
+    for (int c = 0; c < GM_F; ++c) st[c * 32 + lane] = 0.f;
+    bar_sync(1, NT);
+    if (item_s[0].tile < 0) return;
+    setup(0);
+    for (int i = 0;; ++i) {
+        const int b = i & 1;
+        const GridLists L(lbase + b * lsz, nsc, max_segs);
+        float acc[4][4] = {};
+        int cur = -1;         // the super-cell the sums belong to
+        auto flush = [&]() {
+            float2* cp = slots + (size_t)(cur + warp) * GM_PS + fg * GM_WP + 2 * ft;
+#pragma unroll
+            for (int hi = 0; hi < 2; ++hi)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)             // patch rows fg and fg + 8
+                    *reinterpret_cast<float4*>(cp + u * 8 * GM_WP + hi * 8) =
+                        make_float4(acc[hi][2 * u], acc[2 + hi][2 * u], acc[hi][2 * u + 1], acc[2 + hi][2 * u + 1]);
+        };
+        const int half = (ch0 + ch1) >> 1;
+        if (warp == 0 && ch0 >= ch1) bar_arrive(6, 64);
+        for (int chunk = ch0; chunk < ch1; ++chunk) {
+            if (warp == 0 && chunk == half) bar_arrive(6, 64);
+            const int mysc = sc;
+            if (ok) {
+                float2 d;
+                if (MODE == 1) {
+                    const float2 vn = cscale(in.a, in.sc);       // step 8: v_new = c_i r
+                    v[in.m] = vn;
+                    d = csub(vn, in.b);
+                } else {
+                    d = in.a;
+                }
+                const int r0 = (in.c >> 16) - oy, c0 = (in.c & 0xFFFF) - ox;   // footprint origin in the window
+                float wt[J], cw[8];
+                kb_taps<float, J>(in.fy, wt, 0.f, 0.f, kp);
+                class_order<J>(wt, r0 & 7, cw);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) st[c * 32 + (lane ^ ((c & 1) << 4))] = cw[c];
+                const int gam = c0 & 7;
+                kb_taps<float, J>(in.fx, wt, 0.f, 0.f, kp);
+                class_order<J>(wt, gam, cw);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) st[(8 + c) * 32 + (lane ^ ((c & 1) << 4))] = cw[c];
+                st[16 * 32 + lane] = d.x;
+                st[17 * 32 + lane] = d.y;
+            } else {          // no point here: value zero, with the (finite) weights of an earlier one
+                st[16 * 32 + lane] = 0.f;
+                st[17 * 32 + lane] = 0.f;
+            }
+            // the next chunk's loads go out now and land while this one is accumulated
+            const int nxt = (chunk + 1) * 32 + lane;
+            ok = chunk + 1 < ch1 && nxt < total &&
+                 grid_mma_load<MODE>(in, nxt, sc, k, jj, nsc, nact, L, simg, rbuf, v, cell, fxs, fys, perm);
+            __syncwarp();
+#pragma unroll
+            for (int grp = 0; grp < 2; ++grp) {
+                if (chunk * 32 + grp * 16 >= total) break;
+                const int key = __shfl_sync(0xffffffffu, mysc, grp * 16);
+                if (key != cur) {
+                    if (cur >= 0) flush();
+                    cur = key;
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) (&acc[0][0])[q] = 0.f;
+                }
+                grid_mma_group(st, grp, fg, ft, acc);
+            }
+            __syncwarp();
+        }
+        if (cur >= 0) flush();
+        // the next item's first loads go out before this one's window is put together
+        bar_sync(1 + (b ^ 1), NT);
+        const bool more = item_s[b ^ 1].tile >= 0;
+        if (more) setup(b ^ 1);
+        bar_sync(3, NCT);
+        if (i > 0) bar_sync(5, NT);
+        // the window, block of 8 x 8 cells by block, two cells a lane: block (by, bx) is covered by
+        // the patches of the super-cells (by, bx) .. (by - 1, bx - 1)
+        for (int by = 0, bx = warp; ; bx += nc) {
+            while (bx > nsd) { bx -= nsd + 1; ++by; }
+            if (by > nsd) break;
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int a = q >> 1, c = q & 1, sy = by - a, sx = bx - c;
+                if (sy < 0 || sy >= nsd || sx < 0 || sx >= nsd) continue;
+                const int2 si = L.sinfo[sy * nsd + sx];
+                const float2* sp = slots + si.x * GM_PS + (8 * a + fg) * GM_WP + 8 * c + 2 * ft;
+#pragma unroll 1
+                for (int e = 0; e < si.y; ++e, sp += GM_PS) {
+                    const float4 x = *reinterpret_cast<const float4*>(sp);
+                    sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+                }
+            }
+            const int ex = 8 * bx + 2 * ft;
+            *reinterpret_cast<float4*>(wbuf + ((ex >> 2) * W + 8 * by + fg) * 4 + (ex & 3)) = sum;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        bar_sync(4, NT);
+        if (!more) return;
+    }
+}
+
 // ---------------------------------------------------------------- launchers
 
 template <typename R, int J, int MODE>
 static cudaError_t launch_degrid(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out, const DualArgs* a,
-                                 const int32_t* tiles, const int32_t* count, int ctas, cudaStream_t s,
-                                 int batch = 1) {
+                                 cudaStream_t s, int batch = 1) {
     if constexpr (J <= 8)
-        if (p->g_mode == PD_G_CSR) return launch_degrid_csr<R, J, MODE>(p, grid, out, a, tiles, count, ctas, s, batch);
+        if (p->g_mode == PD_G_CSR) return launch_degrid_csr<R, J, MODE>(p, grid, out, a, s, batch);
     const Geo& g = p->g;
     const int ms = std::max(p->max_tile_segs, 1);
     const size_t win = sizeof(R) == 4 ? (size_t)2 * g.ext * ((g.ext + 2) & ~1) : (size_t)g.ext * g.ext;
     const size_t smem = win * sizeof(cplx_t<R>) + (size_t)16 * ms * sizeof(double) + (size_t)(2 * ms + 1) * sizeof(int);
     cudaError_t e = ensure_smem(k_degrid<R, J, MODE>, smem);
     if (e) return e;
-    // CTAs stride over the heaviest-first tile list: launch only as many as are
-    // resident at once, so none starts its share late
+    // items are claimed one at a time: launch only as many CTAs as are resident at once
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid<R, J, MODE>, 256, smem) == cudaSuccess &&
-        per_sm > 0)
-        ctas = std::min(ctas, per_sm * p->num_sms);
-    if ((e = cudaMemsetAsync(p->sched + 4, 0, sizeof(int32_t), s))) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid<R, J, MODE>, 256, smem))) return e;
+    const int ctas = (int)std::min<int64_t>((int64_t)p->n_ditems * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
     k_degrid<R, J, MODE><<<ctas, 256, smem, s>>>(
         grid, out, a ? (const cplx_t<R>*)a->y : nullptr, a ? (const cplx_t<R>*)a->v : nullptr,
         (cplx_t<R>*)p->rbuf, p->cell, (const R*)p->fx, (const R*)p->fy, p->perm, p->seg_start, p->seg_block,
-        p->tile_seg_start, a ? a->block_active : nullptr, tiles, count, p->seg_part, ms, g, R(2.0 / g.J),
-        R(g.beta), p->kbpoly, p->sched + 4, batch, (int64_t)(g.nx / 4 + 1) * 4 * g.Ky, (int64_t)p->M);
+        a ? a->block_active : nullptr, a ? a->ditems : p->ditems, a ? a->nditems : p->counts_all + 2,
+        a ? a->tile_on : nullptr, p->seg_part, ms, g, R(2.0 / g.J), R(g.beta), p->kbpoly, p->sched + 4, batch,
+        (int64_t)(g.nx / 4 + 1) * 4 * g.Ky, (int64_t)p->M);
     return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t degrid_plain(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out_user, cudaStream_t s, int batch) {
-    const int ctas = (int)std::min<int64_t>((int64_t)p->g.ntiles * batch, (int64_t)p->num_sms * 8);
     cudaError_t e = cudaSuccess;
-    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 0>(p, grid, out_user, nullptr, p->tile_order,
-                                                        p->counts_all + 1, ctas, s, batch)));
+    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 0>(p, grid, out_user, nullptr, s, batch)));
     return e;
 }
 
 template <typename R>
-cudaError_t degrid_dual(const pd_plan* p, const cplx_t<R>* grid, const DualArgs& a, const int32_t* tiles,
-                        const int32_t* counts, cudaStream_t s) {
-    const int ctas = std::min(p->g.ntiles, p->num_sms * 8);
+static cudaError_t block_norms(const pd_plan* p, const int32_t* active, const double* eps, double* res_norm,
+                               int norm_only, cudaStream_t s) {
+    k_block_norms<R><<<(p->d * 32 + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_slot_start, p->block_slot_list,
+                                                             active, eps, p->blk_norm, (R*)p->blk_scale, res_norm,
+                                                             p->d, norm_only);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t degrid_dual(const pd_plan* p, const cplx_t<R>* grid, const DualArgs& a, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     prof_mark(PH_DEGRID, 0, s);
-    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 1>(p, grid, nullptr, &a, tiles, counts + 1, ctas, s)));
+    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 1>(p, grid, nullptr, &a, s)));
     prof_mark(PH_DEGRID, 1, s);
     if (e) return e;
     prof_mark(PH_NORMS, 0, s);
-    k_block_norms<R><<<(p->d * 32 + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_seg_start, p->block_seg_list,
-                                                       a.block_active, a.eps, p->blk_norm, (R*)p->blk_scale,
-                                                       a.res_norm, p->d, 0);
+    e = block_norms<R>(p, a.block_active, a.eps, a.res_norm, 0, s);
     prof_mark(PH_NORMS, 1, s);
-    return cudaGetLastError();
+    return e;
 }
 
 template <typename R>
@@ -622,16 +1196,58 @@ cudaError_t degrid_res_norms(const pd_plan* p, const cplx_t<R>* grid, const cplx
                              cudaStream_t s) {
     // every block: the residual part of the pd-mode pass (its r output goes to the
     // plan's scratch and v is not needed, so y stands in for it), then ||G_i b - y_i||
-    const int ctas = std::min(p->g.ntiles, p->num_sms * 8);
-    DualArgs a{y, (void*)y, nullptr, nullptr, res_norm};
+    DualArgs a{y, (void*)y, nullptr, nullptr, res_norm, nullptr, p->ditems, p->counts_all + 2};
     cudaError_t e = cudaSuccess;
-    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 1>(p, grid, nullptr, &a, p->tile_order, p->counts_all + 1,
-                                                        ctas, s)));
-    if (e) return e;
-    k_block_norms<R><<<(p->d * 32 + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_seg_start, p->block_seg_list,
-                                                       nullptr, nullptr, nullptr, nullptr, res_norm, p->d, 1);
+    PD_J_DISPATCH(p->g.J, (e = launch_degrid<R, JJ, 1>(p, grid, nullptr, &a, s)));
+    return e ? e : block_norms<R>(p, nullptr, nullptr, res_norm, 1, s);
+}
+
+// Whether the plan grids with k_grid_mma (FP32 taps evaluated in the kernel, J <= 8, and the
+// segment lists fit), its warps per CTA and its part size.
+void grid_setup(pd_plan* p) {
+    const Geo& g = p->g;
+    const int ms = std::max(p->max_tile_segs, 1);
+    // Seven working warps and the feeding one: 2 CTAs per SM by registers (at 16.8M points on a
+    // 4096^2 grid 3 / 5 / 7 / 10 / 15 working warps take 445 / 415 / 360 / 485 / 448 us).
+    p->grid_warps = 8;
+    // Parts of a tile are added to U one after the other, so only a tile well above a CTA's
+    // share of the points is split (at the same size 2048 points a part cost 23% more than
+    // whole tiles of up to 9100).
+    p->grid_part = (int)std::max<int64_t>(4096, p->M / (2 * p->num_sms));
+    bool ok = p->prec == PD_F32 && g.J <= 8 && p->g_mode == PD_G_ON_THE_FLY && g.tile >= SC;
+    const size_t smem = ok ? grid_mma_smem(g.tile, p->grid_warps - 1, ms) : 0;
+    ok = ok && smem <= (size_t)p->max_smem - 1024;
+    p->grid_smem = ok ? smem : 0;
+}
+
+template <int J, int MODE>
+static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const DualArgs* a, int32_t* pend, float2* U,
+                                   cudaStream_t s, int batch) {
+    const Geo& g = p->g;
+    cudaError_t e;
+    if ((e = ensure_smem(k_grid_mma<J, MODE>, p->grid_smem))) return e;
+    int per_sm = 1;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid_mma<J, MODE>, p->grid_warps * 32,
+                                                           p->grid_smem)))
+        return e;
+    const int ctas = (int)std::min<int64_t>((int64_t)p->n_items * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
+    k_grid_mma<J, MODE><<<ctas, p->grid_warps * 32, p->grid_smem, s>>>(
+        src, (const float2*)p->rbuf, a ? (float2*)a->v : nullptr, (const float*)p->blk_scale,
+        a ? a->block_active : nullptr, p->cell, (const float*)p->fx, (const float*)p->fy, p->perm, p->seg_start,
+        p->seg_block, p->seg_sc_start, p->tile_info, a ? a->tile_on : nullptr, a ? a->items : p->items,
+        a ? a->nitems : p->nitems, pend, U, std::max(p->max_tile_segs, 1), g, p->kbpoly, p->sched + 8, batch,
+        (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     return cudaGetLastError();
 }
+
+#define PD_J8_DISPATCH(J_, CALL)                         \
+    switch (J_) {                                        \
+        case 2: { constexpr int JJ = 2; CALL; } break;   \
+        case 4: { constexpr int JJ = 4; CALL; } break;   \
+        case 6: { constexpr int JJ = 6; CALL; } break;   \
+        case 8: { constexpr int JJ = 8; CALL; } break;   \
+        default: return cudaErrorInvalidValue;           \
+    }
 
 template <typename R, int J, int MODE>
 static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const DualArgs* a, const int32_t* tiles,
@@ -658,7 +1274,7 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
             ctas8 = std::min(ctas8, per_sm * p->num_sms);
         k_grid8w<R, J, MODE><<<ctas8, nw * 32, smem8, s>>>(
             src, rb, vv, (const R*)p->blk_scale, act, p->cell, (const R*)p->fx, (const R*)p->fy, p->perm,
-            p->seg_start, p->seg_block, p->tile_seg_start, p->seg_sc_start, tiles, count, U, ms, g, toj, beta,
+            p->seg_start, p->seg_block, p->tile_seg_start, p->seg_sc_start, tiles, count, a ? a->tile_on : nullptr, U, ms, g, toj, beta,
             p->kbpoly, next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     } else {
         const size_t smem = (size_t)2 * g.ext * g.ext * sizeof(R) + lists;
@@ -667,7 +1283,7 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
             k_grid<R, J, MODE><<<ctas, 256, smem, s>>>(src ? src + (int64_t)b * p->M : src, rb, vv,
                                                       (const R*)p->blk_scale, act, p->cell, (const R*)p->fx,
                                                       (const R*)p->fy, p->perm, p->seg_start, p->seg_block,
-                                                      p->tile_seg_start, tiles, count,
+                                                      p->tile_seg_start, tiles, count, a ? a->tile_on : nullptr,
                                                       U + (int64_t)b * g.Kx * g.Ky, ms, g, toj, beta, p->kbpoly);
     }
     return cudaGetLastError();
@@ -678,10 +1294,19 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
 template <typename R>
 static cudaError_t launch_grid(const pd_plan* p, int mode, const cplx_t<R>* src, const DualArgs* a,
                                const int32_t* const* tiles, const int32_t* counts4, cplx_t<R>* U, cudaStream_t s,
-                               int batch = 1) {
+                               int batch = 1, int32_t* pend = nullptr) {
     const Geo& g = p->g;
     cudaError_t e = cudaSuccess;
     prof_mark(PH_GRID, 0, s);
+    if constexpr (sizeof(R) == 4) {
+        if (p->grid_smem) {
+            int32_t* pd = pend ? pend : p->pend;
+            if (mode == 0) PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 0>(p, src, a, pd, U, s, batch)))
+            else PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 1>(p, src, a, pd, U, s, 1)))
+            prof_mark(PH_GRID, 1, s);
+            return e;
+        }
+    }
     if ((e = cudaMemsetAsync(p->sched, 0, 4 * sizeof(int32_t), s))) return e;
     for (int c = 0; c < 4 && !e; ++c) {
         if (mode == 0) {
@@ -697,13 +1322,16 @@ static cudaError_t launch_grid(const pd_plan* p, int mode, const cplx_t<R>* src,
 }
 
 template <typename R>
-cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch) {
+cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch, int32_t* pend) {
     // U = G^T y: every window is added to a zeroed grid
-    cudaError_t e = cudaMemsetAsync(U, 0, (size_t)batch * p->g.Kx * p->g.Ky * sizeof(cplx_t<R>), s);
+    cudaError_t e;
+    const int64_t cells = (int64_t)batch * p->g.Kx * p->g.Ky;
+    if (p->grid_smem) e = grid_begin(p, nullptr, pend ? pend : p->pend, (float4*)U, cells / 2, batch, s);
+    else e = cudaMemsetAsync(U, 0, (size_t)cells * sizeof(cplx_t<R>), s);
     if (e) return e;
     const int q = p->g.ntiles / 4;
     const int32_t* lists[4] = {p->colour_tiles, p->colour_tiles + q, p->colour_tiles + 2 * q, p->colour_tiles + 3 * q};
-    return launch_grid<R>(p, 0, y_user, nullptr, lists, p->colour_counts, U, s, batch);
+    return launch_grid<R>(p, 0, y_user, nullptr, lists, p->colour_counts, U, s, batch, pend);
 }
 
 template <typename R>
@@ -716,12 +1344,10 @@ template cudaError_t degrid_plain<float>(const pd_plan*, const float2*, float2*,
 template cudaError_t degrid_plain<double>(const pd_plan*, const double2*, double2*, cudaStream_t, int);
 template cudaError_t degrid_res_norms<float>(const pd_plan*, const float2*, const float2*, double*, cudaStream_t);
 template cudaError_t degrid_res_norms<double>(const pd_plan*, const double2*, const double2*, double*, cudaStream_t);
-template cudaError_t degrid_dual<float>(const pd_plan*, const float2*, const DualArgs&, const int32_t*,
-                                        const int32_t*, cudaStream_t);
-template cudaError_t degrid_dual<double>(const pd_plan*, const double2*, const DualArgs&, const int32_t*,
-                                         const int32_t*, cudaStream_t);
-template cudaError_t grid_plain<float>(const pd_plan*, const float2*, float2*, cudaStream_t, int);
-template cudaError_t grid_plain<double>(const pd_plan*, const double2*, double2*, cudaStream_t, int);
+template cudaError_t degrid_dual<float>(const pd_plan*, const float2*, const DualArgs&, cudaStream_t);
+template cudaError_t degrid_dual<double>(const pd_plan*, const double2*, const DualArgs&, cudaStream_t);
+template cudaError_t grid_plain<float>(const pd_plan*, const float2*, float2*, cudaStream_t, int, int32_t*);
+template cudaError_t grid_plain<double>(const pd_plan*, const double2*, double2*, cudaStream_t, int, int32_t*);
 template cudaError_t grid_dual<float>(const pd_plan*, const DualArgs&, const int32_t* const*, const int32_t*,
                                       float2*, cudaStream_t);
 template cudaError_t grid_dual<double>(const pd_plan*, const DualArgs&, const int32_t* const*, const int32_t*,

@@ -19,11 +19,13 @@ __device__ __forceinline__ void kb_taps(R frac, R* w, R two_over_j, R beta, cons
         for (int a = 0; a < J / 2; ++a) {
             float ev = kp.c[a][KB_DEG], od = kp.c[a][KB_DEG - 1];
 #pragma unroll
-            for (int k = KB_DEG - 2; k >= 0; k -= 2) ev = fmaf(ev, x2, kp.c[a][k]);
+            for (int k = KB_DEG - 2; k >= 2; k -= 2) ev = fmaf(ev, x2, kp.c[a][k]);
 #pragma unroll
             for (int k = KB_DEG - 3; k >= 1; k -= 2) od = fmaf(od, x2, kp.c[a][k]);
-            w[a] = fmaf(x, od, ev);
-            w[J - 1 - a] = fmaf(-x, od, ev);
+            // the constant term last, with the part that its rounding left: one rounding of w
+            ev = fmaf(ev, x2, kp.lo[a]);
+            w[a] = kp.c[a][0] + fmaf(x, od, ev);
+            w[J - 1 - a] = kp.c[a][0] + fmaf(-x, od, ev);
         }
     } else {
 #pragma unroll
@@ -98,7 +100,7 @@ template <typename R, int MODE>
 __device__ __forceinline__ cplx_t<R> grid_value(int m, const cplx_t<R>* __restrict__ src,
                                                 const cplx_t<R>* __restrict__ rbuf, cplx_t<R>* __restrict__ v,
                                                 const int32_t* __restrict__ perm, R sc) {
-    if (MODE == 0) return src[perm[m]];
+    if (MODE == 0) return vis_conj(perm[m], src[vis_index(perm[m])]);
     const cplx_t<R> r = rbuf[m], vo = v[m];
     const cplx_t<R> vn = cscale(r, sc);
     v[m] = vn;
@@ -110,7 +112,7 @@ __device__ __forceinline__ cplx_t<R> grid_value(int m, const cplx_t<R>* __restri
 template <typename R, class V>
 __device__ __forceinline__ void add_window(cplx_t<R>* __restrict__ U, int oy, int ox, const Geo& g, const V& val) {
     using C2 = cplx_t<R>;
-    const int E = g.ext, H = g.halo_lo;
+    const int E = g.ext;
     constexpr int EB = 8;
     for (int i0 = threadIdx.x; i0 < E * E; i0 += EB * (int)blockDim.x) {
         C2 uo[EB];
@@ -121,7 +123,7 @@ __device__ __forceinline__ void add_window(cplx_t<R>* __restrict__ U, int oy, in
             off[k] = -1;
             if (i < E * E) {
                 const int ey = i / E, ex = i - ey * E;
-                off[k] = panel_off((oy - H + ey) & (g.Ky - 1), (ox - H + ex) & (g.Kx - 1), g.Ky);
+                off[k] = panel_off((oy + ey) & (g.Ky - 1), (ox + ex) & (g.Kx - 1), g.Ky);
                 uo[k] = U[off[k]];
             }
         }
@@ -132,6 +134,35 @@ __device__ __forceinline__ void add_window(cplx_t<R>* __restrict__ U, int oy, in
             const int ey = i / E, ex = i - ey * E;
             U[off[k]] = cadd(uo[k], val(ey, ex));
         }
+    }
+}
+
+// Thread 0: the next item (claimed in order by whichever CTA is free) whose tile is on, for
+// image w mod batch of a batch, into *it; its number is returned (>= n * batch: none left).
+__device__ __forceinline__ int claim_item(int* sched, const TileItem* __restrict__ items, int n, int batch,
+                                          const int32_t* __restrict__ tile_on, TileItem* it) {
+    for (;;) {
+        const int w = atomicAdd(sched, 1);
+        if (w >= n * batch) return w;
+        const TileItem t = items[w / batch];
+        if (tile_on && !tile_on[t.tile]) continue;
+        *it = t;
+        return w;
+    }
+}
+// The same over a list of tiles.
+__device__ __forceinline__ int claim_tile(int* next, const int32_t* __restrict__ list, int n, int batch,
+                                          const int32_t* __restrict__ tile_on) {
+    for (;;) {
+        const int w = atomicAdd(next, 1);
+        if (w >= n * batch || !tile_on || tile_on[list[w / batch]]) return w;
+    }
+}
+// Thread 0 of each CTA at the end: the last one sets the counters back for the next launch.
+__device__ __forceinline__ void leave_items(int* sched) {
+    if (atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
+        sched[0] = 0;
+        sched[1] = 0;
     }
 }
 
@@ -153,7 +184,7 @@ __device__ __forceinline__ void add_window(cplx_t<R>* __restrict__ U, int oy, in
 // g_mode is PD_G_CSR.
 template <typename R, int J, int MODE>
 cudaError_t launch_degrid_csr(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out, const DualArgs* a,
-                              const int32_t* tiles, const int32_t* count, int ctas, cudaStream_t s, int batch);
+                              cudaStream_t s, int batch);
 template <typename R, int J, int MODE>
 cudaError_t launch_grid_csr(const pd_plan* p, const cplx_t<R>* src, const DualArgs* a, const int32_t* tiles,
                             const int32_t* count, cplx_t<R>* U, int* next_tile, cudaStream_t s, int batch);

@@ -42,10 +42,10 @@ __global__ void k_build_csr(const int32_t* __restrict__ cell, const R* __restric
     R* vp = val + m * (J * J);
 #pragma unroll
     for (int b = 0; b < J; ++b) {
-        const int ky = (by - g.halo_lo + b) & (g.Ky - 1);
+        const int ky = (by + b) & (g.Ky - 1);
 #pragma unroll
         for (int a = 0; a < J; ++a) {
-            cp[b * J + a] = (ky << 16) | ((bx - g.halo_lo + a) & (g.Kx - 1));
+            cp[b * J + a] = (ky << 16) | ((bx + a) & (g.Kx - 1));
             vp[b * J + a] = (R)(wy[b] * wx[a]);
         }
     }
@@ -53,8 +53,8 @@ __global__ void k_build_csr(const int32_t* __restrict__ cell, const R* __restric
 
 // Row m of the DDE-aware G (Sec. 2): the JK x JK interpolation kernel convolved with the
 // point's d x d Fourier-domain DDE kernel D_m (offsets -h .. h), a footprint of
-// g.J = JK + d - 1 cells per axis starting g.halo_lo = JK/2 - 1 + h cells before the base
-// cell. Entry (b', a') = sum over b + i = b', a + j = a' of phi_y(b) phi_x(a) D_m[i][j],
+// g.J = JK + d - 1 cells per axis from the point's cell (JK/2 - 1 + h before floor(g)) on.
+// Entry (b', a') = sum over b + i = b', a + j = a' of phi_y(b) phi_x(a) D_m[i][j],
 // summed in FP64 and rounded once.
 template <typename R, int JK>
 __global__ void k_build_csr_dde(const int32_t* __restrict__ cell, const R* __restrict__ fxs,
@@ -75,7 +75,7 @@ __global__ void k_build_csr_dde(const int32_t* __restrict__ cell, const R* __res
     int32_t* cp = col + m * Jf * Jf;
     cplx_t<R>* vp = val + m * Jf * Jf;
     for (int bq = 0; bq < Jf; ++bq) {
-        const int ky = (by - g.halo_lo + bq) & (g.Ky - 1);
+        const int ky = (by + bq) & (g.Ky - 1);
         for (int aq = 0; aq < Jf; ++aq) {
             double re = 0.0, im = 0.0;
             for (int i = 0; i < dw; ++i) {
@@ -89,7 +89,7 @@ __global__ void k_build_csr_dde(const int32_t* __restrict__ cell, const R* __res
                     im += w * D[i * dw + j].y;
                 }
             }
-            cp[bq * Jf + aq] = (ky << 16) | ((bx - g.halo_lo + aq) & (g.Kx - 1));
+            cp[bq * Jf + aq] = (ky << 16) | ((bx + aq) & (g.Kx - 1));
             vp[bq * Jf + aq] = mk<cplx_t<R>>((R)re, (R)im);
         }
     }
@@ -189,33 +189,34 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
     const cplx_t<R>* __restrict__ grid, cplx_t<R>* __restrict__ out, const cplx_t<R>* __restrict__ y,
     const cplx_t<R>* __restrict__ v, cplx_t<R>* __restrict__ rbuf, const int32_t* __restrict__ col,
     const W* __restrict__ val, const int32_t* __restrict__ perm, const int32_t* __restrict__ seg_start,
-    const int32_t* __restrict__ seg_block, const int32_t* __restrict__ tile_seg_start,
-    const int32_t* __restrict__ active, const int32_t* __restrict__ list, const int32_t* __restrict__ count,
-    double* __restrict__ seg_part, int max_segs, Geo g, int* __restrict__ next_tile, int batch, int64_t gstride,
-    int64_t ostride) {
+    const int32_t* __restrict__ seg_block, const int32_t* __restrict__ active, const TileItem* __restrict__ items,
+    const int32_t* __restrict__ nitems, const int32_t* __restrict__ tile_on, double* __restrict__ seg_part,
+    int max_segs, Geo g, int* __restrict__ sched, int batch, int64_t gstride, int64_t ostride) {
     using C2 = cplx_t<R>;
     constexpr int GL = 8;   // lanes per visibility, lane b of a group on footprint row b (b < J)
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int E = g.ext, H = g.halo_lo;
+    const int E = g.ext;
     C2* win = reinterpret_cast<C2*>(smraw);                              // [E][E]
     double* part = reinterpret_cast<double*>(win + E * E + (E * E & 1)); // [8 warps][max_segs][2]
     int* act_seg = reinterpret_cast<int*>(part + 16 * max_segs);
     int* act_pre = act_seg + max_segs;
-    __shared__ int nact_s, tile_s;
+    __shared__ int nact_s, item_s;
+    __shared__ TileItem ti_s;
     const int warp = threadIdx.x >> 5, grp = threadIdx.x / GL, b = threadIdx.x % GL;
     const int ngrp = blockDim.x / GL;
-    const int n = *count;
+    const int n = *nitems;
+    if (threadIdx.x == 0) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
     for (;;) {
-        if (threadIdx.x == 0) tile_s = atomicAdd(next_tile, 1);
         __syncthreads();
-        const int w = tile_s;
+        const int w = item_s;
         if (w >= n * batch) break;
-        const int t = list[w / batch], img = w % batch;
+        const TileItem ti = ti_s;
+        const int t = ti.tile, img = w % batch;
         const C2* gimg = grid + (int64_t)img * gstride;
         C2* oimg = MODE == 0 ? out + (int64_t)img * ostride : out;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
-        const int wy0 = ty * g.tile - H, wx0 = tx * g.tile - H;     // window origin (unwrapped)
-        const int seg0 = tile_seg_start[t], nseg_t = tile_seg_start[t + 1] - seg0;
+        const int wy0 = ty * g.tile, wx0 = tx * g.tile;     // window origin
+        const int seg0 = ti.seg0, nseg_t = ti.nseg;
         list_active_segments(seg0, nseg_t, seg_block, MODE == 1 ? active : nullptr, seg_start, act_seg, act_pre,
                              &nact_s);
         for (int i = threadIdx.x; i < E * E; i += blockDim.x) {
@@ -225,10 +226,12 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
         if (MODE == 1)
             for (int i = threadIdx.x; i < 16 * nseg_t; i += blockDim.x) part[i] = 0.0;
         __syncthreads();
-        const int nact = nact_s, total = act_pre[nact];
+        // this part's positions of the tile's active points
+        const int nact = nact_s, all = act_pre[nact];
+        const int first = (int)((int64_t)all * ti.part / ti.parts), total = (int)((int64_t)all * (ti.part + 1) / ti.parts);
         double* mypart = part + 2 * nseg_t * warp;
         int j = 0;
-        for (int base = 0; base < total; base += ngrp) {
+        for (int base = first; base < total; base += ngrp) {
             const int pos = base + grp;
             const bool ok = pos < total;
             int m = 0;
@@ -256,7 +259,7 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
             R ar = R(0), ad = R(0);
             if (lead) {
                 if (MODE == 0) {
-                    oimg[perm[m]] = mk<C2>(sx, sy);
+                    oimg[vis_index(perm[m])] = vis_conj(perm[m], mk<C2>(sx, sy));
                 } else {
                     const C2 yy = y[m], vv = v[m];
                     const R dx = sx - yy.x, dy = sy - yy.y;
@@ -269,6 +272,7 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
             if (MODE == 1) warp_seg_add(lead, j, ar, ad, mypart);
         }
         __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
         if (MODE == 1) {
             for (int k = threadIdx.x; k < nact; k += blockDim.x) {
                 double sr = 0.0, sd = 0.0;
@@ -276,17 +280,18 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
                     sr += part[2 * nseg_t * wp + 2 * k];
                     sd += part[2 * nseg_t * wp + 2 * k + 1];
                 }
-                seg_part[2 * act_seg[k]] = sr;
-                seg_part[2 * act_seg[k] + 1] = sd;
+                const int64_t slot = (int64_t)ti.slot0 + act_seg[k] - seg0;
+                seg_part[2 * slot] = sr;
+                seg_part[2 * slot + 1] = sd;
             }
         }
-        __syncthreads();
     }
+    if (threadIdx.x == 0) leave_items(sched);
 }
 
 template <typename R, typename W, int J, int MODE>
 static cudaError_t degrid_csr_w(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out, const DualArgs* a,
-                                const int32_t* tiles, const int32_t* count, int ctas, cudaStream_t s, int batch) {
+                                cudaStream_t s, int batch) {
     const Geo& g = p->g;
     const int ms = std::max(p->max_tile_segs, 1);
     const size_t win = (size_t)g.ext * g.ext + (g.ext * g.ext & 1);
@@ -294,23 +299,22 @@ static cudaError_t degrid_csr_w(const pd_plan* p, const cplx_t<R>* grid, cplx_t<
     cudaError_t e = ensure_smem(k_degrid_csr<R, W, J, MODE>, smem);
     if (e) return e;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid_csr<R, W, J, MODE>, 256, smem) ==
-            cudaSuccess && per_sm > 0)
-        ctas = std::min(ctas, per_sm * p->num_sms);
-    if ((e = cudaMemsetAsync(p->sched + 4, 0, sizeof(int32_t), s))) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid_csr<R, W, J, MODE>, 256, smem))) return e;
+    const int ctas = (int)std::min<int64_t>((int64_t)p->n_ditems * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
     k_degrid_csr<R, W, J, MODE><<<ctas, 256, smem, s>>>(
         grid, out, a ? (const cplx_t<R>*)a->y : nullptr, a ? (const cplx_t<R>*)a->v : nullptr,
         (cplx_t<R>*)p->rbuf, p->csr_col, (const W*)p->csr_val, p->perm, p->seg_start, p->seg_block,
-        p->tile_seg_start, a ? a->block_active : nullptr, tiles, count, p->seg_part, ms, g, p->sched + 4, batch,
-        (int64_t)(g.nx / 4 + 1) * 4 * g.Ky, (int64_t)p->M);
+        a ? a->block_active : nullptr, a ? a->ditems : p->ditems, a ? a->nditems : p->counts_all + 2,
+        a ? a->tile_on : nullptr, p->seg_part, ms, g, p->sched + 4, batch, (int64_t)(g.nx / 4 + 1) * 4 * g.Ky,
+        (int64_t)p->M);
     return cudaGetLastError();
 }
 
 template <typename R, int J, int MODE>
 cudaError_t launch_degrid_csr(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out, const DualArgs* a,
-                              const int32_t* tiles, const int32_t* count, int ctas, cudaStream_t s, int batch) {
-    return p->csr_cplx ? degrid_csr_w<R, cplx_t<R>, J, MODE>(p, grid, out, a, tiles, count, ctas, s, batch)
-                       : degrid_csr_w<R, R, J, MODE>(p, grid, out, a, tiles, count, ctas, s, batch);
+                              cudaStream_t s, int batch) {
+    return p->csr_cplx ? degrid_csr_w<R, cplx_t<R>, J, MODE>(p, grid, out, a, s, batch)
+                       : degrid_csr_w<R, R, J, MODE>(p, grid, out, a, s, batch);
 }
 
 // ---------------------------------------------------------------- gridding
@@ -353,7 +357,7 @@ __device__ __forceinline__ void grid_raw(GridRaw<R>& in, int pos, int& j, const 
         in.b = v[m];
         in.sc = scale[seg_block[sg]];
     } else {
-        in.a = src[perm[m]];
+        in.a = vis_conj(perm[m], src[vis_index(perm[m])]);
     }
 }
 
@@ -375,13 +379,13 @@ __global__ void __launch_bounds__(256, 2) k_grid_csr(
     const R* __restrict__ scale, const int32_t* __restrict__ active, const int32_t* __restrict__ col,
     const W* __restrict__ val, const int32_t* __restrict__ perm, const int32_t* __restrict__ seg_start,
     const int32_t* __restrict__ seg_block, const int32_t* __restrict__ tile_seg_start,
-    const int32_t* __restrict__ list, const int32_t* __restrict__ count, cplx_t<R>* __restrict__ U, int max_segs,
-    Geo g, int* __restrict__ next_tile, int batch, int64_t sstride, int64_t ustride) {
+    const int32_t* __restrict__ list, const int32_t* __restrict__ count, const int32_t* __restrict__ tile_on,
+    cplx_t<R>* __restrict__ U, int max_segs, Geo g, int* __restrict__ next_tile, int batch, int64_t sstride, int64_t ustride) {
     using C2 = cplx_t<R>;
     constexpr int NE = J * J;                 // entries per row of G (<= 64: two per lane)
     constexpr int PB = 8;                     // visibilities whose entries are loaded together
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int E = g.ext, EE = E * E, H = g.halo_lo;
+    const int E = g.ext, EE = E * E;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     C2* wins = reinterpret_cast<C2*>(smraw);                 // [nw][E][E]
     int* act_seg = reinterpret_cast<int*>(wins + (size_t)nw * EE);
@@ -392,7 +396,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_csr(
     const int e0 = 2 * lane;
     const bool has = e0 < NE;                 // J^2 is even: entries e0, e0 + 1 together
     for (;;) {
-        if (threadIdx.x == 0) tile_s = atomicAdd(next_tile, 1);
+        if (threadIdx.x == 0) tile_s = claim_tile(next_tile, list, n, batch, tile_on);
         __syncthreads();
         const int w = tile_s;
         if (w >= n * batch) break;
@@ -401,7 +405,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_csr(
         C2* uimg = U + (int64_t)img * ustride;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
         const int oy = ty * g.tile, ox = tx * g.tile;
-        const int wy0 = oy - H, wx0 = ox - H;
+        const int wy0 = oy, wx0 = ox;
         const int seg0 = tile_seg_start[t], nseg_t = tile_seg_start[t + 1] - seg0;
         list_active_segments(seg0, nseg_t, seg_block, MODE == 1 ? active : nullptr, seg_start, act_seg, act_pre,
                              &nact_s);
@@ -481,7 +485,7 @@ static cudaError_t grid_csr_w(const pd_plan* p, const cplx_t<R>* src, const Dual
     k_grid_csr<R, W, J, MODE><<<ctas, nw * 32, smem, s>>>(
         src, (const cplx_t<R>*)p->rbuf, a ? (cplx_t<R>*)a->v : nullptr, (const R*)p->blk_scale,
         a ? a->block_active : nullptr, p->csr_col, (const W*)p->csr_val, p->perm, p->seg_start, p->seg_block,
-        p->tile_seg_start, tiles, count, U, ms, g, next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
+        p->tile_seg_start, tiles, count, a ? a->tile_on : nullptr, U, ms, g, next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     return cudaGetLastError();
 }
 
@@ -494,11 +498,9 @@ cudaError_t launch_grid_csr(const pd_plan* p, const cplx_t<R>* src, const DualAr
 
 #define PD_CSR_INST(R_, J_)                                                                                      \
     template cudaError_t launch_degrid_csr<R_, J_, 0>(const pd_plan*, const cplx_t<R_>*, cplx_t<R_>*,            \
-                                                      const DualArgs*, const int32_t*, const int32_t*, int,      \
-                                                      cudaStream_t, int);                                        \
+                                                      const DualArgs*, cudaStream_t, int);                       \
     template cudaError_t launch_degrid_csr<R_, J_, 1>(const pd_plan*, const cplx_t<R_>*, cplx_t<R_>*,            \
-                                                      const DualArgs*, const int32_t*, const int32_t*, int,      \
-                                                      cudaStream_t, int);                                        \
+                                                      const DualArgs*, cudaStream_t, int);                       \
     template cudaError_t launch_grid_csr<R_, J_, 0>(const pd_plan*, const cplx_t<R_>*, const DualArgs*,          \
                                                     const int32_t*, const int32_t*, cplx_t<R_>*, int*,           \
                                                     cudaStream_t, int);                                          \

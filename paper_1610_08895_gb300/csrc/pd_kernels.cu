@@ -11,201 +11,165 @@ namespace pdgb {
 
 constexpr int SEL_NT = 1024;
 
-// Exclusive scan of per-thread counts over a 1024-thread block; returns the total.
-__device__ int block_excl_scan(int v, int* sh, int& excl) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) sh[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        int w = sh[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        sh[lane] = w;
-    }
-    __syncthreads();
-    const int before = warp > 0 ? sh[warp - 1] : 0;
-    excl = before + x - v;
-    const int total = sh[31];
-    __syncthreads();
-    return total;
+// Tile t of the heaviest-first list: on if a block with points in it is active; its flag for
+// the degridding and gridding launches, the parts that the gridding has to add for it, and
+// the numbers of active segments and tiles.
+__device__ __forceinline__ void flag_tile(int t, const int4* __restrict__ tile_info, const int32_t* __restrict__ seg_block,
+                                          const int32_t* block_active, int32_t* __restrict__ tile_on,
+                                          int32_t* __restrict__ pend, int& segs, int& tiles) {
+    const int4 ti = tile_info[t];
+    int n = 0;
+    for (int k = 0; k < ti.y; ++k) n += block_active[seg_block[ti.x + k]];
+    tile_on[t] = n > 0;
+    pend[t] = n > 0 ? ti.z : 0;
+    segs += n;
+    tiles += n > 0;
 }
 
 // Step 3: Philox draws u(seed, t, stream, index) < p for blocks (stream 0) and
 // bases (stream 1); with adaptive = 1 the block probabilities are first set by
 // eq. (prob-choice) from the current residual norms. Then the tiles holding a
-// visibility of an active block are compacted, heaviest first, into the list read
-// by the persistent degridding and gridding launches.
+// visibility of an active block are flagged (here for up to SEL_TILES tiles, one or two a
+// thread; more of them in k_flag_tiles, where every SM takes part).
+constexpr int SEL_TILES = 2 * SEL_NT;
+constexpr int SEL_D = 4096 / SEL_NT;      // blocks per thread at most
 __global__ void __launch_bounds__(SEL_NT) k_select(
     uint64_t seed, int adaptive, double an, double pmin, double pmax, int64_t* __restrict__ tptr,
     double* __restrict__ p_block, const double* __restrict__ p_basis, const double* __restrict__ res_norm,
     const double* __restrict__ eps, int d, int b, int32_t* __restrict__ block_active,
-    int32_t* __restrict__ basis_active, const int32_t* __restrict__ tile_order,
-    const int32_t* __restrict__ tile_seg_start, const int32_t* __restrict__ seg_block, int ntiles,
-    int32_t* __restrict__ tile_active, int32_t* __restrict__ act_tiles, int32_t* __restrict__ act_col, int ntx,
+    int32_t* __restrict__ basis_active, const int32_t* __restrict__ tile_order, const int4* __restrict__ tile_info,
+    const int32_t* __restrict__ seg_block, int ntiles, int32_t* __restrict__ tile_on, int32_t* __restrict__ pend,
     int32_t* __restrict__ counts) {
-    __shared__ int shi[32];
     __shared__ double shd[32];
-    __shared__ double q_sh, cap_sh;
     __shared__ int64_t t_sh;
+    __shared__ int cnt_sh[2];
     const int tid = threadIdx.x;
     if (tid == 0) {
         const int64_t t = *tptr + 1;
         *tptr = t;
         t_sh = t;
+        cnt_sh[0] = cnt_sh[1] = 0;
     }
+    __syncthreads();
     if (adaptive) {
         // c_i = max(||r_i|| - eps_i, 0)^2 / eps_i^2; p_i = p_min + min(q_i + a, p_max - p_min)
-        double csum = 0.0;
-        for (int i = tid; i < d; i += SEL_NT) {
-            const double e = eps[i], r = res_norm[i];
-            const double c = r > e ? (r - e) * (r - e) / (e * e) : 0.0;
-            csum += c;
+        double c[SEL_D], csum = 0.0;
+#pragma unroll
+        for (int u = 0; u < SEL_D; ++u) {
+            const int i = tid + u * SEL_NT;
+            c[u] = 0.0;
+            if (i < d) {
+                const double e = eps[i], r = res_norm[i];
+                c[u] = r > e ? (r - e) * (r - e) / (e * e) : 0.0;
+            }
+            csum += c[u];
         }
-        csum = block_sum(csum, shd);
-        if (tid == 0) shd[0] = csum;
-        __syncthreads();
-        csum = shd[0];
-        __syncthreads();
-        const double cap = pmax - pmin;
-        const double target = an - d * pmin;
+        auto all_sum = [&](double v) {
+            v = block_sum(v, shd);
+            if (tid == 0) shd[0] = v;
+            __syncthreads();
+            v = shd[0];
+            __syncthreads();
+            return v;
+        };
+        csum = all_sum(csum);
+        const double cap = pmax - pmin, target = an - d * pmin;
         if (csum == 0.0) {
             for (int i = tid; i < d; i += SEL_NT) p_block[i] = an / d;
         } else {
             const double qs = target / csum;
-            // a = 0 unless some q_i exceeds the cap (then some p_i saturates at p_max)
+            // a = 0 unless some q_i exceeds the cap (then some p_i saturates at p_max). f(a) =
+            // sum min(q_i + a, cap) is concave, so Newton's steps from 0 stay left of the root and
+            // each one passes a breakpoint or lands on it: a handful of steps instead of a bisection
+            // to double precision (80 steps of one block-wide sum each)
+            double a = 0.0;
             int sat = 0;
-            for (int i = tid; i < d; i += SEL_NT) {
-                const double e = eps[i], r = res_norm[i];
-                const double c = r > e ? (r - e) * (r - e) / (e * e) : 0.0;
-                sat |= (qs * c > cap);
-            }
+#pragma unroll
+            for (int u = 0; u < SEL_D; ++u) sat |= qs * c[u] > cap;
             sat = __syncthreads_or(sat);
-            double lo = 0.0, hi = 0.0;
-            if (sat) {
-                // f(a) = sum min(q_i + a, cap) is non-decreasing: bisection to double precision
-                hi = cap;
-                for (int it = 0; it < 80; ++it) {
-                    const double mid = 0.5 * (lo + hi);
-                    double f = 0.0;
-                    for (int i = tid; i < d; i += SEL_NT) {
-                        const double e = eps[i], r = res_norm[i];
-                        const double c = r > e ? (r - e) * (r - e) / (e * e) : 0.0;
-                        f += fmin(qs * c + mid, cap);
-                    }
-                    f = block_sum(f, shd);
-                    if (tid == 0) shd[0] = f;
-                    __syncthreads();
-                    f = shd[0];
-                    __syncthreads();
-                    if (f < target) lo = mid; else hi = mid;
+            for (int it = 0; sat && it <= d; ++it) {
+                double f = 0.0, fr = 0.0;
+#pragma unroll
+                for (int u = 0; u < SEL_D; ++u) {
+                    if (tid + u * SEL_NT >= d) break;
+                    const double q = qs * c[u] + a;
+                    f += fmin(q, cap);
+                    fr += q < cap ? 1.0 : 0.0;
                 }
+                f = all_sum(f);
+                fr = all_sum(fr);
+                const double next = fr > 0.0 ? a + (target - f) / fr : a;
+                if (!(next > a)) break;
+                a = next;
             }
-            if (tid == 0) { q_sh = qs; cap_sh = hi; }
-            __syncthreads();
-            const double a = cap_sh;
-            for (int i = tid; i < d; i += SEL_NT) {
-                const double e = eps[i], r = res_norm[i];
-                const double c = r > e ? (r - e) * (r - e) / (e * e) : 0.0;
-                p_block[i] = pmin + fmin(q_sh * c + a, cap);
-            }
+#pragma unroll
+            for (int u = 0; u < SEL_D; ++u)
+                if (tid + u * SEL_NT < d) p_block[tid + u * SEL_NT] = pmin + fmin(qs * c[u] + a, cap);
         }
     }
     __syncthreads();
     const int64_t t = t_sh;
     for (int i = tid; i < d; i += SEL_NT) block_active[i] = philox_uniform(seed, (uint64_t)t, 0, i) < p_block[i];
     for (int j = tid; j < b; j += SEL_NT) basis_active[j] = philox_uniform(seed, (uint64_t)t, 1, j) < p_basis[j];
-    __syncthreads();
-    // active tiles, in the static heaviest-first order (all of them for the degridding,
-    // and split by colour for the gridding); count active segments too
-    {
-        const int per = (ntiles + SEL_NT - 1) / SEL_NT;
-        const int k0 = min(ntiles, tid * per), k1 = min(ntiles, k0 + per);
-        int mine = 0, segs = 0, mc[4] = {0, 0, 0, 0};
-        // the flags of this thread's tiles, kept in registers for the compaction pass
-        // below (up to 128 tiles per thread; beyond that it reads tile_active back)
-        constexpr int FW = 4;
-        uint32_t onm[FW] = {0u, 0u, 0u, 0u};
-        // batches of tiles whose independent loads go out together
-        constexpr int TB = 8;
-        for (int kb = k0; kb < k1; kb += TB) {
-            int tt[TB], s0[TB], s1[TB];
-#pragma unroll
-            for (int i = 0; i < TB; ++i) tt[i] = kb + i < k1 ? tile_order[kb + i] : -1;
-#pragma unroll
-            for (int i = 0; i < TB; ++i) {
-                s0[i] = tt[i] >= 0 ? tile_seg_start[tt[i]] : 0;
-                s1[i] = tt[i] >= 0 ? tile_seg_start[tt[i] + 1] : 0;
-            }
-#pragma unroll
-            for (int i = 0; i < TB; ++i) {
-                if (tt[i] < 0) continue;
-                int on = 0;
-                for (int sg = s0[i]; sg < s1[i]; ++sg) {
-                    const int a = block_active[seg_block[sg]];
-                    on |= a;
-                    segs += a;
-                }
-                tile_active[tt[i]] = on;
-                const int li = kb + i - k0;
-#pragma unroll
-                for (int f = 0; f < FW; ++f)
-                    if (on && (li >> 5) == f) onm[f] |= 1u << (li & 31);
-                mine += on;
-                const int col = tile_colour(tt[i], ntx);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) mc[c] += on && col == c;
-            }
-        }
-        int excl, sexcl, cex[4];
-        const int total = block_excl_scan(mine, shi, excl);
-        const int stotal = block_excl_scan(segs, shi, sexcl);
-        int ctot[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ctot[c] = block_excl_scan(mc[c], shi, cex[c]);
-        const int q = ntiles / 4;
-        for (int k = k0; k < k1; ++k) {
-            const int li = k - k0;
-            bool on;
-            if (li < 32 * FW) {
-                uint32_t w = onm[0];
-#pragma unroll
-                for (int f = 1; f < FW; ++f) w = (li >> 5) == f ? onm[f] : w;
-                on = (w >> (li & 31)) & 1u;
-            } else {
-                on = tile_active[tile_order[k]];
-            }
-            if (on) {
-                const int tt = tile_order[k];
-                act_tiles[excl++] = tt;
-                const int col = tile_colour(tt, ntx);
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (col == c) act_col[c * q + cex[c]++] = tt;
-            }
-        }
-        if (tid == 0) {
-            counts[0] = stotal;
-            counts[1] = total;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) counts[2 + c] = ctot[c];
-        }
+    if (ntiles > SEL_TILES) {
+        if (tid < 2) counts[tid] = 0;
+        return;
     }
+    __syncthreads();
+    int segs = 0, tiles = 0;
+    for (int k = tid; k < ntiles; k += SEL_NT)
+        flag_tile(tile_order[k], tile_info, seg_block, block_active, tile_on, pend, segs, tiles);
+    if (segs) { atomicAdd(&cnt_sh[0], segs); atomicAdd(&cnt_sh[1], tiles); }
+    __syncthreads();
+    if (tid < 2) counts[tid] = cnt_sh[tid];
+}
+
+__global__ void __launch_bounds__(256) k_flag_tiles(const int32_t* __restrict__ tile_order,
+                                                    const int4* __restrict__ tile_info,
+                                                    const int32_t* __restrict__ seg_block,
+                                                    const int32_t* __restrict__ block_active, int ntiles,
+                                                    int32_t* __restrict__ tile_on, int32_t* __restrict__ pend,
+                                                    int32_t* __restrict__ counts) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    int segs = 0, tiles = 0;
+    if (k < ntiles) flag_tile(tile_order[k], tile_info, seg_block, block_active, tile_on, pend, segs, tiles);
+    segs = __reduce_add_sync(0xffffffffu, segs);
+    tiles = __reduce_add_sync(0xffffffffu, tiles);
+    if ((threadIdx.x & 31) == 0 && segs) { atomicAdd(counts, segs); atomicAdd(counts + 1, tiles); }
 }
 
 cudaError_t select_active(const pd_plan* p, pd_state* st, const SelectArgs& a, cudaStream_t s) {
     prof_mark(PH_SELECT, 0, s);
+    const int nt = p->ntiles_nonempty;
     k_select<<<1, SEL_NT, 0, s>>>(a.seed, a.adaptive, a.n, a.p_min, a.p_max, st->t, st->p_block, st->p_basis,
                                  st->res_norm, st->eps, p->d, p->b, st->block_active, st->basis_active,
-                                 p->tile_order, p->tile_seg_start, p->seg_block, p->g.ntiles,
-                                 st->tile_active, st->act_tiles, st->act_col, p->g.ntx, st->counts);
+                                 p->tile_order, p->tile_info, p->seg_block, nt, st->tile_active, p->pend, st->counts);
+    if (nt > SEL_TILES)
+        k_flag_tiles<<<(nt + 255) / 256, 256, 0, s>>>(p->tile_order, p->tile_info, p->seg_block, st->block_active, nt,
+                                                      st->tile_active, p->pend, st->counts);
     prof_mark(PH_SELECT, 1, s);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) k_grid_begin(const int4* __restrict__ tile_info, const int32_t* __restrict__ seg_block,
+                                                    const int32_t* __restrict__ active, int ntiles,
+                                                    int32_t* __restrict__ pend, float4* __restrict__ U, int64_t n4,
+                                                    int batch) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < (int64_t)ntiles * batch; i += step) {
+        const int4 ti = tile_info[i % ntiles];
+        int on = active == nullptr && ti.y > 0;
+        if (active)
+            for (int k = 0; k < ti.y; ++k) on |= active[seg_block[ti.x + k]];
+        pend[i] = on ? ti.z : 0;
+    }
+    for (int64_t i = i0; i < n4; i += step) U[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+cudaError_t grid_begin(const pd_plan* p, const int32_t* active, int32_t* pend, float4* U, int64_t n4, int batch,
+                       cudaStream_t s) {
+    const int64_t n = std::max<int64_t>((int64_t)p->g.ntiles * batch, U ? n4 / 4 : 0);
+    const int ctas = (int)std::min<int64_t>((n + 255) / 256, (int64_t)p->num_sms * 8);
+    k_grid_begin<<<ctas, 256, 0, s>>>(p->tile_info, p->seg_block, active, p->g.ntiles, pend, U, U ? n4 : 0, batch);
     return cudaGetLastError();
 }
 
@@ -268,57 +232,67 @@ template <typename C>
 __global__ void k_gather(const C* __restrict__ user, C* __restrict__ internal, const int32_t* __restrict__ perm,
                          int64_t m) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        internal[i] = user[perm[i]];
+        internal[i] = vis_conj(perm[i], user[vis_index(perm[i])]);
 }
 template <typename C>
 __global__ void k_scatter(const C* __restrict__ internal, C* __restrict__ user, const int32_t* __restrict__ perm,
                           int64_t m) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-        user[perm[i]] = internal[i];
+        user[vis_index(perm[i])] = vis_conj(perm[i], internal[i]);
+}
+template <typename R>
+cudaError_t gather_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
+    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
+    k_gather<<<ctas, 256, 0, s>>>(src, dst, perm, p->M);
+    return cudaGetLastError();
+}
+template <typename R>
+cudaError_t scatter_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
+    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
+    k_scatter<<<ctas, 256, 0, s>>>(src, dst, perm, p->M);
+    return cudaGetLastError();
 }
 template <typename R>
 cudaError_t gather_internal(const pd_plan* p, const cplx_t<R>* user, cplx_t<R>* internal, cudaStream_t s) {
-    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
-    k_gather<<<ctas, 256, 0, s>>>(user, internal, p->perm, p->M);
-    return cudaGetLastError();
+    return gather_by<R>(p, p->perm, user, internal, s);
 }
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s) {
-    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
-    k_scatter<<<ctas, 256, 0, s>>>(internal, user, p->perm, p->M);
-    return cudaGetLastError();
+    return scatter_by<R>(p, p->perm, internal, user, s);
 }
 
-// ||y_i|| per block (= ||Phi_i x^(0) - y_i|| for x^(0) = 0): segment partials, then
-// a fixed-order sum per block.
+// ||y_i|| per block (= ||Phi_i x^(0) - y_i|| for x^(0) = 0): partial sums of every slot, one
+// warp each, then a fixed-order sum per block, one warp each.
 template <typename R>
-__global__ void k_seg_sq(const cplx_t<R>* __restrict__ y, const int32_t* __restrict__ seg_start, int nseg,
-                         double* __restrict__ part) {
-    __shared__ double sh[32];
-    for (int sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
+__global__ void __launch_bounds__(256) k_slot_sq(const cplx_t<R>* __restrict__ y, const SegSlot* __restrict__ range,
+                                                 int64_t nslot, double* __restrict__ part) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < nslot; k += step) {
+        const SegSlot r = range[k];
         double a = 0.0;
-        for (int m = seg_start[sg] + threadIdx.x; m < seg_start[sg + 1]; m += blockDim.x)
-            a += (double)y[m].x * y[m].x + (double)y[m].y * y[m].y;
-        a = block_sum(a, sh);
-        if (threadIdx.x == 0) part[2 * sg + 1] = a;
+        for (int m = r.start + lane; m < r.end; m += 32) a += (double)y[m].x * y[m].x + (double)y[m].y * y[m].y;
+        a = warp_sum(a);
+        if (lane == 0) part[2 * k + 1] = a;
     }
 }
-__global__ void k_block_sqrt(const double* __restrict__ part, const int32_t* __restrict__ bss,
-                             const int32_t* __restrict__ bsl, int d, double* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_block_sqrt(const double* __restrict__ part, const int32_t* __restrict__ bss,
+                                                    const int32_t* __restrict__ bsl, int d, double* __restrict__ out) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= d) return;
     double a = 0.0;
-    for (int k = bss[i]; k < bss[i + 1]; ++k) a += part[2 * bsl[k] + 1];
-    out[i] = sqrt(a);
+    for (int k = bss[i] + lane; k < bss[i + 1]; k += 32) a += part[2 * (int64_t)bsl[k] + 1];
+    a = warp_sum(a);
+    if (lane == 0) out[i] = sqrt(a);
 }
 cudaError_t init_res_norm(const pd_plan* p, pd_state* st, cudaStream_t s) {
-    const int ctas = (int)std::min<int64_t>(std::max<int64_t>(p->nseg, 1), (int64_t)p->num_sms * 8);
+    const int ctas = (int)std::min<int64_t>((p->nslot + 7) / 8, (int64_t)p->num_sms * 16);
     if (p->prec == PD_F64)
-        k_seg_sq<double><<<ctas, 256, 0, s>>>((const double2*)st->y, p->seg_start, (int)p->nseg, p->seg_part);
+        k_slot_sq<double><<<ctas, 256, 0, s>>>((const double2*)st->y, p->slot_range, p->nslot, p->seg_part);
     else
-        k_seg_sq<float><<<ctas, 256, 0, s>>>((const float2*)st->y, p->seg_start, (int)p->nseg, p->seg_part);
-    k_block_sqrt<<<(p->d + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_seg_start, p->block_seg_list, p->d,
-                                                    st->res_norm);
+        k_slot_sq<float><<<ctas, 256, 0, s>>>((const float2*)st->y, p->slot_range, p->nslot, p->seg_part);
+    k_block_sqrt<<<(p->d * 32 + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_slot_start, p->block_slot_list, p->d,
+                                                         st->res_norm);
     return cudaGetLastError();
 }
 
@@ -374,6 +348,10 @@ template cudaError_t norm2<float>(const pd_plan*, const float*, int64_t, double*
 template cudaError_t norm2<double>(const pd_plan*, const double*, int64_t, double*, cudaStream_t);
 template cudaError_t scale_copy<float>(const float*, float*, int64_t, double, cudaStream_t);
 template cudaError_t scale_copy<double>(const double*, double*, int64_t, double, cudaStream_t);
+template cudaError_t gather_by<float>(const pd_plan*, const int32_t*, const float2*, float2*, cudaStream_t);
+template cudaError_t gather_by<double>(const pd_plan*, const int32_t*, const double2*, double2*, cudaStream_t);
+template cudaError_t scatter_by<float>(const pd_plan*, const int32_t*, const float2*, float2*, cudaStream_t);
+template cudaError_t scatter_by<double>(const pd_plan*, const int32_t*, const double2*, double2*, cudaStream_t);
 template cudaError_t gather_internal<float>(const pd_plan*, const float2*, float2*, cudaStream_t);
 template cudaError_t gather_internal<double>(const pd_plan*, const double2*, double2*, cudaStream_t);
 template cudaError_t scatter_user<float>(const pd_plan*, const float2*, float2*, cudaStream_t);

@@ -24,8 +24,6 @@ struct Geo {
     double beta;
     int tile, logT, ntx, nty, ntiles;
     int ext;        // T + J - 1: extended tile edge of the gridding accumulator
-    int halo_lo;    // J/2 - 1 cells before the tile
-    int halo_hi;    // J/2 cells after the tile
 };
 
 // Tile colour classes of the gridding: (tile row parity, tile column parity). Two tiles
@@ -37,13 +35,36 @@ __host__ __device__ __forceinline__ int tile_colour(int t, int ntx) { return (((
 // Monomial coefficients (in x = 2 f - 1) of the per-tap Chebyshev interpolants of the
 // Kaiser-Bessel weight phi(f + J/2 - 1 - a), used by the FP32 kernels.
 constexpr int KB_DEG = 10;
+// lo: what the constant terms' rounding to FP32 left.
 struct KbPoly {
     float c[16][KB_DEG + 1];
+    float lo[16];
 };
 
-// Super-cells of SC x SC base cells inside a tile: the visibilities of a segment are
-// sorted by super-cell, then row-major by base cell (the gridding's super-rows).
+// One degridding work item: a part of a tile's points. slot0: where the part's per-segment
+// sums go in seg_part (one pair for each of the tile's segments).
+struct TileItem {
+    int32_t tile, part, parts, slot0;
+    int32_t seg0, nseg, pad0, pad1;
+};
+// A slot of seg_part: the part's share of one segment's points.
+struct SegSlot {
+    int32_t start, end;
+};
+
+// Super-cells of SC x SC cells inside a tile: the visibilities of a segment are sorted by
+// the super-cell of their footprint's first cell, then row-major by that cell.
 constexpr int SC = 8;
+
+// The image is real, so the visibility at -(u, v) is the conjugate of the one at (u, v):
+// points with u < 0 are held at -(u, v) as conjugates (unless G has DDEs, or the point is
+// on a grid line), which leaves norms, duals and Re(Phi^H .) as they are and halves the tiles that hold points. perm
+// carries the flag in its sign bit; these read and write a value in the user's convention.
+__host__ __device__ __forceinline__ int vis_index(int q) { return q & 0x7fffffff; }
+template <typename C> __device__ __forceinline__ C vis_conj(int q, C v) {
+    if (q < 0) v.y = -v.y;
+    return v;
+}
 
 // Element offset of grid cell (ky, kx) in the column-panel layout [Kx/PW][K][PW].
 __host__ __device__ __forceinline__ int64_t panel_off(int ky, int kx, int K) {
@@ -63,16 +84,24 @@ struct pd_plan {
     int64_t nseg;
     int ntiles_nonempty;
     int num_sms;
+    int max_smem;              // opt-in shared memory per CTA (bytes)
     int device;
 
     // host copies of the static tables
-    std::vector<int32_t> h_tile_seg_start, h_seg_block, h_block_seg_start, h_block_seg_list;
+    std::vector<int32_t> h_tile_seg_start, h_seg_block;
+
+    // checkpoints keep the visibilities in the order of their own tiles and base cells, whatever
+    // the plan's internal order is: device list of the internal index of each (sign bit: held
+    // as a conjugate), made by the first save or load
+    std::vector<int32_t> h_base;   // base cell (by << 16 | bx) of each point, user order
+    int ck_tile = 0;
+    int32_t* ck_perm = nullptr;
 
     // device: visibilities in internal (tile, block, row, column) order
-    int32_t* cell = nullptr;       // (by << 16) | bx of floor(g), mod K
+    int32_t* cell = nullptr;       // (by << 16) | bx of the footprint's first cell, mod K
     void* fx = nullptr;            // real [M]: fractional part of g_x
     void* fy = nullptr;
-    int32_t* perm = nullptr;       // internal -> user index
+    int32_t* perm = nullptr;       // internal -> user index; sign bit set: held as its conjugate (see vis_user)
     int g_mode = PD_G_ON_THE_FLY;  // PD_G_CSR: G stored explicitly, below
     int kb_J = 0;                  // interpolation kernel width (g.J is the footprint: kb_J + dde - 1)
     int dde = 0;                   // DDE kernel width d (0: none)
@@ -88,18 +117,34 @@ struct pd_plan {
     std::vector<int32_t> h_sc_start;       // (host, only during plan construction)
     int max_tile_segs = 0;                 // most (tile, block) segments in one tile
     pdgb::KbPoly kbpoly{};
-    int32_t* block_seg_start = nullptr;    // [d + 1] into block_seg_list
-    int32_t* block_seg_list = nullptr;     // [nseg] segments of each block, tile order
+    int32_t* block_slot_start = nullptr;   // [d + 1] into block_slot_list
+    int32_t* block_slot_list = nullptr;    // [nslot] seg_part slots of each block, in a fixed order
     int32_t* tile_order = nullptr;         // [ntiles] tiles by decreasing visibility count
     int32_t* colour_tiles = nullptr;       // [4][ntiles/4] tiles of each colour, heaviest first
-    int32_t* colour_counts = nullptr;      // [4] ntiles/4 each
-    int32_t* counts_all = nullptr;         // {nseg, ntiles}
+    int32_t* colour_counts = nullptr;      // [4] tiles of each colour that hold visibilities
+    // FP32 gridding (k_grid_mma): a tile's points are cut into parts of about grid_part points,
+    // and (tile, part) items are claimed tile colour by tile colour, heaviest tile first
+    int grid_part = 0, grid_warps = 0, n_items = 0;
+    size_t grid_smem = 0;                  // 0: the plan grids with the other kernels
+    int4* tile_info = nullptr;             // [ntiles] {first segment, segments, parts, place in the order of items}
+    int2* items = nullptr;                 // [nitems] {tile, part}
+    int32_t* nitems = nullptr;             // device count
+    int32_t* pend = nullptr;               // [ntiles] parts of the running launch not yet added to U
+    int32_t* bpend = nullptr;              // the same for each image of a batch
+    pdgb::TileItem* ditems = nullptr;      // [n_ditems] degridding items, heaviest tile first
+    int n_ditems = 0;
+    int64_t nslot = 0;                     // slots of seg_part
+    pdgb::SegSlot* slot_range = nullptr;   // [nslot] points of each slot (init_res_norm)
+    std::vector<pdgb::TileItem> h_ditems;
+    int32_t* counts_all = nullptr;         // {nseg, tiles that hold visibilities, n_ditems}
     int32_t* ones_block = nullptr;         // all blocks active
     int32_t* ones_basis = nullptr;
 
     // tables
     void* cx = nullptr;            // real [nx] deapodisation
     void* cy = nullptr;            // real [ny]
+    void* cxl = nullptr;           // FP32: what rounding cx and cy to float left
+    void* cyl = nullptr;
     void* twx = nullptr;           // complex [Kx]: exp(-2 pi i k / Kx)
     void* twy = nullptr;           // complex [Ky]
     void* filt = nullptr;          // real [b][MAX_FILTER] low-pass filters (0 for Dirac)
@@ -116,15 +161,16 @@ struct pd_plan {
     void* bgb = nullptr;
     void* bgu = nullptr;
     void* rbuf = nullptr;          // complex [M] residuals r = v + G b - y (internal order)
-    double* seg_part = nullptr;    // [2 * nseg] per-segment FP64 partial norms
+    double* seg_part = nullptr;    // [2 * nslot] FP64 partial norms of each segment's share of a part
     double* blk_norm = nullptr;    // [2 * d]: ||r_i||^2, ||G_i b - y_i||^2
     void* blk_scale = nullptr;     // real [d]: max(0, 1 - eps_i / ||r_i||)
     void* ll[2] = {nullptr, nullptr};  // real [b][ny/2][nx/2] wavelet approximation ping-pong
     void* ds = nullptr;            // real [b][ny][nx] change of the sparsity duals
     void* synpart = nullptr;       // real [b][ny][nx] level-0 synthesis of each basis
     double* red = nullptr;         // reduction scratch
-    int32_t* sched = nullptr;      // [8] work counters of the dynamically scheduled launches (0-3 gridding
-                                   // colours, 4 degridding)
+    int32_t* sched = nullptr;      // [16] work counters of the dynamically scheduled launches: 0-3 gridding
+                                   // colours (zeroed before each launch); 4-5 degridding, 8-9 k_grid_mma (next
+                                   // item, CTAs done: left at zero by every launch); 10: a wait gave up
     int red_len = 0;
     size_t device_bytes = 0;
     std::vector<void*> allocs;     // every device allocation of the plan
@@ -147,10 +193,8 @@ struct pd_state {
     double* p_basis = nullptr;     // [b]
     int32_t* block_active = nullptr;   // [d]
     int32_t* basis_active = nullptr;   // [b]
-    int32_t* act_tiles = nullptr;      // [ntiles] tiles holding an active block, heaviest first
-    int32_t* act_col = nullptr;        // [4][ntiles/4] the same tiles split by colour
     int32_t* tile_active = nullptr;    // [ntiles]: tile holds a visibility of an active block
-    int32_t* counts = nullptr;         // {active segments, active tiles, active tiles of colour 0..3}
+    int32_t* counts = nullptr;         // {active segments, active tiles}
     int64_t* t = nullptr;              // iteration counter (device)
     double* diag = nullptr;            // [2]: ||dx||^2, ||x||^2
     double* prim_part = nullptr;       // [2 * ny / rows-per-CTA]
@@ -169,10 +213,13 @@ struct pd_state {
     // plain per-block form (pd_params.per_block): one-hot activity flags, each block's tiles
     int32_t* pb_eye_blocks = nullptr;  // [d][d]
     int32_t* pb_eye_bases = nullptr;   // [b][b]
-    int32_t* pb_tiles = nullptr;       // tiles of block i at pb_tiles[h_pb_off[i] ...]
-    int32_t* pb_counts = nullptr;      // [d][2]: {0, number of tiles of block i}
+    pdgb::TileItem* pb_ditems = nullptr;   // degridding items of block i at pb_ditems[h_pb_off[i] ...]
+    int32_t* pb_counts = nullptr;      // [d] number of them
     int32_t* pb_col = nullptr;         // tiles of block i and colour c at pb_col[h_pb_off[4 i + c] ...]
     int32_t* pb_ccounts = nullptr;     // [d][4] number of tiles of block i per colour
+    int2* pb_items = nullptr;          // k_grid_mma's items of block i at pb_items[h_pb_item_off[i] ...]
+    int32_t* pb_nitems = nullptr;      // [d]
+    std::vector<int32_t> h_pb_item_off;
     std::vector<int32_t> h_pb_off;
     std::vector<int32_t> h_act, h_actb;
     int64_t h_t = 0;
@@ -215,12 +262,19 @@ cudaError_t inv_fft(const pd_plan* p, const cplx_t<R>* grid, R* out, const Prima
 int inv_rows_ctas(const pd_plan* p);
 
 // ---- gridding.cu
+// decides whether the plan grids with k_grid_mma, with how many warps and which part size
+void grid_setup(pd_plan* p);
 struct DualArgs {
     const void* y;        // internal-order data (pd mode) or user-order input (plain mode)
     void* v;              // dual (pd mode)
     const int32_t* block_active;
     const double* eps;
     double* res_norm;     // updated for active blocks
+    const int32_t* tile_on = nullptr;   // [ntiles] flags of the tiles to work on (nullptr: every listed one)
+    const TileItem* ditems = nullptr;   // degridding items and their device count
+    const int32_t* nditems = nullptr;
+    const int2* items = nullptr;        // k_grid_mma's work items and their device count
+    const int32_t* nitems = nullptr;
 };
 // plain degrid of `batch` half grids (stride: one image's half grid) into out (user order, stride M)
 template <typename R>
@@ -229,15 +283,15 @@ cudaError_t degrid_plain(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out
 template <typename R>
 cudaError_t degrid_res_norms(const pd_plan* p, const cplx_t<R>* grid, const cplx_t<R>* y, double* res_norm,
                              cudaStream_t s);
-// pd degrid over the listed tiles: r = v + G b - y, segment partial norms, then block scales
+// pd degrid over a's items: r = v + G b - y, segment partial norms, then block scales
 template <typename R>
-cudaError_t degrid_dual(const pd_plan* p, const cplx_t<R>* grid, const DualArgs& a, const int32_t* tiles,
-                        const int32_t* counts, cudaStream_t s);
+cudaError_t degrid_dual(const pd_plan* p, const cplx_t<R>* grid, const DualArgs& a, cudaStream_t s);
 // G in CSR form (PD_G_CSR): the J^2 (cell, weight) entries of every visibility
 cudaError_t build_csr(pd_plan* p, cudaStream_t s);
 // plain grid: U = G^T y_user (U overwritten) for `batch` inputs (stride M) and grids (stride Kx Ky)
 template <typename R>
-cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch = 1);
+cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch = 1,
+                       int32_t* pend = nullptr);
 // pd grid over the listed tiles, one launch per colour (tiles[c]: device list of colour c,
 // counts4[c]: device count): v <- scale * r, U += G^T (v_new - v_old)
 template <typename R>
@@ -278,8 +332,16 @@ template <typename R>
 cudaError_t scale_copy(const R* x, R* y, int64_t n, double scale, cudaStream_t s);
 template <typename R>
 cudaError_t gather_internal(const pd_plan* p, const cplx_t<R>* user, cplx_t<R>* internal, cudaStream_t s);
+// the same through another list of places (checkpoints)
+template <typename R>
+cudaError_t gather_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
+template <typename R>
+cudaError_t scatter_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s);
+// pend[t] = parts of the tiles that hold a point of an active block (all of them: active null), else 0;
+// and U = 0 where given (n4 float4 elements), for `batch` images
+cudaError_t grid_begin(const pd_plan* p, const int32_t* active, int32_t* pend, float4* U, int64_t n4, int batch, cudaStream_t s);
 cudaError_t init_res_norm(const pd_plan* p, pd_state* st, cudaStream_t s);
 
 }  // namespace pdgb

@@ -1,0 +1,92 @@
+"""Points at the edges of the gridding's and degridding's work items: one point, chunks of 32
+with a remainder, a tile so heavy that it is split into parts, points on grid lines and at
+the band edges (which are not held as conjugates), every kernel width and tile size; the
+fixed order of the sums; the order in which a checkpoint keeps the visibilities."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_util import TOL_OP32, TOL_OP64, rel  # noqa: E402
+from oracle import measurement as meas  # noqa: E402
+from paper_1610_08895_gb300 import synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import __graft_entry__ as ge
+    ge.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+
+
+def _points(kind, m, n, seed=0):
+    rng = np.random.default_rng(seed)
+    if kind == "cluster":           # all in one tile
+        return np.array([0.7, -1.1]) + rng.uniform(0.0, 6.0 * np.pi / n, size=(m, 2))
+    if kind == "lines":             # integer grid coordinates in x, in y, in both, and the band edges
+        k = rng.integers(-n, n, size=(m, 2)) * (np.pi / n)
+        f = rng.uniform(-np.pi, np.pi, size=(m, 2))
+        uv = np.where(rng.integers(0, 2, size=(m, 2)) == 0, k, f)
+        uv[:4] = [[-np.pi, -np.pi], [0.0, 0.0], [-np.pi, 0.3], [0.3, -np.pi]]
+        return uv
+    return synth.uv_gaussian(m, seed=seed + 1)
+
+
+CASES = [
+    # kind, m, n, blocks, J, tile
+    ("gauss", 1, 16, 1, 8, 0), ("gauss", 31, 16, 2, 6, 8), ("gauss", 33, 32, 3, 4, 16), ("gauss", 65, 32, 1, 2, 2),
+    ("gauss", 4097, 64, 5, 8, 8), ("gauss", 3000, 64, 7, 8, 64), ("lines", 2000, 32, 4, 8, 16),
+    ("lines", 1500, 32, 2, 6, 8), ("lines", 1200, 32, 3, 4, 32), ("lines", 700, 32, 1, 2, 16),
+    ("cluster", 9001, 64, 3, 8, 16), ("cluster", 8500, 128, 40, 6, 32), ("cluster", 3001, 64, 2, 12, 16),
+]
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("case", CASES)
+def test_operators_at_the_edges_of_work_items(case, precision):
+    from paper_1610_08895_gb300.api import Plan
+    kind, m, n, nb, J, tile = case
+    if kind == "lines" and precision == "f32" and J <= 4:
+        pytest.skip("the kernel's jump at |t| = J/2 is above FP32 rounding: a fraction that rounds to a grid "
+                    "line takes another set of taps than the FP64 oracle")
+    uv = _points(kind, m, n)
+    geo = meas.Geometry(n, n, J)
+    plan = Plan(n, n, uv, (np.arange(m) % nb).astype(np.int32), nb, kernel_width=J, precision=precision, tile=tile)
+    x = synth.random_images(1, n, n, seed=3)[0]
+    v = synth.uniform_vis(m, seed=4)
+    tol = TOL_OP32 if precision == "f32" else TOL_OP64
+    y = plan.pd_apply_phi(torch.tensor(x, dtype=plan.real_dtype, device="cuda")).cpu().numpy()
+    assert rel(y, geo.phi(x, uv)) < tol
+    vt = torch.tensor(v, dtype=plan.cplx_dtype, device="cuda")
+    xa = plan.pd_apply_phi_adj(vt)
+    assert rel(xa.cpu().numpy(), geo.phi_adj(v, uv)) < tol
+    if J <= 8:                      # wider kernels add through shared-memory atomics
+        assert torch.equal(xa, plan.pd_apply_phi_adj(vt))
+
+
+@pytest.mark.parametrize("tile", [0, 16])
+def test_checkpoint_order_of_the_visibilities(tile):
+    """The buffer holds v by (tile, block, 8 x 8 super-cell, row, column, user index) of the base cells."""
+    from paper_1610_08895_gb300.api import Plan, State
+    n, m, nb, J = 64, 3000, 5, 8
+    uv = _points("lines", m, n, seed=2)
+    blk = (np.arange(m) % nb).astype(np.int32)
+    plan = Plan(n, n, uv, blk, nb, kernel_width=J, precision="f64", tile=tile)
+    st = State(plan)
+    st.pd_state_set_data(torch.tensor(synth.uniform_vis(m, seed=5), device="cuda"), np.ones(nb))
+    v0 = synth.uniform_vis(m, seed=6)
+    st.pd_state_set_start(v0=torch.tensor(v0, device="cuda"))
+    buf = st.save()
+    N, T = n * n, tile or 32
+    start = 8 * (2 * N + plan.nbases * N + N)
+    got = buf[start:start + 16 * m].view(np.complex128)
+    base = np.floor(uv * (2 * n) / (2 * np.pi)).astype(np.int64) % (2 * n)
+    bx, by = base[:, 0], base[:, 1]
+    sc = (by % T) // 8 * (T // 8) + (bx % T) // 8
+    order = np.lexsort((np.arange(m), bx, by, sc, blk, (by // T) * (2 * n // T) + bx // T))
+    assert np.array_equal(got, v0[order])
+    other = State(plan)
+    other.load(buf)
+    assert np.array_equal(other.v().cpu().numpy(), v0)
