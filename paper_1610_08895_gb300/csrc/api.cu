@@ -469,6 +469,13 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
                 p->kbpoly.lo[a] = (float)(kp[(size_t)a * (KB_DEG + 1)] - (double)p->kbpoly.c[a][0]);
             }
         }
+        if (p->prec == PD_F64) {
+            double err = 0.0;
+            const std::vector<double> kp = kb_tap_polynomials_ext(p->kb_J, g.beta, KB_DEG64, &err);
+            for (int a = 0; a < p->kb_J; ++a)
+                for (int k = 0; k <= KB_DEG64; ++k) p->kbpoly64.c[a][k] = kp[(size_t)a * (KB_DEG64 + 1) + k];
+            p->kbpoly64.use = err < 1e-16;
+        }
         p->h_filt.assign((size_t)p->b * MAX_FILTER, 0.0);
         p->h_filt_len.assign(p->b, 0);
         for (int k = 0; k < p->b; ++k) {

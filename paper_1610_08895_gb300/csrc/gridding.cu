@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
                                                 const TileItem* __restrict__ items,
                                                 const int32_t* __restrict__ nitems,
                                                 const int32_t* __restrict__ tile_on, double* __restrict__ seg_part,
-                                                int max_segs, Geo g, R two_over_j, R beta, const KbPoly kp,
+                                                int max_segs, Geo g, R two_over_j, R beta, const kb_poly_t<R> kp,
                                                 int* __restrict__ sched, int batch, int64_t gstride,
                                                 int64_t ostride) {
     using C2 = cplx_t<R>;
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(256) k_grid(const cplx_t<R>* __restrict__ src,
                                               const int32_t* __restrict__ list, const int32_t* __restrict__ count,
                                               const int32_t* __restrict__ tile_on, cplx_t<R>* __restrict__ U,
                                               int max_segs,
-                                              Geo g, R two_over_j, R beta, const KbPoly kp) {
+                                              Geo g, R two_over_j, R beta, const kb_poly_t<R> kp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     R* acc = reinterpret_cast<R*>(smraw);   // [ext*ext] re then [ext*ext] im
     int* act_seg = reinterpret_cast<int*>(acc + 2 * g.ext * g.ext);
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
     const int32_t* __restrict__ seg_start, const int32_t* __restrict__ seg_block,
     const int32_t* __restrict__ tile_seg_start, const int32_t* __restrict__ sc_start,
     const int32_t* __restrict__ list, const int32_t* __restrict__ count, const int32_t* __restrict__ tile_on,
-    cplx_t<R>* __restrict__ U, int max_segs, Geo g, R two_over_j, R beta, const KbPoly kp,
+    cplx_t<R>* __restrict__ U, int max_segs, Geo g, R two_over_j, R beta, const kb_poly_t<R> kp,
     int* __restrict__ next_tile, int batch, int64_t istride, int64_t ustride) {
     static_assert(J <= 8 && J % 2 == 0, "class ownership needs J <= 8");
     using C2 = cplx_t<R>;
@@ -1157,7 +1157,7 @@ static cudaError_t launch_degrid(const pd_plan* p, const cplx_t<R>* grid, cplx_t
         grid, out, a ? (const cplx_t<R>*)a->y : nullptr, a ? (const cplx_t<R>*)a->v : nullptr,
         (cplx_t<R>*)p->rbuf, p->cell, (const R*)p->fx, (const R*)p->fy, p->perm, p->seg_start, p->seg_block,
         a ? a->block_active : nullptr, a ? a->ditems : p->ditems, a ? a->nditems : p->counts_all + 2,
-        a ? a->tile_on : nullptr, p->seg_part, ms, g, R(2.0 / g.J), R(g.beta), p->kbpoly, p->sched + 4, batch,
+        a ? a->tile_on : nullptr, p->seg_part, ms, g, R(2.0 / g.J), R(g.beta), kb_poly<R>(p), p->sched + 4, batch,
         (int64_t)(g.nx / 4 + 1) * 4 * g.Ky, (int64_t)p->M);
     return cudaGetLastError();
 }
@@ -1275,7 +1275,7 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
         k_grid8w<R, J, MODE><<<ctas8, nw * 32, smem8, s>>>(
             src, rb, vv, (const R*)p->blk_scale, act, p->cell, (const R*)p->fx, (const R*)p->fy, p->perm,
             p->seg_start, p->seg_block, p->tile_seg_start, p->seg_sc_start, tiles, count, a ? a->tile_on : nullptr, U, ms, g, toj, beta,
-            p->kbpoly, next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
+            kb_poly<R>(p), next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     } else {
         const size_t smem = (size_t)2 * g.ext * g.ext * sizeof(R) + lists;
         if ((e = ensure_smem(k_grid<R, J, MODE>, smem))) return e;
@@ -1284,7 +1284,7 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
                                                       (const R*)p->blk_scale, act, p->cell, (const R*)p->fx,
                                                       (const R*)p->fy, p->perm, p->seg_start, p->seg_block,
                                                       p->tile_seg_start, tiles, count, a ? a->tile_on : nullptr,
-                                                      U + (int64_t)b * g.Kx * g.Ky, ms, g, toj, beta, p->kbpoly);
+                                                      U + (int64_t)b * g.Kx * g.Ky, ms, g, toj, beta, kb_poly<R>(p));
     }
     return cudaGetLastError();
 }

@@ -6,30 +6,41 @@
 
 namespace pdgb {
 
-// The J tap weights phi(frac + J/2 - 1 - a) of one axis. FP32: the plan's per-tap
-// Chebyshev interpolants (degree 10, interpolation error ~3e-11 of phi(0), below FP32
-// resolution) in x = 2 frac - 1. phi is even, so tap J-1-a is tap a at -x: with the
-// polynomial split into even and odd parts p = E(x^2) + x O(x^2), one pass gives both
-// E + x O (tap a) and E - x O (tap J-1-a). FP64: I0 itself.
+// The J tap weights phi(frac + J/2 - 1 - a) of one axis, from the plan's per-tap Chebyshev
+// interpolants in x = 2 frac - 1 (FP32: degree 10, interpolation error ~3e-11 of phi(0);
+// FP64: degree 18, fitted in extended precision, below 1e-17 of phi(0)). phi is even, so tap
+// J-1-a is tap a at -x: with the polynomial split into even and odd parts p = E(x^2) + x O(x^2),
+// one pass gives both E + x O (tap a) and E - x O (tap J-1-a). In FP64, where the GPU has 1/64
+// of its FP32 rate, the 8 x 2 evaluations of I0 were most of both kernels (phi_256_f64 of
+// perf/cases.py: 8.4 ms with them, 4.7 ms with the polynomials).
 template <typename R, int J>
-__device__ __forceinline__ void kb_taps(R frac, R* w, R two_over_j, R beta, const KbPoly& kp) {
-    if constexpr (sizeof(R) == 4) {
-        const float x = 2.0f * frac - 1.0f, x2 = x * x;
+__device__ __forceinline__ void kb_taps(R frac, R* w, R two_over_j, R beta, const kb_poly_t<R>& kp) {
+    constexpr int DEG = sizeof(R) == 4 ? KB_DEG : KB_DEG64;
+    if constexpr (sizeof(R) == 8) {
+        if (!kp.use) {
 #pragma unroll
-        for (int a = 0; a < J / 2; ++a) {
-            float ev = kp.c[a][KB_DEG], od = kp.c[a][KB_DEG - 1];
-#pragma unroll
-            for (int k = KB_DEG - 2; k >= 2; k -= 2) ev = fmaf(ev, x2, kp.c[a][k]);
-#pragma unroll
-            for (int k = KB_DEG - 3; k >= 1; k -= 2) od = fmaf(od, x2, kp.c[a][k]);
-            // the constant term last, with the part that its rounding left: one rounding of w
-            ev = fmaf(ev, x2, kp.lo[a]);
-            w[a] = kp.c[a][0] + fmaf(x, od, ev);
-            w[J - 1 - a] = kp.c[a][0] + fmaf(-x, od, ev);
+            for (int a = 0; a < J; ++a) w[a] = kb_weight<R>(frac + R(J / 2 - 1 - a), two_over_j, beta);
+            return;
         }
-    } else {
+    }
+    const R x = R(2) * frac - R(1), x2 = x * x;
 #pragma unroll
-        for (int a = 0; a < J; ++a) w[a] = kb_weight<R>(frac + R(J / 2 - 1 - a), two_over_j, beta);
+    for (int a = 0; a < J / 2; ++a) {
+        R ev = kp.c[a][DEG], od = kp.c[a][DEG - 1];
+#pragma unroll
+        for (int k = DEG - 2; k >= 2; k -= 2) ev = fma(ev, x2, kp.c[a][k]);
+#pragma unroll
+        for (int k = DEG - 3; k >= 1; k -= 2) od = fma(od, x2, kp.c[a][k]);
+        if constexpr (sizeof(R) == 4) {
+            // the constant term last, with the part that its rounding left: one rounding of w
+            ev = fma(ev, x2, kp.lo[a]);
+            w[a] = kp.c[a][0] + fma(x, od, ev);
+            w[J - 1 - a] = kp.c[a][0] + fma(-x, od, ev);
+        } else {
+            ev = fma(ev, x2, kp.c[a][0]);
+            w[a] = fma(x, od, ev);
+            w[J - 1 - a] = fma(-x, od, ev);
+        }
     }
 }
 

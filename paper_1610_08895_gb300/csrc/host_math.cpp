@@ -2,6 +2,7 @@
 // and FFT twiddles, all computed in FP64.
 #include "host_math.hpp"
 
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -155,6 +156,60 @@ std::vector<double> kb_tap_polynomials(int J, double beta, int deg) {
         }
         for (int i = 0; i < n; ++i) out[(size_t)a * n + i] = mono[i];
     }
+    return out;
+}
+
+// I0(z) by its power series (positive terms only).
+static long double bessel_i0_ext(long double z) {
+    const long double q = z * z / 4.0L;
+    long double term = 1.0L, sum = 1.0L;
+    for (int k = 1; k < 4000; ++k) {
+        term *= q / ((long double)k * k);
+        sum += term;
+        if (term < sum * 1e-22L) break;
+    }
+    return sum;
+}
+
+std::vector<double> kb_tap_polynomials_ext(int J, double beta, int deg, double* err) {
+    using ld = long double;
+    const int n = deg + 1;
+    const ld pi = 3.14159265358979323846264338327950288L;
+    auto phi = [&](ld t) {
+        const ld u = 2.0L * t / J, arg = 1.0L - u * u;
+        return arg > 0 ? bessel_i0_ext((ld)beta * std::sqrt(arg)) : (arg > -1e-15L ? 1.0L : 0.0L);
+    };
+    std::vector<double> out((size_t)J * n, 0.0);
+    ld worst = 0.0L;
+    for (int a = 0; a < J; ++a) {
+        std::vector<ld> fx(n), cheb(n, 0.0L);
+        for (int k = 0; k < n; ++k) fx[k] = phi((std::cos(pi * (k + 0.5L) / n) + 1.0L) / 2.0L + J / 2 - 1 - a);
+        for (int j = 0; j < n; ++j) {
+            ld acc = 0.0L;
+            for (int k = 0; k < n; ++k) acc += fx[k] * std::cos(pi * j * (k + 0.5L) / n);
+            cheb[j] = (j == 0 ? 1.0L : 2.0L) * acc / n;
+        }
+        // sum_j cheb_j T_j in monomials, T_{j+1} = 2 x T_j - T_{j-1}
+        std::vector<ld> prev(n, 0.0L), cur(n, 0.0L), mono(n, 0.0L);
+        cur[0] = 1.0L;
+        for (int j = 0; j < n; ++j) {
+            for (int i = 0; i < n; ++i) mono[i] += cheb[j] * cur[i];
+            std::vector<ld> next(n, 0.0L);
+            for (int i = 0; i + 1 < n; ++i) next[i + 1] = (j == 0 ? 1.0L : 2.0L) * cur[i];
+            if (j > 0)
+                for (int i = 0; i < n; ++i) next[i] -= prev[i];
+            prev = cur;
+            cur = next;
+        }
+        for (int i = 0; i < n; ++i) out[(size_t)a * n + i] = (double)mono[i];
+        for (int k = 0; k <= 2 * n; ++k) {     // between the nodes
+            const ld x = std::cos(pi * k / (2 * n));
+            ld v = 0.0L;
+            for (int i = n - 1; i >= 0; --i) v = v * x + mono[i];
+            worst = std::max(worst, std::abs(v - phi((x + 1.0L) / 2.0L + J / 2 - 1 - a)));
+        }
+    }
+    *err = (double)(worst / phi(0.0L));
     return out;
 }
 

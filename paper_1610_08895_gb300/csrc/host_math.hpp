@@ -16,5 +16,8 @@ std::vector<double> twiddles(int K);
 // Monomial coefficients (in x = 2 f - 1, f in [0, 1)) of the degree-`deg` Chebyshev
 // interpolant of tap a's weight phi(f + J/2 - 1 - a), for a = 0..J-1: [J][deg + 1].
 std::vector<double> kb_tap_polynomials(int J, double beta, int deg);
+// The same fitted in extended precision; *err is the largest deviation of the fit from the
+// weight between the nodes, relative to phi(0), before the coefficients are rounded to FP64.
+std::vector<double> kb_tap_polynomials_ext(int J, double beta, int deg, double* err);
 
 }  // namespace pdgb

@@ -40,6 +40,16 @@ struct KbPoly {
     float c[16][KB_DEG + 1];
     float lo[16];
 };
+// The same for the FP64 kernels; use = 0 where the fit is not exact to FP64 (a caller's own,
+// larger kb_beta): those plans evaluate I0 itself.
+constexpr int KB_DEG64 = 18;
+struct KbPoly64 {
+    double c[16][KB_DEG64 + 1];
+    int use;
+};
+template <typename R> struct KbPolyOf { using type = KbPoly; };
+template <> struct KbPolyOf<double> { using type = KbPoly64; };
+template <typename R> using kb_poly_t = typename KbPolyOf<R>::type;
 
 // One degridding work item: a part of a tile's points. slot0: where the part's per-segment
 // sums go in seg_part (one pair for each of the tile's segments).
@@ -117,6 +127,7 @@ struct pd_plan {
     std::vector<int32_t> h_sc_start;       // (host, only during plan construction)
     int max_tile_segs = 0;                 // most (tile, block) segments in one tile
     pdgb::KbPoly kbpoly{};
+    pdgb::KbPoly64 kbpoly64{};
     int32_t* block_slot_start = nullptr;   // [d + 1] into block_slot_list
     int32_t* block_slot_list = nullptr;    // [nslot] seg_part slots of each block, in a fixed order
     int32_t* tile_order = nullptr;         // [ntiles] tiles by decreasing visibility count
@@ -230,6 +241,11 @@ struct pd_state {
 };
 
 namespace pdgb {
+
+template <typename R> inline const kb_poly_t<R>& kb_poly(const pd_plan* p) {
+    if constexpr (sizeof(R) == 8) return p->kbpoly64;
+    else return p->kbpoly;
+}
 
 // Kernel phases of one iteration, for optional per-phase CUDA-event timing.
 enum Phase {
