@@ -153,6 +153,190 @@ __device__ __forceinline__ void dwt_body(const R* __restrict__ src, R* __restric
     }
 }
 
+// ---- FP32 levels on tiles of T x T per sub-band (both sides of the sub-bands multiples of T)
+// The same filter bank as above, laid out for the FP32 pipes: every thread keeps the taps as
+// pairs (h_j, g_j) and runs both filters in one packed multiply-add per value; rows are staged
+// and filtered in 16-byte pieces (pitches of an odd number of pieces: eight threads of a
+// quarter-warp on eight rows hit distinct banks), and in the column pass a warp's threads take
+// consecutive columns. Bound by instruction issue (2 LF multiply-adds a pixel). The analysis of
+// an iteration at 2048^2 (half of nine bases, four levels): 217 -> 124 us; at 256^2: 54 -> 25 us.
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+          "l"(reinterpret_cast<const unsigned long long&>(c)));
+    return d;
+}
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+
+template <int LF, int T> struct Dwt32Shape {
+    static constexpr int IH = 2 * T + LF - 2;             // staged rows
+    static constexpr int IW4 = (2 * T + LF - 2 + 3) / 4;  // staged 16-byte pieces per row
+    static constexpr int IP = 4 * (IW4 | 1), RP = T + 4;  // pitches: staged rows, row-pass results
+    static constexpr int FLOATS = IH * (IP + 2 * RP);
+};
+template <int T> constexpr size_t dwt32_smem() { return (size_t)Dwt32Shape<MAX_FILTER, T>::FLOATS * sizeof(float); }
+template <int T> constexpr int dwt32_threads() { return T == 32 ? 256 : 128; }
+
+template <int MODE, int LF, int T>
+__device__ __forceinline__ void dwt32_body(const float* __restrict__ src, float* __restrict__ ll_out,
+                                           float* __restrict__ out, float* __restrict__ ds,
+                                           const float* __restrict__ wt, const float* __restrict__ filt, int k, int my,
+                                           int mx, int oy0, int ox0, bool last, int64_t boff, int nx, int64_t ll_off,
+                                           float scale, float alpha, float* sm) {
+    using S = Dwt32Shape<LF, T>;
+    constexpr int NT = dwt32_threads<T>();
+    const int hy = my >> 1, hx = mx >> 1;
+    float* in = sm;                                   // [IH][IP]
+    float* ra = in + S::IH * S::IP;                   // [IH][RP]
+    float* rd = ra + S::IH * S::RP;                   // [IH][RP]
+    // stage the tile and its halo (periodic), several rows' loads in flight
+    {
+        constexpr int N = S::IH * S::IW4, UB = 6;
+#pragma unroll 1
+        for (int base = threadIdx.x; base < N; base += UB * NT) {
+            float4 v[UB];
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int i = base + u * NT, rr = i / S::IW4, q = i - rr * S::IW4;
+                if (i < N)
+                    v[u] = *reinterpret_cast<const float4*>(src + (int64_t)((2 * oy0 + rr) & (my - 1)) * mx +
+                                                            ((2 * ox0 + 4 * q) & (mx - 1)));
+            }
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int i = base + u * NT, rr = i / S::IW4, q = i - rr * S::IW4;
+                if (i < N) *reinterpret_cast<float4*>(in + rr * S::IP + 4 * q) = v[u];
+            }
+        }
+    }
+    float2 hg[LF];
+#pragma unroll
+    for (int j = 0; j < LF; ++j)
+        hg[j] = make_float2(filt[k * MAX_FILTER + j], ((j & 1) ? -1.f : 1.f) * filt[k * MAX_FILTER + LF - 1 - j]);
+    __syncthreads();
+    // row pass: four outputs of one row a thread, consecutive threads on consecutive rows
+#pragma unroll 1
+    for (int it = threadIdx.x; it < S::IH * (T / 4); it += NT) {
+        const int gr = it / S::IH, rr = it - gr * S::IH;
+        constexpr int NX4 = (LF + 6 + 3) / 4;
+        float x[4 * NX4];
+#pragma unroll
+        for (int q = 0; q < NX4; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(in + rr * S::IP + 8 * gr + 4 * q);
+            x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+        }
+        float2 acc[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < LF + 6; ++i) {
+            const float2 xx = dup2(x[i]);
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+                if (i - 2 * o >= 0 && i - 2 * o < LF) acc[o] = ffma2(hg[i - 2 * o], xx, acc[o]);
+        }
+        *reinterpret_cast<float4*>(ra + rr * S::RP + 4 * gr) = make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x);
+        *reinterpret_cast<float4*>(rd + rr * S::RP + 4 * gr) = make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y);
+    }
+    __syncthreads();
+    // column pass: RO output rows of one column of the low- (LL, LH) or high-pass (HL, HH) half
+    constexpr int RO = T == 32 ? 8 : 4;
+    static_assert(2 * T * (T / RO) <= 2 * NT, "at most two items a thread");
+#pragma unroll 1
+    for (int it = threadIdx.x; it < 2 * T * (T / RO); it += NT) {
+        const int c = it % T, r0 = (it / T) % (T / RO) * RO, half = it / (T * (T / RO));
+        const float* rr = half ? rd : ra;
+        const bool store_lo = half || last;
+        const int64_t p_lo = boff + (int64_t)(oy0 + r0) * nx + (half ? hx : 0) + ox0 + c;
+        const int64_t p_hi = p_lo + (int64_t)hy * nx;
+        float so[RO], th[RO];
+        if (MODE == 1) {
+#pragma unroll
+            for (int o = 0; o < RO; ++o) {
+                if (store_lo) so[o] = out[p_lo + (int64_t)o * nx];
+                th[o] = out[p_hi + (int64_t)o * nx];
+            }
+        }
+        float2 acc[RO];
+#pragma unroll
+        for (int o = 0; o < RO; ++o) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < LF + 2 * RO - 2; ++i) {
+            const float2 xx = dup2(rr[(2 * r0 + i) * S::RP + c]);
+#pragma unroll
+            for (int o = 0; o < RO; ++o)
+                if (i - 2 * o >= 0 && i - 2 * o < LF) acc[o] = ffma2(hg[i - 2 * o], xx, acc[o]);
+        }
+#pragma unroll
+        for (int o = 0; o < RO; ++o) {
+            const int64_t pl = p_lo + (int64_t)o * nx, ph = p_hi + (int64_t)o * nx;
+            if (MODE == 0) {
+                if (store_lo) out[pl] = acc[o].x * scale;
+                out[ph] = acc[o].y * scale;
+            } else {
+                // weighted prior: the threshold of each coefficient is alpha times its weight
+                if (store_lo) {
+                    const float sn = clip(so[o] + acc[o].x * scale, wt ? alpha * wt[pl] : alpha);
+                    out[pl] = sn;
+                    ds[pl] = sn - so[o];
+                }
+                const float sn = clip(th[o] + acc[o].y * scale, wt ? alpha * wt[ph] : alpha);
+                out[ph] = sn;
+                ds[ph] = sn - th[o];
+            }
+            if (!half && !last) ll_out[ll_off + (int64_t)(oy0 + r0 + o) * hx + ox0 + c] = acc[o].x;
+        }
+    }
+}
+
+// One FP32 level for every basis in blockIdx.z; level 0 also treats the Dirac bases (the
+// identity, elementwise on the tile's 2T x 2T pixels).
+template <int MODE, int T>
+__global__ void __launch_bounds__(dwt32_threads<T>(), T == 32 ? (MODE == 0 ? 3 : 2) : 6) k_dwt32_level(
+    const float* __restrict__ x0, const float* __restrict__ ll_in, float* __restrict__ ll_out, float* __restrict__ out,
+    float* __restrict__ ds, const float* __restrict__ wt, const float* __restrict__ filt,
+    const int32_t* __restrict__ flen, const int32_t* __restrict__ active, int level, int L, int ny, int nx, float scale,
+    float alpha) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int k = blockIdx.z;
+    const int lf = flen[k];
+    if (lf == 0 && level > 0) return;
+    if (MODE == 1 && !active[k]) return;
+    const int my = ny >> level, mx = nx >> level;
+    const int oy0 = blockIdx.y * T, ox0 = blockIdx.x * T;
+    const int64_t boff = (int64_t)k * ny * nx, ll_off = (int64_t)k * (ny / 2) * (nx / 2);
+    if (lf == 0) {
+        for (int i = threadIdx.x; i < 2 * T * (T / 2); i += dwt32_threads<T>()) {
+            const int rr = i / (T / 2), q = i % (T / 2);
+            const int64_t at = (int64_t)(2 * oy0 + rr) * nx + 2 * ox0 + 4 * q;
+            const float4 x = *reinterpret_cast<const float4*>(x0 + at);
+            float4* o = reinterpret_cast<float4*>(out + boff + at);
+            if (MODE == 0) {
+                *o = make_float4(x.x * scale, x.y * scale, x.z * scale, x.w * scale);
+            } else {
+                const float4 so = *o;
+                float4 a = make_float4(alpha, alpha, alpha, alpha), sn;
+                if (wt) {
+                    const float4 w = *reinterpret_cast<const float4*>(wt + boff + at);
+                    a = make_float4(alpha * w.x, alpha * w.y, alpha * w.z, alpha * w.w);
+                }
+                sn.x = clip(so.x + x.x * scale, a.x); sn.y = clip(so.y + x.y * scale, a.y);
+                sn.z = clip(so.z + x.z * scale, a.z); sn.w = clip(so.w + x.w * scale, a.w);
+                *o = sn;
+                *reinterpret_cast<float4*>(ds + boff + at) =
+                    make_float4(sn.x - so.x, sn.y - so.y, sn.z - so.z, sn.w - so.w);
+            }
+        }
+        return;
+    }
+    const float* src = level == 0 ? x0 : ll_in + ll_off;
+    float* sm = reinterpret_cast<float*>(smraw);
+    PD_LF_DISPATCH(lf, (dwt32_body<MODE, LF, T>(src, ll_out, out, ds, wt, filt, k, my, mx, oy0, ox0, level == L - 1, boff,
+                                                nx, ll_off, scale, alpha, sm)));
+}
+
 // One level for every basis in blockIdx.z. MODE 0: out = coefficient * scale.
 // MODE 1: s/ds update of step 13 (wt: per-coefficient weights of the reweighted prior,
 // same layout as s, or null). The last level also treats the approximation band.
@@ -319,6 +503,146 @@ __device__ __forceinline__ void synth_tile(const R* __restrict__ coef, const R* 
     __syncthreads();
 }
 
+// FP32 tiles of 2P x 2P (P pairs of rows and columns, both sides of the sub-bands multiples of
+// P): an output pair (2m, 2m + 1) takes the tap pairs (h_2i, h_2i+1) and (g_2i, g_2i+1), so
+// each value is one packed multiply-add; bands are staged from a column that is a multiple of
+// four (16-byte pieces) on. The synthesis of an iteration at 2048^2: 192 -> 111 us; at 256^2:
+// 43 -> 27 us.
+template <int LF, int P> struct Idwt32Shape {
+    static constexpr int NK = P + LF / 2 - 1;             // staged rows of a band
+    static constexpr int HA = (LF / 2 - 1 + 3) / 4 * 4;   // staged columns before the tile
+    static constexpr int NC4 = (P + HA) / 4, BP = 4 * (NC4 | 1);
+    static constexpr int FLOATS = 4 * NK * BP + 2 * (2 * P) * BP;
+};
+template <int P> constexpr size_t idwt32_smem() { return (size_t)Idwt32Shape<MAX_FILTER, P>::FLOATS * sizeof(float); }
+template <int P> constexpr int idwt32_threads() { return P == 32 ? 256 : 128; }
+
+template <int LF, int P>
+__device__ __forceinline__ void idwt32_body(const float* __restrict__ coef, const float* __restrict__ ll_in,
+                                            const float* __restrict__ filt, int k, int level, int L, int ny, int nx,
+                                            int oy0, int ox0, float* __restrict__ dst, float* sm) {
+    using S = Idwt32Shape<LF, P>;
+    constexpr int NT = idwt32_threads<P>();
+    const int mx = nx >> level, hy = (ny >> level) >> 1, hx = mx >> 1;
+    float* band = sm;                                 // [4][NK][BP]: LL, LH, HL, HH
+    float* col = sm + 4 * S::NK * S::BP;              // [2][2P][BP]: columns synthesised, low- and high-x half
+    const int64_t boff = (int64_t)k * ny * nx;
+    const bool coarsest = level == L - 1;
+    const float* ll = coarsest ? coef + boff : ll_in + (int64_t)k * (ny / 2) * (nx / 2);
+    const int llp = coarsest ? nx : hx;
+    const int ky0 = oy0 / 2 - (LF / 2 - 1), kx0 = ox0 / 2 - S::HA;
+    {
+        constexpr int N = S::NK * S::NC4, UB = 2;
+#pragma unroll 1
+        for (int base = threadIdx.x; base < N; base += UB * NT) {
+            float4 v[UB][4];
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int i = base + u * NT, rr = i / S::NC4, q = i - rr * S::NC4;
+                if (i < N) {
+                    const int gy = (ky0 + rr) & (hy - 1), gx = (kx0 + 4 * q) & (hx - 1);
+                    const float* c = coef + boff + (int64_t)gy * nx + gx;
+                    v[u][0] = *reinterpret_cast<const float4*>(ll + (int64_t)gy * llp + gx);
+                    v[u][1] = *reinterpret_cast<const float4*>(c + (int64_t)hy * nx);
+                    v[u][2] = *reinterpret_cast<const float4*>(c + hx);
+                    v[u][3] = *reinterpret_cast<const float4*>(c + (int64_t)hy * nx + hx);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UB; ++u) {
+                const int i = base + u * NT, rr = i / S::NC4, q = i - rr * S::NC4;
+                if (i < N) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        *reinterpret_cast<float4*>(band + (e * S::NK + rr) * S::BP + 4 * q) = v[u][e];
+                }
+            }
+        }
+    }
+    float2 hp[LF / 2], gp[LF / 2];                    // tap pairs (even, odd)
+#pragma unroll
+    for (int i = 0; i < LF / 2; ++i) {
+        hp[i] = make_float2(filt[k * MAX_FILTER + 2 * i], filt[k * MAX_FILTER + 2 * i + 1]);
+        gp[i] = make_float2(filt[k * MAX_FILTER + LF - 1 - 2 * i], -filt[k * MAX_FILTER + LF - 2 - 2 * i]);
+    }
+    __syncthreads();
+    // column pass: four row pairs of one column of the low- (LL, LH) or high-x (HL, HH) half
+    constexpr int NC = P + S::HA;
+#pragma unroll 1
+    for (int it = threadIdx.x; it < 2 * NC * (P / 4); it += NT) {
+        const int c = it % NC, q = it / NC, m0 = q % (P / 4) * 4, half = q / (P / 4);
+        const float* b0 = band + 2 * half * S::NK * S::BP + c;
+        const float* b1 = b0 + S::NK * S::BP;
+        float2 acc[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < LF / 2 + 3; ++i) {        // band row m0 + i meets tap pair o + LF/2 - 1 - i of pair o
+            const float2 a = dup2(b0[(m0 + i) * S::BP]), e = dup2(b1[(m0 + i) * S::BP]);
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int j = o + LF / 2 - 1 - i;
+                if (j >= 0 && j < LF / 2) {
+                    acc[o] = ffma2(hp[j], a, acc[o]);
+                    acc[o] = ffma2(gp[j], e, acc[o]);
+                }
+            }
+        }
+        float* w = col + (half * 2 * P + 2 * m0) * S::BP + c;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            w[2 * o * S::BP] = acc[o].x;
+            w[(2 * o + 1) * S::BP] = acc[o].y;
+        }
+    }
+    __syncthreads();
+    // row pass: four column pairs of one row, consecutive threads along the row
+#pragma unroll 1
+    for (int it = threadIdx.x; it < 2 * P * (P / 4); it += NT) {
+        const int rr = it / (P / 4), m0 = it % (P / 4) * 4;
+        constexpr int NV = S::HA + 4;
+        float bl[NV], bh[NV];
+#pragma unroll
+        for (int q = 0; q < NV / 4; ++q) {
+            const float4 a = *reinterpret_cast<const float4*>(col + rr * S::BP + m0 + 4 * q);
+            const float4 e = *reinterpret_cast<const float4*>(col + (2 * P + rr) * S::BP + m0 + 4 * q);
+            bl[4 * q] = a.x; bl[4 * q + 1] = a.y; bl[4 * q + 2] = a.z; bl[4 * q + 3] = a.w;
+            bh[4 * q] = e.x; bh[4 * q + 1] = e.y; bh[4 * q + 2] = e.z; bh[4 * q + 3] = e.w;
+        }
+        float2 acc[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {                // staged column m0 + i meets tap pair o + HA - i of pair o
+            const float2 a = dup2(bl[i]), e = dup2(bh[i]);
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int j = o + S::HA - i;
+                if (j >= 0 && j < LF / 2) {
+                    acc[o] = ffma2(hp[j], a, acc[o]);
+                    acc[o] = ffma2(gp[j], e, acc[o]);
+                }
+            }
+        }
+        float4* o4 = reinterpret_cast<float4*>(dst + (int64_t)(oy0 + rr) * mx + ox0 + 2 * m0);
+        o4[0] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+        o4[1] = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
+    }
+}
+
+template <int P>
+__global__ void __launch_bounds__(idwt32_threads<P>(), P == 32 ? 3 : 6) k_idwt32_level(
+    const float* __restrict__ coef, const float* __restrict__ ll_in, float* __restrict__ ll_out,
+    const float* __restrict__ filt, const int32_t* __restrict__ flen, const int32_t* __restrict__ active, int level,
+    int L, int ny, int nx, int64_t out_stride) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int k = blockIdx.z;
+    const int lf = flen[k];
+    if (lf == 0 || (active && !active[k])) return;
+    PD_LF_DISPATCH(lf, (idwt32_body<LF, P>(coef, ll_in, filt, k, level, L, ny, nx, blockIdx.y * 2 * P, blockIdx.x * 2 * P,
+                                           ll_out + (int64_t)k * out_stride, reinterpret_cast<float*>(smraw))));
+}
+
 // One level of one basis per blockIdx.z: reconstruct the (ny>>level) x (nx>>level)
 // approximation of the next finer level into ll_out + basis * out_stride (at level 0:
 // the basis's full-size synthesis).
@@ -400,37 +724,76 @@ template <typename R> static size_t syn_smem(int ty, int tx) {
     return (size_t)(4 * NKy * NKx + 2 * ty * (NKx | 1) + ty * (tx + 1)) * sizeof(R);
 }
 
+// FP32 tile edge of a level whose sub-bands are hy x hx: 32, or 16 where tiles of 32 would
+// leave SMs without a CTA (at 256^2 the levels are one CTA's latency), 0 below 16 (the
+// generic kernel).
+static int dwt32_tile(int hy, int hx, int b, int sms) {
+    if (hy < 16 || hx < 16) return 0;
+    if (hy < 32 || hx < 32) return 16;
+    return (int64_t)(hy / 32) * (hx / 32) * b >= 2 * (int64_t)sms ? 32 : 16;
+}
+
+// One analysis level of all bases (and, at level 0, the Dirac bases).
+template <int MODE, typename R>
+static cudaError_t analysis_level(const R* x, const R* llin, R* llout, R* out, R* ds, const R* wt, const R* filt,
+                                  const int32_t* flen, const int32_t* active, int b, int lev, int L, int ny, int nx,
+                                  R scale, R alpha, int sms, cudaStream_t s) {
+    const int hy = (ny >> lev) / 2, hx = (nx >> lev) / 2;
+    cudaError_t e;
+    if constexpr (sizeof(R) == 4) {
+        // 16-byte pieces: a caller's image, coefficients or weights may start anywhere
+        const bool al = (((uintptr_t)x | (uintptr_t)out | (uintptr_t)ds | (uintptr_t)wt) & 15) == 0;
+        const int T = al ? dwt32_tile(hy, hx, b, sms) : 0;
+        if (T == 32) {
+            if ((e = ensure_smem(k_dwt32_level<MODE, 32>, dwt32_smem<32>()))) return e;
+            k_dwt32_level<MODE, 32><<<dim3(hx / 32, hy / 32, b), dwt32_threads<32>(), dwt32_smem<32>(), s>>>(
+                x, llin, llout, out, ds, wt, filt, flen, active, lev, L, ny, nx, scale, alpha);
+            return cudaGetLastError();
+        }
+        if (T == 16) {
+            if ((e = ensure_smem(k_dwt32_level<MODE, 16>, dwt32_smem<16>()))) return e;
+            k_dwt32_level<MODE, 16><<<dim3(hx / 16, hy / 16, b), dwt32_threads<16>(), dwt32_smem<16>(), s>>>(
+                x, llin, llout, out, ds, wt, filt, flen, active, lev, L, ny, nx, scale, alpha);
+            return cudaGetLastError();
+        }
+    }
+    if (lev == 0) {
+        const int64_t n = (int64_t)ny * nx;
+        const int dgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 4);
+        k_dirac<R, MODE><<<dgrid, 256, 0, s>>>(x, out, MODE == 0 ? out : ds, wt, flen, active, b, n, scale, alpha);
+        if ((e = cudaGetLastError())) return e;
+    }
+    const int ty = std::min(AT, hy), tx = std::min(AT, hx);
+    const size_t sm = ana_smem<R>(ty, tx);
+    if ((e = ensure_smem(k_dwt_level<R, MODE>, sm))) return e;
+    k_dwt_level<R, MODE><<<dim3((hx + tx - 1) / tx, (hy + ty - 1) / ty, b), NT_W, sm, s>>>(
+        x, llin, llout, out, ds, wt, filt, flen, active, lev, L, ny, nx, scale, alpha);
+    return cudaGetLastError();
+}
+
+template <int MODE, typename R>
+static cudaError_t analysis_t(const pd_plan* p, const R* x, R* out, R* ds, const int32_t* active, R alpha,
+                              cudaStream_t s, const R* wt) {
+    const int ny = p->g.ny, nx = p->g.nx, b = p->b, L = p->L;
+    const R scale = R(1.0 / std::sqrt((double)b));
+    if (p->n_wavelet == 0) {
+        const int64_t n = (int64_t)ny * nx;
+        const int dgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)p->num_sms * 4);
+        k_dirac<R, MODE><<<dgrid, 256, 0, s>>>(x, out, MODE == 0 ? out : ds, wt, p->filt_len, active, b, n, scale, alpha);
+        return cudaGetLastError();
+    }
+    cudaError_t e = cudaSuccess;
+    for (int lev = 0; lev < L && !e; ++lev)
+        e = analysis_level<MODE, R>(x, (const R*)p->ll[(lev + 1) & 1], (R*)p->ll[lev & 1], out, ds, wt,
+                                    (const R*)p->filt, p->filt_len, active, b, lev, L, ny, nx, scale, alpha, p->num_sms, s);
+    return e;
+}
+
 template <typename R>
 static cudaError_t analysis(const pd_plan* p, const R* x, R* out, R* ds, const int32_t* active, int mode, R alpha,
                             cudaStream_t s, const R* wt = nullptr) {
-    cudaError_t e;
-    const int ny = p->g.ny, nx = p->g.nx, b = p->b, L = p->L;
-    const R scale = R(1.0 / std::sqrt((double)b));
-    const int64_t n = (int64_t)ny * nx;
-    int dgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)p->num_sms * 4);
-    if (mode == 0)
-        k_dirac<R, 0><<<dgrid, 256, 0, s>>>(x, out, out, nullptr, p->filt_len, active, b, n, scale, alpha);
-    else
-        k_dirac<R, 1><<<dgrid, 256, 0, s>>>(x, out, ds, wt, p->filt_len, active, b, n, scale, alpha);
-    if ((e = cudaGetLastError())) return e;
-    if (p->n_wavelet == 0) return cudaSuccess;
-    for (int lev = 0; lev < L; ++lev) {
-        const int hy = (ny >> lev) / 2, hx = (nx >> lev) / 2;
-        const int ty = std::min(AT, hy), tx = std::min(AT, hx);
-        dim3 grid((hx + tx - 1) / tx, (hy + ty - 1) / ty, b);
-        const R* llin = (const R*)p->ll[(lev + 1) & 1];
-        R* llout = (R*)p->ll[lev & 1];
-        const size_t sm = ana_smem<R>(ty, tx);
-        if ((e = ensure_smem(k_dwt_level<R, 0>, sm)) || (e = ensure_smem(k_dwt_level<R, 1>, sm))) return e;
-        if (mode == 0)
-            k_dwt_level<R, 0><<<grid, NT_W, sm, s>>>(x, llin, llout, out, nullptr, nullptr, (const R*)p->filt,
-                                                     p->filt_len, active, lev, L, ny, nx, scale, alpha);
-        else
-            k_dwt_level<R, 1><<<grid, NT_W, sm, s>>>(x, llin, llout, out, ds, wt, (const R*)p->filt, p->filt_len,
-                                                     active, lev, L, ny, nx, scale, alpha);
-        if ((e = cudaGetLastError())) return e;
-    }
-    return cudaSuccess;
+    return mode == 0 ? analysis_t<0, R>(p, x, out, ds, active, alpha, s, nullptr)
+                     : analysis_t<1, R>(p, x, out, ds, active, alpha, s, wt);
 }
 
 template <typename R>
@@ -445,6 +808,25 @@ static cudaError_t synthesis(const pd_plan* p, const R* coef, R* out, const int3
             const int my = ny >> lev, mx = nx >> lev;
             const int ty = std::min(ST, my), tx = std::min(ST, mx);
             dim3 grid((mx + tx - 1) / tx, (my + ty - 1) / ty, b);
+            if constexpr (sizeof(R) == 4) {
+                const int P = ((uintptr_t)coef & 15) == 0 ? dwt32_tile(my / 2, mx / 2, b, p->num_sms) : 0;
+                float* to = lev > 0 ? (float*)p->ll[lev & 1] : (float*)p->synpart;
+                const int64_t st = lev > 0 ? (int64_t)(ny / 2) * (nx / 2) : n;
+                const int32_t* act = mode == 1 ? active : nullptr;
+                if (P == 32) {
+                    if ((e = ensure_smem(k_idwt32_level<32>, idwt32_smem<32>()))) return e;
+                    k_idwt32_level<32><<<dim3(mx / 64, my / 64, b), idwt32_threads<32>(), idwt32_smem<32>(), s>>>(
+                        coef, (const float*)p->ll[(lev + 1) & 1], to, (const float*)p->filt, p->filt_len, act, lev, L, ny,
+                        nx, st);
+                } else if (P == 16) {
+                    if ((e = ensure_smem(k_idwt32_level<16>, idwt32_smem<16>()))) return e;
+                    k_idwt32_level<16><<<dim3(mx / 32, my / 32, b), idwt32_threads<16>(), idwt32_smem<16>(), s>>>(
+                        coef, (const float*)p->ll[(lev + 1) & 1], to, (const float*)p->filt, p->filt_len, act, lev, L, ny,
+                        nx, st);
+                }
+                if ((e = cudaGetLastError())) return e;
+                if (P) continue;
+            }
             if ((e = ensure_smem(k_idwt_level<R>, syn_smem<R>(ty, tx)))) return e;
             // levels L-1 .. 1 rebuild the approximations, level 0 each basis's full image
             R* dst = lev > 0 ? (R*)p->ll[lev & 1] : (R*)p->synpart;
@@ -599,21 +981,17 @@ static pd_status psi_adj_static_t(const R* x, R* coeffs, int nx, int ny, int L, 
     k_psi_call_tables<R><<<1, MAX_BASES * MAX_FILTER, 0, s>>>(bl, db, filt, flen, ones);
     if ((e = cudaGetLastError())) return set_error(PD_ECUDA, cudaGetErrorString(e));
     const R scale = R(1.0 / std::sqrt((double)b));
-    const int64_t n = (int64_t)ny * nx;
-    const int dgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 4);
-    k_dirac<R, 0><<<dgrid, 256, 0, s>>>(x, coeffs, coeffs, nullptr, flen, ones, b, n, scale, R(0));
-    if ((e = cudaGetLastError())) return set_error(PD_ECUDA, cudaGetErrorString(e));
-    if (nwav == 0) return PD_OK;
-    for (int lev = 0; lev < L; ++lev) {
-        const int hy = (ny >> lev) / 2, hx = (nx >> lev) / 2;
-        const int ty = std::min(AT, hy), tx = std::min(AT, hx);
-        dim3 grid((hx + tx - 1) / tx, (hy + ty - 1) / ty, b);
-        const size_t sm = ana_smem<R>(ty, tx);
-        if ((e = ensure_smem(k_dwt_level<R, 0>, sm))) return set_error(PD_ECUDA, cudaGetErrorString(e));
-        k_dwt_level<R, 0><<<grid, NT_W, sm, s>>>(x, ll[(lev + 1) & 1], ll[lev & 1], coeffs, nullptr, nullptr, filt,
-                                                 flen, ones, lev, L, ny, nx, scale, R(0));
+    if (nwav == 0) {
+        const int64_t n = (int64_t)ny * nx;
+        const int dgrid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 4);
+        k_dirac<R, 0><<<dgrid, 256, 0, s>>>(x, coeffs, coeffs, nullptr, flen, ones, b, n, scale, R(0));
         if ((e = cudaGetLastError())) return set_error(PD_ECUDA, cudaGetErrorString(e));
+        return PD_OK;
     }
+    for (int lev = 0; lev < L; ++lev)
+        if ((e = analysis_level<0, R>(x, ll[(lev + 1) & 1], ll[lev & 1], coeffs, nullptr, nullptr, filt, flen, ones, b, lev,
+                                      L, ny, nx, scale, R(0), sms, s)))
+            return set_error(PD_ECUDA, cudaGetErrorString(e));
     return PD_OK;
 }
 
