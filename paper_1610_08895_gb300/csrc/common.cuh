@@ -107,10 +107,18 @@ __device__ __forceinline__ void stage_batched(T* dst, int n, const F& load) {
     }
 }
 
-// Allow a kernel `bytes` of dynamic shared memory. Static plus dynamic shared memory
-// above 48 KB needs the opt-in attribute, so it is always set to the requested size.
+// Allow a kernel `bytes` of dynamic shared memory. Static plus dynamic shared memory above
+// 48 KB needs the opt-in attribute; it is raised where a launch needs more than any launch of
+// that kernel on that device before (launch_cache remembers the largest request).
+cudaError_t launch_smem(const void* kernel, size_t bytes);
 template <typename K> inline cudaError_t ensure_smem(K kernel, size_t bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return launch_smem((const void*)kernel, bytes);
+}
+// Resident CTAs per SM of a kernel at a block size and dynamic shared memory size, asked for
+// once per device.
+cudaError_t launch_occupancy(const void* kernel, int threads, size_t smem, int* per_sm);
+template <typename K> inline cudaError_t occupancy(int* per_sm, K kernel, int threads, size_t smem) {
+    return launch_occupancy((const void*)kernel, threads, smem, per_sm);
 }
 
 }  // namespace pdgb

@@ -1151,7 +1151,7 @@ static cudaError_t launch_degrid(const pd_plan* p, const cplx_t<R>* grid, cplx_t
     if (e) return e;
     // items are claimed one at a time: launch only as many CTAs as are resident at once
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid<R, J, MODE>, 256, smem))) return e;
+    if ((e = occupancy(&per_sm, k_degrid<R, J, MODE>, 256, smem))) return e;
     const int ctas = (int)std::min<int64_t>((int64_t)p->n_ditems * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
     k_degrid<R, J, MODE><<<ctas, 256, smem, s>>>(
         grid, out, a ? (const cplx_t<R>*)a->y : nullptr, a ? (const cplx_t<R>*)a->v : nullptr,
@@ -1227,7 +1227,7 @@ static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const Du
     cudaError_t e;
     if ((e = ensure_smem(k_grid_mma<J, MODE>, p->grid_smem))) return e;
     int per_sm = 1;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid_mma<J, MODE>, p->grid_warps * 32,
+    if ((e = occupancy(&per_sm, k_grid_mma<J, MODE>, p->grid_warps * 32,
                                                            p->grid_smem)))
         return e;
     const int ctas = (int)std::min<int64_t>((int64_t)p->n_items * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
@@ -1269,7 +1269,7 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
         if ((e = ensure_smem(k_grid8w<R, J, MODE>, smem8))) return e;
         int per_sm = 0;
         int ctas8 = std::min(g.ntiles * batch, p->num_sms * 16);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid8w<R, J, MODE>, nw * 32, smem8) ==
+        if (occupancy(&per_sm, k_grid8w<R, J, MODE>, nw * 32, smem8) ==
                 cudaSuccess && per_sm > 0)
             ctas8 = std::min(ctas8, per_sm * p->num_sms);
         k_grid8w<R, J, MODE><<<ctas8, nw * 32, smem8, s>>>(

@@ -299,7 +299,7 @@ static cudaError_t degrid_csr_w(const pd_plan* p, const cplx_t<R>* grid, cplx_t<
     cudaError_t e = ensure_smem(k_degrid_csr<R, W, J, MODE>, smem);
     if (e) return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid_csr<R, W, J, MODE>, 256, smem))) return e;
+    if ((e = occupancy(&per_sm, k_degrid_csr<R, W, J, MODE>, 256, smem))) return e;
     const int ctas = (int)std::min<int64_t>((int64_t)p->n_ditems * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
     k_degrid_csr<R, W, J, MODE><<<ctas, 256, smem, s>>>(
         grid, out, a ? (const cplx_t<R>*)a->y : nullptr, a ? (const cplx_t<R>*)a->v : nullptr,
@@ -479,7 +479,7 @@ static cudaError_t grid_csr_w(const pd_plan* p, const cplx_t<R>* src, const Dual
     cudaError_t e = ensure_smem(k_grid_csr<R, W, J, MODE>, smem);
     if (e) return e;
     int per_sm = 0, ctas = std::min(g.ntiles * batch, p->num_sms * 8);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grid_csr<R, W, J, MODE>, nw * 32, smem) ==
+    if (occupancy(&per_sm, k_grid_csr<R, W, J, MODE>, nw * 32, smem) ==
             cudaSuccess && per_sm > 0)
         ctas = std::min(ctas, per_sm * p->num_sms);
     k_grid_csr<R, W, J, MODE><<<ctas, nw * 32, smem, s>>>(
