@@ -362,30 +362,47 @@ __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN
     __syncthreads();
     fft_smem<R, N, +1, 2 * P::PAIRS>(s, twx);
     R adx = R(0), ax = R(0);
-    for (int e = threadIdx.x; e < P::PAIRS * N; e += NT) {
-        const int pr = e / N, ix = e % N;
-        const int lc = ix - N / 2;
-        const int m = padi<R>(lc & (N - 1));
-        const C2 w = cconj(__ldg(&twx[lc & (Kx - 1)]));
-        const C2* ev = s + (2 * pr) * S::PN;
-        const C2 z = cadd(ev[m], cmul(w, ev[S::PN + m]));
-        const R c = cx[ix], cl = cxl[ix];
+    // pixels of several steps at a time: their x and s~ loads go out together
+    constexpr int EB = sizeof(R) == 4 ? 4 : 2;
+    for (int e0 = threadIdx.x; e0 < P::PAIRS * N; e0 += EB * NT) {
+        R xo[EB][2], so[EB][2];
+        if (mode == 1) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int iy = iy0 + 2 * pr + h;
-            const R g = deapodise(h ? z.y : z.x, c, cl, cy[iy], cyl[iy]);
-            const int64_t idx = (int64_t)iy * N + ix;
-            if (mode == 0) {
-                out[idx] = g;
-            } else {
-                const R xo = xs[idx];
-                R xn = xo - tau * (sigma * st_[idx] + varsigma * g);
-                xn = xn > R(0) ? xn : R(0);
-                xt[idx] = R(2) * xn - xo;
-                xs[idx] = xn;
-                const R dd = xn - xo;
-                adx += dd * dd;
-                ax += xn * xn;
+            for (int u = 0; u < EB; ++u) {
+                const int e = e0 + u * NT;
+                if (e >= P::PAIRS * N) break;
+                const int64_t idx = (int64_t)(iy0 + 2 * (e / N)) * N + e % N;
+                xo[u][0] = xs[idx]; xo[u][1] = xs[idx + N];
+                so[u][0] = st_[idx]; so[u][1] = st_[idx + N];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < EB; ++u) {
+            const int e = e0 + u * NT;
+            if (e >= P::PAIRS * N) break;
+            const int pr = e / N, ix = e % N;
+            const int lc = ix - N / 2;
+            const int m = padi<R>(lc & (N - 1));
+            const C2 w = cconj(__ldg(&twx[lc & (Kx - 1)]));
+            const C2* ev = s + (2 * pr) * S::PN;
+            const C2 z = cadd(ev[m], cmul(w, ev[S::PN + m]));
+            const R c = cx[ix], cl = cxl[ix];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int iy = iy0 + 2 * pr + h;
+                const R g = deapodise(h ? z.y : z.x, c, cl, cy[iy], cyl[iy]);
+                const int64_t idx = (int64_t)iy * N + ix;
+                if (mode == 0) {
+                    out[idx] = g;
+                } else {
+                    R xn = xo[u][h] - tau * (sigma * so[u][h] + varsigma * g);
+                    xn = xn > R(0) ? xn : R(0);
+                    xt[idx] = R(2) * xn - xo[u][h];
+                    xs[idx] = xn;
+                    const R dd = xn - xo[u][h];
+                    adx += dd * dd;
+                    ax += xn * xn;
+                }
             }
         }
     }

@@ -271,7 +271,13 @@ __global__ void __launch_bounds__(256) k_slot_sq(const cplx_t<R>* __restrict__ y
     for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < nslot; k += step) {
         const SegSlot r = range[k];
         double a = 0.0;
-        for (int m = r.start + lane; m < r.end; m += 32) a += (double)y[m].x * y[m].x + (double)y[m].y * y[m].y;
+        for (int m0 = r.start + lane; m0 < r.end; m0 += 4 * 32) {
+            cplx_t<R> v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = m0 + 32 * u < r.end ? y[m0 + 32 * u] : mk<cplx_t<R>>(R(0), R(0));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a += (double)v[u].x * v[u].x + (double)v[u].y * v[u].y;
+        }
         a = warp_sum(a);
         if (lane == 0) part[2 * k + 1] = a;
     }
