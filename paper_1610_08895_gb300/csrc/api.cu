@@ -163,8 +163,13 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     // default tile: 16 cells, so that small grids still make enough work items and dense ones
     // no long ones; 32 for FP32 grids of 2048^2 cells and more, whose items fill the GPU anyway
     // and then spend less on windows. At least two tiles per grid side, for the tile colours.
+    // Tiles of 8 spread the work of a stored G (real rows) and of the FP64 kernels up to 1024^2
+    // cells best.
     const bool fly32 = d->precision == PD_F32 && d->g_mode == PD_G_ON_THE_FLY && d->kernel_width <= 8;
-    int T = d->tile ? d->tile : (fly32 && (int64_t)g.Kx * g.Ky >= (int64_t)2048 * 2048 ? 32 : 16);
+    const int64_t cells = (int64_t)g.Kx * g.Ky;
+    int T = d->tile ? d->tile
+            : fly32 ? (cells >= (int64_t)2048 * 2048 ? 32 : 16)
+            : (d->g_mode == PD_G_CSR && !dde) || (d->g_mode != PD_G_CSR && cells <= (int64_t)1024 * 1024) ? 8 : 16;
     auto fit = [&](int t) {
         while (t > std::min(g.Kx, g.Ky) / 2) t >>= 1;
         while (t < g.J) t <<= 1;
@@ -218,10 +223,11 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         if (blk < 0 || blk >= p->d) return fail(PD_EINVAL, "block_of_vis out of range");
         double gxv = u * g.Kx / (2.0 * M_PI), gyv = v * g.Ky / (2.0 * M_PI);
         p->h_base[m] = base_cell(gxv, gyv);
-        // Held at -(u, v) as its conjugate. A point on a grid line (to the working precision)
+        // Held at -(u, v) as its conjugate, where G is evaluated in the kernels (a stored G gains
+        // nothing: its rows are read all the same). A point on a grid line (to the working precision)
         // stays where it is: its taps reach J/2 cells to one side only, and the mirrored ones
         // would to the other.
-        if (!dde && u < 0 && inside(gxv) && inside(gyv)) {
+        if (p->g_mode == PD_G_ON_THE_FLY && u < 0 && inside(gxv) && inside(gyv)) {
             gxv = -gxv;
             gyv = -gyv;
             flip[m] = 1;
@@ -808,7 +814,7 @@ static pd_status set_start_t(pd_plan* p, pd_state* st, const void* x0, const voi
     } else {
         CU(cudaMemsetAsync(st->v, 0, p->M * p->csz, s));
         CU(cudaMemsetAsync(st->u, 0, K * p->csz, s));
-    }
+        }
     CU(cudaMemsetAsync(st->t, 0, sizeof(int64_t), s));
     CU(cudaMemsetAsync(st->diag, 0, 2 * sizeof(double), s));
     // residual norms of the adaptive probabilities: ||Phi_i x^(0) - y_i||

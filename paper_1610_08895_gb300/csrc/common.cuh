@@ -62,6 +62,16 @@ __host__ __device__ inline double philox_uniform(uint64_t seed, uint64_t t, uint
     return (double)(philox_word0(t, stream, index, 0, seed, 0) >> 11) * (1.0 / 9007199254740992.0);
 }
 
+// Packed FP32 multiply-add: a b + c in both halves, one instruction.
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+          "l"(reinterpret_cast<const unsigned long long&>(c)));
+    return d;
+}
+
 // Deterministic block-wide sum of a double for any blockDim.x that is a multiple
 // of 32 (fixed shuffle tree per warp, then warp 0). sh must hold 32 doubles.
 // The result is valid in thread 0.

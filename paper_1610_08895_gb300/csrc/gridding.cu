@@ -89,11 +89,14 @@ __device__ __forceinline__ void stage_window_pairs(float2* win, const float2* __
     }
 }
 
+// Bound by the shared-memory pipe (32 16-byte window reads a point). Four CTAs per SM: five
+// leave 48 registers and spill (16.8M points, half active, 4096^2 grid: 222 us against 231;
+// packed multiply-adds of the (re, im) pairs did not help either way: 238 us).
 // MODE 0 (plain): out_user[perm[m]] = (G grid)_m for every visibility of the listed tiles.
 // MODE 1 (pd): for visibilities of active blocks r = v + G b - y, with FP64 sums of
 // ||r||^2 and ||G b - y||^2 per (tile, block) segment (per-warp slots, summed in warp order).
 template <typename R, int J, int MODE>
-__global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_degrid(const cplx_t<R>* __restrict__ grid, cplx_t<R>* __restrict__ out,
+__global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 4 : 3) : 1) k_degrid(const cplx_t<R>* __restrict__ grid, cplx_t<R>* __restrict__ out,
                                                 const cplx_t<R>* __restrict__ y, const cplx_t<R>* __restrict__ v,
                                                 cplx_t<R>* __restrict__ rbuf, const int32_t* __restrict__ cell,
                                                 const R* __restrict__ fxs, const R* __restrict__ fys,
@@ -128,9 +131,8 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
         __syncthreads();
         const int w = item_s;
         if (w >= n * batch) break;
-        // item w / batch of the heaviest-first list for image w mod batch (a batch of plain applications)
         const TileItem ti = ti_s;
-        const int t = ti.tile, img = w % batch;
+        const int t = ti.tile, img = w / n;
         const cplx_t<R>* gimg = grid + (int64_t)img * gstride;
         cplx_t<R>* oimg = MODE == 0 ? out + (int64_t)img * ostride : out;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
@@ -234,28 +236,35 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 5 : 3) : 1) k_
     if (threadIdx.x == 0) leave_items(sched);
 }
 
-// Per-block FP64 norms summed over the block's seg_part slots in a fixed order (one warp per
-// block: lane-strided partial sums, then a fixed shuffle tree), the ball scale
+// Per-block FP64 norms summed over the block's seg_part slots in a fixed order (one CTA per
+// block: thread-strided partial sums, then a fixed tree; one warp per block took 48 us for the
+// 1,500 slots of each of 64 blocks in tiles of 8 cells), the ball scale
 // c_i = max(0, 1 - eps_i/||r_i||) of step 8 (so v_new = c_i r_i = z - P_B(z)), and the
 // residual norm ||G_i b - y_i|| for the adaptive probabilities of Sec. 4.
 // norm_only (active == nullptr: every block): only the residual norm is written.
 template <typename R>
-__global__ void k_block_norms(const double* __restrict__ part, const int32_t* __restrict__ bss,
+__global__ void __launch_bounds__(128) k_block_norms(const double* __restrict__ part, const int32_t* __restrict__ bss,
                               const int32_t* __restrict__ bsl, const int32_t* __restrict__ active,
                               const double* __restrict__ eps, double* __restrict__ bnorm, R* __restrict__ scale,
                               double* __restrict__ res_norm, int d, int norm_only) {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= d || (active && !active[i])) return;     // whole warps leave together
+    __shared__ double sh[32];
+    const int i = blockIdx.x;
+    if (active && !active[i]) return;
     double sr = 0.0, sd = 0.0;
-    for (int k = bss[i] + lane; k < bss[i + 1]; k += 32) {
-        const int sg = bsl[k];
-        sr += part[2 * sg];
-        sd += part[2 * sg + 1];
+    const int end = bss[i + 1];
+    for (int k0 = bss[i] + threadIdx.x; k0 < end; k0 += 4 * (int)blockDim.x) {
+        double2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = k0 + u * (int)blockDim.x;
+            v[u] = k < end ? *reinterpret_cast<const double2*>(part + 2 * (int64_t)bsl[k]) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { sr += v[u].x; sd += v[u].y; }
     }
-    sr = warp_sum(sr);
-    sd = warp_sum(sd);
-    if (lane != 0) return;
+    sr = block_sum(sr, sh);
+    sd = block_sum(sd, sh);
+    if (threadIdx.x != 0) return;
     if (norm_only) {
         res_norm[i] = sqrt(sd);
         return;
@@ -370,7 +379,15 @@ template <typename R> __device__ __forceinline__ void st4(R* p, R a, R b, R c, R
 }
 // lo, hi += the class weight's low / high part times ry
 template <typename C2, typename R> __device__ __forceinline__ void acc_cand(C2& lo, C2& hi, R w, C2 ry) {
-    const R wl = w > R(0) ? w : R(0), wh = w < R(0) ? -w : R(0);
+    R wl, wh;
+    if constexpr (sizeof(R) == 8) {      // by the sign bit: a comparison would take the FP64 pipe
+        const bool neg = __double2hiint(w) < 0;
+        wl = neg ? 0.0 : w;
+        wh = neg ? -w : 0.0;
+    } else {
+        wl = w > R(0) ? w : R(0);
+        wh = w < R(0) ? -w : R(0);
+    }
     lo.x += wl * ry.x; lo.y += wl * ry.y;
     hi.x += wh * ry.x; hi.y += wh * ry.y;
 }
@@ -465,8 +482,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
         __syncthreads();
         const int w = tile_s;
         if (w >= n * batch) break;
-        // work item w: tile w / batch of the list for image w mod batch (plain gridding of a batch)
-        const int t = list[w / batch], img = w % batch;
+        const int t = list[w % n], img = w / n;   // image by image of a batch
         const cplx_t<R>* simg = MODE == 0 ? src + (int64_t)img * istride : src;
         cplx_t<R>* Uimg = U + (int64_t)img * ustride;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
@@ -837,9 +853,9 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
     if (warp == nc) {
         // ---------------------------------------------------------------- the feeding warp
         int* act_seg = reinterpret_cast<int*>(lbase + 2 * lsz);
-        const int nitem = *nitems * batch;
+        const int nlist = *nitems, nitem = nlist * batch;
         // claims the next item with an active block (items are claimed in order by whichever CTA is
-        // free; item w: items[w / batch] for image w mod batch of a batch) and lists it in buffer b
+        // free, a batch image by image) and lists it in buffer b
         auto prepare = [&](int b) -> bool {
             const GridLists L(lbase + b * lsz, nsc, max_segs);
             int w;
@@ -852,7 +868,7 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
                     if (lane == 0) item_s[b].tile = -1;
                     return false;
                 }
-                it = items[w / batch];
+                it = items[w % nlist];
                 ti = tile_info[it.x];
                 if (!tile_on || tile_on[it.x]) break;
             }
@@ -934,7 +950,7 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
                 }
                 L.sinfo[sc] = si;
             }
-            if (lane == 0) item_s[b] = GridItem{it.x, w % batch, it.y, ti.z, nact, padded, cbeg, nchunk};
+            if (lane == 0) item_s[b] = GridItem{it.x, w / nlist, it.y, ti.z, nact, padded, cbeg, nchunk};
             return true;
         };
         bool have = prepare(0);
@@ -1172,7 +1188,7 @@ cudaError_t degrid_plain(const pd_plan* p, const cplx_t<R>* grid, cplx_t<R>* out
 template <typename R>
 static cudaError_t block_norms(const pd_plan* p, const int32_t* active, const double* eps, double* res_norm,
                                int norm_only, cudaStream_t s) {
-    k_block_norms<R><<<(p->d * 32 + 127) / 128, 128, 0, s>>>(p->seg_part, p->block_slot_start, p->block_slot_list,
+    k_block_norms<R><<<p->d, 128, 0, s>>>(p->seg_part, p->block_slot_start, p->block_slot_list,
                                                              active, eps, p->blk_norm, (R*)p->blk_scale, res_norm,
                                                              p->d, norm_only);
     return cudaGetLastError();

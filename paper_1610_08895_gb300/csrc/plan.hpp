@@ -67,7 +67,7 @@ struct SegSlot {
 constexpr int SC = 8;
 
 // The image is real, so the visibility at -(u, v) is the conjugate of the one at (u, v):
-// points with u < 0 are held at -(u, v) as conjugates (unless G has DDEs, or the point is
+// points with u < 0 are held at -(u, v) as conjugates (unless G is stored, or the point is
 // on a grid line), which leaves norms, duals and Re(Phi^H .) as they are and halves the tiles that hold points. perm
 // carries the flag in its sign bit; these read and write a value in the user's convention.
 __host__ __device__ __forceinline__ int vis_index(int q) { return q & 0x7fffffff; }

@@ -160,14 +160,6 @@ __device__ __forceinline__ void dwt_body(const R* __restrict__ src, R* __restric
 // quarter-warp on eight rows hit distinct banks), and in the column pass a warp's threads take
 // consecutive columns. Bound by instruction issue (2 LF multiply-adds a pixel). The analysis of
 // an iteration at 2048^2 (half of nine bases, four levels): 217 -> 124 us; at 256^2: 54 -> 25 us.
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(reinterpret_cast<unsigned long long&>(d))
-        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
-          "l"(reinterpret_cast<const unsigned long long&>(c)));
-    return d;
-}
 __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 
 template <int LF, int T> struct Dwt32Shape {
