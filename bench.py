@@ -147,7 +147,7 @@ class Clocks:
 
 
 # committed ncu summaries with the measured DRAM traffic of a kernel, per bench phase
-PROFILE_OF_PHASE = {"grid_dual": "k_grid8w_gridding_c5.md", "degrid_dual": "k_degrid_degridding_c5.md"}
+PROFILE_OF_PHASE = {"grid_dual": "k_grid_mma_gridding_c5.md", "degrid_dual": "k_degrid_degridding_c5.md"}
 
 
 def kernel_source_hash(path, name):
@@ -285,10 +285,10 @@ def run_cufft(n, stream, reps=20):
             "ifft2_ms": round(_time_ms(lambda: torch.fft.ifft2(g), reps, stream), 4)}
 
 
-# our kernels per iteration: draws; 2 forward passes; degridding + block norms; 4 gridding
-# colour launches; L analysis levels + the Dirac basis; L synthesis levels + the ordered
-# sum; 2 inverse passes; the primal norm sums
-KERNELS_PER_ITER = lambda L: 1 + 2 + 2 + 4 + (L + 1) + (L + 1) + 2 + 1   # noqa: E731
+# our kernels per iteration: draws (a second launch flags the tiles of the large workloads, not
+# counted); 2 forward passes; degridding + block norms; gridding; L analysis levels (the Dirac
+# basis in the first); L synthesis levels + the ordered sum; 2 inverse passes; the primal norm sums
+KERNELS_PER_ITER = lambda L: 1 + 2 + 2 + 1 + L + (L + 1) + 2 + 1   # noqa: E731
 
 
 # ---------------------------------------------------------------------------------------------
@@ -637,7 +637,7 @@ def run_profile_target(args):
     """A short, deterministic launch sequence for ncu: plan, y from synthetic noise, start
     values x^(0) = x~^(0) = the test image, then args.profile_run eager iterations (per
     iteration: draws, 4 analysis + 4 synthesis levels and the sum, 2 forward passes,
-    degridding, block norms, 4 gridding colour launches, 2 inverse passes, primal sums)."""
+    degridding, block norms, gridding, 2 inverse passes, primal sums)."""
     import torch
     import __graft_entry__ as ge
     ge.build()

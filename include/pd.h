@@ -285,7 +285,7 @@ typedef struct {
     int32_t per_block;             /* 1: the plain per-block form, for comparison with the batched
                                       one: the host draws the active sets (same Philox draws) and
                                       launches the degridding, ball projection and gridding
-                                      (four tile-colour launches) once per active block and the
+                                      (FP64: four tile-colour launches) once per active block and the
                                       wavelet analysis and synthesis once per active basis;
                                       same results up to rounding
                                       order. Needs adaptive = 0 and use_graph = 0; synchronises
