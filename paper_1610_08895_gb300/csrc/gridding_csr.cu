@@ -373,8 +373,12 @@ __device__ __forceinline__ cplx_t<R> grid_raw_value(const GridRaw<R>& in, cplx_t
 // Each warp takes a contiguous share of the tile's active visibilities (fixed by the
 // warp index, so the summation order is too) and adds them one at a time into its own
 // E x E window; the windows are then summed in warp order and added to U.
-template <typename R, typename W, int J, int MODE>
-__global__ void __launch_bounds__(256, sizeof(W) == sizeof(R) ? 4 : 2) k_grid_csr(
+// PB: visibilities whose entries are loaded together. Eight, with two CTAs per SM; real weights
+// in tiles of 8 cells, whose windows leave room, four with four CTAs (4.2M visibilities, half
+// active, 2048^2 grid: 356 us against 534 us with eight and two, 393 us with two and six; in
+// tiles of 16 eight and two are better, 570 against 836 us).
+template <typename R, typename W, int J, int MODE, int PB>
+__global__ void __launch_bounds__(256, PB == 4 ? 4 : 2) k_grid_csr(
     const cplx_t<R>* __restrict__ src, const cplx_t<R>* __restrict__ rbuf, cplx_t<R>* __restrict__ v,
     const R* __restrict__ scale, const int32_t* __restrict__ active, const int32_t* __restrict__ col,
     const W* __restrict__ val, const int32_t* __restrict__ perm, const int32_t* __restrict__ seg_start,
@@ -383,10 +387,6 @@ __global__ void __launch_bounds__(256, sizeof(W) == sizeof(R) ? 4 : 2) k_grid_cs
     cplx_t<R>* __restrict__ U, int max_segs, Geo g, int* __restrict__ next_tile, int batch, int64_t sstride, int64_t ustride) {
     using C2 = cplx_t<R>;
     constexpr int NE = J * J;                 // entries per row of G (<= 64: two per lane)
-    // visibilities whose entries are loaded together: real weights four, with four CTAs per SM at
-    // tiles of 8 cells (4.2M visibilities, half active, 2048^2 grid: 356 us against 534 us with
-    // eight and two CTAs and 393 us with two and six); complex ones eight, with two CTAs
-    constexpr int PB = sizeof(W) == sizeof(R) ? 4 : 8;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int E = g.ext, EE = E * E;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -470,8 +470,8 @@ __global__ void __launch_bounds__(256, sizeof(W) == sizeof(R) ? 4 : 2) k_grid_cs
     }
 }
 
-template <typename R, typename W, int J, int MODE>
-static cudaError_t grid_csr_w(const pd_plan* p, const cplx_t<R>* src, const DualArgs* a, const int32_t* tiles,
+template <typename R, typename W, int J, int MODE, int PB>
+static cudaError_t grid_csr_pb(const pd_plan* p, const cplx_t<R>* src, const DualArgs* a, const int32_t* tiles,
                               const int32_t* count, cplx_t<R>* U, int* next_tile, cudaStream_t s, int batch) {
     const Geo& g = p->g;
     const int ms = std::max(p->max_tile_segs, 1);
@@ -479,17 +479,25 @@ static cudaError_t grid_csr_w(const pd_plan* p, const cplx_t<R>* src, const Dual
     // eight warps unless their windows do not fit (large tiles in FP64)
     const int nw = (int)std::max<size_t>(1, std::min<size_t>(8, ((size_t)200 << 10) / winb));
     const size_t smem = nw * winb + (size_t)(2 * ms + 1) * sizeof(int);
-    cudaError_t e = ensure_smem(k_grid_csr<R, W, J, MODE>, smem);
+    cudaError_t e = ensure_smem(k_grid_csr<R, W, J, MODE, PB>, smem);
     if (e) return e;
     int per_sm = 0, ctas = std::min(g.ntiles * batch, p->num_sms * 8);
-    if (occupancy(&per_sm, k_grid_csr<R, W, J, MODE>, nw * 32, smem) ==
+    if (occupancy(&per_sm, k_grid_csr<R, W, J, MODE, PB>, nw * 32, smem) ==
             cudaSuccess && per_sm > 0)
         ctas = std::min(ctas, per_sm * p->num_sms);
-    k_grid_csr<R, W, J, MODE><<<ctas, nw * 32, smem, s>>>(
+    k_grid_csr<R, W, J, MODE, PB><<<ctas, nw * 32, smem, s>>>(
         src, (const cplx_t<R>*)p->rbuf, a ? (cplx_t<R>*)a->v : nullptr, (const R*)p->blk_scale,
         a ? a->block_active : nullptr, p->csr_col, (const W*)p->csr_val, p->perm, p->seg_start, p->seg_block,
         p->tile_seg_start, tiles, count, a ? a->tile_on : nullptr, U, ms, g, next_tile, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     return cudaGetLastError();
+}
+
+template <typename R, typename W, int J, int MODE>
+static cudaError_t grid_csr_w(const pd_plan* p, const cplx_t<R>* src, const DualArgs* a, const int32_t* tiles,
+                              const int32_t* count, cplx_t<R>* U, int* next_tile, cudaStream_t s, int batch) {
+    if constexpr (std::is_same<W, float>::value)
+        if (p->g.tile == 8) return grid_csr_pb<R, W, J, MODE, 4>(p, src, a, tiles, count, U, next_tile, s, batch);
+    return grid_csr_pb<R, W, J, MODE, 8>(p, src, a, tiles, count, U, next_tile, s, batch);
 }
 
 template <typename R, int J, int MODE>

@@ -667,8 +667,10 @@ __global__ void __launch_bounds__(NT_W) k_idwt_level(const R* __restrict__ coef,
 // active bases in basis order: MODE 0: out = acc * scale, MODE 1: out += acc * scale
 // (the s~ update of step 14). Four consecutive pixels per thread.
 template <typename R> struct Quad { R a, b, c, d; };
-template <typename R> __device__ __forceinline__ Quad<R> ldq(const R* p) {
-    if constexpr (sizeof(R) == 4) {
+template <typename R, bool VEC> __device__ __forceinline__ Quad<R> ldq(const R* p) {
+    if constexpr (!VEC) {
+        return {p[0], p[1], p[2], p[3]};
+    } else if constexpr (sizeof(R) == 4) {
         const float4 q = *reinterpret_cast<const float4*>(p);
         return {q.x, q.y, q.z, q.w};
     } else {
@@ -676,8 +678,10 @@ template <typename R> __device__ __forceinline__ Quad<R> ldq(const R* p) {
         return {q0.x, q0.y, q1.x, q1.y};
     }
 }
-template <typename R> __device__ __forceinline__ void stq(R* p, const Quad<R>& v) {
-    if constexpr (sizeof(R) == 4) {
+template <typename R, bool VEC> __device__ __forceinline__ void stq(R* p, const Quad<R>& v) {
+    if constexpr (!VEC) {
+        p[0] = v.a; p[1] = v.b; p[2] = v.c; p[3] = v.d;
+    } else if constexpr (sizeof(R) == 4) {
         *reinterpret_cast<float4*>(p) = make_float4(v.a, v.b, v.c, v.d);
     } else {
         *reinterpret_cast<double2*>(p) = make_double2(v.a, v.b);
@@ -685,7 +689,8 @@ template <typename R> __device__ __forceinline__ void stq(R* p, const Quad<R>& v
     }
 }
 
-template <typename R, int MODE>
+// VEC: both the coefficients and the output are 16-byte aligned (a caller's may start anywhere).
+template <typename R, int MODE, bool VEC>
 __global__ void __launch_bounds__(256) k_syn_sum(const R* __restrict__ coef, const R* __restrict__ part,
                                                  const int32_t* __restrict__ flen, const int32_t* __restrict__ active,
                                                  int b, int64_t n, R* __restrict__ out, R scale) {
@@ -694,15 +699,15 @@ __global__ void __launch_bounds__(256) k_syn_sum(const R* __restrict__ coef, con
         Quad<R> acc{R(0), R(0), R(0), R(0)};
         for (int k = 0; k < b; ++k) {
             if (MODE == 1 && !active[k]) continue;
-            const Quad<R> v = ldq((flen[k] == 0 ? coef : part) + (int64_t)k * n + i);
+            const Quad<R> v = ldq<R, VEC>((flen[k] == 0 ? coef : part) + (int64_t)k * n + i);
             acc.a += v.a; acc.b += v.b; acc.c += v.c; acc.d += v.d;
         }
         Quad<R> o{acc.a * scale, acc.b * scale, acc.c * scale, acc.d * scale};
         if (MODE == 1) {
-            const Quad<R> prev = ldq(out + i);
+            const Quad<R> prev = ldq<R, VEC>(out + i);
             o.a += prev.a; o.b += prev.b; o.c += prev.c; o.d += prev.d;
         }
-        stq(out + i, o);
+        stq<R, VEC>(out + i, o);
     }
 }
 
@@ -830,10 +835,12 @@ static cudaError_t synthesis(const pd_plan* p, const R* coef, R* out, const int3
         }
     }
     const int ctas = (int)std::min<int64_t>((n / 4 + 255) / 256, (int64_t)p->num_sms * 8);
-    if (mode == 0)
-        k_syn_sum<R, 0><<<ctas, 256, 0, s>>>(coef, (const R*)p->synpart, p->filt_len, active, b, n, out, scale);
-    else
-        k_syn_sum<R, 1><<<ctas, 256, 0, s>>>(coef, (const R*)p->synpart, p->filt_len, active, b, n, out, scale);
+    const bool vec = (((uintptr_t)coef | (uintptr_t)out) & 15) == 0;
+    auto sum = [&](auto kernel) {
+        kernel<<<ctas, 256, 0, s>>>(coef, (const R*)p->synpart, p->filt_len, active, b, n, out, scale);
+    };
+    if (mode == 0) vec ? sum(k_syn_sum<R, 0, true>) : sum(k_syn_sum<R, 0, false>);
+    else vec ? sum(k_syn_sum<R, 1, true>) : sum(k_syn_sum<R, 1, false>);
     return cudaGetLastError();
 }
 

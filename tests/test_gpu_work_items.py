@@ -90,3 +90,23 @@ def test_checkpoint_order_of_the_visibilities(tile):
     other = State(plan)
     other.load(buf)
     assert np.array_equal(other.v().cpu().numpy(), v0)
+
+
+@pytest.mark.parametrize("n,levels", [(16, 2), (32, 1), (64, 3), (128, 2), (256, 4)])
+def test_dictionary_on_buffers_that_start_anywhere(n, levels):
+    """Psi^H and Psi on 4-byte aligned buffers equal the aligned ones: the 16-byte kernels and
+    the general ones they give way to (and each of their tile sizes) compute the same filters."""
+    from paper_1610_08895_gb300.api import Plan
+    ids = (0, 1, 2, 5, 8)
+    plan = Plan(n, n, np.zeros((1, 2)), np.zeros(1, np.int32), 1, basis_ids=ids, levels=levels)
+    x = torch.tensor(synth.random_images(1, n, n, seed=1)[0], dtype=torch.float32, device="cuda")
+    big = torch.zeros(n * n + 1, dtype=torch.float32, device="cuda")
+    odd = big[1:].view(n, n)
+    odd.copy_(x)
+    a = plan.pd_apply_psi_adj(x)
+    coeffs = torch.zeros(a.numel() + 1, dtype=torch.float32, device="cuda")[1:].view_as(a)
+    b = plan.pd_apply_psi_adj(odd, coeffs)
+    assert rel(b.cpu().numpy(), a.cpu().numpy()) < 2e-6        # 2 x 16 taps a level, summed in another order
+    back = plan.pd_apply_psi(b, torch.zeros(n * n + 1, dtype=torch.float32, device="cuda")[1:].view(n, n))
+    assert rel(back.cpu().numpy(), x.cpu().numpy()) < TOL_OP32
+    assert rel(plan.pd_apply_psi(a).cpu().numpy(), x.cpu().numpy()) < TOL_OP32
