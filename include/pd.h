@@ -389,7 +389,9 @@ pd_status pd_state_report(const pd_plan* plan, const pd_state* st, int64_t* t, d
  * pd_state_bytes() bytes to host `buf`; pd_state_load restores it (same plan).
  * The counter-based draws make a resumed run identical to an uninterrupted one. v and y are
  * stored by the base cells of the points in tiles of `tile` (0: 32) cells, independently of the
- * plan's internal order; the first save or load of a plan sorts the points once on the host.
+ * plan's internal order; the first save or load of a plan sorts the points once on the host
+ * (PD_ENOMEM if that finds no memory). Both touch the state and no scratch of the plan: other
+ * states of the plan may iterate on other streams meanwhile, and any thread may save its own.
  */
 size_t pd_state_bytes(const pd_plan* plan);
 pd_status pd_state_save(const pd_plan* plan, const pd_state* st, void* buf, void* stream);

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -749,6 +750,8 @@ extern "C" pd_status pd_state_create(pd_plan* p, pd_state** out) {
               !dalloc(A, B, &st->basis_active, p->b) &&
               !dalloc(A, B, &st->tile_active, p->g.ntiles) && !dalloc(A, B, &st->counts, 2) && !dalloc(A, B, &st->t, 1) && !dalloc(A, B, &st->diag, 2) &&
               !dalloc(A, B, &st->prim_part, 2 * (size_t)inv_rows_ctas(p)) && !dalloc(A, B, &st->status, 1);
+    st->ck_cap = std::min<int64_t>(p->M, 1 << 20);
+    ok = ok && !dalloc_bytes(A, B, &st->ck_vis, st->ck_cap * p->csz) && !dalloc(A, B, &st->ck_idx, st->ck_cap);
     if (!ok) {
         pd_state_destroy(st);
         return fail(PD_ENOMEM, "pd_state_create: device allocation failed");
@@ -1304,8 +1307,10 @@ static std::vector<Part> state_parts(const pd_plan* p, const pd_state* st) {
             {st->res_norm, p->d * sizeof(double), false}, {st->p_block, p->d * sizeof(double), false},
             {st->p_basis, p->b * sizeof(double), false}, {st->t, sizeof(int64_t), false}};
 }
+// The plan's ck_order, made on first use; any thread may ask.
 static pd_status ensure_ck(pd_plan* p) {
-    if (p->ck_perm) return PD_OK;
+    std::lock_guard<std::mutex> lock(p->ck_mu);
+    if (!p->ck_order.empty()) return PD_OK;
     const int64_t M = p->M;
     std::vector<int32_t> perm(M), seg(p->nseg + 1);
     CU(cudaMemcpy(perm.data(), p->perm, M * sizeof(int32_t), cudaMemcpyDeviceToHost));
@@ -1331,8 +1336,47 @@ static pd_status ensure_ck(pd_plan* p) {
     });
     std::vector<int32_t> out(M);
     for (int64_t i = 0; i < M; ++i) out[i] = key[i].at;
-    CU(dalloc(p->allocs, p->device_bytes, &p->ck_perm, M));
-    CU(upload(p->ck_perm, out));
+    p->ck_order = std::move(out);
+    return PD_OK;
+}
+// One array of visibilities out of or into a checkpoint, piece by piece through the state's staging.
+template <typename R>
+static cudaError_t copy_vis(const pd_state* st, void* dev, unsigned char* host, bool save, cudaStream_t s) {
+    const pd_plan* p = st->plan;
+    using C = cplx_t<R>;
+    cudaError_t e;
+    for (int64_t i = 0; i < p->M; i += st->ck_cap) {
+        const int64_t n = std::min(st->ck_cap, p->M - i);
+        if ((e = cudaMemcpyAsync(st->ck_idx, p->ck_order.data() + i, n * sizeof(int32_t), cudaMemcpyHostToDevice, s)))
+            return e;
+        if (save) {
+            if ((e = gather_by<R>(n, st->ck_idx, (const C*)dev, (C*)st->ck_vis, s)) ||
+                (e = cudaMemcpyAsync(host + i * sizeof(C), st->ck_vis, n * sizeof(C), cudaMemcpyDeviceToHost, s)))
+                return e;
+        } else {
+            if ((e = cudaMemcpyAsync(st->ck_vis, host + i * sizeof(C), n * sizeof(C), cudaMemcpyHostToDevice, s)) ||
+                (e = scatter_by<R>(n, st->ck_idx, (const C*)st->ck_vis, (C*)dev, s)))
+                return e;
+        }
+    }
+    return cudaSuccess;
+}
+static pd_status copy_state(pd_state* st, unsigned char* c, bool save, cudaStream_t s) {
+    const pd_plan* p = st->plan;
+    pd_status e = ensure_ck(st->plan);
+    if (e != PD_OK) return e;
+    std::lock_guard<std::mutex> lock(st->ck_mu);
+    for (const Part& q : state_parts(p, st)) {
+        if (q.vis) {
+            if (p->prec == PD_F64) CU(copy_vis<double>(st, q.dev, c, save, s));
+            else CU(copy_vis<float>(st, q.dev, c, save, s));
+        } else {
+            CU(save ? cudaMemcpyAsync(c, q.dev, q.bytes, cudaMemcpyDeviceToHost, s)
+                    : cudaMemcpyAsync(q.dev, c, q.bytes, cudaMemcpyHostToDevice, s));
+        }
+        c += q.bytes;
+    }
+    CU(cudaStreamSynchronize(s));
     return PD_OK;
 }
 extern "C" size_t pd_state_bytes(const pd_plan* p) {
@@ -1344,37 +1388,19 @@ extern "C" size_t pd_state_bytes(const pd_plan* p) {
 }
 extern "C" pd_status pd_state_save(const pd_plan* p, const pd_state* st, void* buf, void* stream) {
     if (!p || !st || !buf || st->plan != p) return fail(PD_EINVAL, "pd_state_save: bad argument");
-    pd_status e = ensure_ck(st->plan);
-    if (e != PD_OK) return e;
-    cudaStream_t s = (cudaStream_t)stream;
-    unsigned char* c = (unsigned char*)buf;
-    for (const Part& q : state_parts(p, st)) {
-        if (q.vis) {      // through the plan's residual scratch
-            if (p->prec == PD_F64) CU(gather_by<double>(p, p->ck_perm, (const double2*)q.dev, (double2*)p->rbuf, s));
-            else CU(gather_by<float>(p, p->ck_perm, (const float2*)q.dev, (float2*)p->rbuf, s));
-        }
-        CU(cudaMemcpyAsync(c, q.vis ? p->rbuf : q.dev, q.bytes, cudaMemcpyDeviceToHost, s));
-        c += q.bytes;
+    try {
+        return copy_state(const_cast<pd_state*>(st), (unsigned char*)buf, true, (cudaStream_t)stream);
+    } catch (const std::bad_alloc&) {
+        return fail(PD_ENOMEM, "pd_state_save: no host memory to order the visibilities");
     }
-    CU(cudaStreamSynchronize(s));
-    return PD_OK;
 }
 extern "C" pd_status pd_state_load(const pd_plan* p, pd_state* st, const void* buf, void* stream) {
     if (!p || !st || !buf || st->plan != p) return fail(PD_EINVAL, "pd_state_load: bad argument");
-    pd_status e = ensure_ck(st->plan);
-    if (e != PD_OK) return e;
-    cudaStream_t s = (cudaStream_t)stream;
-    const unsigned char* c = (const unsigned char*)buf;
-    for (const Part& q : state_parts(p, st)) {
-        CU(cudaMemcpyAsync(q.vis ? p->rbuf : q.dev, c, q.bytes, cudaMemcpyHostToDevice, s));
-        if (q.vis) {
-            if (p->prec == PD_F64) CU(scatter_by<double>(p, p->ck_perm, (const double2*)p->rbuf, (double2*)q.dev, s));
-            else CU(scatter_by<float>(p, p->ck_perm, (const float2*)p->rbuf, (float2*)q.dev, s));
-        }
-        c += q.bytes;
+    try {
+        return copy_state(st, (unsigned char*)const_cast<void*>(buf), false, (cudaStream_t)stream);
+    } catch (const std::bad_alloc&) {
+        return fail(PD_ENOMEM, "pd_state_load: no host memory to order the visibilities");
     }
-    CU(cudaStreamSynchronize(s));
-    return PD_OK;
 }
 
 extern "C" pd_status pd_plan_autotune(const pd_plan_desc* desc, const int32_t* candidates, int32_t ncand,

@@ -241,24 +241,24 @@ __global__ void k_scatter(const C* __restrict__ internal, C* __restrict__ user, 
         user[vis_index(perm[i])] = vis_conj(perm[i], internal[i]);
 }
 template <typename R>
-cudaError_t gather_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
-    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
-    k_gather<<<ctas, 256, 0, s>>>(src, dst, perm, p->M);
+cudaError_t gather_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
+    const int ctas = (int)std::min<int64_t>(4096, (m + 255) / 256);
+    k_gather<<<ctas, 256, 0, s>>>(src, dst, perm, m);
     return cudaGetLastError();
 }
 template <typename R>
-cudaError_t scatter_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
-    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
-    k_scatter<<<ctas, 256, 0, s>>>(src, dst, perm, p->M);
+cudaError_t scatter_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s) {
+    const int ctas = (int)std::min<int64_t>(4096, (m + 255) / 256);
+    k_scatter<<<ctas, 256, 0, s>>>(src, dst, perm, m);
     return cudaGetLastError();
 }
 template <typename R>
 cudaError_t gather_internal(const pd_plan* p, const cplx_t<R>* user, cplx_t<R>* internal, cudaStream_t s) {
-    return gather_by<R>(p, p->perm, user, internal, s);
+    return gather_by<R>(p->M, p->perm, user, internal, s);
 }
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s) {
-    return scatter_by<R>(p, p->perm, internal, user, s);
+    return scatter_by<R>(p->M, p->perm, internal, user, s);
 }
 
 // ||y_i|| per block (= ||Phi_i x^(0) - y_i|| for x^(0) = 0): partial sums of every slot, one
@@ -354,10 +354,10 @@ template cudaError_t norm2<float>(const pd_plan*, const float*, int64_t, double*
 template cudaError_t norm2<double>(const pd_plan*, const double*, int64_t, double*, cudaStream_t);
 template cudaError_t scale_copy<float>(const float*, float*, int64_t, double, cudaStream_t);
 template cudaError_t scale_copy<double>(const double*, double*, int64_t, double, cudaStream_t);
-template cudaError_t gather_by<float>(const pd_plan*, const int32_t*, const float2*, float2*, cudaStream_t);
-template cudaError_t gather_by<double>(const pd_plan*, const int32_t*, const double2*, double2*, cudaStream_t);
-template cudaError_t scatter_by<float>(const pd_plan*, const int32_t*, const float2*, float2*, cudaStream_t);
-template cudaError_t scatter_by<double>(const pd_plan*, const int32_t*, const double2*, double2*, cudaStream_t);
+template cudaError_t gather_by<float>(int64_t, const int32_t*, const float2*, float2*, cudaStream_t);
+template cudaError_t gather_by<double>(int64_t, const int32_t*, const double2*, double2*, cudaStream_t);
+template cudaError_t scatter_by<float>(int64_t, const int32_t*, const float2*, float2*, cudaStream_t);
+template cudaError_t scatter_by<double>(int64_t, const int32_t*, const double2*, double2*, cudaStream_t);
 template cudaError_t gather_internal<float>(const pd_plan*, const float2*, float2*, cudaStream_t);
 template cudaError_t gather_internal<double>(const pd_plan*, const double2*, double2*, cudaStream_t);
 template cudaError_t scatter_user<float>(const pd_plan*, const float2*, float2*, cudaStream_t);

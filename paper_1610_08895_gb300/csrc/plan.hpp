@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -101,11 +102,12 @@ struct pd_plan {
     std::vector<int32_t> h_tile_seg_start, h_seg_block;
 
     // checkpoints keep the visibilities in the order of their own tiles and base cells, whatever
-    // the plan's internal order is: device list of the internal index of each (sign bit: held
-    // as a conjugate), made by the first save or load
+    // the plan's internal order is: host list of the internal index of each (sign bit: held
+    // as a conjugate), made by the first save or load under the lock and only read after that
     std::vector<int32_t> h_base;   // base cell (by << 16 | bx) of each point, user order
     int ck_tile = 0;
-    int32_t* ck_perm = nullptr;
+    std::mutex ck_mu;
+    std::vector<int32_t> ck_order;
 
     // device: visibilities in internal (tile, block, row, column) order
     int32_t* cell = nullptr;       // (by << 16) | bx of the footprint's first cell, mod K
@@ -209,6 +211,13 @@ struct pd_state {
     int64_t* t = nullptr;              // iteration counter (device)
     double* diag = nullptr;            // [2]: ||dx||^2, ||x||^2
     double* prim_part = nullptr;       // [2 * ny / rows-per-CTA]
+    // staging of a checkpoint's visibilities (the state's own: other states of the plan may be
+    // iterating on other streams meanwhile): ck_cap of them and their internal indices, one save
+    // or load at a time
+    std::mutex ck_mu;
+    int64_t ck_cap = 0;
+    void* ck_vis = nullptr;
+    int32_t* ck_idx = nullptr;
     int32_t* status = nullptr;         // device status word
     std::vector<void*> allocs;
     size_t device_bytes = 0;
@@ -348,11 +357,11 @@ template <typename R>
 cudaError_t scale_copy(const R* x, R* y, int64_t n, double scale, cudaStream_t s);
 template <typename R>
 cudaError_t gather_internal(const pd_plan* p, const cplx_t<R>* user, cplx_t<R>* internal, cudaStream_t s);
-// the same through another list of places (checkpoints)
+// the same through another list of m places (checkpoints)
 template <typename R>
-cudaError_t gather_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
+cudaError_t gather_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
 template <typename R>
-cudaError_t scatter_by(const pd_plan* p, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
+cudaError_t scatter_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s);
 // pend[t] = parts of the tiles that hold a point of an active block (all of them: active null), else 0;
