@@ -550,6 +550,16 @@ extern "C" pd_status pd_plan_info(const pd_plan* p, int32_t* ky, int32_t* kx, do
     return PD_OK;
 }
 
+// Tests only, not in pd.h: sets the work counters of the plan's launches to `value`, as launches that
+// did not end or overlapped would leave them.
+extern "C" pd_status pd_test_work_counters(pd_plan* p, int32_t value) {
+    if (!p) return fail(PD_EINVAL, "pd_test_work_counters: null plan");
+    const std::vector<int32_t> c(10, value);
+    CU(cudaDeviceSynchronize());
+    CU(cudaMemcpy(p->sched, c.data(), c.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    return PD_OK;
+}
+
 // ------------------------------------------------------------------ operators
 // Scratch of a batch of operator applications (one launch per pass for the whole batch):
 // the plan's own buffers for one image, otherwise buffers kept by the plan and grown to

@@ -255,12 +255,14 @@ __global__ void __launch_bounds__(PassShape<R, N>::NT_ROWS, PassShape<R, N>::MIN
 template <typename R, int N>
 __global__ void __launch_bounds__(PassShape<R, N>::NT_COLS, PassShape<R, N>::MIN_CTAS_COLS) k_fwd_cols(
     const cplx_t<R>* __restrict__ t1, cplx_t<R>* __restrict__ gb, const cplx_t<R>* __restrict__ twy,
-    int64_t t1_stride, int64_t gb_stride) {
+    int64_t t1_stride, int64_t gb_stride, int* __restrict__ sched) {
     using C2 = cplx_t<R>;
     using S = Shape<R, N>;
     using P = PassShape<R, N>;
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* s = reinterpret_cast<C2*>(smraw);
+    // the degridding that reads this grid starts from its first item, whatever an earlier launch left
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) sched[threadIdx.x] = 0;
     t1 += (int64_t)blockIdx.y * t1_stride;
     gb += (int64_t)blockIdx.y * gb_stride;
     constexpr int NT = P::NT_COLS, CQ = P::CQ, Ky = 2 * N, PER = 4 / CQ;
@@ -452,7 +454,7 @@ static cudaError_t launch_fwd_cols(const pd_plan* p, const cplx_t<R>* t1, cplx_t
     cudaError_t e;
     if ((e = ensure_smem(k_fwd_cols<R, N>, P::SMEM_COLS))) return e;
     k_fwd_cols<R, N><<<dim3((p->g.nx / 4 + 1) * (4 / P::CQ), batch), P::NT_COLS, P::SMEM_COLS, s>>>(
-        t1, gb, (const cplx_t<R>*)p->twy, t1_elems(p), gb_elems(p));
+        t1, gb, (const cplx_t<R>*)p->twy, t1_elems(p), gb_elems(p), p->sched + 4);
     return cudaGetLastError();
 }
 template <typename R, int N>

@@ -1005,11 +1005,6 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
             if (lane == 0) atomicSub(pd + im.tile, 1);
             have = next;
         }
-        // the last CTA to leave sets the counters back for the next launch
-        if (lane == 0 && atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
-            sched[0] = 0;
-            sched[1] = 0;
-        }
         return;
     }
     // -------------------------------------------------------------------- the working warps

@@ -172,7 +172,8 @@ __device__ __forceinline__ int claim_tile(int* next, const int32_t* __restrict__
         if (w >= n * batch || !tile_on || tile_on[list[w % n]]) return w;
     }
 }
-// Thread 0 of each CTA at the end: the last one sets the counters back for the next launch.
+// Thread 0 of each CTA at the end: the last one sets the counters back for the next launch on the
+// same grid (the forward FFT sets them too).
 __device__ __forceinline__ void leave_items(int* sched) {
     if (atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
         sched[0] = 0;

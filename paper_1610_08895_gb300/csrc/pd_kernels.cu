@@ -26,6 +26,7 @@ __device__ __forceinline__ void flag_tile(int t, const int4* __restrict__ tile_i
     tiles += n > 0;
 }
 
+// next_item: the gridding's work counter, set to the first item here.
 // Step 3: Philox draws u(seed, t, stream, index) < p for blocks (stream 0) and
 // bases (stream 1); with adaptive = 1 the block probabilities are first set by
 // eq. (prob-choice) from the current residual norms. Then the tiles holding a
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(SEL_NT) k_select(
     const double* __restrict__ eps, int d, int b, int32_t* __restrict__ block_active,
     int32_t* __restrict__ basis_active, const int32_t* __restrict__ tile_order, const int4* __restrict__ tile_info,
     const int32_t* __restrict__ seg_block, int ntiles, int32_t* __restrict__ tile_on, int32_t* __restrict__ pend,
-    int32_t* __restrict__ counts) {
+    int32_t* __restrict__ next_item, int32_t* __restrict__ counts) {
     __shared__ double shd[32];
     __shared__ int64_t t_sh;
     __shared__ int cnt_sh[2];
@@ -49,6 +50,7 @@ __global__ void __launch_bounds__(SEL_NT) k_select(
         *tptr = t;
         t_sh = t;
         cnt_sh[0] = cnt_sh[1] = 0;
+        *next_item = 0;
     }
     __syncthreads();
     if (adaptive) {
@@ -143,7 +145,8 @@ cudaError_t select_active(const pd_plan* p, pd_state* st, const SelectArgs& a, c
     const int nt = p->ntiles_nonempty;
     k_select<<<1, SEL_NT, 0, s>>>(a.seed, a.adaptive, a.n, a.p_min, a.p_max, st->t, st->p_block, st->p_basis,
                                  st->res_norm, st->eps, p->d, p->b, st->block_active, st->basis_active,
-                                 p->tile_order, p->tile_info, p->seg_block, nt, st->tile_active, p->pend, st->counts);
+                                 p->tile_order, p->tile_info, p->seg_block, nt, st->tile_active, p->pend, p->sched + 8,
+                                 st->counts);
     if (nt > SEL_TILES)
         k_flag_tiles<<<(nt + 255) / 256, 256, 0, s>>>(p->tile_order, p->tile_info, p->seg_block, st->block_active, nt,
                                                       st->tile_active, p->pend, st->counts);
@@ -153,8 +156,9 @@ cudaError_t select_active(const pd_plan* p, pd_state* st, const SelectArgs& a, c
 
 __global__ void __launch_bounds__(256) k_grid_begin(const int4* __restrict__ tile_info, const int32_t* __restrict__ seg_block,
                                                     const int32_t* __restrict__ active, int ntiles,
-                                                    int32_t* __restrict__ pend, float4* __restrict__ U, int64_t n4,
-                                                    int batch) {
+                                                    int32_t* __restrict__ pend, int32_t* __restrict__ next_item,
+                                                    float4* __restrict__ U, int64_t n4, int batch) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *next_item = 0;
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = i0; i < (int64_t)ntiles * batch; i += step) {
         const int4 ti = tile_info[i % ntiles];
@@ -169,7 +173,8 @@ cudaError_t grid_begin(const pd_plan* p, const int32_t* active, int32_t* pend, f
                        cudaStream_t s) {
     const int64_t n = std::max<int64_t>((int64_t)p->g.ntiles * batch, U ? n4 / 4 : 0);
     const int ctas = (int)std::min<int64_t>((n + 255) / 256, (int64_t)p->num_sms * 8);
-    k_grid_begin<<<ctas, 256, 0, s>>>(p->tile_info, p->seg_block, active, p->g.ntiles, pend, U, U ? n4 : 0, batch);
+    k_grid_begin<<<ctas, 256, 0, s>>>(p->tile_info, p->seg_block, active, p->g.ntiles, pend, p->sched + 8, U,
+                                       U ? n4 : 0, batch);
     return cudaGetLastError();
 }
 

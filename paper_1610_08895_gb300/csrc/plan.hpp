@@ -182,8 +182,9 @@ struct pd_plan {
     void* synpart = nullptr;       // real [b][ny][nx] level-0 synthesis of each basis
     double* red = nullptr;         // reduction scratch
     int32_t* sched = nullptr;      // [16] work counters of the dynamically scheduled launches: 0-3 gridding
-                                   // colours (zeroed before each launch); 4-5 degridding, 8-9 k_grid_mma (next
-                                   // item, CTAs done: left at zero by every launch); 10: a wait gave up
+                                   // colours (zeroed before each launch); 4-5 degridding (next item, CTAs done:
+                                   // zeroed by the forward FFT and by every launch); 8 k_grid_mma (next item:
+                                   // zeroed with pend); 10: a wait gave up
     int red_len = 0;
     size_t device_bytes = 0;
     std::vector<void*> allocs;     // every device allocation of the plan
@@ -364,8 +365,8 @@ template <typename R>
 cudaError_t scatter_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s);
-// pend[t] = parts of the tiles that hold a point of an active block (all of them: active null), else 0;
-// and U = 0 where given (n4 float4 elements), for `batch` images
+// pend[t] = parts of the tiles that hold a point of an active block (all of them: active null), else 0,
+// the gridding's work counter = 0, and U = 0 where given (n4 float4 elements), for `batch` images
 cudaError_t grid_begin(const pd_plan* p, const int32_t* active, int32_t* pend, float4* U, int64_t n4, int batch, cudaStream_t s);
 cudaError_t init_res_norm(const pd_plan* p, pd_state* st, cudaStream_t s);
 

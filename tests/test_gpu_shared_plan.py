@@ -1,5 +1,6 @@
 """Several states of one plan: what may run side by side on different streams and threads, and
 what each call leaves of the plan's shared scratch to the others."""
+import ctypes
 import threading
 
 import numpy as np
@@ -7,7 +8,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from gpu_util import make_problem  # noqa: E402
+from gpu_util import make_problem, rel  # noqa: E402
 from paper_1610_08895_gb300 import synth  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -78,3 +79,39 @@ def test_first_checkpoints_from_several_threads():
         assert np.array_equal(bufs[k], states[k].save())
         states[k].load(bufs[k])
         assert np.array_equal(bufs[k], states[k].save())
+
+
+@pytest.mark.parametrize("kw", [dict(precision="f32"), dict(precision="f64"), dict(precision="f32", g_mode="csr")])
+def test_launches_start_from_their_first_item_whatever_an_earlier_one_left(kw):
+    """Counters that an earlier launch left anywhere (it overlapped another one, say) do not reach the
+    next call: Phi, Phi^H, an iteration and a batch are what they are on untouched counters."""
+    from paper_1610_08895_gb300 import _binding as B
+    from paper_1610_08895_gb300.api import Plan, State
+    n, m = 64, 5000
+    uv = synth.uv_gaussian(m, seed=1)
+    plan = Plan(n, n, uv, (np.arange(m) % 4).astype(np.int32), 4, basis_ids=(0, 1), levels=2, **kw)
+    st = State(plan)
+    x = torch.tensor(synth.random_images(2, n, n, seed=3), dtype=plan.real_dtype, device="cuda")
+    y = torch.tensor(np.stack([synth.uniform_vis(m, seed=k) for k in (4, 5)]), dtype=plan.cplx_dtype, device="cuda")
+
+    def everything():
+        yield plan.pd_apply_phi(x[0])
+        yield plan.pd_apply_phi(x)
+        yield plan.pd_apply_phi_adj(y[0])
+        yield plan.pd_apply_phi_adj(y)
+        for form in (dict(), dict(use_graph=True), dict(per_block=True)):
+            st.pd_state_set_data(y[0], np.ones(4))
+            spoil()
+            st.pd_iterate(2, 0.49, 1.0, 1e-4, 1e-3, seed=1, p_block=[0.9] * 4, p_basis=[0.9] * 2, **form)
+            yield st.x()
+            yield st.v()
+
+    spoil = lambda: None  # noqa: E731
+    want = [t.clone() for t in everything()]
+    hook = B.load().pd_test_work_counters
+    hook.argtypes = [ctypes.c_void_p, ctypes.c_int32]
+    spoil = lambda: B.check(hook(plan.handle, 12345))  # noqa: E731
+    spoil()
+    for got, ref in zip(everything(), want):
+        assert rel(got.cpu().numpy(), ref.cpu().numpy()) < 1e-6 and torch.isfinite(torch.view_as_real(got) if got.is_complex() else got).all()
+        spoil()
