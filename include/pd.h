@@ -44,7 +44,7 @@ typedef enum {
     PD_EINVAL = 1,      /* invalid argument (sizes, ranges, null pointers) */
     PD_ENOMEM = 2,      /* device or host allocation failed */
     PD_ECUDA = 3,       /* a CUDA runtime call or kernel launch failed */
-    PD_ETIMEOUT = 4,    /* a bounded device wait gave up (pd_state_report) */
+    PD_ETIMEOUT = 4,    /* a bounded device wait gave up: results complete, see pd_plan_status */
     PD_ENOTCONV = 5,    /* power iteration did not reach its tolerance */
     PD_ENOTSUP = 6      /* valid but unsupported configuration */
 } pd_status;
@@ -152,6 +152,18 @@ const char* pd_last_error(void);
 pd_status pd_plan_info(const pd_plan* plan, int32_t* ky, int32_t* kx, double* beta,
                        int32_t* tile, int64_t* nsegments, int64_t* ntiles_nonempty,
                        int64_t* device_bytes);
+
+/*
+ * PD_ETIMEOUT if a wait of a plain application on this plan (pd_apply_phi_adj) ever gave up,
+ * PD_OK otherwise; synchronises `stream`. The FP32 gridding adds overlapping tiles in a fixed
+ * order, for which a thread block waits for another one of the launch; the wait is bounded
+ * (some seconds), and a launch in which it runs out goes on: its sums are complete, but their
+ * order, and so their rounding, depended on timing. Calls that return host results say so
+ * themselves, with every output written: pd_operator_norms and pd_state_set_start for their own
+ * applications, pd_state_report for everything gridded into that state's U since its last
+ * pd_state_set_data, pd_state_set_start or pd_state_load.
+ */
+pd_status pd_plan_status(const pd_plan* plan, void* stream);
 
 /* Daubechies low-pass filter of basis id k (1..8) as derived by the plan,
  * written to host h[2k] (largest tap first, sum sqrt(2)). */
@@ -378,7 +390,8 @@ pd_status pd_state_get_v(const pd_plan* plan, const pd_state* st, void* v, void*
  * NULL) and the activity of the last draw (host int32 [nblocks] and
  * [nbases], may be NULL), and the size of the last iteration's work lists (host
  * int32 [2]: (tile, block) segments of active blocks, tiles holding an active
- * block; may be NULL).
+ * block; may be NULL). Errors: PD_EINVAL, PD_ECUDA, PD_ETIMEOUT (see pd_plan_status; the
+ * outputs are written all the same, and every report of the state returns it).
  */
 pd_status pd_state_report(const pd_plan* plan, const pd_state* st, int64_t* t, double* dx2,
                           double* x2, double* res_norm, double* p_block, int32_t* block_active,

@@ -55,6 +55,7 @@ _SIGS = {
                          ctypes.c_int),
     "pd_last_error": ([], ctypes.c_char_p),
     "pd_plan_info": ([_VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP], ctypes.c_int),
+    "pd_plan_status": ([_VP, _VP], ctypes.c_int),
     "pd_daubechies_filter": ([ctypes.c_int32, _VP], ctypes.c_int),
     "pd_apply_phi": ([_VP, _VP, _VP, ctypes.c_int32, _VP], ctypes.c_int),
     "pd_apply_phi_adj": ([_VP, _VP, _VP, ctypes.c_int32, _VP], ctypes.c_int),

@@ -94,6 +94,10 @@ class Plan:
         return {"ky": ky.value, "kx": kx.value, "beta": beta.value, "tile": tile.value,
                 "nsegments": ns.value, "ntiles_nonempty": nc.value, "device_bytes": nb.value}
 
+    def pd_plan_status(self):
+        """Raises PDError (PD_ETIMEOUT) if a wait of a plain application on this plan ever gave up."""
+        B.call("pd_plan_status", self._h, _stream())
+
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
             B.load().pd_plan_destroy(self._h)

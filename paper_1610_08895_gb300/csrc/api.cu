@@ -560,6 +560,28 @@ extern "C" pd_status pd_test_work_counters(pd_plan* p, int32_t value) {
     return PD_OK;
 }
 
+// A wait of the ordered adds that gave up leaves U complete, its sums in an order of their own.
+static const char* k_gave_up = "a wait of the gridding's ordered adds gave up: its sums are complete, "
+                               "but their order, and so their rounding, depended on timing";
+
+extern "C" pd_status pd_plan_status(const pd_plan* p, void* stream) {
+    if (!p) return fail(PD_EINVAL, "pd_plan_status: null plan");
+    cudaStream_t s = (cudaStream_t)stream;
+    int32_t gave_up = 0;
+    CU(cudaMemcpyAsync(&gave_up, p->sched + 10, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+    return gave_up ? fail(PD_ETIMEOUT, k_gave_up) : PD_OK;
+}
+
+// Tests only, not in pd.h: the poll limit of the ordered adds' waits, and whether launches start
+// with one part too many pending, so that waits run out.
+extern "C" pd_status pd_test_ordered_adds(pd_plan* p, int32_t polls, int32_t hold) {
+    if (!p || polls < 1) return fail(PD_EINVAL, "pd_test_ordered_adds: bad argument");
+    p->wait_polls = polls;
+    p->test_hold = hold;
+    return PD_OK;
+}
+
 // ------------------------------------------------------------------ operators
 // Scratch of a batch of operator applications (one launch per pass for the whole batch):
 // the plan's own buffers for one image, otherwise buffers kept by the plan and grown to
@@ -606,12 +628,13 @@ static pd_status apply_phi_t(pd_plan* p, const void* x, void* y, int batch, cuda
     return PD_OK;
 }
 template <typename R>
-static pd_status apply_phi_adj_t(pd_plan* p, const void* y, void* x, int batch, cudaStream_t s) {
+static pd_status apply_phi_adj_t(pd_plan* p, const void* y, void* x, int batch, cudaStream_t s,
+                                 int32_t* gave_up = nullptr) {
     void *t1, *gb, *gu;
     int32_t* pend;
     pd_status st = ensure_batch(p, batch, &t1, &gb, &gu, &pend);
     if (st != PD_OK) return st;
-    CU(grid_plain<R>(p, (const cplx_t<R>*)y, (cplx_t<R>*)gu, s, batch, pend));
+    CU(grid_plain<R>(p, (const cplx_t<R>*)y, (cplx_t<R>*)gu, s, batch, pend, gave_up));
     CU(inv_fft<R>(p, (const cplx_t<R>*)gu, (R*)x, nullptr, s, batch, (cplx_t<R>*)t1));
     return PD_OK;
 }
@@ -685,18 +708,21 @@ static pd_status norms_t(pd_plan* p, const void* x0, int max_iter, double tol, d
     R *xa, *xb, *coef;
     cplx_t<R>* vis;
     double* dn;
+    int32_t* flag;
     auto cleanup = [&]() { free_all(tmp); };
     if (dalloc(tmp, bytes, &xa, N) || dalloc(tmp, bytes, &xb, N) || dalloc(tmp, bytes, &coef, N * p->b) ||
-        dalloc(tmp, bytes, &vis, p->M) || dalloc(tmp, bytes, &dn, 1)) {
+        dalloc(tmp, bytes, &vis, p->M) || dalloc(tmp, bytes, &dn, 1) || dalloc(tmp, bytes, &flag, 1) ||
+        cudaMemsetAsync(flag, 0, sizeof(int32_t), s)) {
         cleanup();
         return fail(PD_ENOMEM, "pd_operator_norms: temporary allocation failed");
     }
     int it1 = 0, it2 = 0;
     double l1 = 0, l2 = 0;
+    int32_t gave_up = 0;
     pd_status st1 = power_t<R>(p, (const R*)x0, max_iter, tol, xa, xb, dn,
                                [&](R* a, R* b) {
                                    pd_status q = apply_phi_t<R>(p, a, vis, 1, s);
-                                   return q != PD_OK ? q : apply_phi_adj_t<R>(p, vis, b, 1, s);
+                                   return q != PD_OK ? q : apply_phi_adj_t<R>(p, vis, b, 1, s, flag);
                                },
                                &l1, &it1, s);
     if (st1 != PD_OK && st1 != PD_ENOTCONV) { cleanup(); return st1; }
@@ -707,11 +733,15 @@ static pd_status norms_t(pd_plan* p, const void* x0, int max_iter, double tol, d
                                    return e ? fail(PD_ECUDA, cudaGetErrorString(e)) : PD_OK;
                                },
                                &l2, &it2, s);
+    cudaError_t ef = cudaMemcpyAsync(&gave_up, flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    if (!ef) ef = cudaStreamSynchronize(s);
     cleanup();
+    CU(ef);
     if (st2 != PD_OK && st2 != PD_ENOTCONV) return st2;
     if (phi2) *phi2 = l1;
     if (psi2) *psi2 = l2;
     if (iters) *iters = std::max(it1, it2);
+    if (gave_up) return fail(PD_ETIMEOUT, k_gave_up);
     if (st1 == PD_ENOTCONV || st2 == PD_ENOTCONV) return fail(PD_ENOTCONV, "power method: max_iter reached");
     return PD_OK;
 }
@@ -758,8 +788,12 @@ extern "C" pd_status pd_state_create(pd_plan* p, pd_state** out) {
               !dalloc(A, B, &st->res_norm, p->d) && !dalloc(A, B, &st->p_block, p->d) &&
               !dalloc(A, B, &st->p_basis, p->b) && !dalloc(A, B, &st->block_active, p->d) &&
               !dalloc(A, B, &st->basis_active, p->b) &&
-              !dalloc(A, B, &st->tile_active, p->g.ntiles) && !dalloc(A, B, &st->counts, 2) && !dalloc(A, B, &st->t, 1) && !dalloc(A, B, &st->diag, 2) &&
-              !dalloc(A, B, &st->prim_part, 2 * (size_t)inv_rows_ctas(p)) && !dalloc(A, B, &st->status, 1);
+              !dalloc(A, B, &st->tile_active, p->g.ntiles) && !dalloc(A, B, &st->counts, 2) && !dalloc(A, B, &st->t, 4) &&
+              !dalloc(A, B, &st->prim_part, 2 * (size_t)inv_rows_ctas(p));
+    if (ok) {          // t, diag and status side by side: a report reads them in one copy
+        st->diag = (double*)(st->t + 1);
+        st->status = (int32_t*)(st->t + 3);
+    }
     st->ck_cap = std::min<int64_t>(p->M, 1 << 20);
     ok = ok && !dalloc_bytes(A, B, &st->ck_vis, st->ck_cap * p->csz) && !dalloc(A, B, &st->ck_idx, st->ck_cap);
     if (!ok) {
@@ -767,6 +801,7 @@ extern "C" pd_status pd_state_create(pd_plan* p, pd_state** out) {
         return fail(PD_ENOMEM, "pd_state_create: device allocation failed");
     }
     for (void* q : A) cudaMemset(q, 0, 16);
+    CU(cudaMemset(st->t, 0, 4 * sizeof(int64_t)));
     CU(cudaMemset(st->x, 0, N * p->rsz));
     CU(cudaMemset(st->xt, 0, N * p->rsz));
     CU(cudaMemset(st->s, 0, N * p->b * p->rsz));
@@ -794,8 +829,7 @@ extern "C" pd_status pd_state_set_data(pd_plan* p, pd_state* st, const void* y, 
     CU(cudaMemsetAsync(st->st, 0, N * p->rsz, s));
     CU(cudaMemsetAsync(st->v, 0, p->M * p->csz, s));
     CU(cudaMemsetAsync(st->u, 0, K * p->csz, s));
-    CU(cudaMemsetAsync(st->t, 0, sizeof(int64_t), s));
-    CU(cudaMemsetAsync(st->diag, 0, 2 * sizeof(double), s));
+    CU(cudaMemsetAsync(st->t, 0, 4 * sizeof(int64_t), s));      // t, diag, status
     if (st->syn_at) CU(cudaMemsetAsync(st->syn_at, 0, N * p->b * p->rsz, s));
     if (st->syn_u) CU(cudaMemsetAsync(st->syn_u, 0, N * p->rsz, s));
     std::vector<double> ones_d(p->d, 1.0), ones_b(p->b, 1.0);
@@ -810,6 +844,7 @@ template <typename R>
 static pd_status set_start_t(pd_plan* p, pd_state* st, const void* x0, const void* xt0, const void* s0,
                              const void* v0, cudaStream_t s) {
     const size_t N = (size_t)p->g.nx * p->g.ny, K = (size_t)p->g.Kx * p->g.Ky;
+    CU(cudaMemsetAsync(st->t, 0, 4 * sizeof(int64_t), s));      // t, diag, status
     if (x0) CU(cudaMemcpyAsync(st->x, x0, N * p->rsz, cudaMemcpyDeviceToDevice, s));
     else CU(cudaMemsetAsync(st->x, 0, N * p->rsz, s));
     if (xt0) CU(cudaMemcpyAsync(st->xt, xt0, N * p->rsz, cudaMemcpyDeviceToDevice, s));
@@ -823,13 +858,11 @@ static pd_status set_start_t(pd_plan* p, pd_state* st, const void* x0, const voi
     }
     if (v0) {
         CU(gather_internal<R>(p, (const cplx_t<R>*)v0, (cplx_t<R>*)st->v, s));
-        CU(grid_plain<R>(p, (const cplx_t<R>*)v0, (cplx_t<R>*)st->u, s));   // U = G^T v
+        CU(grid_plain<R>(p, (const cplx_t<R>*)v0, (cplx_t<R>*)st->u, s, 1, nullptr, st->status));   // U = G^T v
     } else {
         CU(cudaMemsetAsync(st->v, 0, p->M * p->csz, s));
         CU(cudaMemsetAsync(st->u, 0, K * p->csz, s));
-        }
-    CU(cudaMemsetAsync(st->t, 0, sizeof(int64_t), s));
-    CU(cudaMemsetAsync(st->diag, 0, 2 * sizeof(double), s));
+    }
     // residual norms of the adaptive probabilities: ||Phi_i x^(0) - y_i||
     if (x0) {
         CU(fwd_fft<R>(p, (const R*)st->x, (cplx_t<R>*)p->gridb, s));
@@ -837,8 +870,10 @@ static pd_status set_start_t(pd_plan* p, pd_state* st, const void* x0, const voi
     } else {
         CU(init_res_norm(p, st, s));
     }
+    int32_t gave_up = 0;
+    CU(cudaMemcpyAsync(&gave_up, st->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    return PD_OK;
+    return gave_up ? fail(PD_ETIMEOUT, k_gave_up) : PD_OK;
 }
 
 extern "C" pd_status pd_state_set_start(pd_plan* p, pd_state* st, const void* x0, const void* x_tilde0,
@@ -884,7 +919,7 @@ static cudaError_t enqueue_dual(pd_plan* p, pd_state* st, const pd_params* prm, 
     if (concurrent && (e = cudaEventRecord(st->ev_join, ps))) return e;
     if ((e = fwd_fft<R>(p, (const R*)st->xt, (cplx_t<R>*)p->gridb, s))) return e;
     DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm, st->tile_active,
-                p->ditems, p->counts_all + 2, p->items, p->nitems};
+                p->ditems, p->counts_all + 2, p->items, p->nitems, st->status};
     if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, s))) return e;
     {
         const int q = p->g.ntiles / 4;
@@ -1019,6 +1054,7 @@ static cudaError_t enqueue_iteration_per_block(pd_plan* p, pd_state* st, const p
         for (int c = 0; c < 4; ++c) lists[c] = st->pb_col + st->h_pb_off[d + 1 + 4 * i + c];
         if (p->grid_smem) {
             if ((e = grid_begin(p, da.block_active, p->pend, nullptr, 0, 1, s))) return e;
+            da.gave_up = st->status;
             da.items = st->pb_items + st->h_pb_item_off[i];
             da.nitems = st->pb_nitems + i;
         }
@@ -1105,7 +1141,7 @@ static cudaError_t enqueue_synthesis(pd_plan* p, pd_state* st, const pd_params* 
     if ((e = psi_plain<R>(p, (const R*)st->syn_at, (R*)st->xt, s))) return e;            // x~ = Psi alpha~
     if ((e = fwd_fft<R>(p, (const R*)st->xt, (cplx_t<R>*)p->gridb, s))) return e;        // b~ = F Z x~
     DualArgs da{st->y, st->v, st->block_active, st->eps, st->res_norm, st->tile_active,
-                p->ditems, p->counts_all + 2, p->items, p->nitems};
+                p->ditems, p->counts_all + 2, p->items, p->nitems, st->status};
     if ((e = degrid_dual<R>(p, (const cplx_t<R>*)p->gridb, da, s))) return e;
     {
         const int q = p->g.ntiles / 4;
@@ -1283,25 +1319,19 @@ extern "C" pd_status pd_state_report(const pd_plan* p, const pd_state* st, int64
                                      int32_t* work, void* stream) {
     if (!p || !st || st->plan != p) return fail(PD_EINVAL, "pd_state_report: bad argument");
     cudaStream_t s = (cudaStream_t)stream;
-    int64_t th = 0;
-    double dg[2] = {0, 0};
-    CU(cudaMemcpyAsync(&th, st->t, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(dg, st->diag, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    struct { int64_t t; double diag[2]; int32_t gave_up, pad; } h{};
+    static_assert(sizeof(h) == 4 * sizeof(int64_t), "t, diag and status as in pd_state_create");
+    CU(cudaMemcpyAsync(&h, st->t, sizeof(h), cudaMemcpyDeviceToHost, s));
     if (res_norm) CU(cudaMemcpyAsync(res_norm, st->res_norm, p->d * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (p_block) CU(cudaMemcpyAsync(p_block, st->p_block, p->d * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (block_active) CU(cudaMemcpyAsync(block_active, st->block_active, p->d * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (basis_active) CU(cudaMemcpyAsync(basis_active, st->basis_active, p->b * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    int32_t gave_up = 0;
-    CU(cudaMemcpyAsync(&gave_up, p->sched + 10, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (work) CU(cudaMemcpyAsync(work, st->counts, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    if (gave_up) {
-        CU(cudaMemsetAsync(p->sched + 10, 0, sizeof(int32_t), s));
-        return fail(PD_ETIMEOUT, "a wait of the gridding gave up: the state is not valid");
-    }
-    if (t) *t = th;
-    if (dx2) *dx2 = dg[0];
-    if (x2) *x2 = dg[1];
+    if (t) *t = h.t;
+    if (dx2) *dx2 = h.diag[0];
+    if (x2) *x2 = h.diag[1];
+    if (h.gave_up) return fail(PD_ETIMEOUT, k_gave_up);
     return PD_OK;
 }
 
@@ -1386,6 +1416,7 @@ static pd_status copy_state(pd_state* st, unsigned char* c, bool save, cudaStrea
         }
         c += q.bytes;
     }
+    if (!save) CU(cudaMemsetAsync(st->status, 0, sizeof(int32_t), s));
     CU(cudaStreamSynchronize(s));
     return PD_OK;
 }

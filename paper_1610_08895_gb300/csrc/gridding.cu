@@ -658,7 +658,6 @@ constexpr int GM_F = 18;       // floats per staged point: 8 row classes, 8 colu
 constexpr int GM_WP = 18;      // patch pitch (complex)
 constexpr int GM_PS = 16 * GM_WP;   // patch slot (complex)
 constexpr int GM_MAXW = 16;    // warps per CTA, the feeding one included
-constexpr int GM_SPIN = 1 << 22;
 
 __device__ __forceinline__ int ld_acquire(const int32_t* p) {
     int v;
@@ -833,10 +832,9 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
     const float2* __restrict__ src, const float2* __restrict__ rbuf, float2* __restrict__ v,
     const float* __restrict__ scale, const int32_t* __restrict__ active, const int32_t* __restrict__ cell,
     const float* __restrict__ fxs, const float* __restrict__ fys, const int32_t* __restrict__ perm,
-    const int32_t* __restrict__ seg_start, const int32_t* __restrict__ seg_block,
-    const int32_t* __restrict__ sc_start, const int4* __restrict__ tile_info, const int32_t* __restrict__ tile_on,
+    const int32_t* __restrict__ seg_block, const int32_t* __restrict__ sc_start, const int4* __restrict__ tile_info, const int32_t* __restrict__ tile_on,
     const int2* __restrict__ items, const int32_t* __restrict__ nitems, int32_t* pend, float2* U, int max_segs, Geo g,
-    const KbPoly kp, int* sched, int batch, int64_t istride, int64_t ustride) {
+    const KbPoly kp, int* sched, int32_t* gave_up, int polls, int batch, int64_t istride, int64_t ustride) {
     static_assert(J <= 8 && J % 2 == 0, "a super-cell's window is 16 x 16 for J <= 8");
     extern __shared__ __align__(16) unsigned char smraw[];
     const int T = g.tile, nsd = T >> 3, nsc = nsd * nsd, W = T + 8;
@@ -967,7 +965,8 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
             // U in the order of the items, so that the sums do not depend on timing. Earlier items
             // are claimed earlier and a CTA takes its items in order, so the first unfinished one
             // is being worked on and never waits: this wait ends. Its limit is a safeguard (some
-            // seconds), after which the launch goes on and sets its error flag.
+            // seconds), after which the launch sets its flag and goes on: the adds are atomic, so that
+            // U is still complete and only the order of its sums is lost.
             const GridItem& im = item_s[b];
             const int ty = im.tile / g.ntx, tx = im.tile - ty * g.ntx;
             int32_t* pd = pend + (int64_t)im.img * g.ntiles;
@@ -977,7 +976,7 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
                 if (t2 == im.tile || tile_info[t2].w < tile_info[im.tile].w) {
                     int tries = 0;
                     while (ld_acquire(pd + t2) > upto)
-                        if (++tries > GM_SPIN) { atomicExch(sched + 2, 1); break; }
+                        if (++tries > polls) { atomicExch(gave_up, 1); break; }
                 }
             }
             __syncwarp();
@@ -1231,9 +1230,15 @@ void grid_setup(pd_plan* p) {
     p->grid_smem = ok ? smem : 0;
 }
 
+// Tests only (pd_test_ordered_adds): one part too many pending for the first item's tile, so that
+// the waits for it run out.
+__global__ void k_hold(const int2* items, const int32_t* nitems, int32_t* pend) {
+    if (*nitems > 0) pend[items[0].x] += 1;
+}
+
 template <int J, int MODE>
 static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const DualArgs* a, int32_t* pend, float2* U,
-                                   cudaStream_t s, int batch) {
+                                   int32_t* gave_up, cudaStream_t s, int batch) {
     const Geo& g = p->g;
     cudaError_t e;
     if ((e = ensure_smem(k_grid_mma<J, MODE>, p->grid_smem))) return e;
@@ -1242,12 +1247,13 @@ static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const Du
                                                            p->grid_smem)))
         return e;
     const int ctas = (int)std::min<int64_t>((int64_t)p->n_items * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
+    if (p->test_hold) k_hold<<<1, 1, 0, s>>>(a ? a->items : p->items, a ? a->nitems : p->nitems, pend);
     k_grid_mma<J, MODE><<<ctas, p->grid_warps * 32, p->grid_smem, s>>>(
         src, (const float2*)p->rbuf, a ? (float2*)a->v : nullptr, (const float*)p->blk_scale,
-        a ? a->block_active : nullptr, p->cell, (const float*)p->fx, (const float*)p->fy, p->perm, p->seg_start,
+        a ? a->block_active : nullptr, p->cell, (const float*)p->fx, (const float*)p->fy, p->perm,
         p->seg_block, p->seg_sc_start, p->tile_info, a ? a->tile_on : nullptr, a ? a->items : p->items,
-        a ? a->nitems : p->nitems, pend, U, std::max(p->max_tile_segs, 1), g, p->kbpoly, p->sched + 8, batch,
-        (int64_t)p->M, (int64_t)g.Kx * g.Ky);
+        a ? a->nitems : p->nitems, pend, U, std::max(p->max_tile_segs, 1), g, p->kbpoly, p->sched + 8, gave_up,
+        p->wait_polls, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     return cudaGetLastError();
 }
 
@@ -1305,15 +1311,17 @@ static cudaError_t launch_grid_j(const pd_plan* p, const cplx_t<R>* src, const D
 template <typename R>
 static cudaError_t launch_grid(const pd_plan* p, int mode, const cplx_t<R>* src, const DualArgs* a,
                                const int32_t* const* tiles, const int32_t* counts4, cplx_t<R>* U, cudaStream_t s,
-                               int batch = 1, int32_t* pend = nullptr) {
+                               int batch = 1, int32_t* pend = nullptr, int32_t* gave_up = nullptr) {
     const Geo& g = p->g;
     cudaError_t e = cudaSuccess;
     prof_mark(PH_GRID, 0, s);
     if constexpr (sizeof(R) == 4) {
         if (p->grid_smem) {
             int32_t* pd = pend ? pend : p->pend;
-            if (mode == 0) PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 0>(p, src, a, pd, U, s, batch)))
-            else PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 1>(p, src, a, pd, U, s, 1)))
+            int32_t* gu = a ? a->gave_up : gave_up;
+            if (!gu) gu = p->sched + 10;
+            if (mode == 0) PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 0>(p, src, a, pd, U, gu, s, batch)))
+            else PD_J8_DISPATCH(g.J, (e = launch_grid_mma<JJ, 1>(p, src, a, pd, U, gu, s, 1)))
             prof_mark(PH_GRID, 1, s);
             return e;
         }
@@ -1333,7 +1341,8 @@ static cudaError_t launch_grid(const pd_plan* p, int mode, const cplx_t<R>* src,
 }
 
 template <typename R>
-cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch, int32_t* pend) {
+cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch, int32_t* pend,
+                       int32_t* gave_up) {
     // U = G^T y: every window is added to a zeroed grid
     cudaError_t e;
     const int64_t cells = (int64_t)batch * p->g.Kx * p->g.Ky;
@@ -1342,7 +1351,7 @@ cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, 
     if (e) return e;
     const int q = p->g.ntiles / 4;
     const int32_t* lists[4] = {p->colour_tiles, p->colour_tiles + q, p->colour_tiles + 2 * q, p->colour_tiles + 3 * q};
-    return launch_grid<R>(p, 0, y_user, nullptr, lists, p->colour_counts, U, s, batch, pend);
+    return launch_grid<R>(p, 0, y_user, nullptr, lists, p->colour_counts, U, s, batch, pend, gave_up);
 }
 
 template <typename R>
@@ -1357,8 +1366,8 @@ template cudaError_t degrid_res_norms<float>(const pd_plan*, const float2*, cons
 template cudaError_t degrid_res_norms<double>(const pd_plan*, const double2*, const double2*, double*, cudaStream_t);
 template cudaError_t degrid_dual<float>(const pd_plan*, const float2*, const DualArgs&, cudaStream_t);
 template cudaError_t degrid_dual<double>(const pd_plan*, const double2*, const DualArgs&, cudaStream_t);
-template cudaError_t grid_plain<float>(const pd_plan*, const float2*, float2*, cudaStream_t, int, int32_t*);
-template cudaError_t grid_plain<double>(const pd_plan*, const double2*, double2*, cudaStream_t, int, int32_t*);
+template cudaError_t grid_plain<float>(const pd_plan*, const float2*, float2*, cudaStream_t, int, int32_t*, int32_t*);
+template cudaError_t grid_plain<double>(const pd_plan*, const double2*, double2*, cudaStream_t, int, int32_t*, int32_t*);
 template cudaError_t grid_dual<float>(const pd_plan*, const DualArgs&, const int32_t* const*, const int32_t*,
                                       float2*, cudaStream_t);
 template cudaError_t grid_dual<double>(const pd_plan*, const DualArgs&, const int32_t* const*, const int32_t*,

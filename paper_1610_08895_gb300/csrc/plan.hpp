@@ -144,6 +144,8 @@ struct pd_plan {
     int32_t* nitems = nullptr;             // device count
     int32_t* pend = nullptr;               // [ntiles] parts of the running launch not yet added to U
     int32_t* bpend = nullptr;              // the same for each image of a batch
+    int32_t wait_polls = 1 << 22;          // polls (some seconds) after which a wait of the ordered adds gives up
+    int32_t test_hold = 0;                 // tests only: launches start with one part too many pending
     pdgb::TileItem* ditems = nullptr;      // [n_ditems] degridding items, heaviest tile first
     int n_ditems = 0;
     int64_t nslot = 0;                     // slots of seg_part
@@ -184,7 +186,7 @@ struct pd_plan {
     int32_t* sched = nullptr;      // [16] work counters of the dynamically scheduled launches: 0-3 gridding
                                    // colours (zeroed before each launch); 4-5 degridding (next item, CTAs done:
                                    // zeroed by the forward FFT and by every launch); 8 k_grid_mma (next item:
-                                   // zeroed with pend); 10: a wait gave up
+                                   // zeroed with pend); 10: a wait of a plain application gave up
     int red_len = 0;
     size_t device_bytes = 0;
     std::vector<void*> allocs;     // every device allocation of the plan
@@ -219,7 +221,7 @@ struct pd_state {
     int64_t ck_cap = 0;
     void* ck_vis = nullptr;
     int32_t* ck_idx = nullptr;
-    int32_t* status = nullptr;         // device status word
+    int32_t* status = nullptr;         // set: a wait of the gridding into this state's U gave up
     std::vector<void*> allocs;
     size_t device_bytes = 0;
     // CUDA graph of one iteration
@@ -301,6 +303,7 @@ struct DualArgs {
     const int32_t* nditems = nullptr;
     const int2* items = nullptr;        // k_grid_mma's work items and their device count
     const int32_t* nitems = nullptr;
+    int32_t* gave_up = nullptr;         // set if a wait of the ordered adds gives up
 };
 // plain degrid of `batch` half grids (stride: one image's half grid) into out (user order, stride M)
 template <typename R>
@@ -317,7 +320,7 @@ cudaError_t build_csr(pd_plan* p, cudaStream_t s);
 // plain grid: U = G^T y_user (U overwritten) for `batch` inputs (stride M) and grids (stride Kx Ky)
 template <typename R>
 cudaError_t grid_plain(const pd_plan* p, const cplx_t<R>* y_user, cplx_t<R>* U, cudaStream_t s, int batch = 1,
-                       int32_t* pend = nullptr);
+                       int32_t* pend = nullptr, int32_t* gave_up = nullptr);
 // pd grid over the listed tiles, one launch per colour (tiles[c]: device list of colour c,
 // counts4[c]: device count): v <- scale * r, U += G^T (v_new - v_old)
 template <typename R>

@@ -110,3 +110,64 @@ def test_dictionary_on_buffers_that_start_anywhere(n, levels):
     back = plan.pd_apply_psi(b, torch.zeros(n * n + 1, dtype=torch.float32, device="cuda")[1:].view(n, n))
     assert rel(back.cpu().numpy(), x.cpu().numpy()) < TOL_OP32
     assert rel(plan.pd_apply_psi(a).cpu().numpy(), x.cpu().numpy()) < TOL_OP32
+
+
+def _hold(plan, polls, hold):
+    import ctypes
+    from paper_1610_08895_gb300 import _binding as B
+    hook = B.load().pd_test_ordered_adds
+    hook.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32]
+    B.check(hook(plan.handle, polls, hold))
+
+
+def _timeout(call):
+    from paper_1610_08895_gb300 import _binding as B
+    with pytest.raises(B.PDError) as e:
+        call()
+    return e.value.status == B.PD_ETIMEOUT
+
+
+def test_a_wait_of_the_ordered_adds_that_gives_up():
+    """A short limit and one part too many pending: the launch ends, the sums are complete, every state
+    keeps its own flag until its data are set anew, plain applications theirs, and the next call
+    is as if nothing had been."""
+    from paper_1610_08895_gb300.api import Plan, State
+    n, m, nb, J = 64, 6000, 4, 8
+    uv = _points("gauss", m, n)
+    geo = meas.Geometry(n, n, J)
+    plan = Plan(n, n, uv, (np.arange(m) % nb).astype(np.int32), nb, kernel_width=J, basis_ids=(0, 1), levels=2)
+    v = synth.uniform_vis(m, seed=4)
+    vt = torch.tensor(v, dtype=plan.cplx_dtype, device="cuda")
+    kw = dict(tau=0.49, sigma=1.0, varsigma=1e-4, kappa=1e-3, seed=1, p_block=[1.0] * nb, p_basis=[1.0] * 2)
+    a, b = State(plan), State(plan)
+    for st in (a, b):
+        st.pd_state_set_data(vt, np.ones(nb))
+    want = plan.pd_apply_phi_adj(vt)
+    a.pd_iterate(3, **kw)
+    want_x, start = a.x(), b.save()
+    a.report()
+    plan.pd_plan_status()
+    a.pd_state_set_data(vt, np.ones(nb))
+    _hold(plan, 8, 1)
+    for form in (dict(), dict(use_graph=True), dict(per_block=True)):
+        a.pd_state_set_data(vt, np.ones(nb))
+        a.report()
+        a.pd_iterate(3, **kw, **form)
+        assert rel(a.x().cpu().numpy(), want_x.cpu().numpy()) < 1e-5      # complete; another order of the sums
+        assert _timeout(a.report) and _timeout(a.report)
+    plan.pd_plan_status()                                                   # not a plain application's
+    xa = plan.pd_apply_phi_adj(vt)
+    assert rel(xa.cpu().numpy(), geo.phi_adj(v, uv)) < TOL_OP32
+    assert _timeout(plan.pd_plan_status)
+    x0 = torch.tensor(synth.random_images(1, n, n, seed=3)[0], dtype=plan.real_dtype, device="cuda")
+    assert _timeout(lambda: plan.pd_operator_norms(x0, 3, 0.0))
+    b.report()                                                              # nor another state's
+    assert _timeout(lambda: b.pd_state_set_start(v0=vt)) and _timeout(b.report)
+    _hold(plan, 1 << 22, 0)
+    assert torch.equal(plan.pd_apply_phi_adj(vt), want)
+    assert _timeout(a.report)
+    b.load(start)
+    b.report()
+    a.pd_state_set_data(vt, np.ones(nb))
+    a.pd_iterate(3, **kw)
+    assert a.report()["t"] == 3 and torch.equal(a.x(), want_x)
