@@ -353,11 +353,15 @@ pd_status pd_synthesis_iterate(pd_plan* plan, pd_state* st, const pd_params* par
  * replicated (every rank runs the same primal update).
  * pd_iterate_dual: steps 3-14 (draws, F Z x~, degridding and the l2-ball update of this
  * rank's active blocks, gridding of their dual change into the state's U, the sparsity
- * dual update). The caller then sums U over the ranks (pd_state_u gives the device
+ * dual update). The caller then sums U over the ranks (pd_state_u_folded gives the device
  * pointer of the state's U, complex [Kx/4][Ky][4] column panels, Kx*Ky elements; the
- * sum must go to another buffer, since U keeps this rank's own part). U stands for G^T v up
- * to the symmetry of a real image: most visibilities with u < 0 are gridded as their
- * conjugates at -(u, v), which leaves Re(Z^T F^H U) as it is; pd_iterate_primal takes either.
+ * sum must go to another buffer, since U keeps this rank's own part). The state's U has the
+ * Hermitian part of G^T v, which is all that Re(Z^T F^H U) takes: most visibilities with u < 0
+ * are gridded as their conjugates at -(u, v).
+ * pd_state_u: G^T v itself, in the same layout, at an address that stays valid and is brought up
+ * to date by every call that changes v, on that call's stream. The first call allocates the grid
+ * (PD_ENOMEM) and synchronises the device; from then on each such call takes two more griddings.
+ * Either grid, or a sum of either over ranks, may be passed to pd_iterate_primal.
  * pd_iterate_primal: steps 17-18 with the summed U (device, same layout; NULL = the
  * state's own U). adaptive must be 0 (the residual norms would differ between ranks).
  * Both asynchronous on `stream`; pd_iterate_dual + pd_iterate_primal(NULL) equals one
@@ -366,6 +370,7 @@ pd_status pd_synthesis_iterate(pd_plan* plan, pd_state* st, const pd_params* par
 pd_status pd_iterate_dual(pd_plan* plan, pd_state* st, const pd_params* params, void* stream);
 pd_status pd_iterate_primal(pd_plan* plan, pd_state* st, const pd_params* params, const void* u, void* stream);
 pd_status pd_state_u(pd_state* st, void** u, int64_t* elements);
+pd_status pd_state_u_folded(pd_state* st, void** u, int64_t* elements);
 
 /*
  * Per-phase kernel times accumulated by iterations run with params.profile = 1:

@@ -74,6 +74,7 @@ _SIGS = {
     "pd_iterate_dual": ([_VP, _VP, ctypes.POINTER(PdParams), _VP], ctypes.c_int),
     "pd_iterate_primal": ([_VP, _VP, ctypes.POINTER(PdParams), _VP, _VP], ctypes.c_int),
     "pd_state_u": ([_VP, ctypes.POINTER(_VP), _VP], ctypes.c_int),
+    "pd_state_u_folded": ([_VP, ctypes.POINTER(_VP), _VP], ctypes.c_int),
     "pd_state_get_x": ([_VP, _VP, _VP], ctypes.c_int),
     "pd_state_get_x_tilde": ([_VP, _VP, _VP], ctypes.c_int),
     "pd_state_get_s": ([_VP, _VP, _VP], ctypes.c_int),

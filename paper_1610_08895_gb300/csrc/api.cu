@@ -232,6 +232,7 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
             gxv = -gxv;
             gyv = -gyv;
             flip[m] = 1;
+            p->folded = true;
         }
         double flx, fly, fx, fy;
         split(gxv, flx, fx);
@@ -830,6 +831,7 @@ extern "C" pd_status pd_state_set_data(pd_plan* p, pd_state* st, const void* y, 
     CU(cudaMemsetAsync(st->v, 0, p->M * p->csz, s));
     CU(cudaMemsetAsync(st->u, 0, K * p->csz, s));
     CU(cudaMemsetAsync(st->t, 0, 4 * sizeof(int64_t), s));      // t, diag, status
+    if (st->u_out) CU(cudaMemsetAsync(st->u_out, 0, K * p->csz, s));
     if (st->syn_at) CU(cudaMemsetAsync(st->syn_at, 0, N * p->b * p->rsz, s));
     if (st->syn_u) CU(cudaMemsetAsync(st->syn_u, 0, N * p->rsz, s));
     std::vector<double> ones_d(p->d, 1.0), ones_b(p->b, 1.0);
@@ -837,6 +839,14 @@ extern "C" pd_status pd_state_set_data(pd_plan* p, pd_state* st, const void* y, 
     CU(cudaMemcpyAsync(st->p_basis, ones_b.data(), p->b * sizeof(double), cudaMemcpyHostToDevice, s));
     CU(init_res_norm(p, st, s));
     CU(cudaStreamSynchronize(s));
+    return PD_OK;
+}
+
+// The grid that pd_state_u handed out, after anything that changed v.
+static pd_status refresh_u(pd_state* st, cudaStream_t s) {
+    if (!st->u_out) return PD_OK;
+    if (st->plan->prec == PD_F64) CU(unfolded_u<double>(st->plan, st, (double2*)st->u_out, s));
+    else CU(unfolded_u<float>(st->plan, st, (float2*)st->u_out, s));
     return PD_OK;
 }
 
@@ -870,6 +880,8 @@ static pd_status set_start_t(pd_plan* p, pd_state* st, const void* x0, const voi
     } else {
         CU(init_res_norm(p, st, s));
     }
+    const pd_status eu = refresh_u(st, s);
+    if (eu != PD_OK) return eu;
     int32_t gave_up = 0;
     CU(cudaMemcpyAsync(&gave_up, st->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
@@ -1111,7 +1123,7 @@ extern "C" pd_status pd_iterate_dual(pd_plan* p, pd_state* st, const pd_params* 
     if (p->prec == PD_F64) CU(enqueue_dual<double>(p, st, prm, s, true));
     else CU(enqueue_dual<float>(p, st, prm, s, true));
     CU(cudaStreamWaitEvent(s, st->ev_join, 0));
-    return PD_OK;
+    return refresh_u(st, s);
 }
 
 extern "C" pd_status pd_iterate_primal(pd_plan* p, pd_state* st, const pd_params* prm, const void* u, void* stream) {
@@ -1123,9 +1135,29 @@ extern "C" pd_status pd_iterate_primal(pd_plan* p, pd_state* st, const pd_params
     return PD_OK;
 }
 
+extern "C" pd_status pd_state_u_folded(pd_state* st, void** u, int64_t* elements) {
+    if (!st || !u) return fail(PD_EINVAL, "pd_state_u_folded: bad argument");
+    *u = st->u;
+    if (elements) *elements = (int64_t)st->plan->g.Kx * st->plan->g.Ky;
+    return PD_OK;
+}
 extern "C" pd_status pd_state_u(pd_state* st, void** u, int64_t* elements) {
     if (!st || !u) return fail(PD_EINVAL, "pd_state_u: bad argument");
-    *u = st->u;
+    if (!st->plan->folded) return pd_state_u_folded(st, u, elements);
+    if (!st->u_out) {
+        const pd_plan* p = st->plan;
+        const size_t K = (size_t)p->g.Kx * p->g.Ky;
+        if (dalloc_bytes(st->allocs, st->device_bytes, &st->u_out, K * p->csz)) {
+            st->u_out = nullptr;
+            (void)cudaGetLastError();
+            return fail(PD_ENOMEM, "pd_state_u: device allocation failed");
+        }
+        CU(cudaDeviceSynchronize());       // the state's work may be on any stream
+        const pd_status e = refresh_u(st, 0);
+        if (e != PD_OK) return e;
+        CU(cudaDeviceSynchronize());
+    }
+    *u = st->u_out;
     if (elements) *elements = (int64_t)st->plan->g.Kx * st->plan->g.Ky;
     return PD_OK;
 }
@@ -1186,6 +1218,8 @@ extern "C" pd_status pd_synthesis_iterate(pd_plan* p, pd_state* st, const pd_par
     // the image x = Psi alpha for pd_state_get_x
     if (p->prec == PD_F64) CU(psi_plain<double>(p, (const double*)st->s, (double*)st->x, s));
     else CU(psi_plain<float>(p, (const float*)st->s, (float*)st->x, s));
+    const pd_status eu = refresh_u(st, s);
+    if (eu != PD_OK) return eu;
     CU(cudaStreamSynchronize(s));   // the host vector of ones is read by the copy above
     return PD_OK;
 }
@@ -1218,7 +1252,7 @@ extern "C" pd_status pd_iterate(pd_plan* p, pd_state* st, const pd_params* prm, 
             if (p->prec == PD_F64) CU(enqueue_iteration_per_block<double>(p, st, prm, s));
             else CU(enqueue_iteration_per_block<float>(p, st, prm, s));
         }
-        return PD_OK;
+        return refresh_u(st, s);
     }
     if (prm->use_graph) {
         // The caller's stream may be the legacy default stream, which cannot be captured:
@@ -1274,7 +1308,7 @@ extern "C" pd_status pd_iterate(pd_plan* p, pd_state* st, const pd_params* prm, 
             else CU(enqueue_iteration<float>(p, st, prm, s));
         }
     }
-    return PD_OK;
+    return refresh_u(st, s);
 }
 
 extern "C" pd_status pd_state_profile(pd_state* st, double* ms, int64_t* iterations, int32_t n, int32_t reset) {
@@ -1416,7 +1450,11 @@ static pd_status copy_state(pd_state* st, unsigned char* c, bool save, cudaStrea
         }
         c += q.bytes;
     }
-    if (!save) CU(cudaMemsetAsync(st->status, 0, sizeof(int32_t), s));
+    if (!save) {
+        CU(cudaMemsetAsync(st->status, 0, sizeof(int32_t), s));
+        e = refresh_u(st, s);
+        if (e != PD_OK) return e;
+    }
     CU(cudaStreamSynchronize(s));
     return PD_OK;
 }

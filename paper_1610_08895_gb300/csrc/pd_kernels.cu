@@ -257,6 +257,43 @@ cudaError_t scatter_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cpl
     k_scatter<<<ctas, 256, 0, s>>>(src, dst, perm, m);
     return cudaGetLastError();
 }
+// The visibilities that are held as their conjugates (held = 1) or the others, in user order and
+// convention, zeros in the place of the rest.
+template <typename C>
+__global__ void k_scatter_side(const C* __restrict__ internal, C* __restrict__ user, const int32_t* __restrict__ perm,
+                               int64_t m, int held) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+        C v = vis_conj(perm[i], internal[i]);
+        if ((perm[i] < 0) != (held != 0)) v.x = v.y = 0;
+        user[vis_index(perm[i])] = v;
+    }
+}
+// U[k] += conj W[-k] over the whole grid.
+template <typename C>
+__global__ void k_add_mirrored(C* __restrict__ U, const C* __restrict__ W, int Ky, int Kx) {
+    const int64_t n = (int64_t)Ky * Kx;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int ky = (int)(i / PW % Ky), kx = (int)(i / PW / Ky) * PW + (int)(i % PW);
+        const C w = W[panel_off((Ky - ky) & (Ky - 1), (Kx - kx) & (Kx - 1), Ky)];
+        C u = U[i];
+        u.x += w.x;
+        u.y -= w.y;
+        U[i] = u;
+    }
+}
+template <typename R>
+cudaError_t unfolded_u(const pd_plan* p, const pd_state* st, cplx_t<R>* out, cudaStream_t s) {
+    cplx_t<R>* user = (cplx_t<R>*)p->rbuf;
+    cplx_t<R>* grid[2] = {out, (cplx_t<R>*)p->gridu};
+    const int ctas = (int)std::min<int64_t>(4096, (p->M + 255) / 256);
+    cudaError_t e;
+    for (int held = 0; held < 2; ++held) {
+        k_scatter_side<<<ctas, 256, 0, s>>>((const cplx_t<R>*)st->v, user, p->perm, p->M, held);
+        if ((e = cudaGetLastError()) || (e = grid_plain<R>(p, user, grid[held], s, 1, nullptr, st->status))) return e;
+    }
+    k_add_mirrored<<<p->num_sms * 8, 256, 0, s>>>(out, (const cplx_t<R>*)grid[1], p->g.Ky, p->g.Kx);
+    return cudaGetLastError();
+}
 template <typename R>
 cudaError_t gather_internal(const pd_plan* p, const cplx_t<R>* user, cplx_t<R>* internal, cudaStream_t s) {
     return gather_by<R>(p->M, p->perm, user, internal, s);
@@ -363,6 +400,8 @@ template cudaError_t gather_by<float>(int64_t, const int32_t*, const float2*, fl
 template cudaError_t gather_by<double>(int64_t, const int32_t*, const double2*, double2*, cudaStream_t);
 template cudaError_t scatter_by<float>(int64_t, const int32_t*, const float2*, float2*, cudaStream_t);
 template cudaError_t scatter_by<double>(int64_t, const int32_t*, const double2*, double2*, cudaStream_t);
+template cudaError_t unfolded_u<float>(const pd_plan*, const pd_state*, float2*, cudaStream_t);
+template cudaError_t unfolded_u<double>(const pd_plan*, const pd_state*, double2*, cudaStream_t);
 template cudaError_t gather_internal<float>(const pd_plan*, const float2*, float2*, cudaStream_t);
 template cudaError_t gather_internal<double>(const pd_plan*, const double2*, double2*, cudaStream_t);
 template cudaError_t scatter_user<float>(const pd_plan*, const float2*, float2*, cudaStream_t);

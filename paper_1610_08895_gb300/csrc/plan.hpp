@@ -108,6 +108,7 @@ struct pd_plan {
     int ck_tile = 0;
     std::mutex ck_mu;
     std::vector<int32_t> ck_order;
+    bool folded = false;           // some visibility is held as its conjugate
 
     // device: visibilities in internal (tile, block, row, column) order
     int32_t* cell = nullptr;       // (by << 16) | bx of the footprint's first cell, mod K
@@ -213,6 +214,7 @@ struct pd_state {
     int32_t* counts = nullptr;         // {active segments, active tiles}
     int64_t* t = nullptr;              // iteration counter (device)
     double* diag = nullptr;            // [2]: ||dx||^2, ||x||^2
+    void* u_out = nullptr;             // complex grid: G^T v itself, kept up to date once pd_state_u was called
     double* prim_part = nullptr;       // [2 * ny / rows-per-CTA]
     // staging of a checkpoint's visibilities (the state's own: other states of the plan may be
     // iterating on other streams meanwhile): ck_cap of them and their internal indices, one save
@@ -366,6 +368,10 @@ template <typename R>
 cudaError_t gather_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
 template <typename R>
 cudaError_t scatter_by(int64_t m, const int32_t* perm, const cplx_t<R>* src, cplx_t<R>* dst, cudaStream_t s);
+// out = G^T v of a state, every visibility at its own (u, v): two plain griddings, of the
+// visibilities held as conjugates and of the others (uses the plan's rbuf and gridu)
+template <typename R>
+cudaError_t unfolded_u(const pd_plan* p, const pd_state* st, cplx_t<R>* out, cudaStream_t s);
 template <typename R>
 cudaError_t scatter_user(const pd_plan* p, const cplx_t<R>* internal, cplx_t<R>* user, cudaStream_t s);
 // pend[t] = parts of the tiles that hold a point of an active block (all of them: active null), else 0,

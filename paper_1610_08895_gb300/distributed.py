@@ -9,8 +9,8 @@ grid. Every rank plans only its own visibilities but with the global block count
 the counter-based draws of Algorithm 1 step 3 are the same everywhere; the primal
 variables x, x~ and the sparsity duals s are replicated (every rank runs the same
 primal and sparsity updates on the same data). Per iteration the one exchange is a sum
-over ranks of U_r = G_r^T v_r (the rank's gridded dual sum), a full complex grid of
-Kx Ky elements: one all-reduce.
+over ranks of U_r (the rank's gridded dual sum: a complex grid of Kx Ky elements with the
+Hermitian part of G_r^T v_r, which is what the primal step takes): one all-reduce.
 
 `run(engine, niter, all_reduce)` drives any rank-local engine (dual_step, u_sum_buffer,
 primal_step); `GpuShard` is the engine on this library's C ABI.
@@ -78,7 +78,7 @@ class GpuShard:
         self.params = B.PdParams(p_block=pb.ctypes.data, p_basis=ps.ctypes.data, seed=int(self.kw.pop("seed", 0)),
                                  **{k: float(v) for k, v in self.kw.items()})
         ptr, n = ctypes.c_void_p(), ctypes.c_int64()
-        B.call("pd_state_u", self.state._h, ctypes.byref(ptr), ctypes.byref(n))
+        B.call("pd_state_u_folded", self.state._h, ctypes.byref(ptr), ctypes.byref(n))
         typestr = "<c8" if p.cplx_dtype == torch.complex64 else "<c16"
         self.u_local = torch.as_tensor(_DevArray(ptr.value, n.value, typestr), device="cuda")
         self.u_sum = torch.empty_like(self.u_local)

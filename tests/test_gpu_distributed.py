@@ -57,3 +57,69 @@ def test_two_shards_match_oracle_and_unsplit_iteration(precision):
     st.pd_state_set_data(torch.tensor(prob.y, dtype=cdt, device="cuda"), prob.eps)
     st.pd_iterate(niter, **kw)
     assert rel(x0_, st.x().cpu().numpy()) < (1e-12 if precision == "f64" else 1e-5)
+
+
+@pytest.mark.parametrize("precision,J", [("f64", 8), ("f32", 8), ("f32", 12), ("f64", 2)])
+def test_state_u_is_the_gridded_dual_sum(precision, J):
+    """pd_state_u's grid is G^T v of the oracle, every visibility at its own (u, v), at the same address
+    after each call that changes v; pd_iterate_primal takes it or the folded one alike."""
+    import ctypes
+
+    from oracle import measurement as meas
+    from paper_1610_08895_gb300 import _binding as B
+    from paper_1610_08895_gb300 import distributed as D
+    from paper_1610_08895_gb300.api import Plan, State
+    n, ny, m = 64, 32, 3000
+    rng = np.random.default_rng(7)
+    uv = rng.uniform(-np.pi, np.pi, size=(m, 2))
+    uv[:50] = rng.integers(-32, 32, size=(50, 2)) * (np.pi / 64)          # on grid lines of both axes
+    geo = meas.Geometry(ny, n, J)
+    plan = Plan(n, ny, uv, (np.arange(m) % 4).astype(np.int32), 4, kernel_width=J, basis_ids=(0, 1), levels=2,
+                precision=precision)
+    st = State(plan)
+    st.pd_state_set_data(torch.tensor(synth.uniform_vis(m, seed=5), dtype=plan.cplx_dtype, device="cuda"), np.ones(4))
+    v0 = torch.tensor(synth.uniform_vis(m, seed=6), dtype=plan.cplx_dtype, device="cuda")
+
+    def view(name):
+        ptr, k = ctypes.c_void_p(), ctypes.c_int64()
+        B.call(name, st._h, ctypes.byref(ptr), ctypes.byref(k))
+        typestr = "<c8" if precision == "f32" else "<c16"
+        return ptr.value, torch.as_tensor(D._DevArray(ptr.value, k.value, typestr), device="cuda")
+
+    addr, u = view("pd_state_u")
+    tol = 1e-12 if precision == "f64" else 1e-5
+
+    def check():
+        torch.cuda.synchronize()
+        got = u.cpu().numpy().reshape(2 * n // 4, 2 * ny, 4).transpose(1, 0, 2).reshape(2 * ny, 2 * n)
+        want = geo.grid(st.v().cpu().numpy().astype(complex), uv).reshape(2 * ny, 2 * n)
+        assert rel(got, want) < tol if np.any(want) else not np.any(got)
+        assert view("pd_state_u")[0] == addr
+
+    kw = dict(tau=0.49, sigma=1.0, varsigma=1e-4, kappa=1e-3, seed=1, p_block=[0.6] * 4, p_basis=[1.0] * 2)
+    check()
+    st.pd_state_set_start(v0=v0)
+    check()
+    buf = st.save()
+    for form in (dict(), dict(use_graph=True), dict(per_block=True)):
+        st.pd_iterate(3, **kw, **form)
+        check()
+    st.load(buf)
+    check()
+    pb, ps = np.full(4, 0.6), np.ones(2)
+    prm = B.PdParams(tau=0.49, sigma=1.0, varsigma=1e-4, kappa=1e-3, psi_norm=1.0, seed=1, p_block=pb.ctypes.data,
+                     p_basis=ps.ctypes.data)
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    B.call("pd_iterate_dual", plan.handle, st._h, ctypes.byref(prm), stream)
+    check()
+    after = st.save()
+    out = []
+    for grid in (None, u.clone(), view("pd_state_u_folded")[1].clone()):
+        st.load(after)
+        B.call("pd_iterate_primal", plan.handle, st._h, ctypes.byref(prm),
+               ctypes.c_void_p(0 if grid is None else grid.data_ptr()), stream)
+        out.append(st.x().cpu().numpy())
+    assert rel(out[1], out[0]) < tol and rel(out[2], out[0]) < tol
+    st.pd_state_set_data(v0, np.ones(4))
+    st.pd_synthesis_iterate(2, 0.49, 1.0, 1e-4, 1e-3, seed=1, p_block=[0.6] * 4)
+    check()
