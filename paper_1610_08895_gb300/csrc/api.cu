@@ -479,9 +479,11 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         }
         if (p->prec == PD_F64) {
             double err = 0.0;
-            const std::vector<double> kp = kb_tap_polynomials_ext(p->kb_J, g.beta, KB_DEG64, &err);
-            for (int a = 0; a < p->kb_J; ++a)
-                for (int k = 0; k <= KB_DEG64; ++k) p->kbpoly64.c[a][k] = kp[(size_t)a * (KB_DEG64 + 1) + k];
+            std::vector<double> inner, edge;
+            kb_tap_polynomials_ext(p->kb_J, g.beta, KB_DEG64, kb_outer(p->kb_J), kb_edge_deg(p->kb_J), inner, edge, &err);
+            for (int a = 0; a < p->kb_J / 2; ++a)
+                for (int k = 0; k <= KB_DEG64; ++k) p->kbpoly64.c[a][k] = inner[(size_t)a * (KB_DEG64 + 1) + k];
+            std::copy(edge.begin(), edge.end(), p->kbpoly64.e);
             p->kbpoly64.use = err < 1e-16;
         }
         p->h_filt.assign((size_t)p->b * MAX_FILTER, 0.0);

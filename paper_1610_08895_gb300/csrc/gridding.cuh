@@ -24,8 +24,27 @@ __device__ __forceinline__ void kb_taps(R frac, R* w, R two_over_j, R beta, cons
         }
     }
     const R x = R(2) * frac - R(1), x2 = x * x;
+    constexpr int OUT = sizeof(R) == 8 ? kb_outer(J) : 0;
+    if constexpr (sizeof(R) == 8) {
+        // FP64, outermost taps: the weight falls to 1e-7 of phi(0) and less there, so a fit that is
+        // exact to phi(0) is not to the weight itself (1.7e-12 of it at J = 8). s = q (2 - q), q the
+        // distance to the kernel's end in half-widths, has no cancellation at that end.
 #pragma unroll
-    for (int a = 0; a < J / 2; ++a) {
+        for (int a = 0; a < OUT; ++a) {
+            const double q0 = (a + 1 - frac) * two_over_j, q1 = (a + frac) * two_over_j;
+            const double s0 = q0 * (2.0 - q0), s1 = q1 * (2.0 - q1);
+            double w0 = kp.e[kb_edge_deg(J)], w1 = w0;
+#pragma unroll
+            for (int k = kb_edge_deg(J) - 1; k >= 0; --k) {
+                w0 = fma(w0, s0, kp.e[k]);
+                w1 = fma(w1, s1, kp.e[k]);
+            }
+            w[a] = w0;
+            w[J - 1 - a] = w1;
+        }
+    }
+#pragma unroll
+    for (int a = OUT; a < J / 2; ++a) {
         R ev = kp.c[a][DEG], od = kp.c[a][DEG - 1];
 #pragma unroll
         for (int k = DEG - 2; k >= 2; k -= 2) ev = fma(ev, x2, kp.c[a][k]);

@@ -159,58 +159,85 @@ std::vector<double> kb_tap_polynomials(int J, double beta, int deg) {
     return out;
 }
 
-// I0(z) by its power series (positive terms only).
-static long double bessel_i0_ext(long double z) {
-    const long double q = z * z / 4.0L;
-    long double term = 1.0L, sum = 1.0L;
-    for (int k = 1; k < 4000; ++k) {
-        term *= q / ((long double)k * k);
-        sum += term;
-        if (term < sum * 1e-22L) break;
-    }
-    return sum;
-}
-
-std::vector<double> kb_tap_polynomials_ext(int J, double beta, int deg, double* err) {
+// phi(t) = I0(beta sqrt(s)) with s = 1 - (2 t / J)^2 by its power series: positive terms
+// (beta^2 / 4)^k s^k / (k!)^2, so that it is exact to its own rounding at every t.
+void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg, std::vector<double>& inner,
+                            std::vector<double>& edge, double* err) {
     using ld = long double;
     const int n = deg + 1;
     const ld pi = 3.14159265358979323846264338327950288L;
+    inner.assign((size_t)(J / 2) * n, 0.0);
+    edge.assign(edge_deg + 1, 0.0);
+    *err = 1.0;
+    if (!(beta <= 64.0)) return;          // steeper than the degrees in use can follow
+    std::vector<ld> c(1, 1.0L);
+    for (int k = 1; c.back() > 1e-21L || k <= edge_deg; ++k) c.push_back(c.back() * ((ld)beta * beta / 4.0L) / ((ld)k * k));
     auto phi = [&](ld t) {
-        const ld u = 2.0L * t / J, arg = 1.0L - u * u;
-        return arg > 0 ? bessel_i0_ext((ld)beta * std::sqrt(arg)) : (arg > -1e-15L ? 1.0L : 0.0L);
+        const ld u = 2.0L * t / J, q = 1.0L - u * u;
+        ld v = 0.0L;
+        for (size_t k = c.size(); k-- > 0;) v = v * q + c[k];
+        return v;
     };
-    std::vector<double> out((size_t)J * n, 0.0);
+    const ld phi0 = phi(0.0L);
     ld worst = 0.0L;
-    for (int a = 0; a < J; ++a) {
-        std::vector<ld> fx(n), cheb(n, 0.0L);
-        for (int k = 0; k < n; ++k) fx[k] = phi((std::cos(pi * (k + 0.5L) / n) + 1.0L) / 2.0L + J / 2 - 1 - a);
+    // cos(pi i / (2 n)), for the nodes and the interpolation
+    std::vector<ld> cs(4 * n);
+    for (int i = 0; i < 4 * n; ++i) cs[i] = std::cos(pi * i / (2 * n));
+    std::vector<ld> mono, prev, cur, next, fx(n), cheb(n);
+    for (int a = outer; a < J / 2; ++a) {
+        for (int k = 0; k < n; ++k) fx[k] = phi((cs[2 * k + 1] + 1.0L) / 2.0L + J / 2 - 1 - a);
         for (int j = 0; j < n; ++j) {
             ld acc = 0.0L;
-            for (int k = 0; k < n; ++k) acc += fx[k] * std::cos(pi * j * (k + 0.5L) / n);
+            for (int k = 0; k < n; ++k) acc += fx[k] * cs[j * (2 * k + 1) % (4 * n)];
             cheb[j] = (j == 0 ? 1.0L : 2.0L) * acc / n;
         }
         // sum_j cheb_j T_j in monomials, T_{j+1} = 2 x T_j - T_{j-1}
-        std::vector<ld> prev(n, 0.0L), cur(n, 0.0L), mono(n, 0.0L);
+        mono.assign(n, 0.0L);
+        prev.assign(n, 0.0L);
+        cur.assign(n, 0.0L);
         cur[0] = 1.0L;
         for (int j = 0; j < n; ++j) {
-            for (int i = 0; i < n; ++i) mono[i] += cheb[j] * cur[i];
-            std::vector<ld> next(n, 0.0L);
+            for (int i = 0; i <= j; ++i) mono[i] += cheb[j] * cur[i];
+            next.assign(n, 0.0L);
             for (int i = 0; i + 1 < n; ++i) next[i + 1] = (j == 0 ? 1.0L : 2.0L) * cur[i];
             if (j > 0)
                 for (int i = 0; i < n; ++i) next[i] -= prev[i];
-            prev = cur;
-            cur = next;
+            prev.swap(cur);
+            cur.swap(next);
         }
-        for (int i = 0; i < n; ++i) out[(size_t)a * n + i] = (double)mono[i];
-        for (int k = 0; k <= 2 * n; ++k) {     // between the nodes
-            const ld x = std::cos(pi * k / (2 * n));
+        for (int i = 0; i < n; ++i) inner[(size_t)a * n + i] = (double)mono[i];
+        for (int k = 0; k <= n; ++k) {         // between the nodes, and the ends
+            const ld x = cs[2 * k];
             ld v = 0.0L;
             for (int i = n - 1; i >= 0; --i) v = v * x + mono[i];
-            worst = std::max(worst, std::abs(v - phi((x + 1.0L) / 2.0L + J / 2 - 1 - a)));
+            worst = std::max(worst, std::abs(v - phi((x + 1.0L) / 2.0L + J / 2 - 1 - a)) / phi0);
         }
     }
-    *err = (double)(worst / phi(0.0L));
-    return out;
+    // the outer taps, s in [0, s1]: the series economised (Lanczos 1938): its highest term, replaced by
+    // that term's best approximation of lower degree on [0, s1], again and again
+    const ld q1 = (ld)(J / 2 - outer) / (J / 2), s1 = 1.0L - q1 * q1;
+    const int K = (int)c.size() - 1;
+    std::vector<ld> y(K + 1);
+    ld pw = 1.0L, dropped = 0.0L;
+    for (int k = 0; k <= K; ++k, pw *= s1) y[k] = c[k] * pw;
+    std::vector<std::vector<ld>> T(K + 1);     // T_k(2 y - 1) / 2^(2 k - 1): leading coefficient 1
+    for (int k = 0; k <= K; ++k) {
+        T[k].assign(k + 1, 0.0L);
+        if (k == 0) T[0][0] = 1.0L;
+        else if (k == 1) { T[1][0] = -0.5L; T[1][1] = 1.0L; }
+        else
+            for (int i = 0; i <= k; ++i)       // T_k = (4 y - 2) T_{k-1} - T_{k-2}
+                T[k][i] = (i > 0 ? T[k - 1][i - 1] : 0.0L) - (i < k ? T[k - 1][i] / 2.0L : 0.0L) -
+                          (i < k - 1 ? T[k - 2][i] / (k == 2 ? 8.0L : 16.0L) : 0.0L);
+    }
+    for (int k = K; k > edge_deg; --k) {
+        const ld top = y[k];
+        for (int i = 0; i <= k; ++i) y[i] -= top * T[k][i];
+        dropped += std::abs(std::ldexp(top, 1 - 2 * k));
+    }
+    pw = 1.0L;
+    for (int k = 0; k <= edge_deg; ++k, pw *= s1) edge[k] = (double)(y[k] / pw);
+    *err = (double)std::max(worst, dropped);   // phi >= 1 on the outer taps
 }
 
 }  // namespace pdgb

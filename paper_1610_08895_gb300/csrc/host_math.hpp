@@ -16,8 +16,13 @@ std::vector<double> twiddles(int K);
 // Monomial coefficients (in x = 2 f - 1, f in [0, 1)) of the degree-`deg` Chebyshev
 // interpolant of tap a's weight phi(f + J/2 - 1 - a), for a = 0..J-1: [J][deg + 1].
 std::vector<double> kb_tap_polynomials(int J, double beta, int deg);
-// The same fitted in extended precision; *err is the largest deviation of the fit from the
-// weight between the nodes, relative to phi(0), before the coefficients are rounded to FP64.
-std::vector<double> kb_tap_polynomials_ext(int J, double beta, int deg, double* err);
+// The weights for FP64, fitted in extended precision. Taps outer <= a < J/2: the same monomials,
+// [J/2][deg + 1]. The `outer` outermost taps on either side, where the weight falls to 1 / I0(beta)
+// of its largest value: one polynomial in s = 1 - (2 t / J)^2, [edge_deg + 1], exact to the weight
+// itself there. *err: the larger of the first fit's deviation between the nodes relative to phi(0)
+// and the second one's relative to the weight, before the coefficients are rounded to FP64 (1: not
+// fitted, beta too large).
+void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg, std::vector<double>& inner,
+                            std::vector<double>& edge, double* err);
 
 }  // namespace pdgb

@@ -44,8 +44,13 @@ struct KbPoly {
 // The same for the FP64 kernels; use = 0 where the fit is not exact to FP64 (a caller's own,
 // larger kb_beta): those plans evaluate I0 itself.
 constexpr int KB_DEG64 = 18;
+// The outermost taps (kb_outer of them on either side) by a polynomial in s = 1 - (2 t / J)^2.
+constexpr int KB_EDGE_MAX = 31;
+__host__ __device__ constexpr int kb_outer(int J) { return J > 8 ? 2 : 1; }
+__host__ __device__ constexpr int kb_edge_deg(int J) { return J > 8 ? KB_EDGE_MAX : 20; }
 struct KbPoly64 {
-    double c[16][KB_DEG64 + 1];
+    double c[8][KB_DEG64 + 1];
+    double e[KB_EDGE_MAX + 1];
     int use;
 };
 template <typename R> struct KbPolyOf { using type = KbPoly; };

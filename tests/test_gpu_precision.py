@@ -51,3 +51,38 @@ def test_fp32_gridding_has_no_bias(J):
         scales.append((np.vdot(ref, got) / np.vdot(ref, ref)).real - 1.0)
         assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 1.2e-7      # two units of rounding
     assert abs(np.mean(scales)) < 1e-8, scales
+
+
+def _kb(t, J, beta):
+    """I0(beta sqrt(1 - (2 t / J)^2)) by its power series in extended precision."""
+    s = 1 - (2 * t / J) ** 2
+    q, term, out = np.longdouble(beta) ** 2 / 4, np.ones_like(s), np.ones_like(s)
+    for k in range(1, 400):
+        term = term * q * s / (np.longdouble(k) * k)
+        out = out + term
+        if np.all(term < out * 1e-22):
+            break
+    return np.where(s > 0, out, 0)
+
+
+@pytest.mark.parametrize("J", [2, 4, 6, 8, 10, 16])
+def test_fp64_taps_are_exact_to_themselves(J):
+    """G^T of single points in FP64 plans: every cell of the footprint to 1e-13 of its own value, the outermost
+    ones (some 1e-14 of the largest at J = 8) included. Two taps of at most 20 roundings of 1.1e-16 each; the
+    oracle's own argument rounding is up to beta^2 / 2 * 1.1e-16 = 8e-14 there, so the weights are taken
+    in extended precision."""
+    beta = np.longdouble(meas.kb_beta_default(J, 2.0))
+    rng = np.random.default_rng(J)
+    n = 32
+    for fx, fy in [(0.5, 0.25), (1e-6, 1 - 1e-6), (0.999, 0.001)] + [tuple(rng.random(2)) for _ in range(4)]:
+        g = np.array([5 + fx, 9 + fy])
+        uv = (g * (np.pi / n))[None]
+        got = _gridded(n, n, uv, np.array([1.0 + 0j]), J, "f64")
+        g = (uv[0] * 2 * n / (2.0 * np.pi)).astype(np.longdouble)        # as the plan rounds it
+        base = np.floor(g).astype(int)
+        cells = [(base[k] - J // 2 + 1 + np.arange(J)) for k in range(2)]
+        w = [_kb(g[k] - cells[k], J, beta) for k in range(2)]
+        want = np.outer(w[1], w[0])
+        have = got[np.ix_(cells[1] % (2 * n), cells[0] % (2 * n))]
+        assert np.all(have.imag == 0)
+        assert np.max(np.abs(have.real / want - 1)) < 1e-13
