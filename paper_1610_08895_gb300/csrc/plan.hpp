@@ -47,7 +47,9 @@ constexpr int KB_DEG64 = 18;
 // The outermost taps (kb_outer of them on either side) by a polynomial in s = 1 - (2 t / J)^2.
 constexpr int KB_EDGE_MAX = 31;
 __host__ __device__ constexpr int kb_outer(int J) { return J > 8 ? 2 : 1; }
-__host__ __device__ constexpr int kb_edge_deg(int J) { return J > 8 ? KB_EDGE_MAX : 20; }
+__host__ __device__ constexpr int kb_edge_deg(int J) {
+    return J > 8 ? KB_EDGE_MAX : J == 8 ? 19 : J == 6 ? 17 : J == 4 ? 15 : 11;
+}
 struct KbPoly64 {
     double c[8][KB_DEG64 + 1];
     double e[KB_EDGE_MAX + 1];
