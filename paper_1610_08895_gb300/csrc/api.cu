@@ -161,28 +161,10 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     p->csr_cplx = dde > 0;
     g.J = Jfoot;   // tiles, windows and halos follow the footprint; weights use kb_J
     g.beta = d->kb_beta > 0 ? d->kb_beta : kb_beta_default(p->kb_J);
-    // default tile: 16 cells, so that small grids still make enough work items and dense ones
-    // no long ones; 32 for FP32 grids of 2048^2 cells and more, whose items fill the GPU anyway
-    // and then spend less on windows. At least two tiles per grid side, for the tile colours.
-    // Tiles of 8 spread the work of a stored G (real rows) and of the FP64 kernels up to 1024^2
-    // cells best.
-    const bool fly32 = d->precision == PD_F32 && d->g_mode == PD_G_ON_THE_FLY && d->kernel_width <= 8;
-    const int64_t cells = (int64_t)g.Kx * g.Ky;
-    int T = d->tile ? d->tile
-            : fly32 ? (cells >= (int64_t)2048 * 2048 ? 32 : 16)
-            : (d->g_mode == PD_G_CSR && !dde) || (d->g_mode != PD_G_CSR && cells <= (int64_t)1024 * 1024) ? 8 : 16;
-    auto fit = [&](int t) {
-        while (t > std::min(g.Kx, g.Ky) / 2) t >>= 1;
-        while (t < g.J) t <<= 1;
-        return t;
-    };
-    T = fit(T);
-    p->ck_tile = fit(d->tile ? d->tile : 32);
-    if (T > std::min(g.Kx, g.Ky) / 2) return fail(PD_ENOTSUP, "grid side below twice the kernel width");
-    g.tile = T; g.logT = ilog2(T);
-    g.ntx = g.Kx / T; g.nty = g.Ky / T; g.ntiles = g.ntx * g.nty;
-    g.ext = T + g.J - 1;
     const int halo_lo = g.J / 2 - 1;   // footprint cells before the base cell floor(g)
+    int least = 2;
+    while (least < g.J) least <<= 1;
+    if (least > std::min(g.Kx, g.Ky) / 2) return fail(PD_ENOTSUP, "grid side below twice the kernel width");
     p->M = d->nvis; p->d = d->nblocks; p->b = d->nbases; p->L = d->levels;
     p->basis_ids.assign(d->basis_ids, d->basis_ids + d->nbases);
     p->n_wavelet = 0;
@@ -243,6 +225,33 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         frx[m] = fx;
         fry[m] = fy;
     }
+    // default tile: 16 cells, so that small grids still make enough work items and dense ones
+    // no long ones; 32 for FP32 grids of 2048^2 cells and more, whose items fill the GPU anyway
+    // and then spend less on windows. At least two tiles per grid side, for the tile colours.
+    // Tiles of 8 spread the work of the FP64 kernels (real rows of a stored G among them) best up
+    // to 1024^2 cells. A stored G in FP32: see stored_tile.
+    const bool fly32 = d->precision == PD_F32 && d->g_mode == PD_G_ON_THE_FLY && d->kernel_width <= 8;
+    const int64_t cells = (int64_t)g.Kx * g.Ky;
+    auto fit = [&](int t) {
+        while (t > std::min(g.Kx, g.Ky) / 2) t >>= 1;
+        while (t < g.J) t <<= 1;
+        return t;
+    };
+    const bool many = p->d > 1024;     // blocks that could share one large tile: see the limit below
+    int T = d->tile;
+    if (!T && p->g_mode == PD_G_CSR && p->prec == PD_F32) {
+        std::vector<int32_t> cell(M);
+        for (int64_t m = 0; m < M; ++m) cell[m] = (by[m] << 16) | bx[m];
+        T = many ? (dde ? 16 : 8) : stored_tile(cell, g.Kx, g.Ky, p->csr_cplx, p->num_sms);
+    } else if (!T) {
+        T = fly32 ? (cells >= (int64_t)2048 * 2048 ? 32 : 16)
+            : !dde && (cells <= (int64_t)1024 * 1024 || (many && p->g_mode == PD_G_CSR)) ? 8 : 16;
+    }
+    T = fit(T);
+    p->ck_tile = fit(d->tile ? d->tile : 32);
+    g.tile = T; g.logT = ilog2(T);
+    g.ntx = g.Kx / T; g.nty = g.Ky / T; g.ntiles = g.ntx * g.nty;
+    g.ext = T + g.J - 1;
     // a fifth of an SM's share of the points (five CTAs per SM), at least four rounds of a CTA
     const int degrid_part = (int)std::max<int64_t>(1024, M / ((int64_t)p->num_sms * 5));
     const int64_t nbucket = (int64_t)g.ntiles * p->d;

@@ -240,4 +240,46 @@ void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg
     *err = (double)std::max(worst, dropped);   // phi >= 1 on the outer taps
 }
 
+// The gridding of a stored G (four launches by tile colour, one CTA a tile) takes about a + b n
+// for a tile of n points, and a launch lasts as long as its heaviest tile or as the average over the
+// resident CTAs, with some of the shorter of the two on top. Measured on GB300 (J = 8, real rows):
+// a = 4.5, 5 and 7 us for tiles of 8, 16 and 32, b = 0.045, 0.025 and 0.025 us; four CTAs per SM for
+// tiles of 8, two for the others and for complex rows. Larger tiles stage fewer window cells a point, in the
+// degridding too, and win within 5%. Phi^H in tiles of 8 / 16 / 32: 262,144 points on 512^2 cells
+// 154 / 294 / 839 us, 1.05M on 1024^2 239 / 211 / 541, 4.19M Gaussian on 2048^2 776 / 728 / 1340,
+// 16.8M on 4096^2 3057 / 2794 / 2350, 1.05M there 1685 / 1100 / 554.
+int stored_tile(const std::vector<int32_t>& cell, int Kx, int Ky, bool cplx, int num_sms) {
+    std::vector<int32_t> n((size_t)(Kx / 8) * (Ky / 8), 0);
+    for (int32_t c : cell) n[(size_t)(c >> 19) * (Kx / 8) + ((c & 0xFFFF) >> 3)]++;
+    const double a[3] = {cplx ? 5.2 : 4.5, 5.0, 7.0};
+    const double b[3] = {cplx ? 0.028 : 0.045, cplx ? 0.028 : 0.025, cplx ? 0.028 : 0.025};
+    double best = 0.0;
+    int tile = 8, w = Kx / 8, h = Ky / 8;
+    for (int k = 0; k < 3; ++k) {
+        if (k > 0) {                       // the counts of tiles twice as large
+            if (w < 4 || h < 4) break;     // two tiles a side at least
+            for (int y = 0; y < h / 2; ++y)
+                for (int x = 0; x < w / 2; ++x) {
+                    const size_t q = (size_t)2 * y * w + 2 * x;
+                    n[(size_t)y * (w / 2) + x] = n[q] + n[q + 1] + n[q + w] + n[q + w + 1];
+                }
+            w /= 2;
+            h /= 2;
+        }
+        int most = 0, used = 0;
+        for (size_t i = 0; i < (size_t)w * h; ++i) {
+            most = std::max(most, n[i]);
+            used += n[i] > 0;
+        }
+        const double ctas = (double)num_sms * (k == 0 && !cplx ? 4 : 2);
+        const double heavy = a[k] + b[k] * most, mean = (used * a[k] + b[k] * (double)cell.size()) / (4.0 * ctas);
+        const double t = std::max(heavy, mean) + 0.4 * std::min(heavy, mean);
+        if (k == 0 || t <= 1.05 * best) {
+            best = k == 0 ? t : std::min(best, t);
+            tile = 8 << k;
+        }
+    }
+    return tile;
+}
+
 }  // namespace pdgb

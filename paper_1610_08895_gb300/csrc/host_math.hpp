@@ -1,6 +1,7 @@
 // Host-side FP64 tables of the plan (filters, deapodisation, twiddles).
 #pragma once
 
+#include <cstdint>
 #include <vector>
 
 namespace pdgb {
@@ -24,5 +25,9 @@ std::vector<double> kb_tap_polynomials(int J, double beta, int deg);
 // fitted, beta too large).
 void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg, std::vector<double>& inner,
                             std::vector<double>& edge, double* err);
+
+// Tile edge (8, 16 or 32) for a stored G in FP32, from where the points' footprints start: cell as
+// (y << 16) | x on a Kx x Ky grid. cplx: complex rows.
+int stored_tile(const std::vector<int32_t>& cell, int Kx, int Ky, bool cplx, int num_sms);
 
 }  // namespace pdgb

@@ -1,0 +1,44 @@
+"""Which kernel variant a call takes: default tiles of a stored G, batches, items with few points."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_util import rel  # noqa: E402
+from paper_1610_08895_gb300 import synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import __graft_entry__ as ge
+    ge.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+
+
+def _uv(kind, m):
+    if kind == "uniform":
+        return np.random.default_rng(3).uniform(-np.pi, np.pi, size=(m, 2))
+    return synth.uv_gaussian(m, seed=1) if kind == "gaussian" else synth.uv_radial(m, seed=1)
+
+
+@pytest.mark.parametrize("n,m,kind,d,dde,tile", [
+    (128, 60000, "gaussian", 4, False, 8), (1024, 200000, "uniform", 1, False, 32), (1024, 200000, "radial", 1, True, 32),
+    (256, 30000, "radial", 1, True, 16), (1024, 60000, "uniform", 1500, False, 8)])
+def test_default_tile_of_a_stored_g_follows_the_points(n, m, kind, d, dde, tile):
+    """Large where tiles hold few points, small where the heaviest tile would be all a launch waits for, and
+    where so many blocks could share a large one that the plan would be refused; the same operator either way."""
+    from paper_1610_08895_gb300.api import Plan
+    uv = _uv(kind, m)
+    kw = dict(kernel_width=4, g_mode="csr")
+    if dde:
+        kw["dde_kernels"] = np.random.default_rng(5).normal(size=(m, 3, 3)) + 0j
+    blk = (np.arange(m) % d).astype(np.int32)
+    plan = Plan(n, n, uv, blk, d, **kw)
+    assert plan.info()["tile"] == tile
+    other = Plan(n, n, uv, blk, d, tile=16, **kw) if d <= 1024 else plan
+    x = torch.tensor(synth.random_images(1, n, n, seed=3)[0], dtype=torch.float32, device="cuda")
+    y = plan.pd_apply_phi(x)
+    assert rel(other.pd_apply_phi(x).cpu().numpy(), y.cpu().numpy()) < 2e-6
+    assert rel(other.pd_apply_phi_adj(y).cpu().numpy(), plan.pd_apply_phi_adj(y).cpu().numpy()) < 2e-6
