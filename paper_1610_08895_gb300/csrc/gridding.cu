@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 4 : 3) : 1) k_
     const int E = g.ext, T = g.tile;
     const int warp = threadIdx.x >> 5;
     const int n = *nitems;
-    if (threadIdx.x == 0) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
+    if (threadIdx.x == 0) item_s = claim_item<false>(sched, items, n, batch, tile_on, &ti_s);
     for (;;) {
         __syncthreads();
         const int w = item_s;
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(256, J <= 8 ? (sizeof(R) == 4 ? 4 : 3) : 1) k_
             if (MODE == 1) warp_seg_add(ok, jcur, ar, ad, mypart);
         }
         __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
+        if (threadIdx.x == blockDim.x - 1) item_s = claim_item<false>(sched, items, n, batch, tile_on, &ti_s);
         if (MODE == 1) {
             for (int k = threadIdx.x; k < nact; k += blockDim.x) {
                 double sr = 0.0, sd = 0.0;
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
     const int n = *count;
     for (;;) {
         // tiles are taken from the heaviest-first list one at a time by whichever CTA is free
-        if (threadIdx.x == 0) tile_s = claim_tile(next_tile, list, n, batch, tile_on);
+        if (threadIdx.x == 0) tile_s = claim_tile<false>(next_tile, list, n, batch, tile_on);
         __syncthreads();
         const int w = tile_s;
         if (w >= n * batch) break;

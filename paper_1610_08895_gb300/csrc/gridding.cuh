@@ -169,26 +169,30 @@ __device__ __forceinline__ void add_window(cplx_t<R>* __restrict__ U, int oy, in
 
 // Thread 0: the next item (claimed in order by whichever CTA is free) whose tile is on, into
 // *it; its number w is returned (>= n * batch: none left). A batch goes image by image (image
-// w / n): the visibilities are read or written in user order, at random, and one image's stay
-// in the L2 cache meanwhile (phi_1024_batch8 of perf/cases.py: 3.20 ms with the images
-// of a tile one after the other, 2.63 ms so).
+// w / n) where G is evaluated: the visibilities are read or written in user order, at random, and
+// one image's stay in the L2 cache meanwhile (eight images of 1024^2, 4.19M points each: Phi 1405 ->
+// 837 us). Where G is stored the images of an item follow one another (image w % batch): its rows
+// come from HBM once for all of them (four images of 512^2, 524,288 points, complex rows: Phi^H 467
+// us, image by image 512).
+template <bool STORED>
 __device__ __forceinline__ int claim_item(int* sched, const TileItem* __restrict__ items, int n, int batch,
                                           const int32_t* __restrict__ tile_on, TileItem* it) {
     for (;;) {
         const int w = atomicAdd(sched, 1);
         if (w >= n * batch) return w;
-        const TileItem t = items[w % n];
+        const TileItem t = items[STORED ? w / batch : w % n];
         if (tile_on && !tile_on[t.tile]) continue;
         *it = t;
         return w;
     }
 }
 // The same over a list of tiles.
+template <bool STORED>
 __device__ __forceinline__ int claim_tile(int* next, const int32_t* __restrict__ list, int n, int batch,
                                           const int32_t* __restrict__ tile_on) {
     for (;;) {
         const int w = atomicAdd(next, 1);
-        if (w >= n * batch || !tile_on || tile_on[list[w % n]]) return w;
+        if (w >= n * batch || !tile_on || tile_on[list[STORED ? w / batch : w % n]]) return w;
     }
 }
 // Thread 0 of each CTA at the end: the last one sets the counters back for the next launch on the

@@ -205,13 +205,13 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
     const int warp = threadIdx.x >> 5, grp = threadIdx.x / GL, b = threadIdx.x % GL;
     const int ngrp = blockDim.x / GL;
     const int n = *nitems;
-    if (threadIdx.x == 0) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
+    if (threadIdx.x == 0) item_s = claim_item<true>(sched, items, n, batch, tile_on, &ti_s);
     for (;;) {
         __syncthreads();
         const int w = item_s;
         if (w >= n * batch) break;
         const TileItem ti = ti_s;
-        const int t = ti.tile, img = w / n;
+        const int t = ti.tile, img = w % batch;
         const C2* gimg = grid + (int64_t)img * gstride;
         C2* oimg = MODE == 0 ? out + (int64_t)img * ostride : out;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(256) k_degrid_csr(
             if (MODE == 1) warp_seg_add(lead, j, ar, ad, mypart);
         }
         __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) item_s = claim_item(sched, items, n, batch, tile_on, &ti_s);
+        if (threadIdx.x == blockDim.x - 1) item_s = claim_item<true>(sched, items, n, batch, tile_on, &ti_s);
         if (MODE == 1) {
             for (int k = threadIdx.x; k < nact; k += blockDim.x) {
                 double sr = 0.0, sd = 0.0;
@@ -399,11 +399,11 @@ __global__ void __launch_bounds__(256, PB == 4 ? 4 : 2) k_grid_csr(
     const int e0 = 2 * lane;
     const bool has = e0 < NE;                 // J^2 is even: entries e0, e0 + 1 together
     for (;;) {
-        if (threadIdx.x == 0) tile_s = claim_tile(next_tile, list, n, batch, tile_on);
+        if (threadIdx.x == 0) tile_s = claim_tile<true>(next_tile, list, n, batch, tile_on);
         __syncthreads();
         const int w = tile_s;
         if (w >= n * batch) break;
-        const int t = list[w % n], img = w / n;
+        const int t = list[w / batch], img = w % batch;
         const C2* simg = MODE == 0 ? src + (int64_t)img * sstride : src;
         C2* uimg = U + (int64_t)img * ustride;
         const int ty = t / g.ntx, tx = t - ty * g.ntx;

@@ -42,3 +42,25 @@ def test_default_tile_of_a_stored_g_follows_the_points(n, m, kind, d, dde, tile)
     y = plan.pd_apply_phi(x)
     assert rel(other.pd_apply_phi(x).cpu().numpy(), y.cpu().numpy()) < 2e-6
     assert rel(other.pd_apply_phi_adj(y).cpu().numpy(), plan.pd_apply_phi_adj(y).cpu().numpy()) < 2e-6
+
+
+@pytest.mark.parametrize("n,m,b,kw", [
+    (256, 65536, 8, dict()), (64, 5000, 3, dict(kernel_width=6)), (64, 3000, 2, dict(kernel_width=12)),
+    (64, 5000, 3, dict(precision="f64")), (64, 5000, 3, dict(g_mode="csr")), (128, 9001, 5, dict(g_mode="csr", precision="f64")),
+    (64, 5000, 4, dict(g_mode="csr", kernel_width=6, dde=True))])
+def test_a_batch_is_its_images_one_by_one(n, m, b, kw):
+    from paper_1610_08895_gb300.api import Plan
+    kw = dict(kw)
+    if kw.pop("dde", False):
+        kw["dde_kernels"] = np.random.default_rng(5).normal(size=(m, 3, 3)) + 0j
+    plan = Plan(n, n, _uv("gaussian", m), np.zeros(m, np.int32), 1, **kw)
+    x = torch.tensor(synth.random_images(b, n, n, seed=3), dtype=plan.real_dtype, device="cuda")
+    v = torch.tensor(np.stack([synth.uniform_vis(m, seed=k) for k in range(b)]), dtype=plan.cplx_dtype, device="cuda")
+    y, xa = plan.pd_apply_phi(x), plan.pd_apply_phi_adj(v)
+    for k in range(b):
+        assert torch.equal(y[k], plan.pd_apply_phi(x[k].contiguous()))
+        one = plan.pd_apply_phi_adj(v[k].contiguous())
+        if kw.get("kernel_width", 8) <= 8:
+            assert torch.equal(xa[k], one)
+        else:                                   # wider kernels add through shared-memory atomics
+            assert rel(xa[k].cpu().numpy(), one.cpu().numpy()) < 2e-6
