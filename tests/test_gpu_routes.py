@@ -64,3 +64,24 @@ def test_a_batch_is_its_images_one_by_one(n, m, b, kw):
             assert torch.equal(xa[k], one)
         else:                                   # wider kernels add through shared-memory atomics
             assert rel(xa[k].cpu().numpy(), one.cpu().numpy()) < 2e-6
+
+
+@pytest.mark.parametrize("J", [8, 12])
+def test_residual_norms_where_items_hold_few_points(J):
+    """2,000 items of some 50 points, worked on by smaller blocks, with many blocks of data to an item."""
+    from oracle import measurement as meas
+    from paper_1610_08895_gb300.api import Plan, State
+    n, m, d = 512, 100001, 37
+    uv = _uv("uniform", m)
+    blk = (np.arange(m) % d).astype(np.int32)
+    plan = Plan(n, n, uv, blk, d, kernel_width=J)
+    x = synth.random_images(1, n, n, seed=3)[0]
+    y = synth.uniform_vis(m, seed=4)
+    want = meas.Geometry(n, n, J).phi(x, uv)
+    xt = torch.tensor(x, dtype=torch.float32, device="cuda")
+    assert rel(plan.pd_apply_phi(xt).cpu().numpy(), want) < 1e-5
+    st = State(plan)
+    st.pd_state_set_data(torch.tensor(y, dtype=torch.complex64, device="cuda"), np.ones(d))
+    st.pd_state_set_start(x0=xt)
+    norms = np.sqrt(np.bincount(blk, weights=np.abs(want - y) ** 2, minlength=d))
+    assert np.max(np.abs(st.report()["res_norm"] / norms - 1)) < 1e-5
