@@ -92,6 +92,7 @@ static void free_all(std::vector<void*>& list) {
 extern "C" pd_status pd_plan_destroy(pd_plan* p) {
     if (!p) return PD_OK;
     free_all(p->allocs);
+    if (p->ck_list) cudaFree(p->ck_list);
     delete p;
     return PD_OK;
 }
@@ -175,53 +176,40 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
 
     // ---- visibilities: first footprint cell, fraction, (tile, block) order
     const int64_t M = p->M;
-    std::vector<int32_t> bx(M), by(M);
+    std::vector<int32_t> cell(M);          // the footprint's first cell, halo_lo cells before the base cell
     std::vector<double> frx(M), fry(M);
     std::vector<unsigned char> flip(M, 0);
-    // integer part and fraction; a fraction that rounds to 1 in the working precision moves to
-    // the next cell
-    auto split = [&](double x, double& fl, double& fr) {
-        fl = std::floor(x);
-        fr = x - fl;
-        if (p->prec == PD_F32 && (float)fr >= 1.0f) { fl += 1.0; fr = 0.0; }
-    };
-    auto base_cell = [&](double x, double y) {
-        double flx, fly, fr;
-        split(x, flx, fr);
-        split(y, fly, fr);
-        return (int32_t)(((((int64_t)fly % g.Ky) + g.Ky) % g.Ky) << 16 | ((((int64_t)flx % g.Kx) + g.Kx) % g.Kx));
-    };
-    // neither fraction x nor its mirror image 1 - x rounds to a grid line
-    auto inside = [&](double x) {
-        const double fr = x - std::floor(x);
-        return p->prec == PD_F32 ? (float)fr > 0.0f && (float)fr < 1.0f && (float)(1.0 - fr) < 1.0f
-                                 : fr > 0.0 && fr < 1.0 && 1.0 - fr < 1.0;
-    };
-    p->h_base.resize(M);
+    const bool f32 = p->prec == PD_F32, fold = p->g_mode == PD_G_ON_THE_FLY;
     for (int64_t m = 0; m < M; ++m) {
         const double u = d->uv[2 * m], v = d->uv[2 * m + 1];
         if (!(u >= -M_PI && u < M_PI && v >= -M_PI && v < M_PI))
             return fail(PD_EINVAL, "uv points must lie in [-pi, pi)^2");
         const int blk = d->block_of_vis[m];
         if (blk < 0 || blk >= p->d) return fail(PD_EINVAL, "block_of_vis out of range");
-        double gxv = u * g.Kx / (2.0 * M_PI), gyv = v * g.Ky / (2.0 * M_PI);
-        p->h_base[m] = base_cell(gxv, gyv);
+        const double gx = u * g.Kx / (2.0 * M_PI), gy = v * g.Ky / (2.0 * M_PI);
+        double flx = std::floor(gx), fly = std::floor(gy), fx = gx - flx, fy = gy - fly;
         // Held at -(u, v) as its conjugate, where G is evaluated in the kernels (a stored G gains
-        // nothing: its rows are read all the same). A point on a grid line (to the working precision)
-        // stays where it is: its taps reach J/2 cells to one side only, and the mirrored ones
-        // would to the other.
-        if (p->g_mode == PD_G_ON_THE_FLY && u < 0 && inside(gxv) && inside(gyv)) {
-            gxv = -gxv;
-            gyv = -gyv;
-            flip[m] = 1;
-            p->folded = true;
+        // nothing: its rows are read all the same). A point on a grid line (a fraction or its mirror
+        // image rounds to one in the working precision) stays where it is: its taps reach J/2 cells
+        // to one side only, and the mirrored ones would to the other.
+        if (fold && u < 0) {
+            const double rx = std::ceil(gx) - gx, ry = std::ceil(gy) - gy;
+            const bool in = f32 ? (float)fx > 0.0f && (float)fx < 1.0f && (float)(1.0 - fx) < 1.0f &&
+                                      (float)fy > 0.0f && (float)fy < 1.0f && (float)(1.0 - fy) < 1.0f
+                                : fx > 0.0 && 1.0 - fx < 1.0 && fy > 0.0 && 1.0 - fy < 1.0;
+            if (in) {
+                flx = -std::ceil(gx);
+                fly = -std::ceil(gy);
+                fx = rx;
+                fy = ry;
+                flip[m] = 1;
+                p->folded = true;
+            }
         }
-        double flx, fly, fx, fy;
-        split(gxv, flx, fx);
-        split(gyv, fly, fy);
-        // the footprint's first cell, halo_lo cells before the base cell
-        bx[m] = (int32_t)((((int64_t)flx - halo_lo) % g.Kx + g.Kx) % g.Kx);
-        by[m] = (int32_t)((((int64_t)fly - halo_lo) % g.Ky + g.Ky) % g.Ky);
+        // a fraction that rounds to 1 in the working precision moves to the next cell
+        if (f32 && (float)fx >= 1.0f) { flx += 1.0; fx = 0.0; }
+        if (f32 && (float)fy >= 1.0f) { fly += 1.0; fy = 0.0; }
+        cell[m] = (((int32_t)fly - halo_lo) & (g.Ky - 1)) << 16 | (((int32_t)flx - halo_lo) & (g.Kx - 1));
         frx[m] = fx;
         fry[m] = fy;
     }
@@ -240,8 +228,6 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     const bool many = p->d > 1024;     // blocks that could share one large tile: see the limit below
     int T = d->tile;
     if (!T && p->g_mode == PD_G_CSR && p->prec == PD_F32) {
-        std::vector<int32_t> cell(M);
-        for (int64_t m = 0; m < M; ++m) cell[m] = (by[m] << 16) | bx[m];
         T = many ? (dde ? 16 : 8) : stored_tile(cell, g.Kx, g.Ky, p->csr_cplx, p->num_sms);
     } else if (!T) {
         T = fly32 ? (cells >= (int64_t)2048 * 2048 ? 32 : 16)
@@ -254,37 +240,11 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     g.ext = T + g.J - 1;
     // a fifth of an SM's share of the points (five CTAs per SM), at least four rounds of a CTA
     const int degrid_part = (int)std::max<int64_t>(1024, M / ((int64_t)p->num_sms * 5));
-    const int64_t nbucket = (int64_t)g.ntiles * p->d;
-    std::vector<int32_t> order(M);
+    PointOrder po = order_points(cell, d->block_of_vis, p->d, g.logT, g.ntx, g.ntiles);
+    std::vector<int32_t>& order = po.order;
     {
-        std::vector<int64_t> key(M);
-        for (int64_t m = 0; m < M; ++m) {
-            const int t = (by[m] >> g.logT) * g.ntx + (bx[m] >> g.logT);
-            key[m] = (int64_t)t * p->d + d->block_of_vis[m];
-        }
-        if (nbucket <= (int64_t)1 << 25) {
-            std::vector<int64_t> cnt(nbucket + 1, 0);
-            for (int64_t m = 0; m < M; ++m) cnt[key[m] + 1]++;
-            for (int64_t k = 0; k < nbucket; ++k) cnt[k + 1] += cnt[k];
-            for (int64_t m = 0; m < M; ++m) order[cnt[key[m]]++] = (int32_t)m;
-        } else {
-            std::iota(order.begin(), order.end(), 0);
-            std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b2) { return key[a] < key[b2]; });
-        }
-        // segments = runs of equal (tile, block)
-        std::vector<int32_t> seg_start, seg_block, seg_tile;
-        int64_t prev = -1;
-        for (int64_t i = 0; i < M; ++i) {
-            const int64_t k = key[order[i]];
-            if (k != prev) {
-                seg_start.push_back((int32_t)i);
-                seg_block.push_back((int32_t)(k % p->d));
-                seg_tile.push_back((int32_t)(k / p->d));
-                prev = k;
-            }
-        }
+        const std::vector<int32_t>&seg_start = po.seg_start, &seg_block = po.seg_block, &seg_tile = po.seg_tile;
         p->nseg = (int64_t)seg_block.size();
-        seg_start.push_back((int32_t)M);
         std::vector<int32_t> tile_seg_start(g.ntiles + 1, 0);
         {
             int64_t s = 0;
@@ -298,29 +258,20 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
             p->max_tile_segs = std::max(p->max_tile_segs, tile_seg_start[t + 1] - tile_seg_start[t]);
         if (p->max_tile_segs > 1024)
             return fail(PD_ENOTSUP, "more than 1024 blocks share one gridding tile; use a smaller tile");
-        // within each segment: by 8 x 8 super-cell, then row-major by cell (stable: ties
-        // keep user order), so that the points of one super-cell row are consecutive
+        // the points of each segment are by 8 x 8 super-cell: where each one's start (the gridding's
+        // per-warp ranges)
         p->nsc_side = std::max(1, g.tile / SC);
-        auto scell_of = [&](int32_t m) {
-            const int ly = by[m] & (g.tile - 1), lx = bx[m] & (g.tile - 1);
-            return (ly / SC) * p->nsc_side + lx / SC;
-        };
         const int nsc = p->nsc_side * p->nsc_side;
         std::vector<int32_t> sc_start((size_t)p->nseg * (nsc + 1));
         for (int64_t sg = 0; sg < p->nseg; ++sg) {
-            std::stable_sort(order.begin() + seg_start[sg], order.begin() + seg_start[sg + 1],
-                             [&](int32_t a, int32_t b2) {
-                                 const int sa = scell_of(a), sb = scell_of(b2);
-                                 if (sa != sb) return sa < sb;
-                                 return (by[a] != by[b2]) ? by[a] < by[b2] : bx[a] < bx[b2];
-                             });
-            // start of each super-cell's points inside the segment (the gridding's per-warp ranges)
             int32_t* o = &sc_start[(size_t)sg * (nsc + 1)];
-            int i = seg_start[sg];
-            for (int k = 0; k <= nsc; ++k) {
-                while (i < seg_start[sg + 1] && scell_of(order[i]) < k) ++i;
-                o[k] = i;
+            int k = 0;
+            for (int32_t i = seg_start[sg]; i < seg_start[sg + 1]; ++i) {
+                const int32_t c = cell[order[i]];
+                const int sc = (((c >> 16) & (g.tile - 1)) / SC) * p->nsc_side + (c & (g.tile - 1)) / SC;
+                while (k <= sc) o[k++] = i;
             }
+            while (k <= nsc) o[k++] = seg_start[sg + 1];
         }
         p->h_sc_start = std::move(sc_start);
         // tiles by decreasing visibility count (heaviest scheduled first)
@@ -425,14 +376,18 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     auto& A = p->allocs;
     size_t& B = p->device_bytes;
     {
-        std::vector<int32_t> cell(M);
-        std::vector<double> fxs(M), fys(M);
-        for (int64_t i = 0; i < M; ++i) {
-            const int32_t m = order[i];
-            cell[i] = (by[m] << 16) | bx[m];
-            fxs[i] = frx[m];
-            fys[i] = fry[m];
-        }
+        std::vector<int32_t> sorted(M);
+        for (int64_t i = 0; i < M; ++i) sorted[i] = cell[order[i]];
+        auto put = [&](void* dst, const std::vector<double>& fr) {
+            if (!f32) {
+                std::vector<double> o(M);
+                for (int64_t i = 0; i < M; ++i) o[i] = fr[order[i]];
+                return upload((double*)dst, o);
+            }
+            std::vector<float> o(M);
+            for (int64_t i = 0; i < M; ++i) o[i] = (float)fr[order[i]];
+            return upload((float*)dst, o);
+        };
         if (dde) {   // DDE kernels in internal order, for the CSR build below
             const size_t per = (size_t)2 * dde * dde;
             p->h_dde.resize((size_t)M * per);
@@ -444,12 +399,12 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
         ALLOC(p->perm, M);
         CU(dalloc_bytes(A, B, &p->fx, M * p->rsz));
         CU(dalloc_bytes(A, B, &p->fy, M * p->rsz));
-        CU(upload(p->cell, cell));
+        CU(upload(p->cell, sorted));
+        CU(put(p->fx, frx));
+        CU(put(p->fy, fry));
         for (int64_t i = 0; i < M; ++i)
             if (flip[order[i]]) order[i] = (int32_t)((uint32_t)order[i] | 0x80000000u);
         CU(upload(p->perm, order));
-        CU(upload_real(p->fx, fxs, p->prec));
-        CU(upload_real(p->fy, fys, p->prec));
     }
     {
         std::vector<int32_t> counts = {(int32_t)p->nseg, p->ntiles_nonempty, p->n_ditems};
@@ -1392,36 +1347,40 @@ static std::vector<Part> state_parts(const pd_plan* p, const pd_state* st) {
             {st->res_norm, p->d * sizeof(double), false}, {st->p_block, p->d * sizeof(double), false},
             {st->p_basis, p->b * sizeof(double), false}, {st->t, sizeof(int64_t), false}};
 }
-// The plan's ck_order, made on first use; any thread may ask.
+// The order of the visibilities in checkpoints, made on first use; any thread may ask.
 static pd_status ensure_ck(pd_plan* p) {
     std::lock_guard<std::mutex> lock(p->ck_mu);
-    if (!p->ck_order.empty()) return PD_OK;
+    if (p->ck_ready) return PD_OK;
     const int64_t M = p->M;
-    std::vector<int32_t> perm(M), seg(p->nseg + 1);
+    const Geo& g = p->g;
+    std::vector<int32_t> perm(M), cell(M), seg(p->nseg + 1), base(M), block(M), at(M);
     CU(cudaMemcpy(perm.data(), p->perm, M * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(cell.data(), p->cell, M * sizeof(int32_t), cudaMemcpyDeviceToHost));
     CU(cudaMemcpy(seg.data(), p->seg_start, (p->nseg + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost));
-    struct Key {
-        int64_t bucket;       // tile, block
-        int64_t in;           // super-cell, row, column
-        int32_t user, at;
-    };
-    std::vector<Key> key(M);
-    const int T = p->ck_tile, logT = ilog2(T), ntx = p->g.Kx / T, side = std::max(1, T / SC);
+    const int halo = g.J / 2 - 1;
     for (int64_t sg = 0; sg < p->nseg; ++sg)
         for (int32_t i = seg[sg]; i < seg[sg + 1]; ++i) {
-            const int32_t m = vis_index(perm[i]), c = p->h_base[m], by = c >> 16, bx = c & 0xFFFF;
-            const int ly = by & (T - 1), lx = bx & (T - 1);
-            key[i] = Key{((int64_t)(by >> logT) * ntx + (bx >> logT)) * p->d + p->h_seg_block[sg],
-                         (((int64_t)(ly / SC) * side + lx / SC) << 32) | c, m,
-                         (int32_t)((uint32_t)i | ((uint32_t)perm[i] & 0x80000000u))};
+            const int32_t m = vis_index(perm[i]);
+            int32_t by = (cell[i] >> 16) + halo, bx = (cell[i] & 0xFFFF) + halo;    // floor(g)
+            if (perm[i] < 0) { by = -1 - by; bx = -1 - bx; }                         // held at -g
+            base[m] = (by & (g.Ky - 1)) << 16 | (bx & (g.Kx - 1));
+            block[m] = p->h_seg_block[sg];
+            at[m] = (int32_t)((uint32_t)i | ((uint32_t)perm[i] & 0x80000000u));
         }
-    std::sort(key.begin(), key.end(), [](const Key& a, const Key& b) {
-        if (a.bucket != b.bucket) return a.bucket < b.bucket;
-        return a.in != b.in ? a.in < b.in : a.user < b.user;
-    });
-    std::vector<int32_t> out(M);
-    for (int64_t i = 0; i < M; ++i) out[i] = key[i].at;
-    p->ck_order = std::move(out);
+    const int T = p->ck_tile, ntx = g.Kx / T;
+    std::vector<int32_t> order = order_points(base, block.data(), p->d, ilog2(T), ntx, ntx * (g.Ky / T)).order;
+    for (int32_t& k : order) k = at[k];
+    // on the device if there is room, else each checkpoint brings it along piece by piece
+    if (cudaMalloc((void**)&p->ck_list, M * sizeof(int32_t)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        p->ck_list = nullptr;
+        p->ck_order = std::move(order);
+    } else if (cudaError_t e = upload(p->ck_list, order)) {
+        cudaFree(p->ck_list);
+        p->ck_list = nullptr;
+        CU(e);
+    }
+    p->ck_ready = true;
     return PD_OK;
 }
 // One array of visibilities out of or into a checkpoint, piece by piece through the state's staging.
@@ -1432,15 +1391,19 @@ static cudaError_t copy_vis(const pd_state* st, void* dev, unsigned char* host, 
     cudaError_t e;
     for (int64_t i = 0; i < p->M; i += st->ck_cap) {
         const int64_t n = std::min(st->ck_cap, p->M - i);
-        if ((e = cudaMemcpyAsync(st->ck_idx, p->ck_order.data() + i, n * sizeof(int32_t), cudaMemcpyHostToDevice, s)))
-            return e;
+        const int32_t* idx = p->ck_list + i;
+        if (!p->ck_list) {
+            idx = st->ck_idx;
+            if ((e = cudaMemcpyAsync(st->ck_idx, p->ck_order.data() + i, n * sizeof(int32_t), cudaMemcpyHostToDevice, s)))
+                return e;
+        }
         if (save) {
-            if ((e = gather_by<R>(n, st->ck_idx, (const C*)dev, (C*)st->ck_vis, s)) ||
+            if ((e = gather_by<R>(n, idx, (const C*)dev, (C*)st->ck_vis, s)) ||
                 (e = cudaMemcpyAsync(host + i * sizeof(C), st->ck_vis, n * sizeof(C), cudaMemcpyDeviceToHost, s)))
                 return e;
         } else {
             if ((e = cudaMemcpyAsync(st->ck_vis, host + i * sizeof(C), n * sizeof(C), cudaMemcpyHostToDevice, s)) ||
-                (e = scatter_by<R>(n, st->ck_idx, (const C*)st->ck_vis, (C*)dev, s)))
+                (e = scatter_by<R>(n, idx, (const C*)st->ck_vis, (C*)dev, s)))
                 return e;
         }
     }

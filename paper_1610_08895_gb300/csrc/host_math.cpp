@@ -282,4 +282,70 @@ int stored_tile(const std::vector<int32_t>& cell, int Kx, int Ky, bool cplx, int
     return tile;
 }
 
+// Stable counting sort of `in` (or 0 .. n - 1) by key(i) in [0, nkeys).
+template <typename Key>
+static std::vector<int32_t> counting_sort(size_t n, const std::vector<int32_t>* in, int64_t nkeys, const Key& key) {
+    std::vector<int32_t> at(nkeys + 1, 0), out(n);
+    for (size_t i = 0; i < n; ++i) at[key((int32_t)i) + 1]++;
+    for (int64_t k = 0; k < nkeys; ++k) at[k + 1] += at[k];
+    for (size_t i = 0; i < n; ++i) {
+        const int32_t m = in ? (*in)[i] : (int32_t)i;
+        out[at[key(m)]++] = m;
+    }
+    return out;
+}
+
+PointOrder order_points(const std::vector<int32_t>& cell, const int32_t* block, int nblocks, int logT, int ntx,
+                        int ntiles) {
+    const size_t n = cell.size();
+    const int T = 1 << logT, side = std::max(1, T / 8);
+    auto tile_of = [&](int32_t m) { return (cell[m] >> (16 + logT)) * ntx + ((cell[m] & 0xFFFF) >> logT); };
+    PointOrder o;
+    // one pass over (tile, block) while its counters stay in reach of the caches, else one over the
+    // blocks and one over the tiles
+    if ((int64_t)ntiles * nblocks <= (int64_t)1 << 25) {
+        o.order = counting_sort(n, nullptr, (int64_t)ntiles * nblocks,
+                                [&](int32_t m) { return (int64_t)tile_of(m) * nblocks + block[m]; });
+    } else {
+        const std::vector<int32_t> by_block = counting_sort(n, nullptr, nblocks, [&](int32_t m) { return block[m]; });
+        o.order = counting_sort(n, &by_block, ntiles, tile_of);
+    }
+    int ptile = -1, pblock = -1;
+    for (size_t i = 0; i < n; ++i) {
+        const int32_t m = o.order[i], t = tile_of(m);
+        if (t != ptile || block[m] != pblock) {
+            o.seg_start.push_back((int32_t)i);
+            o.seg_tile.push_back(ptile = t);
+            o.seg_block.push_back(pblock = block[m]);
+        }
+    }
+    o.seg_start.push_back((int32_t)n);
+    // within a segment: its points are in the order of their indices, so that a stable counting sort
+    // over the tile's cells, or a sort of (cell, index) where the points are fewer, leaves ties so
+    auto place = [&](int32_t m) {
+        const int ly = (cell[m] >> 16) & (T - 1), lx = cell[m] & (T - 1);
+        return ((uint64_t)((ly >> 3) * side + (lx >> 3)) << 6) | ((ly & 7) << 3) | (lx & 7);
+    };
+    const size_t places = (size_t)side * side << 6;
+    std::vector<uint64_t> key;
+    std::vector<int32_t> at, tmp;
+    for (size_t sg = 0; sg + 1 < o.seg_start.size(); ++sg) {
+        int32_t* p = o.order.data() + o.seg_start[sg];
+        const size_t len = o.seg_start[sg + 1] - o.seg_start[sg];
+        if (len > places / 4) {
+            at.assign(places + 1, 0);
+            tmp.assign(p, p + len);
+            for (int32_t m : tmp) at[place(m) + 1]++;
+            for (size_t k = 0; k < places; ++k) at[k + 1] += at[k];
+            for (int32_t m : tmp) p[at[place(m)]++] = m;
+        } else {
+            key.resize(len);
+            for (size_t i = 0; i < len; ++i) key[i] = place(p[i]) << 31 | (uint32_t)p[i];
+            std::sort(key.begin(), key.end());
+            for (size_t i = 0; i < len; ++i) p[i] = (int32_t)(key[i] & 0x7fffffffu);
+        }
+    }
+    return o;
+}
+
 }  // namespace pdgb

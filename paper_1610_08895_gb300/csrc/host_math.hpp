@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstdint>
 #include <vector>
 
 namespace pdgb {
@@ -29,5 +30,15 @@ void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg
 // Tile edge (8, 16 or 32) for a stored G in FP32, from where the points' footprints start: cell as
 // (y << 16) | x on a Kx x Ky grid. cplx: complex rows.
 int stored_tile(const std::vector<int32_t>& cell, int Kx, int Ky, bool cplx, int num_sms);
+
+// Points by (tile, block), then 8 x 8 super-cell, row, column and index. cell: (y << 16) | x, in
+// tiles of 2^logT cells, ntx of them in a row. Segments are the runs of one (tile, block).
+struct PointOrder {
+    std::vector<int32_t> order;           // [n] indices of the points
+    std::vector<int32_t> seg_start;       // [segments + 1]
+    std::vector<int32_t> seg_block, seg_tile;
+};
+PointOrder order_points(const std::vector<int32_t>& cell, const int32_t* block, int nblocks, int logT, int ntx,
+                        int ntiles);
 
 }  // namespace pdgb

@@ -108,12 +108,15 @@ struct pd_plan {
     // host copies of the static tables
     std::vector<int32_t> h_tile_seg_start, h_seg_block;
 
-    // checkpoints keep the visibilities in the order of their own tiles and base cells, whatever
-    // the plan's internal order is: host list of the internal index of each (sign bit: held
-    // as a conjugate), made by the first save or load under the lock and only read after that
-    std::vector<int32_t> h_base;   // base cell (by << 16 | bx) of each point, user order
+    // checkpoints keep the visibilities in the order of their base cells in tiles of ck_tile cells,
+    // whatever the plan's internal order is: list of the internal index of each (sign bit: held as a
+    // conjugate), made by the first save or load under the lock and only read after that; on the
+    // device (outside of allocs, which only calls that are ordered on the plan may touch), or on the
+    // host if there was no room
     int ck_tile = 0;
     std::mutex ck_mu;
+    bool ck_ready = false;
+    int32_t* ck_list = nullptr;
     std::vector<int32_t> ck_order;
     bool folded = false;           // some visibility is held as its conjugate
 

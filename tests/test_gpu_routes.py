@@ -85,3 +85,26 @@ def test_residual_norms_where_items_hold_few_points(J):
     st.pd_state_set_start(x0=xt)
     norms = np.sqrt(np.bincount(blk, weights=np.abs(want - y) ** 2, minlength=d))
     assert np.max(np.abs(st.report()["res_norm"] / norms - 1)) < 1e-5
+
+
+@pytest.mark.parametrize("n,tile,d", [(2048, 8, 256), (64, 8, 7), (64, 64, 1)])
+def test_order_of_the_points(n, tile, d):
+    """Plans whose (tile, block) pairs are too many for one counting pass (262,144 tiles, 256 blocks), and segments
+    with many and with few points to a cell: Phi, Phi^H and a checkpoint read back."""
+    from paper_1610_08895_gb300.api import Plan, State
+    m = 20011
+    uv = _uv("gaussian", m)
+    uv[:4000] = uv[:40].repeat(100, axis=0)                     # ties, which stay in the order they came in
+    blk = (np.arange(m) * 31 % d).astype(np.int32)
+    plan, other = Plan(n, n, uv, blk, d, tile=tile), Plan(n, n, uv, blk, d, tile=16)
+    x = torch.tensor(synth.random_images(1, n, n, seed=3)[0], dtype=torch.float32, device="cuda")
+    y = plan.pd_apply_phi(x)
+    assert rel(other.pd_apply_phi(x).cpu().numpy(), y.cpu().numpy()) < 2e-6
+    assert rel(other.pd_apply_phi_adj(y).cpu().numpy(), plan.pd_apply_phi_adj(y).cpu().numpy()) < 2e-6
+    st = State(plan)
+    st.pd_state_set_data(y, np.ones(d))
+    st.pd_state_set_start(v0=y)
+    buf = st.save()
+    st.pd_state_set_data(y, np.ones(d))
+    st.load(buf)
+    assert torch.equal(st.v(), y)
