@@ -761,7 +761,7 @@ extern "C" pd_status pd_state_create(pd_plan* p, pd_state** out) {
         st->diag = (double*)(st->t + 1);
         st->status = (int32_t*)(st->t + 3);
     }
-    st->ck_cap = std::min<int64_t>(p->M, 1 << 20);
+    st->ck_cap = std::min<int64_t>(p->M, 1 << 22);
     ok = ok && !dalloc_bytes(A, B, &st->ck_vis, st->ck_cap * p->csz) && !dalloc(A, B, &st->ck_idx, st->ck_cap);
     if (!ok) {
         pd_state_destroy(st);
