@@ -60,10 +60,12 @@ def test_a_batch_is_its_images_one_by_one(n, m, b, kw):
     for k in range(b):
         assert torch.equal(y[k], plan.pd_apply_phi(x[k].contiguous()))
         one = plan.pd_apply_phi_adj(v[k].contiguous())
-        if kw.get("kernel_width", 8) <= 8:
+        if "g_mode" in kw or kw.get("precision") == "f64":
             assert torch.equal(xa[k], one)
-        else:                                   # wider kernels add through shared-memory atomics
+        else:       # a batch's tiles may be shared out to other warps; J > 8 adds through shared-memory atomics
             assert rel(xa[k].cpu().numpy(), one.cpu().numpy()) < 2e-6
+    if kw.get("kernel_width", 8) <= 8:
+        assert torch.equal(xa, plan.pd_apply_phi_adj(v))
 
 
 @pytest.mark.parametrize("J", [8, 12])
