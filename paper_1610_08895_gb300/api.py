@@ -303,9 +303,10 @@ class State:
 
 
 def autotune_tile(nx, ny, uv, block_of_vis, nblocks, kernel_width=8, basis_ids=(0,), levels=1, precision="f32",
-                  candidates=(16, 32, 64), iters=5):
+                  candidates=None, iters=5):
     """pd_plan_autotune: time Algorithm 1 iterations with each candidate gridding tile
-    and return (best tile, {tile: ms per iteration})."""
+    and return (best tile, {tile: ms per iteration}). candidates: by default 16, 32 and 64, and 8 in
+    FP64, where it is the plan's own choice for grids up to 1024^2 cells."""
     B.load()
     uv = np.ascontiguousarray(uv, dtype=np.float64)
     blk = np.ascontiguousarray(block_of_vis, dtype=np.int32)
@@ -314,6 +315,8 @@ def autotune_tile(nx, ny, uv, block_of_vis, nblocks, kernel_width=8, basis_ids=(
     d = B.PdPlanDesc(nx=int(nx), ny=int(ny), osf=2, nvis=len(uv), uv=uv.ctypes.data, nblocks=int(nblocks),
                      block_of_vis=blk.ctypes.data, kernel_width=int(kernel_width), kb_beta=0.0, nbases=len(ids),
                      basis_ids=ids.ctypes.data, levels=int(levels), precision=prec, tile=0)
+    if candidates is None:
+        candidates = (8, 16, 32, 64) if prec == B.PD_F64 and int(kernel_width) <= 8 else (16, 32, 64)
     cand = np.ascontiguousarray(candidates, dtype=np.int32)
     ms = np.zeros(len(cand))
     best = ctypes.c_int32()

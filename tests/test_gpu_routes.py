@@ -110,3 +110,13 @@ def test_order_of_the_points(n, tile, d):
     st.pd_state_set_data(y, np.ones(d))
     st.load(buf)
     assert torch.equal(st.v(), y)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_autotuner_offers_the_tile_that_a_plan_would_choose(precision):
+    from paper_1610_08895_gb300.api import Plan, autotune_tile
+    n, m = 64, 3000
+    uv, blk = _uv("gaussian", m), np.zeros(m, np.int32)
+    best, times = autotune_tile(n, n, uv, blk, 1, precision=precision, iters=1)
+    assert Plan(n, n, uv, blk, 1, precision=precision).info()["tile"] in times
+    assert times[best] == min(t for t in times.values() if t > 0)
