@@ -171,3 +171,44 @@ def test_a_wait_of_the_ordered_adds_that_gives_up():
     a.pd_state_set_data(vt, np.ones(nb))
     a.pd_iterate(3, **kw)
     assert a.report()["t"] == 3 and torch.equal(a.x(), want_x)
+
+
+@pytest.mark.parametrize("precision,form", [("f32", dict()), ("f32", dict(use_graph=True)), ("f32", dict(per_block=True)),
+                                            ("f64", dict()), ("f64", dict(per_block=True))])
+def test_iterations_with_a_tile_that_is_split_into_parts(precision, form):
+    """9,001 points in one tile of 16 cells (three gridding and nine degridding parts) and 400 around it,
+    in blocks of which few are active: parts left without a point, shares that differ from the slots'
+    ranges, and neighbours that add to the same cells. Against the oracle, and twice the same bits."""
+    from gpu_util import TOL_IT32, TOL_IT64
+    from oracle import pd as PD
+    from paper_1610_08895_gb300.api import Plan, State
+    n, nb, J = 64, 11, 8
+    rng = np.random.default_rng(5)
+    g = np.concatenate([np.array([20.0, 36.0]) + rng.uniform(0.0, 12.0, size=(9001, 2)),      # one tile's cells
+                        np.array([10.0, 26.0]) + rng.uniform(0.0, 32.0, size=(400, 2))])
+    uv = g * (np.pi / n)
+    blk = np.sort(rng.integers(0, nb, size=len(uv))).astype(np.int32)
+    blk[9001:] = rng.integers(0, nb, size=400)
+    prob = PD.Problem(meas.Geometry(n, n, J), uv, blk, nb, [0, 1, 2], 2)
+    phix = prob.phi(synth.test_image(n, seed=2))
+    prob.y = phix + 0.05 * np.abs(phix).mean() * synth.complex_noise(len(uv), seed=3)
+    prob.eps = np.array([0.05 * np.abs(phix).mean() * np.sqrt(max(len(ix), 1)) for ix in prob.block_index])
+    kw = dict(tau=0.49, sigma=1.0, varsigma=1.0 / (9001 * n * n / 4.0), kappa=1e-3, psi_norm=1.0, seed=6,
+              p_block=[0.3] * nb, p_basis=[0.7] * 3)
+    ref, draws = PD.pd_run(prob, 12, **kw)
+    assert min(sum(d[0]) for d in draws) <= 2                                   # few active blocks at times
+    plan = Plan(n, n, uv, blk, nb, kernel_width=J, basis_ids=[0, 1, 2], levels=2, precision=precision, tile=16)
+    out = []
+    for _ in range(2):
+        st = State(plan)
+        st.pd_state_set_data(torch.tensor(prob.y, dtype=plan.cplx_dtype, device="cuda"), prob.eps)
+        st.pd_iterate(12, **kw, **form)
+        out.append((st.x(), st.s(), st.v()))
+        rep = st.report()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    tol = TOL_IT64 if precision == "f64" else TOL_IT32
+    assert rel(out[0][0].cpu().numpy(), ref.x) < tol and rel(out[0][2].cpu().numpy(), ref.v) < tol
+    # s holds small differences of much larger analysis coefficients, whose rounding is relative to them
+    scale = np.linalg.norm(prob.psi_adj(ref.x_tilde))
+    assert np.linalg.norm(out[0][1].cpu().numpy() - ref.s) < (TOL_IT64 if precision == "f64" else 1e-5) * scale
+    assert list(rep["block_active"]) == list(draws[-1][0])
