@@ -220,15 +220,17 @@ void kb_tap_polynomials_ext(int J, double beta, int deg, int outer, int edge_deg
     std::vector<ld> y(K + 1);
     ld pw = 1.0L, dropped = 0.0L;
     for (int k = 0; k <= K; ++k, pw *= s1) y[k] = c[k] * pw;
-    std::vector<std::vector<ld>> T(K + 1);     // T_k(2 y - 1) / 2^(2 k - 1): leading coefficient 1
+    // T_k(2 y - 1) / 2^(2 k - 1), leading coefficient 1; in FP64, since the terms they stand for are
+    // below 1e-4 of the value
+    std::vector<std::vector<double>> T(K + 1);
     for (int k = 0; k <= K; ++k) {
-        T[k].assign(k + 1, 0.0L);
-        if (k == 0) T[0][0] = 1.0L;
-        else if (k == 1) { T[1][0] = -0.5L; T[1][1] = 1.0L; }
+        T[k].assign(k + 1, 0.0);
+        if (k == 0) T[0][0] = 1.0;
+        else if (k == 1) { T[1][0] = -0.5; T[1][1] = 1.0; }
         else
             for (int i = 0; i <= k; ++i)       // T_k = (4 y - 2) T_{k-1} - T_{k-2}
-                T[k][i] = (i > 0 ? T[k - 1][i - 1] : 0.0L) - (i < k ? T[k - 1][i] / 2.0L : 0.0L) -
-                          (i < k - 1 ? T[k - 2][i] / (k == 2 ? 8.0L : 16.0L) : 0.0L);
+                T[k][i] = (i > 0 ? T[k - 1][i - 1] : 0.0) - (i < k ? T[k - 1][i] / 2.0 : 0.0) -
+                          (i < k - 1 ? T[k - 2][i] / (k == 2 ? 8.0 : 16.0) : 0.0);
     }
     for (int k = K; k > edge_deg; --k) {
         const ld top = y[k];
