@@ -238,7 +238,7 @@ static pd_status plan_build(pd_plan* p, const pd_plan_desc* d) {
     g.tile = T; g.logT = ilog2(T);
     g.ntx = g.Kx / T; g.nty = g.Ky / T; g.ntiles = g.ntx * g.nty;
     g.ext = T + g.J - 1;
-    // a fifth of an SM's share of the points (five CTAs per SM), at least four rounds of a CTA
+    // a fifth of an SM's share of the points, where four CTAs work at a time, and at least four rounds of one
     const int degrid_part = (int)std::max<int64_t>(1024, M / ((int64_t)p->num_sms * 5));
     PointOrder po = order_points(cell, d->block_of_vis, p->d, g.logT, g.ntx, g.ntiles);
     std::vector<int32_t>& order = po.order;

@@ -72,6 +72,15 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
+// Packed FP32 add, one instruction.
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+    return d;
+}
+
 // Deterministic block-wide sum of a double for any blockDim.x that is a multiple
 // of 32 (fixed shuffle tree per warp, then warp 0). sh must hold 32 doubles.
 // The result is valid in thread 0.

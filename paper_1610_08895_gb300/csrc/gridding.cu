@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // truncates its sums: left at that, Phi^H was up to 8% further from 64-bit arithmetic at J = 6 than
 // with chains of FP32 multiply-adds (1.58e-7 -> 1.70e-7, 512^2 image), so the leading products go
 // through it twice and what the first sum lost is added with the smaller products (1.53e-7; J = 4, 6
-// and 8: 3% to 24% below the chains; 3.5-4% of the time of Phi^H).
+// and 8: 3% to 24% below the chains; 16.8M points on 4096^2 cells, half of them active: 390 -> 407 us).
 // A CTA works on one part of a tile at a time. The part's points, super-cell by super-cell
 // (each padded to a multiple of 16), are cut into chunks of 32 that are shared out evenly
 // among the CTA's working warps; at the end of a super-cell (or of its share) a warp stores
@@ -649,10 +649,9 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // contiguous in U), while they work on the next.
 // What bounds it: instruction issue (about 30 warp instructions a point, 12 of them in the
 // contraction; the split's logic operations share the half-rate ALU pipe) with 16 warps per
-// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 356 us, against 462 us
-// for the FP32 FMA kernel below it in four launches (same windows); 65,536 points on 512^2,
-// where the densest tile was the critical path of each launch: 28 against 154 us; 1.05M on
-// 1024^2: 38 against 233 us. Slower there: 2048-point parts (459 us), 3 or 15 working warps
+// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 407 us, against 478 us
+// for FP32 FMA kernels in four launches; 65,536 points on 512^2, where the densest tile was the
+// critical path of each launch: 29 against 164 us; 1.05M on 1024^2: 56 against 296 us. Slower there: 2048-point parts (459 us), 3 or 15 working warps
 // (442, 448 us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the
 // tiles' weight instead of their colour (3.3 ms: chains of neighbours).
 // Staging (one lane per point) writes the taps by class (patch row / column mod 8),
@@ -758,9 +757,11 @@ __device__ __forceinline__ void grid_mma_group(const float* __restrict__ st, int
             float m[4] = {0.f, 0.f, 0.f, 0.f}, d[4], t[4];
             mma_bf16(m, A[0], b0[0], b1[0]);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                t[e] = ac[e] + m[e];
-                d[e] = ac[e] - t[e];
+            for (int e = 0; e < 4; e += 2) {
+                const float2 a2 = make_float2(ac[e], ac[e + 1]);
+                const float2 t2 = fadd2(a2, make_float2(m[e], m[e + 1]));
+                const float2 d2 = ffma2(t2, make_float2(-1.f, -1.f), a2);
+                t[e] = t2.x; t[e + 1] = t2.y; d[e] = d2.x; d[e + 1] = d2.y;
             }
             mma_bf16(d, A[0], b0[0], b1[0]);
             mma_bf16(d, A[2], b0[0], b1[0]);
@@ -769,7 +770,10 @@ __device__ __forceinline__ void grid_mma_group(const float* __restrict__ st, int
             mma_bf16(d, A[1], b0[0], b1[0]);
             mma_bf16(d, A[0], b0[1], b1[1]);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) ac[e] = t[e] + d[e];
+            for (int e = 0; e < 4; e += 2) {
+                const float2 s2 = fadd2(make_float2(t[e], t[e + 1]), make_float2(d[e], d[e + 1]));
+                ac[e] = s2.x; ac[e + 1] = s2.y;
+            }
         }
     }
 }

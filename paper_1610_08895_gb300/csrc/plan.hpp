@@ -124,7 +124,7 @@ struct pd_plan {
     int32_t* cell = nullptr;       // (by << 16) | bx of the footprint's first cell, mod K
     void* fx = nullptr;            // real [M]: fractional part of g_x
     void* fy = nullptr;
-    int32_t* perm = nullptr;       // internal -> user index; sign bit set: held as its conjugate (see vis_user)
+    int32_t* perm = nullptr;       // internal -> user index; sign bit set: held as its conjugate (see vis_conj)
     int g_mode = PD_G_ON_THE_FLY;  // PD_G_CSR: G stored explicitly, below
     int kb_J = 0;                  // interpolation kernel width (g.J is the footprint: kb_J + dde - 1)
     int dde = 0;                   // DDE kernel width d (0: none)
