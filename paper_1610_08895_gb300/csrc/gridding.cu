@@ -630,15 +630,14 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // The window of one super-cell (8 x 8 footprint origins) is a 16 x 16 patch, and gridding
 // its points is a contraction over them: patch[r][c] = sum_m wy_m[r] (d_m wx_m[c]). A warp
 // runs it on the tensor cores: M = 16 patch rows, N = 2 x 16 patch columns (re, im), K = 16
-// points. Every FP32 operand is split exactly into three bf16 values (8 + 8 + 8 significant
-// bits), and the six products down to 2^-16 of the leading one are accumulated. What is dropped has
-// an rms of 1.4e-8 of the product (1.0e-7 at most, over 4M random pairs), the rounding of an FP32
-// product 2.5e-8 (6.0e-8 at most); keeping two products more took 5% of the kernel's time and less
-// than 1% off the error of Phi^H. The sum of 16 points is added to FP32 registers. The tensor core
+// points. Every FP32 operand is split exactly into three bf16 values, each rounded to nearest (8 + 8 + 8
+// significant bits), and the six products down to 2^-16 of the leading one are accumulated. What is
+// dropped has an rms of 5.7e-9 of the product and 5.3e-8 at most (4M random pairs), the rounding of an
+// FP32 product 2.5e-8 and 6.0e-8 (a truncated middle part: 1.4e-8 and 1.0e-7). The sum of 16 points is added to FP32 registers. The tensor core
 // truncates its sums: left at that, Phi^H was up to 8% further from 64-bit arithmetic at J = 6 than
 // with chains of FP32 multiply-adds (1.58e-7 -> 1.70e-7, 512^2 image), so the leading products go
 // through it twice and what the first sum lost is added with the smaller products (1.53e-7; J = 4, 6
-// and 8: 3% to 24% below the chains; 16.8M points on 4096^2 cells, half of them active: 390 -> 407 us).
+// and 8: 3% to 25% below the chains; 16.8M points on 4096^2 cells, half of them active: 390 -> 400 us).
 // A CTA works on one part of a tile at a time. The part's points, super-cell by super-cell
 // (each padded to a multiple of 16), are cut into chunks of 32 that are shared out evenly
 // among the CTA's working warps; at the end of a super-cell (or of its share) a warp stores
@@ -649,7 +648,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // contiguous in U), while they work on the next.
 // What bounds it: instruction issue (about 30 warp instructions a point, 12 of them in the
 // contraction; the split's logic operations share the half-rate ALU pipe) with 16 warps per
-// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 407 us, against 478 us
+// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 400 us, against 478 us
 // for FP32 FMA kernels in four launches; 65,536 points on 512^2, where the densest tile was the
 // critical path of each launch: 29 against 164 us; 1.05M on 1024^2: 56 against 296 us. Slower there: 2048-point parts (459 us), 3 or 15 working warps
 // (442, 448 us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the
@@ -694,18 +693,23 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// x = s0 + s1 + s2, each part with its low 16 bits zero: exact in bf16. s0 is rounded to
-// nearest, so that the parts' signs differ and the dropped products have no bias (truncated
-// parts measured twice the error of the sum of 16 products: 9.1e-8 against 4.9e-8, and a
-// chain of FP32 multiply-adds 7.3e-8).
-__device__ __forceinline__ void split3(float x, uint32_t* s) {
-    s[0] = (__float_as_uint(x) + 0x8000u) & 0xffff0000u;
-    const float r = x - __uint_as_float(s[0]);
-    s[1] = __float_as_uint(r) & 0xffff0000u;
-    s[2] = __float_as_uint(r - __uint_as_float(s[1]));
+// x = s0 + s1 + s2 for two values at a time, each part rounded to nearest to bf16 (8 bits; the last one
+// exactly), a in the low and b in the high half: the parts' signs differ, so that the dropped
+// products have no bias.
+__device__ __forceinline__ uint32_t bf16_pair(float2 v) {
+    uint32_t p;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p) : "f"(v.y), "f"(v.x));
+    return p;
 }
-// the upper halves of a (low) and b (high)
-__device__ __forceinline__ uint32_t pack_hi(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+__device__ __forceinline__ void split3(float a, float b, uint32_t* s) {
+    float2 r = make_float2(a, b);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        s[i] = bf16_pair(r);
+        if (i < 2) r = ffma2(make_float2(__uint_as_float(s[i] << 16), __uint_as_float(s[i] & 0xffff0000u)),
+                             make_float2(-1.f, -1.f), r);
+    }
+}
 // 0xffff in the half of each negative operand
 __device__ __forceinline__ uint32_t sign_mask(float a, float b) {
     uint32_t m;
@@ -725,23 +729,21 @@ __device__ __forceinline__ void grid_mma_group(const float* __restrict__ st, int
     uint32_t A[3][4];
     {
         const uint32_t m0 = sign_mask(wy.x, wy.y), m1 = sign_mask(wy.z, wy.w);
-        uint32_t s[4][3];
-        split3(fabsf(wy.x), s[0]); split3(fabsf(wy.y), s[1]); split3(fabsf(wy.z), s[2]); split3(fabsf(wy.w), s[3]);
+        uint32_t u[3], v[3];
+        split3(fabsf(wy.x), fabsf(wy.y), u);
+        split3(fabsf(wy.z), fabsf(wy.w), v);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const uint32_t u = pack_hi(s[0][i], s[1][i]), v = pack_hi(s[2][i], s[3][i]);
-            A[i][0] = u & ~m0; A[i][1] = u & m0; A[i][2] = v & ~m1; A[i][3] = v & m1;
+            A[i][0] = u[i] & ~m0; A[i][1] = u[i] & m0; A[i][2] = v[i] & ~m1; A[i][3] = v[i] & m1;
         }
     }
     const uint32_t m0 = sign_mask(wx.x, wx.y), m1 = sign_mask(wx.z, wx.w);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {                       // real, imaginary part
         const float4 dv = h ? di : dr;
-        uint32_t s[4][3], u[3], v[3];
-        split3(fabsf(wx.x) * dv.x, s[0]); split3(fabsf(wx.y) * dv.y, s[1]);
-        split3(fabsf(wx.z) * dv.z, s[2]); split3(fabsf(wx.w) * dv.w, s[3]);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) { u[i] = pack_hi(s[0][i], s[1][i]); v[i] = pack_hi(s[2][i], s[3][i]); }
+        uint32_t u[3], v[3];
+        split3(fabsf(wx.x) * dv.x, fabsf(wx.y) * dv.y, u);
+        split3(fabsf(wx.z) * dv.z, fabsf(wx.w) * dv.w, v);
 #pragma unroll
         for (int hi = 0; hi < 2; ++hi) {                // low, high half of the patch columns
             uint32_t b0[3], b1[3];
