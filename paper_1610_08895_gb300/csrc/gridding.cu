@@ -630,14 +630,15 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // The window of one super-cell (8 x 8 footprint origins) is a 16 x 16 patch, and gridding
 // its points is a contraction over them: patch[r][c] = sum_m wy_m[r] (d_m wx_m[c]). A warp
 // runs it on the tensor cores: M = 16 patch rows, N = 2 x 16 patch columns (re, im), K = 16
-// points. Every FP32 operand is split exactly into three bf16 values, each rounded to nearest (8 + 8 + 8
-// significant bits), and the six products down to 2^-16 of the leading one are accumulated. What is
-// dropped has an rms of 5.7e-9 of the product and 5.3e-8 at most (4M random pairs), the rounding of an
-// FP32 product 2.5e-8 and 6.0e-8 (a truncated middle part: 1.4e-8 and 1.0e-7). The sum of 16 points is added to FP32 registers. The tensor core
-// truncates its sums: left at that, Phi^H was up to 8% further from 64-bit arithmetic at J = 6 than
-// with chains of FP32 multiply-adds (1.58e-7 -> 1.70e-7, 512^2 image), so the leading products go
-// through it twice and what the first sum lost is added with the smaller products (1.53e-7; J = 4, 6
-// and 8: 3% to 25% below the chains; 16.8M points on 4096^2 cells, half of them active: 390 -> 400 us).
+// points. Every FP32 operand is split exactly into three bf16 values, each rounded to nearest
+// (8 + 8 + 8 significant bits), and the six products down to 2^-16 of the leading one are
+// accumulated. What is dropped has an rms of 5.7e-9 of the product and 5.3e-8 at most (4M random
+// pairs), the rounding of an FP32 product 2.5e-8 and 6.0e-8. The sum of 16 points is added to
+// FP32 registers. The tensor core truncates its sums: left at that, Phi^H was up to 8% further
+// from 64-bit arithmetic at J = 6 than with chains of FP32 multiply-adds (512^2 image: 1.58e-7 ->
+// 1.70e-7), so the leading products go through it twice and what the first sum lost is added with
+// the smaller products (1.53e-7; J = 4, 6 and 8: 3% to 25% below the chains; 16.8M points on 4096^2
+// cells, half of them active: 390 -> 400 us).
 // A CTA works on one part of a tile at a time. The part's points, super-cell by super-cell
 // (each padded to a multiple of 16), are cut into chunks of 32 that are shared out evenly
 // among the CTA's working warps; at the end of a super-cell (or of its share) a warp stores
@@ -646,13 +647,15 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // the next item and lists its points while they work on the current one, and it adds the
 // finished window to U with bulk reductions, one per column panel (rows of a panel are
 // contiguous in U), while they work on the next.
-// What bounds it: instruction issue (about 30 warp instructions a point, 12 of them in the
-// contraction; the split's logic operations share the half-rate ALU pipe) with 16 warps per
-// SM by registers. 16.8M points, half of them active, on a 4096^2 grid: 400 us, against 478 us
-// for FP32 FMA kernels in four launches; 65,536 points on 512^2, where the densest tile was the
-// critical path of each launch: 29 against 164 us; 1.05M on 1024^2: 56 against 296 us. Slower there: 2048-point parts (459 us), 3 or 15 working warps
-// (442, 448 us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the
-// tiles' weight instead of their colour (3.3 ms: chains of neighbours).
+// What bounds it: instruction issue and the barriers between the phases of an item (about 30 warp
+// instructions a point, half of them in the contraction) with 16 warps per SM by registers. 16.8M
+// points, half of them active, on a 4096^2 grid: 400 us, against 478 us for FP32 multiply-adds in
+// four launches; 65,536 points on 512^2, where the densest tile was the critical path of each launch:
+// 30 against 164 us; 1.05M on 1024^2: 56 against 296 us. A batch of dense images is the exception:
+// eight of 1024^2 with 4.19M points each, Phi^H 2.10 ms, in four launches 1.73. Slower (timed on an
+// earlier form, 360 us at 16.8M points): 2048-point parts (459 us), 3 or 15 working warps (442, 448
+// us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the tiles' weight
+// instead of their colour (3.3 ms: chains of neighbours).
 // Staging (one lane per point) writes the taps by class (patch row / column mod 8),
 // negated when the tap falls in the upper half of the patch: 18 floats a point, each read
 // once, by the lane whose fragment needs it.
