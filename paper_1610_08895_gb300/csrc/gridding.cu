@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(GW_MAXW * 32) k_grid8w(
 // points, half of them active, on a 4096^2 grid: 400 us, against 478 us for FP32 multiply-adds in
 // four launches; 65,536 points on 512^2, where the densest tile was the critical path of each launch:
 // 30 against 164 us; 1.05M on 1024^2: 56 against 296 us. A batch of dense images is the exception:
-// eight of 1024^2 with 4.19M points each, Phi^H 2.10 ms, in four launches 1.73. Slower (timed on an
+// eight of 1024^2 with 4.19M points each, Phi^H 1.92 ms, in four launches 1.73. Slower (timed on an
 // earlier form, 360 us at 16.8M points): 2048-point parts (459 us), 3 or 15 working warps (442, 448
 // us), 80 or 96 registers for more warps (496, 410 us), waits in the order of the tiles' weight
 // instead of their colour (3.3 ms: chains of neighbours).
@@ -856,7 +856,7 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
     const float* __restrict__ fxs, const float* __restrict__ fys, const int32_t* __restrict__ perm,
     const int32_t* __restrict__ seg_block, const int32_t* __restrict__ sc_start, const int4* __restrict__ tile_info, const int32_t* __restrict__ tile_on,
     const int2* __restrict__ items, const int32_t* __restrict__ nitems, int32_t* pend, float2* U, int max_segs, Geo g,
-    const KbPoly kp, int* sched, int32_t* gave_up, int polls, int batch, int group, int64_t istride, int64_t ustride) {
+    const KbPoly kp, int* sched, int32_t* gave_up, int polls, int batch, int64_t istride, int64_t ustride) {
     static_assert(J <= 8 && J % 2 == 0, "a super-cell's window is 16 x 16 for J <= 8");
     extern __shared__ __align__(16) unsigned char smraw[];
     const int T = g.tile, nsd = T >> 3, nsc = nsd * nsd, W = T + 8;
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
         int* act_seg = reinterpret_cast<int*>(lbase + 2 * lsz);
         const int nlist = *nitems, nitem = nlist * batch;
         // claims the next item with an active block (items are claimed in order by whichever CTA is
-        // free, a batch group by group of images, each group item by item) and lists it in buffer b
+        // free, all images of a batch before the next item) and lists it in buffer b
         auto prepare = [&](int b) -> bool {
             const GridLists L(lbase + b * lsz, nsc, max_segs);
             int w, img;
@@ -888,9 +888,8 @@ __global__ void __launch_bounds__(GM_MAXW * 32) k_grid_mma(
                     if (lane == 0) item_s[b].tile = -1;
                     return false;
                 }
-                const int gi = w / (nlist * group), r = w - gi * nlist * group, gs = min(group, batch - gi * group);
-                it = items[r / gs];
-                img = gi * group + r % gs;
+                it = items[w / batch];
+                img = w % batch;
                 ti = tile_info[it.x];
                 if (!tile_on || tile_on[it.x]) break;
             }
@@ -1271,12 +1270,14 @@ static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const Du
                                    int32_t* gave_up, cudaStream_t s, int batch) {
     const Geo& g = p->g;
     cudaError_t e;
-    // A batch of items with few points is held up by the feeding warps, one chain of loads and adds an
-    // item: three working warps then, and twice the CTAs (64 images of 256^2, 65,536 points: Phi^H 734
-    // us with seven, 590 / 517 / 556 with four / three / two; eight of 512^2, 100,001 points: 320, 256 / 222
-    // / 231; eight of 512^2, 1.05M points, 630 an item: 568, 514 / 497 / 596). Not for one image, whose
-    // items are one or two a CTA, nor where they hold many more points
-    // (eight of 1024^2, 4.19M points, 2300 an item: 2105, 2192 / 2728 / 3624).
+    // A batch goes item by item, all images of each: image by image, overlapping tiles of one image wait
+    // for one another with nothing else to do meanwhile (64 images of 256^2, 65,536 points: Phi^H 997
+    // us, so 734; eight of 1024^2, 4.19M points: 2119, 1920).
+    // Items with few points are held up by the feeding warps, one chain of loads and adds an item:
+    // three working warps then, and twice the CTAs (the 64 images: 734 us with seven, 590 / 517 / 556
+    // with four / three / two; eight of 512^2, 100,001 points: 320, 256 / 222 / 231, with 1.05M, 630 an
+    // item: 568, 514 / 497 / 596). Not for one image, whose items are one or two a CTA, nor where they
+    // hold many more points (the eight of 1024^2, 2300 an item: 2105, 2192 / 2728 / 3624 image by image).
     const bool few = batch > 1 && p->M <= (int64_t)p->n_items * 800 && (int64_t)p->n_items * batch >= (int64_t)p->num_sms * 8;
     const int warps = few ? 4 : p->grid_warps;
     const size_t smem = few ? grid_mma_smem(g.tile, warps - 1, std::max(p->max_tile_segs, 1)) : p->grid_smem;
@@ -1284,18 +1285,13 @@ static cudaError_t launch_grid_mma(const pd_plan* p, const float2* src, const Du
     int per_sm = 1;
     if ((e = occupancy(&per_sm, k_grid_mma<J, MODE>, warps * 32, smem))) return e;
     const int ctas = (int)std::min<int64_t>((int64_t)p->n_items * batch, (int64_t)std::max(per_sm, 1) * p->num_sms);
-    // Overlapping tiles of one image wait for one another, colour by colour, and an image of few items
-    // leaves nothing else to do meanwhile: a batch goes through its items in groups of images, as many
-    // as have their visibilities (read at random) in the L2 cache together (64 images of 256^2, 65,536
-    // points: Phi^H 997 us image by image, 736 so).
-    const int group = (int)std::max<int64_t>(1, std::min<int64_t>(batch, ((int64_t)48 << 20) / (p->M * (int64_t)sizeof(float2))));
     if (p->test_hold) k_hold<<<1, 1, 0, s>>>(a ? a->items : p->items, a ? a->nitems : p->nitems, pend);
     k_grid_mma<J, MODE><<<ctas, warps * 32, smem, s>>>(
         src, (const float2*)p->rbuf, a ? (float2*)a->v : nullptr, (const float*)p->blk_scale,
         a ? a->block_active : nullptr, p->cell, (const float*)p->fx, (const float*)p->fy, p->perm,
         p->seg_block, p->seg_sc_start, p->tile_info, a ? a->tile_on : nullptr, a ? a->items : p->items,
         a ? a->nitems : p->nitems, pend, U, std::max(p->max_tile_segs, 1), g, p->kbpoly, p->sched + 8, gave_up,
-        p->wait_polls, batch, group, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
+        p->wait_polls, batch, (int64_t)p->M, (int64_t)g.Kx * g.Ky);
     return cudaGetLastError();
 }
 
